@@ -310,7 +310,8 @@ __global__ void k_l2l(const uint32_t *d_nc, const uint32_t *cparent, const uint6
 // in shared memory in K-chunks and multiplied as a small GEMM (rows = output coefficients,
 // columns = target boxes); each target's partial local expansion of the slice is written to
 // its own slot [box][slot] and the slots are summed in a fixed order (k_m2l_reduce), so the
-// result does not depend on scheduling.  (FP64 mode and p > 10; the mixed mode uses k_m2l_tc.)
+// result does not depend on scheduling.  (Mixed mode with p > 11; k_m2l_f32 serves p = 11, k_m2l_tc
+// p <= 10, and the FP64 mode runs the operator-sorted lists of m2l_pairs.cuh.)
 // ---------------------------------------------------------------------------------------
 constexpr int M2L_KC = 32;
 constexpr int M2L_NSLICE = NSLICE;  // offsets with dx = -OFF_R..OFF_R, SLICE_OFFS each
@@ -1303,6 +1304,8 @@ __global__ void __launch_bounds__(P2P_THREADS) k_p2p_react(
   }
 }
 
+#include "m2l_pairs.cuh"
+
 // ---------------------------------------------------------------------------------------
 // driver for one group
 // ---------------------------------------------------------------------------------------
@@ -1919,20 +1922,63 @@ static void upward_t(Ctx &c, Group &g, int parts) {
   }
 }
 
-// every multipole-to-local translation of every group and level in one launch
-template <typename T>
-static void m2l_all_t(Ctx &c, std::vector<Group> &groups) {
-  constexpr int TPT = sizeof(T) == 4 ? 4 : 2;
-  constexpr int TT = 16 * TPT;
-  const Tables &tb = sizeof(T) == 8 ? g_tab_d[c.device] : g_tab_f[c.device];
+// FP64: every multipole-to-local translation of every group and level, sorted by operator
+static void m2l_all_f64(Ctx &c, std::vector<Group> &groups) {
+  const Tables &tb = g_tab_d[c.device];
+  std::vector<PairJob> jobs;
+  std::vector<int> ncls;
+  for (int kind = 0; kind < 2; ++kind)  // free-space jobs, then reaction jobs
+    for (auto &g : groups) {
+      const bool react_far = (g.parts & 2) && g.I.np > 0 && !(g.parts & 8);
+      for (int l = 2; l <= g.D; ++l) {
+        const int64_t ntb = g.T.lev[l].n;
+        if (!ntb) continue;
+        PairJob j;
+        j.L = (double2 *)g.Lt[l];
+        j.ntb = (int32_t)ntb;
+        j.t0 = 0;
+        j.bin0 = 0;
+        if (kind == 0 && g.is_free && (g.parts & 1) && l <= g.Df) {
+          j.vlist = g.vfree[l]; j.cls = tb.cls_free; j.ktrow = nullptr; j.tmask = nullptr;
+          j.M = (const double2 *)g.Mfree[l]; j.ops = (const double *)g.op_free[l];
+          j.ntypes = 1; j.nkt = 0;
+          jobs.push_back(j);
+          ncls.push_back(NFREE_CLS);
+        }
+        if (kind == 1 && react_far && g.vreact[l]) {
+          const int64_t nib = g.I.lev[l].n, rows = nib * g.ntypes;
+          uint32_t *tmask = c.arena.get<uint32_t>((size_t)nib);
+          LPB_CUDA(cudaMemsetAsync(tmask, 0, sizeof(uint32_t) * nib, c.stream));
+          k_pair_types<<<(unsigned)((rows + 7) / 8), 256, 0, c.stream>>>((const double2 *)g.Mimg[l], rows, c.K,
+                                                                         g.ntypes, tmask);
+          LPB_LAUNCH();
+          c.launches++;
+          j.vlist = g.vreact[l]; j.cls = tb.cls_react + (size_t)(g.a - 1) * NKT * NOFF; j.ktrow = g.ktrow[l];
+          j.tmask = tmask; j.M = (const double2 *)g.Mimg[l]; j.ops = (const double *)g.op_react[l];
+          j.ntypes = g.ntypes; j.nkt = 2 * c.ws + 1;
+          jobs.push_back(j);
+          ncls.push_back(NREACT_CLS);
+        }
+      }
+    }
+  if (jobs.empty()) return;
+  prof_mark(c, "m2l_prep");
+  launch_pair_m2l(c, jobs, ncls, (const double *)tb.rot);
+}
+
+// mixed mode: every multipole-to-local translation of every group and level in one launch
+static void m2l_all_f32(Ctx &c, std::vector<Group> &groups) {
+  typedef float T;
+  constexpr int TPT = 4, TT = 16 * TPT;
+  const Tables &tb = g_tab_f[c.device];
   std::vector<XJob> jobs;
   int64_t items = 0;
-  typedef typename C2<T>::t T2;
+  typedef C2<T>::t T2;
   std::vector<RJob> rjobs;
   int64_t relem = 0;
   // tensor-core free-space path: mixed precision, 2K - (p+1) <= 128 real coordinates
   const int tc_nc = (2 * c.K - (c.p + 1) + 31) / 32;
-  const bool use_tc = sizeof(T) == 4 && tc_nc <= 4;  // p <= 10
+  const bool use_tc = tc_nc <= 4;  // p <= 10
   std::vector<TJob> tjobs;
   int64_t titems = 0;
   auto add = [&](const int32_t *tlist, const uint32_t *d_ntl, int64_t ntb, const int32_t *vlist,
@@ -2064,7 +2110,7 @@ static void m2l_all_t(Ctx &c, std::vector<Group> &groups) {
     launch_reduce();
     return;
   }
-  if (sizeof(T) == 4 && c.K <= F32_KR) {
+  if (c.K <= F32_KR) {
     // re-count items with the larger tile of the asynchronous FP32 kernel
     int64_t it = 0;
     for (auto &j : jobs) {
@@ -2082,8 +2128,7 @@ static void m2l_all_t(Ctx &c, std::vector<Group> &groups) {
     launch_reduce();
     return;
   }
-  if (c.K <= 80) launch_m2l_t<T, TPT, 5>(c, jobs, items);
-  else if (c.K <= 128) launch_m2l_t<T, TPT, 8>(c, jobs, items);
+  if (c.K <= 128) launch_m2l_t<T, TPT, 8>(c, jobs, items);
   else launch_m2l_t<T, TPT, 10>(c, jobs, items);
   launch_reduce();
 }
@@ -2149,7 +2194,7 @@ void run_fmm_front(Ctx &c, std::vector<Group> &groups) {
   prof_mark(c, "upward");
   // the reaction tables and operators (side stream) are complete before any M2L
   if (c.ev_join) LPB_CUDA(cudaStreamWaitEvent(c.stream, c.ev_join, 0));
-  d ? m2l_all_t<double>(c, groups) : m2l_all_t<float>(c, groups);
+  d ? m2l_all_f64(c, groups) : m2l_all_f32(c, groups);
   prof_mark(c, "m2l");
 }
 
