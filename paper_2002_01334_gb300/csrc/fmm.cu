@@ -8,6 +8,8 @@
 #include "tc.cuh"
 
 #include <algorithm>
+#include <cmath>
+#include <cstring>
 #include <mutex>
 
 namespace lpb {
@@ -796,154 +798,158 @@ __global__ void k_l2p(const uint32_t *d_nb, const uint64_t *bkey, const uint32_t
 }
 
 // ---------------------------------------------------------------------------------------
-// free-space P2P over the near list (27 neighbours incl. the box itself).  One CTA of
-// P2P_TPB threads per target leaf; the sources of all neighbours are streamed through shared
-// memory in full tiles of P2P_SRC (position, charge) records; a thread holds up to two targets
-// (t and t + P2P_TPB), chosen per warp, so each shared-memory record read serves two pairs.
-// Pair math in T, per-tile partial sums in T, per-target accumulation in FP64.  The self pair
-// (r = 0) is dropped by a select, so distinct charges at one point do not interact either.
+// free-space P2P over the near list (the boxes within the separation, incl. the box itself).  A
+// pair of zero distance (the charge itself, or another at the same point) contributes nothing.
 // ---------------------------------------------------------------------------------------
 constexpr int P2P_THREADS = 128;  // reaction near field
-constexpr int P2P_TPB = 64, P2P_SRC = 128;
 
 __device__ __forceinline__ float fexp(float x) { return __expf(x); }
 __device__ __forceinline__ double fexp(double x) { return exp(x); }
-__device__ __forceinline__ float frsqrt(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double frsqrt(double x) { return rsqrt(x); }
 
-template <typename T>
-struct alignas(4 * sizeof(T)) V4 {
-  T x, y, z, w;
+// FP64 near field: one CTA of P64_WARPS warps per leaf, every group of the evaluation in one launch.
+// Bound: the FP64 pipe (half an FMA per clock and SM quarter), so the kernel minimises FP64
+// operations per pair and idle lanes and leaves everything else to the other pipes:
+//  * 28 FP64 operations per pair (21 without the field): 1/r from the special-function unit's
+//    approximation by one third-order step (5 operations), e^{-lambda r} by the table method (Tang,
+//    ACM TOMS 15, 1989: 2^(n/2048) from a table, a cubic for the remainder below 2^-12; 7 operations).
+//    The library's rsqrt and exp take about 45 in all.
+//  * no idle lanes in a leaf's last, partial group of targets: a group of 2^b targets gives each of
+//    them 32 / 2^b lanes, which split the sources; cnt targets take the full groups of 32 and one
+//    group per set bit of the rest.  The warps of the CTA split the sources once more.
+//  * coordinates are read as they are (no shared-memory tiles: a pair's 32 bytes cost nothing beside
+//    its FP64 time) and differences of them are the exact inputs of r.
+// Sums: per lane over its sources, then over the lanes and warps of a target in a fixed order.
+constexpr int P64_WARPS = 8;
+constexpr int EXP_TAB_BITS = 11, EXP_TAB = 1 << EXP_TAB_BITS;
+__device__ double g_exp2_tab[EXP_TAB];  // 2^(j / EXP_TAB)
+
+void upload_exp2(cudaStream_t s) {
+  static double h[EXP_TAB];
+  for (int j = 0; j < EXP_TAB; ++j) h[j] = (double)exp2l((long double)j / EXP_TAB);
+  LPB_CUDA(cudaMemcpyToSymbolAsync(g_exp2_tab, h, sizeof h, 0, cudaMemcpyHostToDevice, s));
+}
+
+struct P64Job {
+  const uint32_t *bstart, *bcount;  // leaf point ranges
+  const int32_t *ulist;             // [nb][NNEAR] near leaves or -1
+  const double *x, *y, *z, *q;      // sorted points
+  const uint32_t *src;              // input index of each point
+  double lam, scale, ce;            // screening; 1 / (4 pi eps); -lambda log2(e) EXP_TAB
+  uint32_t hi_max;                  // high word of the largest r^2 that counts: lambda r <= 700
+  uint32_t nb;
+  int64_t block0;
 };
 
-template <typename T, int NT, bool COMP>
-__device__ __forceinline__ void p2p_free_tile(const V4<T> *__restrict__ sh, const V4<T> *__restrict__ sl, int nn,
-                                              const T (&px)[2], const T (&py)[2], const T (&pz)[2],
-                                              const T (&qx)[2], const T (&qy)[2], const T (&qz)[2], T lam,
-                                              T (&fp)[2], T (&fx)[2], T (&fy)[2], T (&fz)[2]) {
-#pragma unroll 2
-  for (int j = 0; j < nn; ++j) {
-    const V4<T> s = sh[j];
-    V4<T> sL;
-    if (COMP) sL = sl[j];
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      T dx = px[t] - s.x, dy = py[t] - s.y, dz = pz[t] - s.z;
-      if (COMP) {
-        dx += qx[t] - sL.x;
-        dy += qy[t] - sL.y;
-        dz += qz[t] - sL.z;
-      }
-      const T r2 = dx * dx + dy * dy + dz * dz;
-      const T ri = r2 > T(0) ? frsqrt(r2) : T(0);
-      const T r = r2 * ri;
-      const T e = s.w * fexp(-lam * r) * ri;
-      fp[t] += e;
-      const T f = e * (ri * ri) * (T(1) + lam * r);
-      fx[t] += f * dx;
-      fy[t] += f * dy;
-      fz[t] += f * dz;
-    }
+template <bool FIELD>
+__device__ __forceinline__ void p64_pair(double dx, double dy, double dz, double q, double lam, double ce,
+                                         uint32_t hi_max, double &p, double &fx, double &fy, double &fz) {
+  const double r2 = fma(dz, dz, fma(dy, dy, dx * dx));
+  double y0;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(r2));
+  // normal r^2 up to the cut (beyond it e^{-lambda r} < 1e-304); else 1/r = 0 and the pair drops out
+  const uint32_t hi = (uint32_t)__double2hiint(r2) - 0x00100000u;
+  y0 = hi <= hi_max ? y0 : 0.0;
+  const double e = fma(-(r2 * y0), y0, 1.0);
+  const double ri = fma(y0 * e, fma(0.375, e, 0.5), y0);
+  const double r = r2 * ri;
+  const double magic = 6755399441055744.0;  // 1.5 * 2^52: the sum's low word is the rounded integer
+  const double kd = fma(r, ce, magic);
+  const int n = __double2loint(kd);
+  const double f = fma(r, ce, magic - kd);
+  constexpr double u = 0.693147180559945309417 / EXP_TAB;
+  const double pm = f * fma(f, fma(f, u * u * u / 6.0, u * u / 2.0), u);
+  const double t0 = g_exp2_tab[n & (EXP_TAB - 1)];
+  const double t = __hiloint2double(__double2hiint(t0) + ((n >> EXP_TAB_BITS) << 20), __double2loint(t0));
+  const double w = fma(t, pm, t) * ri;
+  p = fma(q, w, p);
+  if (FIELD) {
+    const double g = (q * w) * (ri * (ri + lam));
+    fx = fma(g, dx, fx);
+    fy = fma(g, dy, fy);
+    fz = fma(g, dz, fz);
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(P2P_TPB) k_p2p_free(const uint32_t *d_nb, const uint64_t *bkey,
-                                                      const uint32_t *bstart, const uint32_t *bcount,
-                                                      const int32_t *ulist, const double *x, const double *y,
-                                                      const double *z, const double *q, const uint32_t *src,
-                                                      Geo geo, double lam, double scale, double *phi,
-                                                      double *field) {
-  constexpr bool comp = sizeof(T) == 4;
-  __shared__ V4<T> sh[P2P_SRC], sl[comp ? P2P_SRC : 1];
-  __shared__ uint32_t nb_start[NNEAR], nb_pre[NNEAR + 1];
-  const uint32_t box = blockIdx.x;
-  if (box >= *d_nb) return;
-  double cx, cy, cz;
-  box_center(bkey[box], geo, cx, cy, cz);
-  if (threadIdx.x == 0) {
-    uint32_t acc = 0;
-    for (int o = 0; o < NNEAR; ++o) {
-      const int s = ulist[(size_t)box * NNEAR + o];
-      nb_pre[o] = acc;
-      nb_start[o] = s < 0 ? 0u : bstart[s];
-      acc += s < 0 ? 0u : bcount[s];
+template <bool FIELD>
+__global__ void __launch_bounds__(32 * P64_WARPS) k_p2p_free_f64(const P64Job *jobs, int njobs, double *phi,
+                                                                 double *field) {
+  __shared__ uint32_t nb_start[NNEAR], nb_cnt[NNEAR];
+  __shared__ double part[P64_WARPS][4][32];
+  __shared__ int s_nnb;
+  int lo = 0, hi = njobs - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (jobs[mid].block0 <= (int64_t)blockIdx.x) lo = mid; else hi = mid - 1;
+  }
+  const P64Job &J = jobs[lo];
+  const uint32_t box = (uint32_t)((int64_t)blockIdx.x - J.block0);
+  if (box >= J.nb) return;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t tst = J.bstart[box], tcnt = J.bcount[box];
+  if (warp == 0) {  // the non-empty near boxes, in slot order
+    int nnb = 0;
+    for (int o0 = 0; o0 < NNEAR; o0 += 32) {
+      const int o = o0 + lane;
+      const int sb = o < NNEAR ? J.ulist[(size_t)box * NNEAR + o] : -1;
+      const uint32_t cnt = sb >= 0 ? J.bcount[sb] : 0u;
+      const unsigned m = __ballot_sync(0xffffffffu, cnt > 0);
+      if (cnt > 0) {
+        const int k = nnb + __popc(m & ((1u << lane) - 1u));
+        nb_start[k] = J.bstart[sb];
+        nb_cnt[k] = cnt;
+      }
+      nnb += __popc(m);
     }
-    nb_pre[NNEAR] = acc;
+    if (lane == 0) s_nnb = nnb;
   }
   __syncthreads();
-  const uint32_t stot = nb_pre[NNEAR];
-  const uint32_t tst = bstart[box], tcnt = bcount[box];
-  const T tl = (T)lam;
-  const unsigned full = 0xffffffffu;
-  for (uint32_t t0 = 0; t0 < tcnt; t0 += 2 * P2P_TPB) {
-    T px[2], py[2], pz[2], qx[2], qy[2], qz[2];
-    bool tv[2];
-    uint32_t tk[2];
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      const uint32_t tj = t0 + threadIdx.x + t * P2P_TPB;
-      tv[t] = tj < tcnt;
-      tk[t] = tst + (tv[t] ? tj : 0);
-      const double ox = x[tk[t]] - cx, oy = y[tk[t]] - cy, oz = z[tk[t]] - cz;
-      px[t] = (T)ox;
-      py[t] = (T)oy;
-      pz[t] = (T)oz;
-      qx[t] = comp ? (T)(ox - (double)px[t]) : T(0);
-      qy[t] = comp ? (T)(oy - (double)py[t]) : T(0);
-      qz[t] = comp ? (T)(oz - (double)pz[t]) : T(0);
+  const int nnb = s_nnb;
+  const double *X = J.x, *Yc = J.y, *Z = J.z, *Q = J.q;
+  const double lam = J.lam, ce = J.ce;
+  const uint32_t hi_max = J.hi_max;
+  for (uint32_t t0 = 0; t0 < tcnt;) {
+    const uint32_t left = tcnt - t0;
+    const int lb = left >= 32 ? 5 : 31 - __clz((int)left);  // 2^lb targets in this group
+    const int sub = lane >> lb, nsub = 32 >> lb;            // this lane's share of the sources
+    const uint32_t tk = tst + t0 + (lane & ((1 << lb) - 1));
+    const double px = X[tk], py = Yc[tk], pz = Z[tk];
+    double p = 0.0, fx = 0.0, fy = 0.0, fz = 0.0;
+    // sources first + stride i of the concatenated near boxes
+    const uint32_t stride = (uint32_t)(nsub * P64_WARPS);
+    uint32_t off = (uint32_t)(warp * nsub + sub);
+    int k = 0;
+    for (;; off += stride) {
+      while (k < nnb && off >= nb_cnt[k]) off -= nb_cnt[k++];
+      if (k >= nnb) break;
+      const uint32_t j = nb_start[k] + off;
+      p64_pair<FIELD>(px - X[j], py - Yc[j], pz - Z[j], Q[j], lam, ce, hi_max, p, fx, fy, fz);
     }
-    const bool w2 = __any_sync(full, tv[1]), w1 = __any_sync(full, tv[0]);
-    double aphi[2] = {0, 0}, ax[2] = {0, 0}, ay[2] = {0, 0}, az[2] = {0, 0};
-    for (uint32_t s0 = 0; s0 < stot; s0 += P2P_SRC) {
-      __syncthreads();
-      for (uint32_t jj = threadIdx.x; jj < P2P_SRC; jj += P2P_TPB) {
-        const uint32_t g = s0 + jj;
-        if (g < stot) {
-          int o = 0;
-          while (nb_pre[o + 1] <= g) ++o;  // neighbour holding source g (empty ones skipped)
-          const uint32_t k = nb_start[o] + (g - nb_pre[o]);
-          const double ux = x[k] - cx, uy = y[k] - cy, uz = z[k] - cz;
-          V4<T> h;
-          h.x = (T)ux;
-          h.y = (T)uy;
-          h.z = (T)uz;
-          h.w = (T)q[k];
-          sh[jj] = h;
-          if (comp) {
-            V4<T> lo;
-            lo.x = (T)(ux - (double)h.x);
-            lo.y = (T)(uy - (double)h.y);
-            lo.z = (T)(uz - (double)h.z);
-            lo.w = T(0);
-            sl[jj] = lo;
-          }
-        }
-      }
-      __syncthreads();
-      const int nn = (int)min((uint32_t)P2P_SRC, stot - s0);
-      T fp[2] = {0, 0}, fx[2] = {0, 0}, fy[2] = {0, 0}, fz[2] = {0, 0};
-      if (w2) p2p_free_tile<T, 2, comp>(sh, sl, nn, px, py, pz, qx, qy, qz, tl, fp, fx, fy, fz);
-      else if (w1) p2p_free_tile<T, 1, comp>(sh, sl, nn, px, py, pz, qx, qy, qz, tl, fp, fx, fy, fz);
-#pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        aphi[t] += (double)fp[t];
-        ax[t] += (double)fx[t];
-        ay[t] += (double)fy[t];
-        az[t] += (double)fz[t];
+    for (int o = 16; o >= (1 << lb); o >>= 1) {  // lanes of one target differ in the bits above lb
+      p += __shfl_xor_sync(0xffffffffu, p, o);
+      if (FIELD) {
+        fx += __shfl_xor_sync(0xffffffffu, fx, o);
+        fy += __shfl_xor_sync(0xffffffffu, fy, o);
+        fz += __shfl_xor_sync(0xffffffffu, fz, o);
       }
     }
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      if (!tv[t]) continue;
-      const uint32_t i = src[tk[t]];
-      phi[i] += scale * aphi[t];
-      if (field) {
-        field[3 * i] += scale * ax[t];
-        field[3 * i + 1] += scale * ay[t];
-        field[3 * i + 2] += scale * az[t];
-      }
+    __syncthreads();  // the previous group's sums have been read
+    part[warp][0][lane] = p;
+    if (FIELD) {
+      part[warp][1][lane] = fx;
+      part[warp][2][lane] = fy;
+      part[warp][3][lane] = fz;
     }
+    __syncthreads();
+    const int v = threadIdx.x >> lb, t = threadIdx.x & ((1 << lb) - 1);  // value, target
+    if (v < (FIELD ? 4 : 1)) {
+      double s = 0.0;
+#pragma unroll
+      for (int w = 0; w < P64_WARPS; ++w) s += part[w][v][t];
+      const uint32_t i = J.src[tst + t0 + t];
+      if (v == 0) phi[i] += J.scale * s;
+      else field[3 * (size_t)i + v - 1] += J.scale * s;
+    }
+    t0 += 1u << lb;
   }
 }
 
@@ -1377,6 +1383,7 @@ void init_fmm_tables(Ctx &c) {
   upload_gl16();
   upload_an();
   make_tables(c);
+  upload_exp2(c.stream);
   upload_consts(c.stream);
   make_rotcol(c);
 }
@@ -2133,13 +2140,45 @@ static void m2l_all_f32(Ctx &c, std::vector<Group> &groups) {
   launch_reduce();
 }
 
-// L2L (adding the parent's shifted expansion), L2P and the near fields of one group
+// the FP64 free-space near field of every group, one launch
+static void near_free_f64(Ctx &c, std::vector<Group> &groups, double *phi, double *field) {
+  std::vector<P64Job> jobs;
+  int64_t blocks = 0;
+  for (auto &g : groups) {
+    if (!(g.is_free && (g.parts & 1))) continue;
+    const Level &Lf = g.T.lev[g.Df];
+    if (!Lf.n) continue;
+    P64Job j;
+    j.bstart = Lf.pstart; j.bcount = Lf.pcount; j.ulist = g.ufree;
+    j.x = g.T.x; j.y = g.T.y; j.z = g.T.z; j.q = g.T.q; j.src = g.T.src;
+    j.lam = c.md.lam[g.l];
+    j.scale = 1.0 / (4.0 * PI * c.md.eps[g.l]);
+    j.ce = (double)(-(long double)j.lam * 1.44269504088896340736L * EXP_TAB);
+    const double rmax = 700.0 / j.lam, r2 = std::min(rmax * rmax, 1e300);
+    uint64_t u;
+    std::memcpy(&u, &r2, sizeof u);
+    // (high word - 0x00100000) <= hi_max: normal numbers up to the cut
+    j.hi_max = std::max((uint32_t)(u >> 32), 0x00100000u) - 0x00100000u;
+    j.nb = (uint32_t)Lf.n;
+    j.block0 = blocks;
+    jobs.push_back(j);
+    blocks += Lf.n;
+  }
+  if (jobs.empty()) return;
+  P64Job *dj = c.arena.get<P64Job>(jobs.size());
+  LPB_CUDA(cudaMemcpyAsync(dj, jobs.data(), sizeof(P64Job) * jobs.size(), cudaMemcpyHostToDevice, c.stream));
+  if (field) k_p2p_free_f64<true><<<(unsigned)blocks, 32 * P64_WARPS, 0, c.stream>>>(dj, (int)jobs.size(), phi, field);
+  else k_p2p_free_f64<false><<<(unsigned)blocks, 32 * P64_WARPS, 0, c.stream>>>(dj, (int)jobs.size(), phi, field);
+  LPB_LAUNCH();
+  c.launches++;
+}
+
+// L2L (adding the parent's shifted expansion), L2P and the reaction near field of one group
 template <typename T>
 static void downward_t(Ctx &c, Group &g, int parts, double *phi, double *field) {
   typedef typename C2<T>::t T2;
   const int K = c.K, D = g.D;
   const Tables &tb = sizeof(T) == 8 ? g_tab_d[c.device] : g_tab_f[c.device];
-  const bool dofree = g.is_free && (parts & 1);
   const bool doreact = (parts & 2) && g.I.np > 0;
   const bool react_near = doreact && !(parts & 4);
   for (int l = 3; l <= D; ++l) {
@@ -2152,16 +2191,6 @@ static void downward_t(Ctx &c, Group &g, int parts, double *phi, double *field) 
     c.launches++;
   }
   PT_DISPATCH(launch_l2p, c, g.T.lev[D], g.T.lev[D].n, g.T, geo_at<T>(g, D), c.md.lam[g.l], g.Lt[D], phi, field);
-  if (dofree && sizeof(T) == 8) {
-    // the FP64 free-space near field at the free-space leaves (level Df); the FP32 one runs in
-    // run_near_free, beside the far field
-    const Level &Lf = g.T.lev[g.Df];
-    k_p2p_free<T><<<(unsigned)Lf.n, P2P_TPB, 0, c.stream>>>(
-        Lf.d_n, Lf.key, Lf.pstart, Lf.pcount, g.ufree, g.T.x, g.T.y, g.T.z, g.T.q, g.T.src, geo_at<T>(g, g.Df),
-        c.md.lam[g.l], 1.0 / (4.0 * PI * c.md.eps[g.l]), phi, field);
-    LPB_LAUNCH();
-    c.launches++;
-  }
   if (react_near && g.ureact && g.nodes) {
     k_p2p_react<T><<<(unsigned)g.T.lev[D].n, P2P_THREADS, 0, c.stream>>>(
         g.T.lev[D].d_n, g.T.lev[D].key, g.T.lev[D].start, g.T.lev[D].count, g.ureact, g.T.x, g.T.y, g.T.z, g.T.src,
@@ -2243,6 +2272,7 @@ void run_fmm_back(Ctx &c, std::vector<Group> &groups, double *phi, double *field
   if (c.near_async) LPB_CUDA(cudaStreamWaitEvent(c.stream, c.ev_near, 0));
   for (auto &g : groups)
     d ? downward_t<double>(c, g, g.parts, phi, field) : downward_t<float>(c, g, g.parts, phi, field);
+  if (d) near_free_f64(c, groups, phi, field);
   prof_mark(c, "downward");
 }
 
