@@ -7,10 +7,13 @@
 #include "internal.h"
 #include "tc.cuh"
 
+#include <cuda_fp16.h>
+
 #include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 namespace lpb {
 
@@ -1311,12 +1314,14 @@ __global__ void __launch_bounds__(P2P_THREADS) k_p2p_react(
 }
 
 #include "m2l_pairs.cuh"
+#include "m2l_tc.cuh"
 
 // ---------------------------------------------------------------------------------------
 // driver for one group
 // ---------------------------------------------------------------------------------------
 struct Tables {
   int32_t *cls_free, *cls_react;  // [NOFF], [2][NKT][NOFF]
+  int32_t *tc_free, *tc_react;    // the same for the tensor-core operators (per canonical pair)
   void *rot, *rot4;               // per precision
 };
 Tables g_tab_d[LPB_MAX_DEVICES], g_tab_f[LPB_MAX_DEVICES];  // per device
@@ -1326,19 +1331,26 @@ static void make_tables(Ctx &c) {
   if (!not_done_on_device(g_tab_ready)) return;
   // operator class of every offset that can appear in a far list (|d|_inf >= 2); which offsets
   // do appear is decided by the list builder for the context's separation
-  std::vector<int32_t> cf(NOFF, -1), cr(2 * NKT * NOFF, -1);
+  std::vector<int32_t> cf(NOFF, -1), cr(2 * NKT * NOFF, -1), tf(NOFF, -1), tr(2 * NKT * NOFF, -1);
   std::vector<double> rot(NOFF * (PMAX + 1) * 2), rot4(4 * (PMAX + 1) * 2);
   for (int o = 0; o < NOFF; ++o) {
     int dx, dy, dz;
     off_decode(o, dx, dy, dz);
     const int cheb = cheb3(dx, dy, dz);
-    if (cheb >= 2) cf[o] = rho_index(dx, dy) * NDZ + dz + OFF_R;
+    int kq;
+    bool refl;
+    const int ci = can_of(dx, dy, kq, refl);
+    if (cheb >= 2) {
+      cf[o] = rho_index(dx, dy) * NDZ + dz + OFF_R;
+      tf[o] = ci * NDZ + dz + OFF_R;
+    }
     for (int a = 1; a <= 2; ++a)
       for (int kt = 0; kt < NKT; ++kt) {
         const int ks = (a == 1) ? -dz - 1 - kt : dz - 1 - kt;
         const int kk = kk_index(kt, ks);
         if (cheb < 2 || kk < 0) continue;
         cr[((a - 1) * NKT + kt) * NOFF + o] = rho_index(dx, dy) * NKK + kk;
+        tr[((a - 1) * NKT + kt) * NOFF + o] = ci * NKK + kk;
       }
     const double ph = (dx == 0 && dy == 0) ? 0.0 : atan2(-(double)dy, -(double)dx);
     for (int m = 0; m <= PMAX; ++m) {
@@ -1354,7 +1366,11 @@ static void make_tables(Ctx &c) {
       rot4[(dir * (PMAX + 1) + m) * 2 + 1] = sin(m * ph);
     }
   }
-  int32_t *dcf, *dcr;
+  int32_t *dcf, *dcr, *dtf, *dtr;
+  LPB_CUDA(cudaMalloc(&dtf, sizeof(int32_t) * NOFF));
+  LPB_CUDA(cudaMalloc(&dtr, sizeof(int32_t) * 2 * NKT * NOFF));
+  LPB_CUDA(cudaMemcpy(dtf, tf.data(), sizeof(int32_t) * NOFF, cudaMemcpyHostToDevice));
+  LPB_CUDA(cudaMemcpy(dtr, tr.data(), sizeof(int32_t) * 2 * NKT * NOFF, cudaMemcpyHostToDevice));
   LPB_CUDA(cudaMalloc(&dcf, sizeof(int32_t) * NOFF));
   LPB_CUDA(cudaMalloc(&dcr, sizeof(int32_t) * 2 * NKT * NOFF));
   LPB_CUDA(cudaMemcpy(dcf, cf.data(), sizeof(int32_t) * NOFF, cudaMemcpyHostToDevice));
@@ -1369,14 +1385,14 @@ static void make_tables(Ctx &c) {
   LPB_CUDA(cudaMemcpy(r4d, rot4.data(), sizeof(double) * rot4.size(), cudaMemcpyHostToDevice));
   LPB_CUDA(cudaMemcpy(rf, rotf.data(), sizeof(float) * rotf.size(), cudaMemcpyHostToDevice));
   LPB_CUDA(cudaMemcpy(r4f, rot4f.data(), sizeof(float) * rot4f.size(), cudaMemcpyHostToDevice));
-  g_tab_d[c.device] = Tables{dcf, dcr, rd, r4d};
-  g_tab_f[c.device] = Tables{dcf, dcr, rf, r4f};
+  g_tab_d[c.device] = Tables{dcf, dcr, dtf, dtr, rd, r4d};
+  g_tab_f[c.device] = Tables{dcf, dcr, dtf, dtr, rf, r4f};
   mark_done_on_device(g_tab_ready);
 }
 
 void upload_gl16();
 void upload_an();
-void make_rotcol(Ctx &c);
+void upload_trig(cudaStream_t s);
 void init_fmm_tables(Ctx &c) {
   static std::mutex mu;
   std::lock_guard<std::mutex> lk(mu);
@@ -1384,8 +1400,8 @@ void init_fmm_tables(Ctx &c) {
   upload_an();
   make_tables(c);
   upload_exp2(c.stream);
+  upload_trig(c.stream);
   upload_consts(c.stream);
-  make_rotcol(c);
 }
 
 template <typename T, int PT>
@@ -1407,445 +1423,6 @@ static void launch_l2p(Ctx &c, const Level &Lv, int64_t nb, const PointSet &P, G
                                                                 P.src, geo, lam, c.p, c.K, (const T2 *)L, phi, field);
   LPB_LAUNCH();
   c.launches++;
-}
-
-// ---------------------------------------------------------------------------------------
-// M2L on the tensor cores (tcgen05, TF32 with a three-product split), free space and reaction.
-//
-// Every translation of this library has the azimuth-factored form
-//     X = e^{i mu phi} M,   Y_nm = sum P_{nm,nu mu} Re X_{nu mu} + i sum Q_{nm,nu mu} Im X_{nu mu},
-//     L_nm += e^{-i m phi} Y_nm
-// with real class operators P, Q that do not depend on the azimuth phi of the offset.  In real
-// form (R = 2K - (p+1) coordinates: for m > 0 the pair (Re, Im) in adjacent columns, then the
-// real parts of the m = 0 coefficients; the m = 0 imaginary parts vanish for real charges) the
-// middle step is one real matrix W_c (P between real parts, Q between imaginary parts) per
-// class c and source type.  A CTA owns 128 target boxes (an octant tile, or a run of a target
-// list) and one dx-slice of the offsets.  For every (offset, source type) step it copies the
-// unrotated source rows and W_c into shared memory with cp.async; before the MMAs each thread
-// rotates its own row in place and splits it into TF32 hi + lo (the rotation couples only the
-// adjacent Re, Im columns of one coefficient); it accumulates D = X W_c^T in a fresh TMEM accumulator
-// as hi*hi + hi*lo + lo*hi, and folds D into FP32 registers after the rotation e^{-i m phi}:
-// the tensor core's accumulation loses precision over long chains (measured), a dot product of
-// 32 NC terms per step does not.
-// ---------------------------------------------------------------------------------------
-// real coordinate c -> half-representation index: >= 0 real part, <= -2 imaginary part of
-// index (-code - 2), -1 padding
-__host__ __device__ __forceinline__ int tc_remap(int c, int K, int p) {
-  const int NI = K - (p + 1);  // coefficients with m > 0
-  if (c < 2 * NI) {
-    const int j = c >> 1;
-    int n = 1;
-    while ((n + 1) * n / 2 <= j) ++n;  // entries with m > 0 below degree n: n(n-1)/2
-    const int h = n * (n + 1) / 2 + (j - n * (n - 1) / 2 + 1);
-    return (c & 1) ? -h - 2 : h;
-  }
-  const int n = c - 2 * NI;
-  return n <= p ? n * (n + 1) / 2 : -1;
-}
-
-// (cos m phi, sin m phi) of every far offset's azimuth phi for each real coordinate pair of the
-// tensor-core layout: entry [o][c], [o][c + 1] for the (Re, Im) columns c, c + 1 of a coefficient
-// of order m; (1, 0) for the columns of m = 0 real parts and padding, which no rotation changes.
-// Per context (the layout depends on p); built once in lpbfmm_create.
-void make_rotcol(Ctx &c) {
-  const int R = 2 * c.K - (c.p + 1), NC = (R + 31) / 32, N = 32 * NC;
-  if (NC > 4) return;  // only the tensor-core path (p <= 10) uses it
-  const int NI2 = 2 * (c.K - (c.p + 1));
-  std::vector<float> t((size_t)NOFF * N);
-  for (int o = 0; o < NOFF; ++o) {
-    int dx, dy, dz;
-    off_decode(o, dx, dy, dz);
-    const double ph = (dx == 0 && dy == 0) ? 0.0 : atan2(-(double)dy, -(double)dx);
-    for (int col = 0; col < N; col += 2) {
-      double cs = 1.0, sn = 0.0;
-      if (col < NI2) {
-        const int h = tc_remap(col, c.K, c.p);  // real part of half index h
-        int n = 0;
-        while ((n + 1) * (n + 2) / 2 <= h) ++n;
-        const int m = h - n * (n + 1) / 2;
-        cs = cos(m * ph);
-        sn = sin(m * ph);
-      }
-      t[(size_t)o * N + col] = (float)cs;
-      t[(size_t)o * N + col + 1] = (float)sn;
-    }
-  }
-  LPB_CUDA(cudaMalloc(&c.rotcol, sizeof(float) * t.size()));
-  LPB_CUDA(cudaMemcpy(c.rotcol, t.data(), sizeof(float) * t.size(), cudaMemcpyHostToDevice));
-}
-
-// W_c of every class and source type as the shared-memory image the MMA reads: per (class, type)
-// a block of NC K-chunks, each [hi: ldr rows x 128 bytes][lo: ldr rows x 128 bytes] in the
-// 128-byte swizzled K-major layout (tc::swz), so that one bulk copy moves a class's operator into
-// shared memory.  Classes that used[] marks absent at this level are skipped.
-__global__ void k_tc_pack_w(const float *ops, int ncls_types, int ntypes, const uint8_t *used, int K, int p, int ldr,
-                            float *wimg) {
-  __shared__ int code[256];
-  const int ct = blockIdx.x;
-  if (ct >= ncls_types || (used && !used[ct / ntypes])) return;
-  for (int c = threadIdx.x; c < ldr; c += blockDim.x) code[c] = tc_remap(c, K, p);
-  __syncthreads();
-  const size_t KK = (size_t)K * K;
-  const float *P = ops + (size_t)ct * 2 * KK, *Q = P + KK;
-  const int total = ldr * ldr;
-  unsigned char *blk = (unsigned char *)(wimg + (size_t)ct * 2 * ldr * ldr);
-  const size_t tile = (size_t)ldr * 128;  // bytes of one hi (or lo) chunk tile
-  for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < total; e += gridDim.y * blockDim.x) {
-    const int r = e / ldr, k = e % ldr;
-    const int ro = code[r], ko = code[k];
-    float w = 0.f;
-    if (ro >= 0 && ko >= 0) w = P[(size_t)ro * K + ko];
-    else if (ro <= -2 && ko <= -2) w = Q[(size_t)(-ro - 2) * K + (-ko - 2)];
-    const float h = tc::to_tf32(w);
-    unsigned char *ch = blk + (size_t)(k >> 5) * 2 * tile;
-    *(float *)(ch + tc::swz(r, k & 31)) = h;
-    *(float *)(ch + tile + tc::swz(r, k & 31)) = tc::to_tf32(w - h);
-  }
-}
-
-// unrotated source rows in real-coordinate order (FP32), ldr = 32 NC floats per (box, type); with
-// tmask, bit tau of tmask[box] is set when the row of source type tau has a nonzero entry (a zero
-// row adds nothing, so the M2L may skip that type for that box)
-__global__ void k_tc_pack_raw(const float2 *M, int64_t nrows, int K, int p, int ldr, float *raw, int ntypes,
-                              uint32_t *tmask) {
-  const int64_t total = nrows * ldr;  // a multiple of 32: every warp is full and within one row
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = e / ldr;
-    const int code = tc_remap((int)(e % ldr), K, p);
-    const float v = code >= 0 ? M[b * K + code].x : (code <= -2 ? M[b * K + (-code - 2)].y : 0.f);
-    raw[e] = v;
-    if (tmask) {
-      const unsigned nz = __ballot_sync(0xffffffffu, v != 0.f);
-      if ((threadIdx.x & 31) == 0 && nz) atomicOr(&tmask[b / ntypes], 1u << (int)(b % ntypes));
-    }
-  }
-}
-
-constexpr int TC_MAXSTEP = SLICE_OFFS * 2 * (MAXLAYER - 1);
-
-constexpr int TC_ROWS = 128, TC_WORKERS = 256, TC_THREADS = TC_WORKERS + 32;
-constexpr int TC_WAIT = 1 << 22;  // mbarrier polls before the kernel reports a timeout
-
-__host__ __device__ constexpr int tc_nst(int NC) { return NC <= 5 ? 3 : 2; }
-__host__ __device__ constexpr size_t tc_stage_bytes(int NC) { return (size_t)2 * (TC_ROWS + 32 * NC) * 128; }
-static size_t tc_smem(int NC) { return tc_nst(NC) * tc_stage_bytes(NC) + 1024; }
-
-__device__ __forceinline__ uint64_t to_global(const void *p) {
-  uint64_t g;
-  asm("cvta.to.global.u64 %0, %1;" : "=l"(g) : "l"(p));
-  return g;
-}
-// one arrival that also announces tx bytes to come by bulk copies
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *mbar, uint32_t bytes) {
-  asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.expect_tx.shared::cta.b64 st, [%0], %1;\n}\n" ::"r"(
-                   tc::smem_u32(mbar)),
-               "r"(bytes)
-               : "memory");
-}
-// bulk copy of bytes (multiple of 16, both addresses 16-byte aligned) global -> shared, completing
-// on mbar
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src, uint32_t bytes, uint64_t *mbar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                   tc::smem_u32(dst)),
-               "l"(to_global(src)), "r"(bytes), "r"(tc::smem_u32(mbar))
-               : "memory");
-}
-
-// x rounded to TF32 (10 stored significand bits), to nearest with ties away from zero, in integer
-// arithmetic on the FP32 bits: the rounding of cvt.rna.tf32.f32 for the finite values here, on
-// the integer pipes (the split of every staged source row runs once per step)
-__device__ __forceinline__ float tf32i(float x) {
-  return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
-}
-template <int NC>
-__global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TJob *jobs, int njobs, int K, int p, int *status) {
-  constexpr int N = 32 * NC, NST = tc_nst(NC);
-  constexpr int TCOLS = 2 * N <= 32 ? 32 : (2 * N <= 64 ? 64 : (2 * N <= 128 ? 128 : 256));
-  static_assert(2 * N <= 256, "two accumulators of N columns");
-  constexpr size_t SA = (size_t)TC_ROWS * 128, SB = (size_t)N * 128;  // bytes of one A / B chunk tile
-  extern __shared__ __align__(16) unsigned char tcsm[];  // base rounded up to 1024 below
-  unsigned char *sbase = (unsigned char *)(((uintptr_t)tcsm + 1023) & ~(uintptr_t)1023);
-  __shared__ int tid_[TC_ROWS];
-  __shared__ int steps[TC_MAXSTEP];  // (offset << 4) | source type
-  __shared__ int remap_s[N], mcol[N];  // coordinate -> half index code; m of that coefficient
-  __shared__ int nsteps;
-  __shared__ unsigned tmk[SLICE_OFFS];  // per offset of the slice: the source types some row needs
-  // the rotation columns depend on the offset's azimuth only, i.e. on (dx, dy): a dx-slice needs
-  // OFF_D rows of the table, kept here for the whole CTA
-  __shared__ __align__(16) float rot_s[OFF_D * 128];
-  // full[b]: the workers have staged buffer b (TC_WORKERS arrivals); empty[b]: its MMAs are done;
-  // accbar[a]: a step's MMAs into accumulator a are done; foldbar[a]: the workers have read it
-  // wfull[b]: the operator chunk of buffer b has landed (one bulk copy, issued by thread 0)
-  __shared__ uint64_t full[NST], empty[NST], accbar[2], foldbar[2], wfull[NST];
-  __shared__ uint32_t tbase;
-  int lo = 0, hi = njobs - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (jobs[mid].item0 <= (int64_t)blockIdx.x) lo = mid; else hi = mid - 1;
-  }
-  const TJob &J = jobs[lo];
-  // the fields the pipeline reads, in registers: the inline-assembly memory clobbers of the
-  // barrier and copy instructions would otherwise make the compiler reload them from global
-  // memory after every one
-  const float *const Jraw = J.raw, *const Jwimg = J.wimg, *const Jrotcol = J.rotcol;
-  const int32_t *const Jvlist = J.vlist, *const Jcls = J.cls_of;
-  const int64_t local = (int64_t)blockIdx.x - J.item0;
-  // slice-major: the CTAs resident at one time share a dx-slice, hence the operator classes of
-  // its offsets, which then stay in L2 (a level's reaction operators alone exceed it)
-  const int64_t ntiles = J.pstart ? 8 * ((J.npar + TC_ROWS - 1) / TC_ROWS) : (J.ntb + TC_ROWS - 1) / TC_ROWS;
-  const int slice = (int)(local / ntiles);
-  const int64_t ti = local % ntiles;
-  const int64_t ntl = J.tlist ? (int64_t)*J.d_ntl : J.ntb;
-  if (J.pstart ? (ti >> 3) * TC_ROWS >= J.npar : ti * TC_ROWS >= ntl) return;
-  // worker thread (tid < TC_WORKERS) = (row, half): row = target slot and TMEM lane, half = which
-  // 4 of a chunk's 8 units and which half of the accumulator columns it handles; the last warp
-  // issues the MMAs (lane 0)
-  const int tid = threadIdx.x, warp = tid >> 5, row = tid & (TC_ROWS - 1), hf = (tid >> 7) & 1;
-  const bool worker = tid < TC_WORKERS;
-  const int ntypes = J.ntypes;
-  for (int c = tid; c < N; c += TC_THREADS) {
-    const int code = tc_remap(c, K, p);
-    remap_s[c] = code;
-    mcol[c] = code == -1 ? 0 : cK.mof[code >= 0 ? code : -code - 2];
-  }
-  if (tid < TC_ROWS) {
-    int t = -1;
-    if (J.tlist) {
-      const int64_t j = ti * TC_ROWS + tid;
-      if (j < ntl) t = J.tlist[j];
-    } else if (J.pstart) {
-      const int oct = (int)(ti & 7);
-      const int64_t P = (ti >> 3) * TC_ROWS + tid;
-      if (P < J.npar) {
-        const uint32_t s0 = J.pstart[P], n = J.pcount[P];
-        for (uint32_t k = 0; k < n; ++k)
-          if ((int)(J.ckey[s0 + k] & 7ull) == oct) t = (int)(s0 + k);
-      }
-    } else {
-      const int64_t j = ti * TC_ROWS + tid;
-      if (j < J.ntb) t = (int)j;
-    }
-    tid_[tid] = t;
-  }
-  for (int k = tid; k < SLICE_OFFS; k += TC_THREADS) tmk[k] = 0u;
-  __syncthreads();
-  if (tid < TC_ROWS) {
-    const int t = tid_[tid];
-    if (t >= 0)
-      for (int k = 0; k < SLICE_OFFS; ++k) {
-        const int o = slice * SLICE_OFFS + k;
-        const int sb = J.cls_of[o] >= 0 ? J.vlist[(size_t)t * NOFF + o] : -1;
-        if (sb >= 0) atomicOr(&tmk[k], J.tmask ? J.tmask[sb] : 0xffffffffu);
-      }
-  }
-  __syncthreads();
-  if (tid == 0) {
-    int n = 0;
-    for (int k = 0; k < SLICE_OFFS; ++k)
-      for (int tau = 0; tau < ntypes; ++tau)
-        if ((tmk[k] >> tau) & 1u) steps[n++] = ((slice * SLICE_OFFS + k) << 4) | tau;
-    nsteps = n;
-  }
-  __syncthreads();
-  const int ns = nsteps;
-  if (ns == 0) return;
-  if (warp == 0) tc::tmem_alloc(&tbase, TCOLS);
-  if (tid == 0) {
-    for (int b = 0; b < NST; ++b) {
-      tc::mbar_init(&full[b], TC_WORKERS);
-      tc::mbar_init(&empty[b], 1);
-      tc::mbar_init(&wfull[b], 1);
-    }
-    for (int a = 0; a < 2; ++a) {
-      tc::mbar_init(&accbar[a], 1);
-      tc::mbar_init(&foldbar[a], TC_WORKERS);
-    }
-    tc::mbar_fence_init();
-  }
-  for (int e = tid; e < OFF_D * N; e += TC_THREADS) {
-    const int dyi = e / N;
-    rot_s[e] = Jrotcol[(size_t)off_index(slice - OFF_R, dyi - OFF_R, 0) * N + (e - dyi * N)];
-  }
-  tc::fence_before();
-  __syncthreads();
-  tc::fence_after();
-  // a warp reads the TMEM lanes of its quarter, 32 (warp % 4) .. + 31
-  const uint32_t tmem = tbase, lanebase = (uint32_t)((warp & 3) * 32) << 16;
-  const int S = ns * NC;  // stages: (step, K-chunk)
-  const int myt = worker ? tid_[row] : -1;
-  constexpr uint32_t IDESC = tc::idesc_tf32(TC_ROWS, N);
-  constexpr int NH = N / 2;  // accumulator columns per thread
-  float racc[NH];
-#pragma unroll
-  for (int j = 0; j < NH; ++j) racc[j] = 0.f;
-  // fold the accumulator of step i into racc after the output rotation e^{-i m phi}
-  auto fold = [&](int i) -> bool {
-    const bool ok = tc::mbar_wait(&accbar[i & 1], (uint32_t)((i >> 1) & 1), TC_WAIT);
-    if (ok) {
-      tc::fence_after();
-      const float4 *rr = (const float4 *)(rot_s + ((steps[i] >> 4) / OFF_D % OFF_D) * N + hf * NH);
-      const uint32_t col = (uint32_t)((i & 1) * N + hf * NH);
-#pragma unroll
-      for (int c1 = 0; c1 < NH; c1 += 32) {
-        uint32_t v[4][8];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) tc::tmem_ld8_nw(tmem + lanebase + col + (uint32_t)(c1 + 8 * q), v[q]);
-        tc::tmem_wait_ld();
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int c0 = c1 + 8 * q;
-          const float4 ra = rr[c0 / 4], rb = rr[c0 / 4 + 1];
-          const float cs[4] = {ra.x, ra.z, rb.x, rb.z}, sn[4] = {ra.y, ra.w, rb.y, rb.w};
-#pragma unroll
-          for (int j = 0; j < 8; j += 2) {
-            const float vr = __uint_as_float(v[q][j]), vi = __uint_as_float(v[q][j + 1]);
-            racc[c0 + j] += cs[j / 2] * vr + sn[j / 2] * vi;
-            racc[c0 + j + 1] += cs[j / 2] * vi - sn[j / 2] * vr;
-          }
-        }
-      }
-      tc::fence_before();
-    }
-    return ok;
-  };
-  bool fail = false;
-  int wl_last = -1;  // last stage whose operator chunk thread 0 requested
-  if (worker) {
-    int cur_o = -1, my_src = -1;
-    // stage s is copied at iteration s and rotated / split at iteration s + 1; the MMA thread takes
-    // it from there, so a buffer is refilled NST stages later, once its MMAs are done
-    for (int s = 0; s < S + 1; ++s) {
-      if (s < S) {
-        const int b = s % NST;
-        if (s >= NST && !tc::mbar_wait(&empty[b], (uint32_t)((s / NST - 1) & 1), TC_WAIT)) {
-          fail = true;
-          break;
-        }
-        const int o = steps[s / NC] >> 4, tau = steps[s / NC] & 15, kc = s % NC;
-        if (o != cur_o) {
-          cur_o = o;
-          my_src = myt >= 0 ? Jvlist[(size_t)myt * NOFF + o] : -1;
-        }
-        unsigned char *st = sbase + (size_t)b * tc_stage_bytes(NC);
-        unsigned char *Ah = st, *Bh = st + 2 * SA;
-        if (tid == 0) {
-          // the class operator's K-chunk (hi and lo tiles, one contiguous image) by one bulk copy
-          const size_t ct = (size_t)Jcls[o] * ntypes + tau;
-          const unsigned char *src = (const unsigned char *)(Jwimg + ct * 2 * N * N) + (size_t)kc * 2 * SB;
-          mbar_expect_tx(&wfull[b], (uint32_t)(2 * SB));
-          bulk_g2s(Bh, src, (uint32_t)(2 * SB), &wfull[b]);
-          wl_last = s;
-        }
-        {
-          // this thread's source row chunk, unrotated, into the A-hi slots (rotated next iteration)
-          const bool v = my_src >= 0;
-          const float *g = Jraw + ((size_t)(v ? my_src : 0) * ntypes + tau) * N + kc * 32;
-#pragma unroll
-          for (int u = hf * 4; u < hf * 4 + 4; ++u) cp_async16(Ah + tc::swz16(row, u), g + 4 * u, v);
-        }
-      }
-      cp_commit();
-      const int sc = s - 1;
-      if (sc < 0) continue;
-      asm volatile("cp.async.wait_group 1;\n" ::);
-      const int si = sc / NC, kc = sc % NC;
-      {
-        // rotate this thread's half row by e^{i mu phi} and split it into TF32 hi (in place) + lo
-        unsigned char *st = sbase + (size_t)(sc % NST) * tc_stage_bytes(NC);
-        unsigned char *Ah = st, *Al = st + SA;
-        const float4 *rr = (const float4 *)(rot_s + ((steps[si] >> 4) / OFF_D % OFF_D) * N + kc * 32);
-#pragma unroll
-        for (int uu = 0; uu < 4; ++uu) {
-          const int u = hf * 4 + uu;
-          float4 x = *(float4 *)(Ah + tc::swz16(row, u));
-          const float4 r = rr[u];  // (cos, sin) of the unit's two column pairs
-          const float xr0 = r.x * x.x - r.y * x.y, xi0 = r.y * x.x + r.x * x.y;
-          const float xr1 = r.z * x.z - r.w * x.w, xi1 = r.w * x.z + r.z * x.w;
-          x = make_float4(xr0, xi0, xr1, xi1);
-          float4 h4v, l4v;
-          h4v.x = tf32i(x.x);
-          h4v.y = tf32i(x.y);
-          h4v.z = tf32i(x.z);
-          h4v.w = tf32i(x.w);
-          l4v.x = tf32i(x.x - h4v.x);
-          l4v.y = tf32i(x.y - h4v.y);
-          l4v.z = tf32i(x.z - h4v.z);
-          l4v.w = tf32i(x.w - h4v.w);
-          *(float4 *)(Ah + tc::swz16(row, u)) = h4v;
-          *(float4 *)(Al + tc::swz16(row, u)) = l4v;
-        }
-      }
-      // this thread's copies (B part, its A row) and its stores are in place: hand over to the tensor core
-      tc::fence_async_smem();
-      tc::mbar_arrive(&full[sc % NST]);
-      // step si is handed over in full: fold step si - 1 (its accumulator is reused by step si + 1)
-      if (kc == NC - 1 && si >= 1) {
-        if (!fold(si - 1)) {
-          fail = true;
-          break;
-        }
-        tc::mbar_arrive(&foldbar[(si - 1) & 1]);
-      }
-    }
-    asm volatile("cp.async.wait_group 0;\n" ::);
-    // no bulk copy may still be writing this CTA's shared memory when it exits
-    if (tid == 0 && fail && wl_last >= 0)
-      tc::mbar_wait(&wfull[wl_last % NST], (uint32_t)((wl_last / NST) & 1), TC_WAIT);
-    if (!fail && !fold(ns - 1)) fail = true;
-    if (!fail) {
-      const int t = tid_[row];
-      if (t >= 0) {
-        float2 *Lrow = J.L + ((size_t)t * M2L_NSLOT + J.slot0 + slice) * K;
-#pragma unroll
-        for (int j = 0; j < NH; ++j) {
-          const int code = remap_s[hf * NH + j];
-          if (code >= 0) {
-            Lrow[code].x = racc[j];
-            if (mcol[hf * NH + j] == 0) Lrow[code].y = 0.f;
-          } else if (code <= -2) {
-            Lrow[-code - 2].y = racc[j];
-          }
-        }
-      }
-    }
-  } else if (tid == TC_WORKERS) {
-    // the MMA thread: stage after stage, once the workers have staged it; a step's first chunk
-    // waits until the workers have read the accumulator two steps back
-    int last = -1;
-    for (int sc = 0; sc < S; ++sc) {
-      const int b = sc % NST, si = sc / NC, kc = sc % NC;
-      if (!tc::mbar_wait(&full[b], (uint32_t)((sc / NST) & 1), TC_WAIT) ||
-          !tc::mbar_wait(&wfull[b], (uint32_t)((sc / NST) & 1), TC_WAIT)) {
-        fail = true;
-        break;
-      }
-      if (kc == 0 && si >= 2 && !tc::mbar_wait(&foldbar[si & 1], (uint32_t)(((si - 2) >> 1) & 1), TC_WAIT)) {
-        fail = true;
-        break;
-      }
-      tc::fence_after();
-      unsigned char *st = sbase + (size_t)b * tc_stage_bytes(NC);
-      const uint32_t ah = tc::smem_u32(st), al = ah + (uint32_t)SA, bh = ah + 2 * (uint32_t)SA,
-                     bl = bh + (uint32_t)SB;
-      const uint32_t dacc = tmem + (uint32_t)((si & 1) * N);
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk) {
-        const uint32_t off = kk * 32;
-        tc::mma_tf32(dacc, tc::sdesc(ah + off), tc::sdesc(bh + off), IDESC, (kc | kk) ? 1u : 0u);
-        tc::mma_tf32(dacc, tc::sdesc(ah + off), tc::sdesc(bl + off), IDESC, 1u);
-        tc::mma_tf32(dacc, tc::sdesc(al + off), tc::sdesc(bh + off), IDESC, 1u);
-      }
-      tc::commit(&empty[b]);
-      if (kc == NC - 1) tc::commit(&accbar[si & 1]);
-      last = sc;
-    }
-    // every MMA has completed once the last committed stage's barrier phase completes
-    if (last >= 0) tc::mbar_wait(&empty[last % NST], (uint32_t)((last / NST) & 1), TC_WAIT);
-  }
-  if (fail) atomicExch(status, LPBFMM_ERR_TIMEOUT);
-  tc::fence_before();
-  __syncthreads();
-  if (warp == 0) tc::tmem_free(tmem, TCOLS);
 }
 
 template <typename T, int TPT, int NR>
@@ -1973,6 +1550,20 @@ static void m2l_all_f64(Ctx &c, std::vector<Group> &groups) {
   launch_pair_m2l(c, jobs, ncls, (const double *)tb.rot);
 }
 
+template <int P>
+static void launch_tc_p(const TJob *jobs, int njobs, int64_t items, int *status, cudaStream_t st) {
+  LPB_ATTR_ONCE(k_m2l_tc<P>, tc_smem(tc_chunks(P)));
+  k_m2l_tc<P><<<(unsigned)items, TC_THREADS, tc_smem(tc_chunks(P)), st>>>(jobs, njobs, status);
+}
+static void launch_tc(int p, const TJob *jobs, int njobs, int64_t items, int *status, cudaStream_t st) {
+  switch (p) {
+#define LPB_TC_CASE(P) case P: launch_tc_p<P>(jobs, njobs, items, status, st); break;
+    LPB_TC_CASE(2) LPB_TC_CASE(3) LPB_TC_CASE(4) LPB_TC_CASE(5) LPB_TC_CASE(6) LPB_TC_CASE(7) LPB_TC_CASE(8)
+    LPB_TC_CASE(9) LPB_TC_CASE(10)
+#undef LPB_TC_CASE
+  }
+}
+
 // mixed mode: every multipole-to-local translation of every group and level in one launch
 static void m2l_all_f32(Ctx &c, std::vector<Group> &groups) {
   typedef float T;
@@ -1983,8 +1574,8 @@ static void m2l_all_f32(Ctx &c, std::vector<Group> &groups) {
   typedef C2<T>::t T2;
   std::vector<RJob> rjobs;
   int64_t relem = 0;
-  // tensor-core free-space path: mixed precision, 2K - (p+1) <= 128 real coordinates
-  const int tc_nc = (2 * c.K - (c.p + 1) + 31) / 32;
+  // tensor-core path: 2K - (p+1) <= 128 real coordinates
+  const int tc_nc = tc_chunks(c.p);
   const bool use_tc = tc_nc <= 4;  // p <= 10
   std::vector<TJob> tjobs;
   int64_t titems = 0;
@@ -2014,60 +1605,55 @@ static void m2l_all_f32(Ctx &c, std::vector<Group> &groups) {
       r.part = part; r.L = g.Lt[l]; r.n = ntb * c.K; r.e0 = relem;
       rjobs.push_back(r);
       relem += r.n;
+      const int N = 32 * tc_nc;
+      // split source rows and their masks; operator images
+      auto pack = [&](TJob &j, const void *M, int64_t nsb, const Level &sl, int side, const void *ops, int kind,
+                      int ntypes, const uint8_t *used, int ncls) {
+        __half *rows = c.arena.get<__half>((size_t)nsb * ntypes * 2 * N);
+        float *rs = c.arena.get<float>((size_t)nsb * ntypes), *wsc = c.arena.get<float>((size_t)ncls * ntypes);
+        uint32_t *tmask = c.arena.get<uint32_t>((size_t)nsb);
+        unsigned char *wimg = c.arena.get<unsigned char>((size_t)ncls * ntypes * N * N * 4);
+        LPB_CUDA(cudaMemsetAsync(tmask, 0, sizeof(uint32_t) * nsb, c.stream));
+        const int64_t nr = nsb * ntypes;
+        k_tc_pack_rows<<<(unsigned)((nr + 7) / 8), 256, 0, c.stream>>>((const float2 *)M, nr, c.K, c.p, tc_nc, ntypes,
+                                                                        sl.key, l, side, c.ws, rows, rs, tmask);
+        LPB_LAUNCH();
+        k_tc_pack_w<<<ncls * ntypes, PACKW_THREADS, sizeof(float) * 2 * c.K * c.K, c.stream>>>(
+            (const float *)ops, kind, ntypes, used, c.ws, c.K, c.p, tc_nc, wimg, wsc);
+        LPB_LAUNCH();
+        c.launches += 2;
+        j.rows = rows; j.rscale = rs; j.tmask = tmask; j.wimg = wimg; j.wscale = wsc; j.ntypes = ntypes;
+        j.L = (float2 *)part; j.ntb = ntb;
+      };
       if (dofree && use_tc) {
-        // tensor-core path: the level's class operators as TF32 hi/lo real matrices
-        const int N = 32 * tc_nc;
-        float *wimg = c.arena.get<float>((size_t)NFREE_CLS * 2 * N * N);
-        k_tc_pack_w<<<dim3(NFREE_CLS, 4), 256, 0, c.stream>>>((const float *)g.op_free[l], NFREE_CLS, 1, nullptr,
-                                                               c.K, c.p, N, wimg);
-        LPB_LAUNCH();
-        c.launches++;
-        float *raw = c.arena.get<float>((size_t)ntb * N);
-        k_tc_pack_raw<<<(unsigned)std::min<int64_t>(4096, (ntb * N + 255) / 256), 256, 0, c.stream>>>(
-            (const float2 *)g.Mfree[l], ntb, c.K, c.p, N, raw, 1, nullptr);
-        LPB_LAUNCH();
-        c.launches++;
         TJob j;
-        j.raw = raw; j.wimg = wimg; j.rotcol = c.rotcol;
-        j.vlist = g.vfree[l]; j.cls_of = tb.cls_free; j.tmask = nullptr; j.tlist = nullptr; j.d_ntl = nullptr;
-        j.L = (float2 *)part; j.ntb = ntb; j.item0 = titems; j.slot0 = 0; j.ntypes = 1;
+        pack(j, g.Mfree[l], ntb, g.T.lev[l], 0, g.op_free[l], 0, 1, nullptr, TC_NFREE);
+        j.vlist = g.vfree[l]; j.cls_of = tb.tc_free; j.tlist = nullptr; j.d_ntl = nullptr;
+        j.item0 = titems; j.slot0 = 0;
         const Level *par = l >= 3 ? &g.T.lev[l - 1] : nullptr;
         j.pstart = par ? par->start : nullptr;
         j.pcount = par ? par->count : nullptr;
         j.ckey = par ? g.T.lev[l].key : nullptr;
         j.npar = par ? par->n : 0;
-        const int64_t tiles = par ? 8 * ((j.npar + TC_ROWS - 1) / TC_ROWS) : (ntb + TC_ROWS - 1) / TC_ROWS;
-        titems += tiles * M2L_NSLICE;
+        j.ntiles = par ? 8 * ((j.npar + TC_ROWS - 1) / TC_ROWS) : (ntb + TC_ROWS - 1) / TC_ROWS;
+        titems += j.ntiles * M2L_NSLICE;
         tjobs.push_back(j);
       } else if (dofree) {
         add(nullptr, nullptr, ntb, g.vfree[l], tb.cls_free, g.Mfree[l], g.op_free[l], part, 1, 0,
             l >= 3 ? &g.T.lev[l - 1] : nullptr, &g.T.lev[l]);
       }
       if (react_far && g.vreact[l] && use_tc && g.ntypes <= 16) {
-        // tensor-core reaction path: class operators per (class, source type)
-        const int N = 32 * tc_nc;
-        const int nct = NREACT_CLS * g.ntypes;
-        float *wimg = c.arena.get<float>((size_t)nct * 2 * N * N);
-        k_tc_pack_w<<<dim3(nct, 4), 256, 0, c.stream>>>((const float *)g.op_react[l], nct, g.ntypes, g.used[l], c.K,
-                                                        c.p, N, wimg);
-        LPB_LAUNCH();
-        c.launches++;
-        const int64_t nir = g.I.lev[l].n * g.ntypes;
-        float *raw = c.arena.get<float>((size_t)nir * N);
-        uint32_t *tmask = c.arena.get<uint32_t>((size_t)g.I.lev[l].n);
-        LPB_CUDA(cudaMemsetAsync(tmask, 0, sizeof(uint32_t) * g.I.lev[l].n, c.stream));
-        k_tc_pack_raw<<<(unsigned)std::min<int64_t>(4096, (nir * N + 255) / 256), 256, 0, c.stream>>>(
-            (const float2 *)g.Mimg[l], nir, c.K, c.p, N, raw, g.ntypes, tmask);
-        LPB_LAUNCH();
-        c.launches++;
+        TJob j;
+        pack(j, g.Mimg[l], g.I.lev[l].n, g.I.lev[l], g.a, g.op_react[l], 1, g.ntypes, g.used[l], TC_NREACT);
+        j.vlist = g.vreact[l]; j.slot0 = M2L_NSLICE;
+        j.pstart = nullptr; j.pcount = nullptr; j.ckey = nullptr; j.npar = 0;
+        // a row is one layer of boxes: at most 4^l of them
+        j.ntiles = (std::min<int64_t>(ntb, (int64_t)1 << (2 * l)) + TC_ROWS - 1) / TC_ROWS;
         for (int kt = 0; kt < 2 * c.ws + 1; ++kt) {
-          TJob j;
-          j.raw = raw; j.wimg = wimg; j.rotcol = c.rotcol;
-          j.vlist = g.vreact[l]; j.cls_of = tb.cls_react + ((g.a - 1) * NKT + kt) * NOFF; j.tmask = tmask;
+          j.cls_of = tb.tc_react + ((g.a - 1) * NKT + kt) * NOFF;
           j.tlist = g.rows[l] + (size_t)kt * ntb; j.d_ntl = g.nrows[l] + kt;
-          j.L = (float2 *)part; j.ntb = ntb; j.item0 = titems; j.slot0 = M2L_NSLICE; j.ntypes = g.ntypes;
-          j.pstart = nullptr; j.pcount = nullptr; j.ckey = nullptr; j.npar = 0;
-          titems += ((ntb + TC_ROWS - 1) / TC_ROWS) * M2L_NSLICE;
+          j.item0 = titems;
+          titems += j.ntiles * M2L_NSLICE;
           tjobs.push_back(j);
         }
       } else if (react_far && g.vreact[l]) {
@@ -2092,16 +1678,7 @@ static void m2l_all_f32(Ctx &c, std::vector<Group> &groups) {
   if (!tjobs.empty()) {
     TJob *dj = c.arena.get<TJob>(tjobs.size());
     LPB_CUDA(cudaMemcpyAsync(dj, tjobs.data(), sizeof(TJob) * tjobs.size(), cudaMemcpyHostToDevice, c.stream));
-    switch (tc_nc) {
-#define LPB_TC_CASE(NCV)                                                                                     \
-  case NCV: {                                                                                                \
-    LPB_ATTR_ONCE(k_m2l_tc<NCV>, tc_smem(NCV));                                                              \
-    k_m2l_tc<NCV><<<(unsigned)titems, TC_THREADS, tc_smem(NCV), c.stream>>>(dj, (int)tjobs.size(), c.K, c.p, c.status); \
-    break;                                                                                                   \
-  }
-      LPB_TC_CASE(1) LPB_TC_CASE(2) LPB_TC_CASE(3) LPB_TC_CASE(4)
-#undef LPB_TC_CASE
-    }
+    launch_tc(c.p, dj, (int)tjobs.size(), titems, c.status, c.stream);
     LPB_LAUNCH();
     c.launches++;
     prof_mark(c, "m2l_tc");
@@ -2306,15 +1883,7 @@ void launch_deferred(const std::vector<Ctx *> &cs, int stage, cudaStream_t st) {
       }
       TJob *dj = c0.arena.get<TJob>(tj.size());
       LPB_CUDA(cudaMemcpyAsync(dj, tj.data(), sizeof(TJob) * tj.size(), cudaMemcpyHostToDevice, st));
-      switch (lead->def.nc) {
-#define LPB_TC_GROUP(NCV)                                                                                    \
-  case NCV:                                                                                                 \
-    LPB_ATTR_ONCE(k_m2l_tc<NCV>, tc_smem(NCV));                                                             \
-    k_m2l_tc<NCV><<<(unsigned)items, TC_THREADS, tc_smem(NCV), st>>>(dj, (int)tj.size(), lead->K, p, c0.status); \
-    break;
-        LPB_TC_GROUP(1) LPB_TC_GROUP(2) LPB_TC_GROUP(3) LPB_TC_GROUP(4)
-#undef LPB_TC_GROUP
-      }
+      launch_tc(p, dj, (int)tj.size(), items, c0.status, st);
       LPB_LAUNCH();
       c0.launches++;
       if (!red.empty()) {

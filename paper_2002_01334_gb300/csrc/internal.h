@@ -196,16 +196,17 @@ struct Group {
 // binary search on the first work item of each job).
 // Tensor-core M2L (k_m2l_tc): one (group, level, row class) of target boxes against one source tree.
 struct TJob {
-  const float *raw;         // source rows [nsb][ntypes][ldr], unrotated real coordinates
-  const float *wimg;        // [ncls][ntypes] operator images (k_tc_pack_w)
-  const float *rotcol;      // [NOFF][ldr] (cos, sin) of m phi per real column pair (make_rotcol)
+  const void *rows;         // source rows [nsb][ntypes][NC][32 hi | 32 lo], split FP16 (k_tc_pack_rows)
+  const float *rscale;      // [nsb][ntypes] inverse power of two of each row
+  const uint32_t *tmask;    // [nsb] source types with a nonzero row (the others are not written)
+  const void *wimg;         // [ncls][ntypes] operator images (k_tc_pack_w)
+  const float *wscale;      // [ncls][ntypes] inverse power of two of each image
   const int32_t *vlist;     // [ntb][NOFF]
   const int32_t *cls_of;    // [NOFF]
-  const uint32_t *tmask;    // [nsb] source types with a nonzero row (nullptr: every type)
   const int32_t *tlist;     // target boxes (nullptr: octant or plain tiles over 0..ntb-1)
   const uint32_t *d_ntl;    // number of entries of tlist (device)
   float2 *L;                // partial sums [ntb][M2L_NSLOT][K]
-  int64_t ntb, item0;
+  int64_t ntb, item0, ntiles;
   int slot0, ntypes;
   const uint32_t *pstart, *pcount;  // octant tiles (nullptr: plain tiles of 128)
   const uint64_t *ckey;
@@ -263,7 +264,6 @@ struct Ctx {
   double *tpoly = nullptr;   // [K][TPK] Legendre-product coefficients
   double *sfac = nullptr;    // [KMAX_TAB+1][KMAX_TAB+1]: sqrt((K+d)! (K-d)!) for d <= K
   double *phat_dir = nullptr;  // [NDIR][(2p+1)(2p+2)/2]: Phat_q^k(cos theta) of the operator directions
-  float *rotcol = nullptr;     // tensor-core M2L: [NOFF][32 NC] (cos, sin) of m phi per real column pair
   // per evaluation: grading of the shared Sommerfeld node set and its Bessel columns
   double stab_lmin = 0.0;
   double *stab_bes = nullptr;

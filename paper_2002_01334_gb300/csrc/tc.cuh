@@ -2,10 +2,10 @@
 // in tensor memory (TMEM), shared-memory matrix descriptors for the 128-byte swizzled K-major
 // layout, mbarrier completion tracking with bounded waits, and TMEM loads.
 //
-// Operand tiles: a K-chunk of 32 TF32 values (128 bytes) per row; rows are 128 bytes apart and
+// Operand tiles: 64 FP16 values (128 bytes) per row; rows are 128 bytes apart and
 // every 8-row group (1024 bytes) is one swizzle atom, in which the 16-byte unit u of row r sits
-// at unit u ^ (r & 7).  Tiles start on 1024-byte boundaries.  An MMA of K = 8 (32 bytes)
-// addresses its slice of the chunk by advancing the descriptor's start address.
+// at unit u ^ (r & 7).  Tiles start on 1024-byte boundaries.  An MMA of K = 16 (32 bytes)
+// addresses its slice of the row by advancing the descriptor's start address.
 #pragma once
 #include <cstdint>
 
@@ -14,10 +14,6 @@ namespace tc {
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// byte offset of element (r, k) (k < 32) inside a swizzled [rows x 32] TF32 tile
-__device__ __forceinline__ uint32_t swz(int r, int k) {
-  return (uint32_t)(r * 128 + (((k >> 2) ^ (r & 7)) << 4) + ((k & 3) << 2));
-}
 // byte offset of the 16-byte unit u (0..7) of row r
 __device__ __forceinline__ uint32_t swz16(int r, int u) { return (uint32_t)(r * 128 + ((u ^ (r & 7)) << 4)); }
 
@@ -32,14 +28,14 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr) {
   return d;
 }
 
-// instruction descriptor: kind::tf32, D in F32, A and B K-major, shape M x N
-__host__ __device__ constexpr uint32_t idesc_tf32(int m, int n) {
-  return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
+// instruction descriptor: kind::f16, A and B in FP16, D in F32, both K-major, shape M x N
+__host__ __device__ constexpr uint32_t idesc_f16(int m, int n) {
+  return (1u << 4) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(m >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n" ::"r"(
+      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
           d_tmem),
       "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
@@ -81,31 +77,16 @@ __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::aft
 // generic-proxy shared-memory writes (st.shared, cp.async) made visible to the tensor core
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;"); }
 
-// whole warp: 8 consecutive 32-bit columns of this warp's 32 TMEM lanes (lane = row)
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
-  uint32_t r[8];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;");
-#pragma unroll
-  for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
-}
-
-// whole warp: 8 consecutive 32-bit columns without waiting; tmem_wait_ld() before using them
-__device__ __forceinline__ void tmem_ld8_nw(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
+// whole warp: 16 consecutive 32-bit columns of this warp's 32 TMEM lanes (lane = row), without waiting;
+// tmem_wait_ld() before using them
+__device__ __forceinline__ void tmem_ld16_nw(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// round to TF32 (nearest, ties away), as the tensor core consumes it
-__device__ __forceinline__ float to_tf32(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return __uint_as_float(r);
-}
 
 }  // namespace tc
 }  // namespace lpb
