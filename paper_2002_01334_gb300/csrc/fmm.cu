@@ -956,275 +956,7 @@ __global__ void __launch_bounds__(32 * P64_WARPS) k_p2p_free_f64(const P64Job *j
   }
 }
 
-// Mixed-precision P2P.  Every point of the target tree carries its offset from its own leaf
-// centre as FP32 hi + lo pairs (k_split_points, once per evaluation).  For a neighbour whose
-// centre lies delta * h away (delta in {-1,0,1}^3), the targets are moved into the
-// neighbour's frame by an exact FP32 two-sum with h = hh + hl, so source records are plain
-// copies: they are staged with cp.async, one neighbour chunk ahead of the one being summed.
-// Per-chunk sums are folded into Kahan-compensated FP32 totals; no FP64 in the pair loop.
-__global__ void k_split_points(const uint32_t *d_nb, const uint64_t *bkey, const uint32_t *bstart,
-                               const uint32_t *bcount, const double *x, const double *y, const double *z,
-                               const double *q, Geo geo, float4 *h4, float4 *l4) {
-  const uint32_t box = blockIdx.x;
-  if (box >= *d_nb) return;
-  double cx, cy, cz;
-  box_center(bkey[box], geo, cx, cy, cz);
-  const uint32_t st = bstart[box], cnt = bcount[box];
-  for (uint32_t j = threadIdx.x; j < cnt; j += blockDim.x) {
-    const uint32_t k = st + j;
-    const double ox = x[k] - cx, oy = y[k] - cy, oz = z[k] - cz;
-    const float hx = (float)ox, hy = (float)oy, hz = (float)oz;
-    h4[k] = make_float4(hx, hy, hz, (float)q[k]);
-    l4[k] = make_float4((float)(ox - (double)hx), (float)(oy - (double)hy), (float)(oz - (double)hz), 0.f);
-  }
-}
-
-__device__ __forceinline__ void two_sum_shift(float hi, float lo, float b, float bl, float &oh, float &ol) {
-  // (hi + lo) + (b + bl) with b exact: oh + ol, the rounding error of hi + b kept in ol
-  const float a = hi + b;
-  const float bb = a - hi;
-  const float e = (hi - (a - bb)) + (b - bb);
-  oh = a;
-  ol = (lo + bl) + e;
-}
-
-__device__ __forceinline__ void kahan_add(float &s, float &c, float v) {
-  const float y = v - c;
-  const float t = s + y;
-  c = (t - s) - y;
-  s = t;
-}
-
-// 2^x on the special-function unit (max. relative error about 2^-22)
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// 1/sqrt(x) on the special-function unit (max. relative error about 2^-22.9; subnormal inputs
-// flushed to zero, which cannot occur for r^2 of distinct points at the FP32 offsets used here)
-__device__ __forceinline__ float rsqrt_approx(float x) {
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// e^{-lambda r} = 2^{(-lambda log2 e) r}; field factor (1 + lambda r) / r^2 = (1/r)(1/r + lambda).
-// MODE by the source box's offset from the target leaf: P2P_SELF (the leaf itself: compensated
-// coordinates, the r = 0 self pair dropped by a select), P2P_TOUCH (a box that touches the leaf:
-// compensated coordinates, r > 0), P2P_APART (a box at least one box away: r >= h, so the FP32
-// rounding of the plain differences, ~2^-23 of 3h, is below 1e-7 of r and the low parts are not
-// used).
-constexpr int P2P_APART = 0, P2P_TOUCH = 1, P2P_SELF = 2;
-template <int NT, int MODE>
-__device__ __forceinline__ void p2p_f32_chunk(const float4 *__restrict__ sh, const float4 *__restrict__ sl, int nn,
-                                              const float (&px)[4], const float (&py)[4], const float (&pz)[4],
-                                              const float (&qx)[4], const float (&qy)[4], const float (&qz)[4],
-                                              float lam, float (&fp)[4], float (&fx)[4], float (&fy)[4],
-                                              float (&fz)[4]) {
-  const float nl2 = -lam * 1.44269504088896341f;
-#pragma unroll 2
-  for (int j = 0; j < nn; ++j) {
-    const float4 s = sh[j];
-    float4 sL = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (MODE != P2P_APART) sL = sl[j];
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      float dx, dy, dz;
-      if (MODE == P2P_APART) {
-        dx = px[t] - s.x;
-        dy = py[t] - s.y;
-        dz = pz[t] - s.z;
-      } else {
-        dx = (px[t] - s.x) + (qx[t] - sL.x);
-        dy = (py[t] - s.y) + (qy[t] - sL.y);
-        dz = (pz[t] - s.z) + (qz[t] - sL.z);
-      }
-      const float r2 = dx * dx + dy * dy + dz * dz;
-      const float ri = (MODE == P2P_SELF) ? (r2 > 0.f ? rsqrt_approx(r2) : 0.f) : rsqrt_approx(r2);
-      const float e = s.w * ex2_approx(nl2 * (r2 * ri)) * ri;
-      fp[t] += e;
-      const float f = e * ri * (ri + lam);
-      fx[t] += f * dx;
-      fy[t] += f * dy;
-      fz[t] += f * dz;
-    }
-  }
-}
-
-// One warp per (target leaf, half) and no block-wide barriers: warp h of a leaf takes the
-// targets 128 i + 64 h + lane + 32 t (t = 0, 1) and streams the sources of the leaf's near boxes
-// through its own double-buffered chunks of P2P_WSRC records.  The near boxes are compacted to the
-// non-empty ones first; a chunk is (near box k, offset within it), walked by a cursor.  Two warps
-// per leaf and an 80-register budget keep 24 warps resident per SM.
-constexpr int P2P_WARPS = 4, P2P_WSRC = 64;
-
-struct P2PCursor {
-  int k;
-  uint32_t off;
-};
-__device__ __forceinline__ void p2p_next(P2PCursor &c, const uint32_t *nb_cnt) {
-  c.off += P2P_WSRC;
-  if (c.off >= nb_cnt[c.k]) {
-    ++c.k;
-    c.off = 0;
-  }
-}
-
-template <int NT>
-__device__ __forceinline__ void p2p_warp_pass(int lane, uint32_t t0, uint32_t tcnt, uint32_t tst,
-                                              const float4 *__restrict__ h4, const float4 *__restrict__ l4,
-                                              const uint32_t *src, float hh, float hl, float lam, double scale,
-                                              double *phi, double *field, float4 (*sh)[P2P_WSRC],
-                                              float4 (*sl)[P2P_WSRC], const uint32_t *nb_start,
-                                              const uint32_t *nb_cnt, const int *nb_o, int nch) {
-  float th[2][3], tl[2][3];
-  uint32_t tk[2];
-  bool tv[2];
-#pragma unroll
-  for (int t = 0; t < 2; ++t) {
-    const uint32_t tj = t0 + lane + 32 * t;
-    tv[t] = t < NT && tj < tcnt;
-    tk[t] = tst + (tv[t] ? tj : 0);
-    const float4 a = h4[tk[t]], b = l4[tk[t]];
-    th[t][0] = a.x; th[t][1] = a.y; th[t][2] = a.z;
-    tl[t][0] = b.x; tl[t][1] = b.y; tl[t][2] = b.z;
-  }
-  auto mode_of = [&](int k) {
-    int ddx, ddy, ddz;
-    near_decode(nb_o[k], ddx, ddy, ddz);
-    const int ch = cheb3(ddx, ddy, ddz);
-    return ch == 0 ? P2P_SELF : (ch == 1 ? P2P_TOUCH : P2P_APART);
-  };
-  auto issue = [&](const P2PCursor &cc, int buf) {
-    const uint32_t first = nb_start[cc.k] + cc.off;
-    const int nn = (int)min((uint32_t)P2P_WSRC, nb_cnt[cc.k] - cc.off);
-    if (mode_of(cc.k) == P2P_APART) {
-      for (int j = lane; j < nn; j += 32) cp_async16(&sh[buf][j], &h4[first + j], true);
-    } else {
-      for (int e = lane; e < 2 * P2P_WSRC; e += 32) {
-        const int j = e >> 1;
-        if (j < nn) {
-          if (e & 1) cp_async16(&sl[buf][j], &l4[first + j], true);
-          else cp_async16(&sh[buf][j], &h4[first + j], true);
-        }
-      }
-    }
-    cp_commit();
-  };
-  float sp[2] = {0, 0}, cp[2] = {0, 0}, sx[2] = {0, 0}, cx[2] = {0, 0};
-  float sy[2] = {0, 0}, cy[2] = {0, 0}, sz[2] = {0, 0}, cz[2] = {0, 0};
-  P2PCursor ci{0, 0u}, cc{0, 0u};  // next chunk to issue, chunk being summed
-  if (nch > 0) {
-    issue(ci, 0);
-    p2p_next(ci, nb_cnt);
-  }
-  for (int c = 0; c < nch; ++c) {
-    const int buf = c & 1;
-    if (c + 1 < nch) {
-      issue(ci, buf ^ 1);
-      p2p_next(ci, nb_cnt);
-      cp_wait1();
-    } else {
-      cp_wait0();
-    }
-    __syncwarp();
-    const int nn = (int)min((uint32_t)P2P_WSRC, nb_cnt[cc.k] - cc.off);
-    int ddx, ddy, ddz;
-    near_decode(nb_o[cc.k], ddx, ddy, ddz);
-    const int mode = mode_of(cc.k);
-    p2p_next(cc, nb_cnt);
-    float px[4], py[4], pz[4], qx[4], qy[4], qz[4];
-    const float dxh = -(float)ddx, dyh = -(float)ddy, dzh = -(float)ddz;
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      two_sum_shift(th[t][0], tl[t][0], dxh * hh, dxh * hl, px[t], qx[t]);
-      two_sum_shift(th[t][1], tl[t][1], dyh * hh, dyh * hl, py[t], qy[t]);
-      two_sum_shift(th[t][2], tl[t][2], dzh * hh, dzh * hl, pz[t], qz[t]);
-    }
-    float fp[4] = {0, 0, 0, 0}, fx[4] = {0, 0, 0, 0}, fy[4] = {0, 0, 0, 0}, fz[4] = {0, 0, 0, 0};
-    if (mode == P2P_APART)
-      p2p_f32_chunk<NT, P2P_APART>(sh[buf], sl[buf], nn, px, py, pz, qx, qy, qz, lam, fp, fx, fy, fz);
-    else if (mode == P2P_TOUCH)
-      p2p_f32_chunk<NT, P2P_TOUCH>(sh[buf], sl[buf], nn, px, py, pz, qx, qy, qz, lam, fp, fx, fy, fz);
-    else
-      p2p_f32_chunk<NT, P2P_SELF>(sh[buf], sl[buf], nn, px, py, pz, qx, qy, qz, lam, fp, fx, fy, fz);
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      kahan_add(sp[t], cp[t], fp[t]);
-      kahan_add(sx[t], cx[t], fx[t]);
-      kahan_add(sy[t], cy[t], fy[t]);
-      kahan_add(sz[t], cz[t], fz[t]);
-    }
-    __syncwarp();  // buffer buf is refilled by the issue of chunk c + 2
-  }
-#pragma unroll
-  for (int t = 0; t < NT; ++t) {
-    if (!tv[t]) continue;
-    const uint32_t i = src[tk[t]];
-    phi[i] += scale * ((double)sp[t] - (double)cp[t]);
-    if (field) {
-      field[3 * i] += scale * ((double)sx[t] - (double)cx[t]);
-      field[3 * i + 1] += scale * ((double)sy[t] - (double)cy[t]);
-      field[3 * i + 2] += scale * ((double)sz[t] - (double)cz[t]);
-    }
-  }
-}
-
-__global__ void __launch_bounds__(32 * P2P_WARPS, 6) k_p2p_free_f32(const P2PJob *jobs, int njobs) {
-  __shared__ __align__(16) float4 sh_[P2P_WARPS][2][P2P_WSRC], sl_[P2P_WARPS][2][P2P_WSRC];
-  __shared__ uint32_t nb_start_[P2P_WARPS][NNEAR], nb_cnt_[P2P_WARPS][NNEAR];
-  __shared__ int nb_o_[P2P_WARPS][NNEAR];
-  int lo = 0, hi = njobs - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (jobs[mid].block0 <= (int64_t)blockIdx.x) lo = mid; else hi = mid - 1;
-  }
-  const P2PJob &J = jobs[lo];
-  const uint32_t *bstart = J.bstart, *bcount = J.bcount, *src = J.src;
-  const int32_t *ulist = J.ulist;
-  const float4 *h4 = J.h4, *l4 = J.l4;
-  const float hh = J.hh, hl = J.hl, lam = J.lam;
-  const double scale = J.scale;
-  double *phi = J.phi, *field = J.field;
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t gw = (uint32_t)((int64_t)blockIdx.x - J.block0) * P2P_WARPS + w;
-  const uint32_t box = gw >> 1, half = gw & 1;
-  if (box >= *J.d_nb) return;
-  const uint32_t tst = bstart[box], tcnt = bcount[box];
-  if (64 * half >= tcnt) return;
-  uint32_t *nb_start = nb_start_[w], *nb_cnt = nb_cnt_[w];
-  int *nb_o = nb_o_[w];
-  // compact the non-empty near boxes (slot order kept) and count their chunks
-  int nnb = 0, nch = 0;
-  for (int o0 = 0; o0 < NNEAR; o0 += 32) {
-    const int o = o0 + lane;
-    const int sb = o < NNEAR ? ulist[(size_t)box * NNEAR + o] : -1;
-    const uint32_t cnt = sb >= 0 ? bcount[sb] : 0u;
-    const unsigned m = __ballot_sync(0xffffffffu, cnt > 0);
-    if (cnt > 0) {
-      const int k = nnb + __popc(m & ((1u << lane) - 1u));
-      nb_start[k] = bstart[sb];
-      nb_cnt[k] = cnt;
-      nb_o[k] = o;
-    }
-    nnb += __popc(m);
-    int ch = (int)((cnt + P2P_WSRC - 1) / P2P_WSRC);
-#pragma unroll
-    for (int s2 = 16; s2; s2 >>= 1) ch += __shfl_xor_sync(0xffffffffu, ch, s2);
-    nch += ch;
-  }
-  __syncwarp();
-  for (uint32_t t0 = 64 * half; t0 < tcnt; t0 += 128) {
-    if (tcnt - t0 > 32)
-      p2p_warp_pass<2>(lane, t0, tcnt, tst, h4, l4, src, hh, hl, lam, scale, phi, field, sh_[w], sl_[w], nb_start,
-                       nb_cnt, nb_o, nch);
-    else
-      p2p_warp_pass<1>(lane, t0, tcnt, tst, h4, l4, src, hh, hl, lam, scale, phi, field, sh_[w], sl_[w], nb_start,
-                       nb_cnt, nb_o, nch);
-  }
-}
+#include "p2p_f32.cuh"
 
 // ---------------------------------------------------------------------------------------
 // reaction near field: target leaf box vs adjacent image leaf boxes across the interface,
@@ -1783,7 +1515,8 @@ static void launch_p2p(Ctx &c, const std::vector<P2PJob> &jobs, int64_t blocks, 
   if (jobs.empty() || blocks <= 0) return;
   P2PJob *dj = c.arena.get<P2PJob>(jobs.size());
   LPB_CUDA(cudaMemcpyAsync(dj, jobs.data(), sizeof(P2PJob) * jobs.size(), cudaMemcpyHostToDevice, st));
-  k_p2p_free_f32<<<(unsigned)blocks, 32 * P2P_WARPS, 0, st>>>(dj, (int)jobs.size());
+  if (jobs[0].field) k_p2p_free_f32<true><<<(unsigned)blocks, 32 * P2P_WARPS, 0, st>>>(dj, (int)jobs.size());
+  else k_p2p_free_f32<false><<<(unsigned)blocks, 32 * P2P_WARPS, 0, st>>>(dj, (int)jobs.size());
   LPB_LAUNCH();
   c.launches++;
 }
@@ -1816,20 +1549,20 @@ void run_near_free(Ctx &c, std::vector<Group> &groups, double *phi, double *fiel
     const unsigned nb = (unsigned)Lf.n;
     if (!nb) continue;
     const int64_t np = g.T.np;
-    float4 *h4 = c.arena.get<float4>((size_t)np), *l4 = c.arena.get<float4>((size_t)np);
+    float *pts = c.arena.get<float>((size_t)np * 7);
     k_split_points<<<nb, 64, 0, c.stream>>>(Lf.d_n, Lf.key, Lf.pstart, Lf.pcount, g.T.x, g.T.y, g.T.z, g.T.q,
-                                             geo_at<float>(g, g.Df), h4, l4);
+                                             geo_at<float>(g, g.Df), pts, np);
     LPB_LAUNCH();
     c.launches++;
     const double hD = g.h(g.Df);
     P2PJob j;
     j.d_nb = Lf.d_n; j.bkey = Lf.key; j.bstart = Lf.pstart; j.bcount = Lf.pcount; j.ulist = g.ufree;
-    j.h4 = h4; j.l4 = l4; j.src = g.T.src; j.phi = phi; j.field = field;
+    j.pts = pts; j.ld = np; j.src = g.T.src; j.phi = phi; j.field = field;
     j.scale = 1.0 / (4.0 * PI * c.md.eps[g.l]);
     j.hh = (float)hD; j.hl = (float)(hD - (double)j.hh); j.lam = (float)c.md.lam[g.l];
     j.block0 = c.def.p2p_blocks;
     c.def.p2p.push_back(j);
-    c.def.p2p_blocks += (2 * (int64_t)nb + P2P_WARPS - 1) / P2P_WARPS;
+    c.def.p2p_blocks += nb;
   }
   if (!c.def.on && !c.def.p2p.empty()) {
     LPB_CUDA(cudaEventRecord(c.ev_p2p[0], c.stream));

@@ -225,7 +225,8 @@ struct P2PJob {
   const uint64_t *bkey;     // leaf keys
   const uint32_t *bstart, *bcount;  // leaf point ranges
   const int32_t *ulist;     // [nb][NNEAR] near leaves or -1
-  const float4 *h4, *l4;    // points as FP32 hi / lo offsets from their leaf centre, charge in h4.w
+  const float *pts;         // [7][ld] offsets from the leaf centre: x, y, z hi, charge, x, y, z lo
+  int64_t ld;
   const uint32_t *src;      // input index of each point
   double *phi, *field;      // outputs (input order)
   double scale;             // 1 / (4 pi eps)

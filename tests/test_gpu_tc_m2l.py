@@ -41,3 +41,35 @@ def test_mixed_matches_fp64_on_the_same_trees(p, ws, scale, layout):
         assert ctx.status() == 0
     (a, fa), (b, fb) = out
     assert rel(b, a) < 1e-6 and rel(fb, fa) < 1e-6, (rel(b, a), rel(fb, fa))
+
+
+@pytest.mark.parametrize("n,lam,spread", [(1, 1.0, 0.1), (2, 1.0, 0.0), (33, 1.0, 0.1), (64, 1e-4, 0.1), (65, 30.0, 0.5),
+                                          (129, 1.0, 0.5), (1000, 1.0, 0.5)])
+def test_fp32_near_field_groups_and_chunks(n, lam, spread):
+    """The FP32 near field alone (depth 2, two-box lists: every pair is near) against the FP64 sum in numpy:
+    one to many target groups, chunks that span leaves and end odd, coincident charges, screening from none to strong.  The pair arithmetic is FP32 with 2^-22 special functions: relative L2 within the
+    1e-6 gate, times lambda r (the exponent's relative rounding) where that is large.  The potential alone
+    equals the potential with the field."""
+    rng = np.random.default_rng(n)
+    xyz = np.column_stack([rng.uniform(-spread, spread, n), rng.uniform(-spread, spread, n),
+                           rng.uniform(-0.6 - spread, -0.6 + spread, n)])
+    if n > 2:
+        xyz[-1] = xyz[0]
+    q = rng.uniform(0.5, 1.0, n)
+    ctx = F.Context([0.0, -1.2], [1.0, 2.0, 5.0], [0.5, lam, 0.8], 4, precision=F.MIXED, uniform_depth=2)
+    args = (torch.tensor(q, device=DEV), torch.tensor(xyz, device=DEV),
+            torch.ones(n, dtype=torch.int32, device=DEV))
+    phi, fld = (t.cpu().numpy() for t in ctx.eval(*args, parts=1))
+    only, _ = ctx.eval(*args, parts=1, field=False)
+    d = xyz[:, None, :] - xyz[None, :, :]
+    r = np.sqrt((d * d).sum(-1))
+    ri = np.divide(1.0, r, out=np.zeros_like(r), where=r > 0)
+    e = q[None, :] * np.exp(-lam * r) * ri / (4 * np.pi * 2.0)
+    ref_p, ref_f = e.sum(1), ((e * (1 + lam * r) * ri * ri)[:, :, None] * d).sum(1)
+    if n <= 2:  # no pair at a distance
+        assert np.all(phi == 0.0) and np.all(fld == 0.0)
+        return
+    tol = 1e-6 * max(1.0, lam * spread / 10)
+    assert np.linalg.norm(phi - ref_p) <= tol * np.linalg.norm(ref_p)
+    assert np.linalg.norm(fld - ref_f) <= tol * np.linalg.norm(ref_f)
+    assert np.array_equal(only.cpu().numpy(), phi)
