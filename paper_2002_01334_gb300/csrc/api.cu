@@ -367,7 +367,7 @@ static void eval_front(Ctx &c, int64_t n, const double *q, const double *xyz, co
   LPB_CUDA(cudaStreamWaitEvent(c.side, c.ev_fork, 0));
   {
     OnStream on(c, c.side);
-    for (auto &g : c.groups) build_operators(c, g, g.parts, 1);
+    build_operators(c, c.groups, 1);
     LPB_CUDA(cudaEventRecord(c.ev_free, c.side));
   }
   per_group([&](int, Group &g) {
@@ -422,7 +422,6 @@ static void eval_front(Ctx &c, int64_t n, const double *q, const double *xyz, co
     for (auto &g : c.groups)
       if (g.I.np) hmin = std::min(hmin, g.h(g.D));
     c.stab_lmin = hmin < 1e300 ? lmin * hmin : lmin;
-    c.stab_bes = nullptr;
   }
   // reaction tables, operators and near-field nodes on the side stream, after the lists (the M2L
   // waits for them)
@@ -430,8 +429,8 @@ static void eval_front(Ctx &c, int64_t n, const double *q, const double *xyz, co
   {
     OnStream on(c, c.side);
     LPB_CUDA(cudaStreamWaitEvent(c.side, c.ev_fork, 0));
+    build_operators(c, c.groups, 2);
     for (auto &g : c.groups) {
-      build_operators(c, g, g.parts, 2);
       if ((g.parts & 2) && g.ureact) {
         double zt, zs;
         z_gaps(g, zt, zs);
@@ -536,7 +535,15 @@ int lpbfmm_create(int n_iface, const double *z_iface, const double *eps, const d
     c->stream = (cudaStream_t)o.stream;
     LPB_CUDA(cudaGetDevice(&c->device));
     if (c->device < 0 || c->device >= LPB_MAX_DEVICES) throw StatusError{LPBFMM_ERR_UNSUPPORTED};
-    std::vector<double> G = gaunt_table(p);
+    std::vector<double> G;
+    {
+      const std::vector<double> g0 = gaunt_table(p);  // [a][c][q] -> [a][q][c]
+      const int NF = (p + 1) * (p + 1), NQ = 2 * p + 1;
+      G.resize(g0.size());
+      for (int x = 0; x < NF; ++x)
+        for (int y = 0; y < NF; ++y)
+          for (int q = 0; q < NQ; ++q) G[((size_t)x * NQ + q) * NF + y] = g0[((size_t)x * NF + y) * NQ + q];
+    }
     std::vector<double> tp = tpoly_table(p, c->tpk);
     LPB_CUDA(cudaMalloc(&c->gaunt, sizeof(double) * G.size()));
     LPB_CUDA(cudaMemcpy(c->gaunt, G.data(), sizeof(double) * G.size(), cudaMemcpyHostToDevice));

@@ -1122,13 +1122,13 @@ static void make_tables(Ctx &c) {
   mark_done_on_device(g_tab_ready);
 }
 
-void upload_gl16();
+void upload_gl();
 void upload_an();
 void upload_trig(cudaStream_t s);
 void init_fmm_tables(Ctx &c) {
   static std::mutex mu;
   std::lock_guard<std::mutex> lk(mu);
-  upload_gl16();
+  upload_gl();
   upload_an();
   make_tables(c);
   upload_exp2(c.stream);

@@ -261,13 +261,12 @@ struct Ctx {
   cudaStream_t stream = nullptr;
   int device = 0;
   // constant tables (device, FP64)
-  double *gaunt = nullptr;   // [(p+1)^2 in][(p+1)^2 out][2p+1]
+  double *gaunt = nullptr;   // [(p+1)^2 a][2p+1][(p+1)^2 c]: int Y_a Y_q conj(Y_c), the column c fastest
   double *tpoly = nullptr;   // [K][TPK] Legendre-product coefficients
   double *sfac = nullptr;    // [KMAX_TAB+1][KMAX_TAB+1]: sqrt((K+d)! (K-d)!) for d <= K
   double *phat_dir = nullptr;  // [NDIR][(2p+1)(2p+2)/2]: Phat_q^k(cos theta) of the operator directions
   // per evaluation: grading of the shared Sommerfeld node set and its Bessel columns
   double stab_lmin = 0.0;
-  double *stab_bes = nullptr;
   int tpk = 0;
   double *adj = nullptr;     // adjoint work space (7 n doubles), grown on demand, kept
   size_t adj_cap = 0;
@@ -339,7 +338,7 @@ void adaptive_lists(Ctx &c, Group &g, int s, int ws, std::vector<int64_t> &rec);
 // ops.cu
 // which: 1 the free-space operators (M2M, L2L, free M2L; need only the depths and roots),
 // 2 the reaction tables and operators (need the interaction lists)
-void build_operators(Ctx &c, Group &g, int parts, int which);
+void build_operators(Ctx &c, std::vector<Group> &groups, int which);
 void build_near_nodes(Ctx &c, Group &g, double zeta_min, double rho_max);
 void stable_noalloc(Ctx &c, int l, int a, int lp, int b, double h, double rho, double zt, double zs, int Kmax,
                     double *out);

@@ -63,6 +63,11 @@ __global__ void k_ops_prep(const OpDesc *descs, int nd, int p, double *prep) {
 
 constexpr int OPS_SPLIT = 4;  // CTAs per descriptor
 
+// Bound: the FP64 pipe (0.63 T FMA/s).  All three kinds are the same sum over q of
+// f_q Phat_q^{mu'-m} G(n, m; nu, mu'; q), mu' = +-mu: the product f_q Phat_q^k is formed once per
+// descriptor, so a term is one FMA (three FP64 operations before: 0.25 ms per free-space group at p = 10,
+// three levels), and the table is read with the column index fastest, so that a warp's loads
+// coalesce.
 template <typename T>
 __global__ void k_build_ops(const OpDesc *descs, const double *prep, const double *phat_dir, int p, int K,
                             const double *gaunt, T *out) {
@@ -70,11 +75,16 @@ __global__ void k_build_ops(const OpDesc *descs, const double *prep, const doubl
   __shared__ double w[NPREP], Pl[NPL_MAX];
   const double *pw = prep + (size_t)blockIdx.x * NPREP;
   for (int e = threadIdx.x; e < NPREP; e += blockDim.x) w[e] = pw[e];
-  const int npl = (2 * p + 1) * (2 * p + 2) / 2;
-  const double *pd = phat_dir + (size_t)d.dir * npl;
-  for (int e = threadIdx.x; e < npl; e += blockDim.x) Pl[e] = pd[e];
   __syncthreads();
-  const double *f = w + PREP_F, *so = w + PREP_SO, *si = w + PREP_SI;
+  const double *so = w + PREP_SO, *si = w + PREP_SI;
+  const int qmax = 2 * p, npl = (qmax + 1) * (qmax + 2) / 2;
+  const double *pd = phat_dir + (size_t)d.dir * npl;
+  for (int e = threadIdx.x; e < npl; e += blockDim.x) {
+    int q, k;
+    hdecode(e, q, k);
+    Pl[e] = w[PREP_F + q] * pd[e];
+  }
+  __syncthreads();
   const int NF = (p + 1) * (p + 1), NQ = 2 * p + 1;
   for (int e = blockIdx.y * blockDim.x + threadIdx.x; e < K * K; e += gridDim.y * blockDim.x) {
     const int o = e / K, i = e % K;
@@ -82,31 +92,25 @@ __global__ void k_build_ops(const OpDesc *descs, const double *prep, const doubl
     hdecode(o, n, m);
     hdecode(i, nu, mu);
     double r[2] = {0.0, 0.0};
+    const double *G = gaunt + (size_t)fidx(n, m) * NQ * NF;
+    const double sc = 4.0 * PI * so[n] * si[nu];
     for (int sgn = 0; sgn < 2; ++sgn) {
       const int mus = sgn ? -mu : mu;
       if (sgn && mu == 0) break;
+      const int k = mus - m, ak = k < 0 ? -k : k;
+      int q0 = n > nu ? n - nu : nu - n;
+      if (q0 < ak) q0 = ak + ((n + nu + ak) & 1);
       double acc = 0.0;
-      for (int q = abs(n - nu); q <= n + nu; q += 2) {
-        if (d.kind == 2 || d.kind == 0) {
-          const int k = m - mus;
-          if (abs(k) > q) continue;
-          acc += f[q] * phat_signed(Pl, q, k) * gaunt[((size_t)fidx(nu, mus) * NF + fidx(n, m)) * NQ + q];
-        } else {
-          const int k = mus - m;
-          if (abs(k) > q) continue;
-          acc += f[q] * phat_signed(Pl, q, k) * gaunt[((size_t)fidx(n, m) * NF + fidx(nu, mus)) * NQ + q];
-        }
-      }
-      acc *= 4.0 * PI * so[n] * si[nu];
-      if (d.kind == 0 && (n & 1)) acc = -acc;
-      r[sgn] = acc;
+      for (int q = q0; q <= n + nu; q += 2) acc = fma(Pl[hidx(q, ak)], G[(size_t)q * NF + fidx(nu, mus)], acc);
+      const bool neg = (k < 0 && (ak & 1)) != (d.kind == 0 && (n & 1));  // Phat_q^{-k} = (-1)^k Phat_q^k
+      r[sgn] = neg ? -acc * sc : acc * sc;
     }
     double P, Q;
     if (mu == 0) { P = r[0]; Q = 0.0; }
     else {
-      const double sg = (mu & 1) ? -1.0 : 1.0;
-      P = r[0] + sg * r[1];
-      Q = r[0] - sg * r[1];
+      const double r1 = (mu & 1) ? -r[1] : r[1];
+      P = r[0] + r1;
+      Q = r[0] - r1;
     }
     out[d.dst + (size_t)o * K + i] = (T)P;
     out[d.dst + (size_t)K * K + (size_t)o * K + i] = (T)Q;
@@ -123,19 +127,19 @@ struct RDesc {
   const uint8_t *used;   // [NREACT_CLS]
   double *stab;          // [NREACT_CLS][ntypes][TS]
   float2 *coef;          // [K*K][NS] double-float (hi, lo) coefficients C_s
-  int64_t dst;           // element offset of class 0, type tau in the op array
+  void *out;             // operators of class 0, type 0 of this level [NREACT_CLS][ntypes][2][K][K]
 };
-
 
 constexpr int MAXPANEL = 1024;
 
 __device__ __forceinline__ int stab_index(int KT, int K, int d, int ij) { return ((K * (KT + 1)) + d) * 4 + ij; }
 
-__device__ void make_panels(double umax, double wmax, double lmin, double *pu, double *pw, int *np) {
+// panels of width at most wmax, graded towards u = 0: at most grow (lmin + u)
+__device__ void make_panels(double umax, double wmax, double lmin, double grow, double *pu, double *pw, int *np) {
   int n = 0;
   double u = 0.0;
   while (u < umax && n < MAXPANEL) {
-    double w = fmin(wmax, 0.5 * (lmin + u));
+    double w = fmin(wmax, grow * (lmin + u));
     if (u + w > umax) w = umax - u;
     pu[n] = u;
     pw[n] = w;
@@ -145,30 +149,38 @@ __device__ void make_panels(double umax, double wmax, double lmin, double *pu, d
   *np = n;
 }
 
-// Gauss-Legendre 16-point rule on [-1,1] (nodes by Newton iteration on the host)
-__constant__ double c_glx[16], c_glw[16];
+// Gauss-Legendre rules on [-1,1] (nodes by Newton iteration on the host): 32 points for the Sommerfeld
+// tables, 16 for the reaction near field
+constexpr int GLN = 32;
+__constant__ double c_glx[16], c_glw[16], c_gl32x[GLN], c_gl32w[GLN];
 static std::atomic<uint64_t> g_gl_ready{0};
-void upload_gl16() {
-  if (!not_done_on_device(g_gl_ready)) return;
-  double x[16], w[16];
-  for (int i = 0; i < 16; ++i) {
-    long double z = cosl(3.14159265358979323846264338L * (i + 0.75L) / 16.5L), dp = 1;
+static void gl_rule(int n, double *x, double *w) {
+  for (int i = 0; i < n; ++i) {
+    long double z = cosl(3.14159265358979323846264338L * (i + 0.75L) / (n + 0.5L)), dp = 1;
     for (int it = 0; it < 100; ++it) {
       long double p0 = 1, p1 = z;
-      for (int k = 2; k <= 16; ++k) { long double p2 = ((2 * k - 1) * z * p1 - (k - 1) * p0) / k; p0 = p1; p1 = p2; }
-      dp = 16 * (z * p1 - p0) / (z * z - 1);
+      for (int k = 2; k <= n; ++k) { long double p2 = ((2 * k - 1) * z * p1 - (k - 1) * p0) / k; p0 = p1; p1 = p2; }
+      dp = n * (z * p1 - p0) / (z * z - 1);
       const long double dz = p1 / dp;
       z -= dz;
       if (fabsl(dz) < 1e-19L) break;
     }
     long double p0 = 1, p1 = z;
-    for (int k = 2; k <= 16; ++k) { long double p2 = ((2 * k - 1) * z * p1 - (k - 1) * p0) / k; p0 = p1; p1 = p2; }
-    dp = 16 * (z * p1 - p0) / (z * z - 1);
+    for (int k = 2; k <= n; ++k) { long double p2 = ((2 * k - 1) * z * p1 - (k - 1) * p0) / k; p0 = p1; p1 = p2; }
+    dp = n * (z * p1 - p0) / (z * z - 1);
     x[i] = (double)z;
     w[i] = (double)(2 / ((1 - z * z) * dp * dp));
   }
-  LPB_CUDA(cudaMemcpyToSymbol(c_glx, x, sizeof x));
-  LPB_CUDA(cudaMemcpyToSymbol(c_glw, w, sizeof w));
+}
+void upload_gl() {
+  if (!not_done_on_device(g_gl_ready)) return;
+  double x[GLN], w[GLN];
+  gl_rule(16, x, w);
+  LPB_CUDA(cudaMemcpyToSymbol(c_glx, x, sizeof(double) * 16));
+  LPB_CUDA(cudaMemcpyToSymbol(c_glw, w, sizeof(double) * 16));
+  gl_rule(GLN, x, w);
+  LPB_CUDA(cudaMemcpyToSymbol(c_gl32x, x, sizeof x));
+  LPB_CUDA(cudaMemcpyToSymbol(c_gl32w, w, sizeof w));
   mark_done_on_device(g_gl_ready);
 }
 __device__ __forceinline__ void gl16(double *x, double *w) {
@@ -176,12 +188,13 @@ __device__ __forceinline__ void gl16(double *x, double *w) {
 }
 
 // Quadrature of S^K S_{K d, ij} for d = 0, 1, K = 0..KT on one composite Gauss-Legendre node
-// set per (component, level) in u = lambda_rho h: panel width min(2/zeta_min, pi/rho_max),
-// graded near u = 0 to resolve the branch points at u = +-i Lambda.  Node data (first kernel):
+// set per (component, level) in u = lambda_rho h: panel width min(6, 3 (Lambda_min + u)), graded near
+// u = 0 to resolve the branch points at u = +-i Lambda.  Node data (k_stab_nodes):
 //   nd[q] = {u, w sigma / u_z, Lam / u_z, Lamp / u'_z, e^{-u_z (k+1/2)} (k < NKT),
-//            e^{-u'_z (k+1/2)} (k < NKT), J0(u rho_r), J1(u rho_r) (r < NRHO)}
-constexpr int ND_ET = 4, ND_ES = ND_ET + NKT, ND_J0 = ND_ES + NKT, ND_J1 = ND_J0 + NRHO;
-constexpr int NDF = ND_J1 + NRHO;
+//            e^{-u'_z (k+1/2)} (k < NKT)}
+// and, shared by every descriptor on the node set, bes[q] = {J0(u rho_r), J1(u rho_r) (r < NRHO)}.
+constexpr int ND_ET = 4, ND_ES = ND_ET + NKT, NDF = ND_ES + NKT, NBES = 2 * NRHO;
+constexpr double ST_WMAX = 6.0, ST_GROW = 3.0;
 
 // host: the u beyond which u^KT e^{-zeta u} has fallen by tol (and e^-3 more) below its peak
 // at u = KT/zeta
@@ -198,28 +211,28 @@ struct NDesc {
   double ucut[NKT];  // truncation point for zeta = k_t + k_s + 1 = 1 .. NKT
   int npan, nq;
   double *nodes;        // [nq][NDF]
-  const double *bes;    // shared J0, J1 columns of this node set [nq][2 NRHO], or null (computed here)
+  const double *bes;    // [nq][NBES]
 };
 
 // J0(u rho_r), J1(u rho_r) at the nodes of one node set, shared by every descriptor using it
 __global__ void k_stab_bessel(NDesc N, double *bes) {
   __shared__ double pu[MAXPANEL], pw[MAXPANEL];
   __shared__ int npan;
-  if (threadIdx.x == 0) make_panels(N.umax, N.wmax, N.lmin, pu, pw, &npan);
+  if (threadIdx.x == 0) make_panels(N.umax, N.wmax, N.lmin, ST_GROW, pu, pw, &npan);
   __syncthreads();
   // one thread per (node, rho value): the node set is short, so a thread per node alone would
   // leave most of the GPU idle
   const int64_t total = (int64_t)N.nq * NRHO;
   for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
     const int j = (int)(e / NRHO), r = (int)(e % NRHO);
-    double *o = bes + (size_t)j * 2 * NRHO;
-    if (j >= npan * 16) {
+    double *o = bes + (size_t)j * NBES;
+    if (j >= npan * GLN) {
       o[r] = 0.0;
       o[NRHO + r] = 0.0;
       continue;
     }
-    const int pi_ = j >> 4, gi = 15 - (j & 15);  // ascending abscissae
-    const double u = pu[pi_] + 0.5 * pw[pi_] * (c_glx[gi] + 1.0);
+    const int pi_ = j / GLN, gi = GLN - 1 - (j % GLN);  // ascending abscissae
+    const double u = pu[pi_] + 0.5 * pw[pi_] * (c_gl32x[gi] + 1.0);
     const double x = u * sqrt((double)rho2_of(r));
     o[r] = j0(x);
     o[NRHO + r] = j1(x);
@@ -231,17 +244,17 @@ __global__ void k_stab_nodes(const RDesc *descs, const NDesc *nds, Medium md) {
   const NDesc N = nds[blockIdx.y];
   __shared__ double pu[MAXPANEL], pw[MAXPANEL];
   __shared__ int npan;
-  if (threadIdx.x == 0) make_panels(N.umax, N.wmax, N.lmin, pu, pw, &npan);
+  if (threadIdx.x == 0) make_panels(N.umax, N.wmax, N.lmin, ST_GROW, pu, pw, &npan);
   __syncthreads();
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < N.nq; j += gridDim.x * blockDim.x) {
     double *o = N.nodes + (size_t)j * NDF;
-    if (j >= npan * 16) {
+    if (j >= npan * GLN) {
       for (int k = 0; k < NDF; ++k) o[k] = 0.0;
       continue;
     }
-    const int pi_ = j >> 4, gi = 15 - (j & 15);  // ascending abscissae
-    const double u = pu[pi_] + 0.5 * pw[pi_] * (c_glx[gi] + 1.0);
-    const double w = 0.5 * pw[pi_] * c_glw[gi];
+    const int pi_ = j / GLN, gi = GLN - 1 - (j % GLN);  // ascending abscissae
+    const double u = pu[pi_] + 0.5 * pw[pi_] * (c_gl32x[gi] + 1.0);
+    const double w = 0.5 * pw[pi_] * c_gl32w[gi];
     const double sg = layer_sigma(md, u / D.h, D.l, D.a, D.lp, D.b);
     const double uz = sqrt(D.Lam * D.Lam + u * u), uzp = sqrt(D.Lamp * D.Lamp + u * u);
     o[0] = u;
@@ -252,126 +265,7 @@ __global__ void k_stab_nodes(const RDesc *descs, const NDesc *nds, Medium md) {
       o[ND_ET + k] = exp(-uz * (k + 0.5));
       o[ND_ES + k] = exp(-uzp * (k + 0.5));
     }
-    if (N.bes) {
-      const double *b = N.bes + (size_t)j * 2 * NRHO;
-      for (int r = 0; r < 2 * NRHO; ++r) o[ND_J0 + r] = b[r];
-    } else {
-      for (int r = 0; r < NRHO; ++r) {
-        const double x = u * sqrt((double)rho2_of(r));
-        o[ND_J0 + r] = j0(x);
-        o[ND_J1 + r] = j1(x);
-      }
-    }
   }
-}
-
-// One CTA per used class.  Per chunk of 256 nodes the power columns u^K (K = 0..KT) and the
-// eight node values v_{d,ij} = w sigma/u_z (Lam/u_z)^i (Lamp/u'_z)^j Z_{kt,ks} J_d(u rho) are
-// staged in shared memory; thread (d, i, j, K) accumulates sum_q u_q^K v_{d,ij}(q), a
-// [KT+1 x Q] x [Q x 8] product in FP64, for the entries with K - d odd: the operators use
-// only those, because K = 1 + |m| + |mu| + 2s and d = |mu - m| differ by an odd number.
-constexpr int SQ_CHUNK = 256, SQ_LD = SQ_CHUNK + 1;
-__global__ void k_stab_quad(const RDesc *descs, const NDesc *nds, int KT, const double *sfac) {
-  const RDesc D = descs[blockIdx.y];
-  const NDesc N = nds[blockIdx.y];
-  const int cls = blockIdx.x;
-  if (D.used && !D.used[cls]) return;
-  extern __shared__ double sqsm[];
-  double *Pw = sqsm;                          // [KT+1][SQ_LD] powers
-  double *V = sqsm + (size_t)(KT + 1) * SQ_LD;  // [8][SQ_LD] node values
-  const int ri = cls / NKK, kk = cls % NKK;
-  int kt, ks;
-  kk_decode(kk, kt, ks);
-  const double ucut = N.ucut[kt + ks];
-  // output of this thread: d, ij, K with K - d odd
-  const int n0 = (KT + 1) / 2, n1 = KT / 2;  // K odd (d = 0): 1,3,..; K even >= 2 (d = 1): 2,4,..
-  const int nout = 4 * (n0 + n1);
-  int od = 0, oij = 0, oK = -1;
-  if ((int)threadIdx.x < nout) {
-    const int t = threadIdx.x;
-    oij = t & 3;
-    const int r = t >> 2;
-    if (r < n0) { od = 0; oK = 2 * r + 1; } else { od = 1; oK = 2 * (r - n0) + 2; }
-  }
-  double acc = 0.0;
-  for (int c0 = 0; c0 < N.nq; c0 += SQ_CHUNK) {
-    const int q = c0 + threadIdx.x;
-    double u = 0.0;
-    if (q < N.nq) {
-      const double *o = N.nodes + (size_t)q * NDF;
-      u = o[0];
-      const double base = o[1] * o[ND_ET + kt] * o[ND_ES + ks];
-      const double j0v = o[ND_J0 + ri], j1v = o[ND_J1 + ri], fi = o[2], fj = o[3];
-      const bool in = u <= ucut && u > 0.0;
-      const double b0 = in ? base * j0v : 0.0, b1 = in ? base * j1v : 0.0;
-      V[0 * SQ_LD + threadIdx.x] = b0;
-      V[1 * SQ_LD + threadIdx.x] = b0 * fj;
-      V[2 * SQ_LD + threadIdx.x] = b0 * fi;
-      V[3 * SQ_LD + threadIdx.x] = b0 * fi * fj;
-      V[4 * SQ_LD + threadIdx.x] = b1;
-      V[5 * SQ_LD + threadIdx.x] = b1 * fj;
-      V[6 * SQ_LD + threadIdx.x] = b1 * fi;
-      V[7 * SQ_LD + threadIdx.x] = b1 * fi * fj;
-    } else {
-      for (int k = 0; k < 8; ++k) V[k * SQ_LD + threadIdx.x] = 0.0;
-    }
-    double pw = 1.0;
-    for (int K = 0; K <= KT; ++K) {
-      Pw[K * SQ_LD + threadIdx.x] = pw;
-      pw *= u;
-    }
-    __syncthreads();
-    if (oK >= 0) {
-      const double *pr = Pw + oK * SQ_LD, *vr = V + (od * 4 + oij) * SQ_LD;
-      const int nn = min(SQ_CHUNK, N.nq - c0);
-      for (int j = 0; j < nn; ++j) acc = fma(pr[j], vr[j], acc);
-    }
-    __syncthreads();
-    if (c0 + SQ_CHUNK < N.nq && N.nodes[(size_t)(c0 + SQ_CHUNK) * NDF] > ucut) break;
-  }
-  double *S = D.stab + ((size_t)(cls - D.cls0) * D.ntypes + D.tau) * (size_t)((KT + 1) * (KT + 1) * 4);
-  if (oK >= 0) {
-    const double nrm = 1.0 / sfac[oK * (KMAX_TAB + 1) + od];
-    S[stab_index(KT, oK, od, oij)] = acc * nrm;
-  }
-  // entries with K - d even for d = 0, 1 are not used by the operators: zero
-  for (int e = threadIdx.x; e < (KT + 1) * 2 * 4; e += blockDim.x) {
-    const int K = e / 8, d = (e >> 2) & 1, ij = e & 3;
-    if (((K - d) & 1) == 0 && K >= d) S[stab_index(KT, K, d, ij)] = 0.0;
-  }
-}
-static size_t stab_quad_smem(int KT) { return sizeof(double) * (size_t)(KT + 1 + 8) * SQ_LD; }
-
-// host: node set of one (component, level) covering every class (zeta >= 1, rho <= sqrt(50) h)
-// number of panels of the graded rule (host mirror of make_panels)
-static int count_panels(double umax, double wmax, double lmin) {
-  int n = 0;
-  double u = 0.0;
-  while (u < umax && n < MAXPANEL) {
-    double w = fmin(wmax, 0.5 * (lmin + u));
-    if (u + w > umax) w = umax - u;
-    u += w;
-    ++n;
-  }
-  return n;
-}
-
-// Panel width 2 in u = lambda_rho h: with rho <= sqrt(50) the Bessel factor J_d(u rho) has
-// derivatives bounded by rho^n, and the 16-point Gauss rule's error term on a width-2 panel,
-// rho^32 2^33 (16!)^4 / (33 (32!)^3), is ~1e-18 of the integrand's scale (~1e-25 for
-// rho <= sqrt(18)); the factors e^{-zeta u} (zeta <= NKT) are smoother still.  The panels are graded towards u = 0, where the
-// branch points u = +-i Lambda of u_z sit.
-static NDesc node_desc(int KT, double tol, double Lam, double Lamp) {
-  NDesc N;
-  N.umax = node_umax(KT, 1.0, tol);
-  for (int z = 0; z < NKT; ++z) N.ucut[z] = node_umax(KT, z + 1.0, tol);
-  N.wmax = 2.0;
-  N.lmin = fmin(Lam, Lamp);
-  N.npan = count_panels(N.umax, N.wmax, N.lmin);
-  N.nq = N.npan * 16;
-  N.nodes = nullptr;
-  N.bes = nullptr;
-  return N;
 }
 
 // a_n = sqrt(n (n+1)) and 1/a_n for n <= 2 KMAX_TAB + 1 (host, long double), for the recurrence
@@ -390,30 +284,161 @@ void upload_an() {
   mark_done_on_device(g_an_ready);
 }
 
-// forward recurrence in d (Sec. 3.5 eq. recurrence1), one warp per class:
-//   S_{K,d+1} = (2d / a_{K+d}) (1/rho) S_{K-1,d} - (a_{K-d} / a_{K+d}) S_{K,d-1}
-__global__ void k_stab_recur(const RDesc *descs, int KT) {
+// Tables of ST_NC classes with one (k_t, k_s) and consecutive rho per CTA: the d = 0, 1 columns by quadrature,
+// then the forward recurrence in d (Sec. 3.5 eq. recurrence1),
+//   S_{K,d+1} = (2d / a_{K+d}) (1/rho) S_{K-1,d} - (a_{K-d} / a_{K+d}) S_{K,d-1}.
+// Only the entries with K - d odd are formed: the operators use no others, because
+// K = 1 + |m| + |mu| + 2s and d = |mu - m| differ by an odd number (and the recurrence stays among them).
+// Quadrature: per chunk of ST_CH nodes the power columns u^K and, per class, the eight node values
+// v_{d,ij} = w sigma/u_z (Lam/u_z)^i (Lamp/u'_z)^j Z_{kt,ks} J_d(u rho) are staged in shared memory; thread
+// (class, d, i, j, K) accumulates sum_q u_q^K v_{d,ij}(q), a [KT+1 x Q] x [Q x 8] product.
+// Bound: the FP64 pipe (86 % busy with one class per CTA and 16-point panels of width 2: 0.26 ms a group
+// at p = 10).  So: the powers once for four classes, nodes beyond the class's cut not at all, and 32-point
+// panels of width 6, which need a third fewer nodes: with |zeta + i rho| <= 8.7 the rule's error on a
+// panel is (e omega / 128)^64, omega <= 26, ~1e-17 of the integrand's scale (16 points on width 2: 1e-14);
+// towards u = 0, panels of 3 (Lambda + u) with the branch points at +-i Lambda: below 1e-20.
+constexpr int ST_NC = 4, ST_CH = 128, ST_LD = ST_CH + 1, ST_THREADS = 384, ST_NOUT = 2;
+static_assert(NRHO % ST_NC == 0, "classes of a CTA share (k_t, k_s)");
+static_assert(4 * KMAX_TAB * ST_NC <= ST_NOUT * ST_THREADS, "outputs per thread");
+__global__ void __launch_bounds__(ST_THREADS) k_stab_table(const RDesc *descs, const NDesc *nds, int KT,
+                                                           const double *sfac) {
   const RDesc D = descs[blockIdx.y];
-  const int cls = blockIdx.x;
-  if (D.used && !D.used[cls]) return;
-  const int ri = cls / NKK;
-  const double rh = sqrt((double)rho2_of(ri));
-  const double irh = rh > 0.0 ? 1.0 / rh : 0.0;
-  double *S = D.stab + ((size_t)(cls - D.cls0) * D.ntypes + D.tau) * (size_t)((KT + 1) * (KT + 1) * 4);
-  const int lane = threadIdx.x;
+  const NDesc N = nds[blockIdx.y];
+  const int kk = blockIdx.x / (NRHO / ST_NC), ri0 = (blockIdx.x % (NRHO / ST_NC)) * ST_NC;
+  unsigned use = 0;
+  for (int r = 0; r < ST_NC; ++r)
+    if (!D.used || D.used[(ri0 + r) * NKK + kk]) use |= 1u << r;
+  if (!use) return;
+  extern __shared__ double stsm[];
+  double *Pw = stsm;                               // [KT+1][ST_LD] powers
+  double *V = Pw + (size_t)(KT + 1) * ST_LD;       // [ST_NC][8][ST_LD] node values
+  double *col = V + (size_t)ST_NC * 8 * ST_LD;     // [3][ST_NC][(KT+1) 4] columns d - 1, d, d + 1
+  const int cl = (KT + 1) * 4;
+  int kt, ks;
+  kk_decode(kk, kt, ks);
+  const double ucut = N.ucut[kt + ks];
+  const int tid = threadIdx.x;
+  // outputs of this thread: class, d, ij, K with K - d odd
+  const int n0 = (KT + 1) / 2, n1 = KT / 2;  // K odd (d = 0): 1,3,..; K even >= 2 (d = 1): 2,4,..
+  const int nout = 4 * (n0 + n1);
+  int orr[ST_NOUT], od[ST_NOUT], oij[ST_NOUT], oK[ST_NOUT];
+  double acc[ST_NOUT];
+#pragma unroll
+  for (int x = 0; x < ST_NOUT; ++x) {
+    const int t = tid + x * ST_THREADS;
+    acc[x] = 0.0;
+    oK[x] = -1;
+    orr[x] = od[x] = oij[x] = 0;
+    if (t < nout * ST_NC && ((use >> (t / nout)) & 1u)) {
+      orr[x] = t / nout;
+      const int o = t % nout, k = o >> 2;
+      oij[x] = o & 3;
+      od[x] = k < n0 ? 0 : 1;
+      oK[x] = k < n0 ? 2 * k + 1 : 2 * (k - n0) + 2;
+    }
+  }
+  for (int c0 = 0; c0 < N.nq; c0 += ST_CH) {
+    bool in = false;
+    if (tid < ST_CH && c0 + tid < N.nq) {
+      const double u = N.nodes[(size_t)(c0 + tid) * NDF];
+      in = u <= ucut && u > 0.0;
+      if (in) {
+        double pw = u;
+        for (int K = 1; K <= KT; ++K) {
+          Pw[K * ST_LD + tid] = pw;
+          pw *= u;
+        }
+      }
+    }
+    const int nn = __syncthreads_count(in);  // the nodes ascend: those within the cut come first
+    for (int e = tid; e < ST_NC * ST_CH; e += ST_THREADS) {
+      const int r = e / ST_CH, j = e % ST_CH;
+      if (j >= nn || !((use >> r) & 1u)) continue;
+      const double *o = N.nodes + (size_t)(c0 + j) * NDF, *bs = N.bes + (size_t)(c0 + j) * NBES + ri0 + r;
+      const double base = o[1] * o[ND_ET + kt] * o[ND_ES + ks], fi = o[2], fj = o[3], ff = fi * fj;
+      const double b0 = base * bs[0], b1 = base * bs[NRHO];
+      double *v = V + (size_t)r * 8 * ST_LD + j;
+      v[0 * ST_LD] = b0;
+      v[1 * ST_LD] = b0 * fj;
+      v[2 * ST_LD] = b0 * fi;
+      v[3 * ST_LD] = b0 * ff;
+      v[4 * ST_LD] = b1;
+      v[5 * ST_LD] = b1 * fj;
+      v[6 * ST_LD] = b1 * fi;
+      v[7 * ST_LD] = b1 * ff;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int x = 0; x < ST_NOUT; ++x)
+      if (oK[x] >= 0) {
+        const double *pr = Pw + oK[x] * ST_LD, *vr = V + (orr[x] * 8 + od[x] * 4 + oij[x]) * ST_LD;
+        double a = acc[x];
+        for (int j = 0; j < nn; ++j) a = fma(pr[j], vr[j], a);
+        acc[x] = a;
+      }
+    __syncthreads();
+    if (nn < ST_CH) break;
+  }
+  const size_t TS = (size_t)(KT + 1) * (KT + 1) * 4;
+  auto table = [&](int r) {
+    return D.stab + ((size_t)((ri0 + r) * NKK + kk - D.cls0) * D.ntypes + D.tau) * TS;
+  };
+#pragma unroll
+  for (int x = 0; x < ST_NOUT; ++x)
+    if (oK[x] >= 0) {
+      const double v = acc[x] * (1.0 / sfac[oK[x] * (KMAX_TAB + 1) + od[x]]);
+      table(orr[x])[stab_index(KT, oK[x], od[x], oij[x])] = v;
+      col[(od[x] * ST_NC + orr[x]) * cl + oK[x] * 4 + oij[x]] = v;
+    }
+  __syncthreads();
   for (int d = 1; d < KT; ++d) {
-    for (int e = lane; e < (KT + 1) * 4; e += 32) {
-      const int K = e >> 2, ij = e & 3;
-      if (K < d + 1) continue;
+    const int per = 4 * ((KT - d) / 2);  // K = d + 2, d + 4, ...
+    const double *c1 = col + (d % 3) * ST_NC * cl, *c0 = col + ((d - 1) % 3) * ST_NC * cl;
+    double *c2 = col + ((d + 1) % 3) * ST_NC * cl;
+    for (int e = tid; e < per * ST_NC; e += ST_THREADS) {
+      const int r = e / per, x = e % per, K = d + 2 + 2 * (x >> 2), ij = x & 3;
+      if (!((use >> r) & 1u)) continue;
+      const double rh = sqrt((double)rho2_of(ri0 + r));
       double v = 0.0;
       if (rh > 0.0) {
         const double ia = c_ian[K + d];
-        v = (2.0 * d * ia * irh) * S[stab_index(KT, K - 1, d, ij)] - (c_an[K - d] * ia) * S[stab_index(KT, K, d - 1, ij)];
+        v = (2.0 * d * ia * (1.0 / rh)) * c1[r * cl + (K - 1) * 4 + ij] - (c_an[K - d] * ia) * c0[r * cl + K * 4 + ij];
       }
-      S[stab_index(KT, K, d + 1, ij)] = v;
+      c2[r * cl + K * 4 + ij] = v;
+      table(r)[stab_index(KT, K, d + 1, ij)] = v;
     }
-    __syncwarp();
+    __syncthreads();
   }
+}
+static size_t stab_table_smem(int KT) {
+  return sizeof(double) * ((size_t)(KT + 1 + ST_NC * 8) * ST_LD + (size_t)3 * ST_NC * (KT + 1) * 4);
+}
+
+// host: node set of one (component, level) covering every class (zeta >= 1, rho <= sqrt(50) h)
+// number of panels of the graded rule (host mirror of make_panels)
+static int count_panels(double umax, double wmax, double lmin, double grow) {
+  int n = 0;
+  double u = 0.0;
+  while (u < umax && n < MAXPANEL) {
+    double w = fmin(wmax, grow * (lmin + u));
+    if (u + w > umax) w = umax - u;
+    u += w;
+    ++n;
+  }
+  return n;
+}
+
+static NDesc node_desc(int KT, double tol, double Lam, double Lamp) {
+  NDesc N;
+  N.umax = node_umax(KT, 1.0, tol);
+  for (int z = 0; z < NKT; ++z) N.ucut[z] = node_umax(KT, z + 1.0, tol);
+  N.wmax = ST_WMAX;
+  N.lmin = fmin(Lam, Lamp);
+  N.npan = count_panels(N.umax, N.wmax, N.lmin, ST_GROW);
+  N.nq = N.npan * GLN;
+  N.nodes = nullptr;
+  N.bes = nullptr;
+  return N;
 }
 
 // C_s(n,m,nu,mu) = sum_{k+k'=s} c^{nm}_k c^{nu mu}_{k'} Lam^{n-m-2k} Lamp^{nu-mu-2k'}
@@ -475,15 +500,23 @@ __device__ __forceinline__ void df_fma(float2 a, float2 b, float2 &acc) {
   acc = make_float2(hi, __fsub_rn(t, __fsub_rn(hi, s)));
 }
 
-// ASM_CC classes per CTA share each entry's decode and coefficient loads
+// ASM_CC classes per CTA share each entry's decode and coefficient loads.  The tables sit in shared memory by
+// (d, t), K = d + 1 + 2t (the entries with K - d odd, no others are read), a quarter of the square
+// [K][d] array, so that six CTAs fit an SM instead of three; rows are padded to an odd number of records.
+// Every level and type of every group in one launch: the levels one after another (300 CTAs each) left
+// most of the GPU idle (0.11 ms a level, 1.55 ms in all at p = 10).
 constexpr int ASM_CC = 4;
+LPB_HD int asm_row(int KT) { return (KT + 1) / 2 * 4 + 1; }
+LPB_HD int asm_size(int p, int KT) { return (2 * p + 1) * asm_row(KT); }
 template <typename T>
-__global__ void k_react_assemble(const RDesc *descs, int p, int K, int KT, const double *sfac, T *out) {
+__global__ void k_react_assemble(const RDesc *descs, int p, int K, int KT, const double *sfac) {
   const RDesc D = descs[blockIdx.y];
   const int cls0 = blockIdx.x * ASM_CC;
   extern __shared__ double asm_sm[];
-  const int TS = (KT + 1) * (KT + 1) * 4;
-  float2 *Sf = (float2 *)asm_sm;  // [ASM_CC][TS]: sqrt((K+d)!(K-d)!) S^K S_{K d, ij}, double-float
+  const size_t TS = (size_t)(KT + 1) * (KT + 1) * 4;
+  const int AR = asm_row(KT), AS = asm_size(p, KT), NT = (KT + 1) / 2;
+  float2 *Sf = (float2 *)asm_sm;  // [ASM_CC][AS]: sqrt((K+d)!(K-d)!) S^K S_{K d, ij}, double-float
+  T *out = (T *)D.out;
   __shared__ double smm[PMAX + 1], rdf[PMAX + 1];
   __shared__ double fa[KHALF_MAX], fb[KHALF_MAX];  // prefactor A(o, i) = fa[o] fb[i]
   __shared__ float faf[KHALF_MAX], fbf[KHALF_MAX];  // the same in FP32 (FP32 operators, p <= 12)
@@ -498,10 +531,11 @@ __global__ void k_react_assemble(const RDesc *descs, int p, int K, int KT, const
   if (!any) return;
   for (int k = 0; k < ASM_CC; ++k) {
     if (!cuse[k]) continue;
-    const double *S = D.stab + ((size_t)(cls0 + k - D.cls0) * D.ntypes + D.tau) * (size_t)TS;
-    for (int e = threadIdx.x; e < TS; e += blockDim.x) {
-      const int Kk = e / ((KT + 1) * 4), d = (e / 4) % (KT + 1);
-      Sf[k * TS + e] = df_split((d <= Kk) ? sfac[Kk * (KMAX_TAB + 1) + d] * S[e] : 0.0);
+    const double *S = D.stab + ((size_t)(cls0 + k - D.cls0) * D.ntypes + D.tau) * TS;
+    for (int e = threadIdx.x; e < (2 * p + 1) * NT * 4; e += blockDim.x) {
+      const int d = e / (NT * 4), x = e % (NT * 4), Kk = d + 1 + 2 * (x >> 2);
+      if (Kk <= KT)
+        Sf[k * AS + d * AR + x] = df_split(sfac[Kk * (KMAX_TAB + 1) + d] * S[stab_index(KT, Kk, d, x & 3)]);
     }
   }
   if (threadIdx.x == 0) {
@@ -549,11 +583,11 @@ __global__ void k_react_assemble(const RDesc *descs, int p, int K, int KT, const
       const int Kk = 1 + m + mu + 2 * s;
       if (s > smax || Kk > KT) break;
       const float2 c = cv[s];
-      const int ip = ((Kk * (KT + 1)) + adp) * 4 + ij, im = ((Kk * (KT + 1)) + dm) * 4 + ij;
+      const int ip = adp * AR + ((m < mu ? m : mu) + s) * 4 + ij, im = dm * AR + s * 4 + ij;
 #pragma unroll
       for (int k = 0; k < ASM_CC; ++k) {
-        df_fma(c, Sf[k * TS + ip], ap[k]);
-        df_fma(c, Sf[k * TS + im], am[k]);
+        df_fma(c, Sf[k * AS + ip], ap[k]);
+        df_fma(c, Sf[k * AS + im], am[k]);
       }
     }
     // signs: (-1)^|d| for d = mu - m < 0 and for d = -mu - m < 0; (-1)^mu of the -mu term
@@ -563,7 +597,7 @@ __global__ void k_react_assemble(const RDesc *descs, int p, int K, int KT, const
       if (!cuse[k]) continue;
       const float2 Xd = fp ? make_float2(-ap[k].x, -ap[k].y) : ap[k];
       const float2 Yd = fm ? make_float2(-am[k].x, -am[k].y) : am[k];
-      T *dP = out + D.dst + (size_t)(cls0 + k) * D.ntypes * 2 * KK + (size_t)D.tau * 2 * KK + (size_t)o * K + i;
+      T *dP = out + (size_t)(cls0 + k) * D.ntypes * 2 * KK + (size_t)D.tau * 2 * KK + (size_t)o * K + i;
       T *dQ = dP + KK;
       if (f32_out) {
         const float Af = faf[o] * fbf[i];
@@ -583,7 +617,7 @@ __global__ void k_react_assemble(const RDesc *descs, int p, int K, int KT, const
     }
   }
 }
-static size_t assemble_smem(int KT) { return ASM_CC * sizeof(double) * (size_t)(KT + 1) * (KT + 1) * 4; }
+static size_t assemble_smem(int p, int KT) { return ASM_CC * sizeof(float2) * (size_t)asm_size(p, KT); }
 
 // near-field reaction quadrature nodes: W = w lr sigma / (4 pi lz_l), lz_l, lz_l'
 __global__ void k_near_nodes(Medium md, int l, int a, int ntypes, double umax, double wmax, double lmin,
@@ -593,7 +627,7 @@ __global__ void k_near_nodes(Medium md, int l, int a, int ntypes, double umax, d
   __shared__ int npan;
   if (threadIdx.x == 0) {
     gl16(gx, gw);
-    make_panels(umax, wmax, lmin, pu, pw, &npan);
+    make_panels(umax, wmax, lmin, 0.5, pu, pw, &npan);
   }
   __syncthreads();
   const int tau = blockIdx.y;
@@ -613,12 +647,20 @@ __global__ void k_near_nodes(Medium md, int l, int a, int ntypes, double umax, d
   }
 }
 
+// nodes and tables of nd descriptors (two launches)
+static void launch_tables(Ctx &c, const RDesc *dr, const NDesc *dn, int nq, unsigned nd, int KT) {
+  k_stab_nodes<<<dim3((unsigned)((nq + 127) / 128), nd), 128, 0, c.stream>>>(dr, dn, c.md);
+  LPB_LAUNCH();
+  LPB_ATTR_ONCE(k_stab_table, stab_table_smem(KMAX_TAB));  // the largest table any order needs
+  k_stab_table<<<dim3(NKK * (NRHO / ST_NC), nd), ST_THREADS, stab_table_smem(KT), c.stream>>>(dr, dn, KT, c.sfac);
+  LPB_LAUNCH();
+}
+
+// the free-space operators of every group: one launch of the radial factors, one of the operators
 template <typename T>
-static void build_ops_t(Ctx &c, Group &g, int parts, int which) {
+static void build_free_t(Ctx &c, std::vector<Group> &groups) {
   const int p = c.p, K = c.K;
   const size_t KK = (size_t)K * K;
-  const double lam_t = c.md.lam[g.l];
-  if (which & 1) {
   std::vector<OpDesc> descs;
   size_t total = 0;
   auto add = [&](int kind, int out_inv, int in_inv, double lam, double bx, double by, double bz, double xout,
@@ -631,163 +673,147 @@ static void build_ops_t(Ctx &c, Group &g, int parts, int which) {
     d.xout = xout; d.xin = xin; d.pref = pref;
     d.dst = (int64_t)(total + offset_in_slot);
     descs.push_back(d);
-      };
-  // layout: per level a block with M2M (free + types), L2L, free M2L classes
+  };
+  // layout: per group and level a block with M2M (free + types), L2L, free M2L classes
   struct Blk { size_t m2m_t, m2m_i, l2l, fm2l; };
-  std::vector<Blk> blk(DMAX + 1);
-  for (int l = 2; l <= g.D; ++l) {
-    const double h = g.h(l), hc = h, hp = 2.0 * h;
-    Blk b{};
-    // M2M: children at level l -> parents at l-1 (only l >= 3)
-    const bool free_l = g.is_free && (parts & 1) && l <= g.Df;  // free-space part lives at levels <= Df
-    if (l >= 3) {
-      if (free_l) {
-        b.m2m_t = total;
+  std::vector<Blk> blk(groups.size() * (DMAX + 1));
+  for (size_t gi = 0; gi < groups.size(); ++gi) {
+    const Group &g = groups[gi];
+    const int parts = g.parts;
+    const double lam_t = c.md.lam[g.l];
+    for (int l = 2; l <= g.D; ++l) {
+      const double h = g.h(l), hc = h, hp = 2.0 * h;
+      Blk b{};
+      // M2M: children at level l -> parents at l-1 (only l >= 3)
+      const bool free_l = g.is_free && (parts & 1) && l <= g.Df;  // free-space part lives at levels <= Df
+      if (l >= 3) {
+        if (free_l) {
+          b.m2m_t = total;
+          for (int cz = 0; cz < 2; ++cz)
+            add(1, 1, 0, lam_t, 0.5 * hc, 0.5 * hc, (cz ? 0.5 : -0.5) * hc, lam_t * hp, lam_t * hc, 1.0,
+                NFREE_CLS + cz, (size_t)cz * 2 * KK);
+          total += 4 * KK;
+        }
+        if (parts & 2) {
+          b.m2m_i = total;
+          for (int t = 0; t < g.ntypes; ++t) {
+            int lp, bb;
+            type_decode(t, lp, bb);
+            const double la = c.md.lam[lp];
+            for (int cz = 0; cz < 2; ++cz)
+              add(1, 1, 0, la, 0.5 * hc, 0.5 * hc, (cz ? 0.5 : -0.5) * hc, la * hp, la * hc, 1.0, NFREE_CLS + cz,
+                  ((size_t)t * 2 + cz) * 2 * KK);
+          }
+          total += (size_t)g.ntypes * 4 * KK;
+        }
+        // L2L: parent (l-1) -> child at l
+        b.l2l = total;
         for (int cz = 0; cz < 2; ++cz)
-          add(1, 1, 0, lam_t, 0.5 * hc, 0.5 * hc, (cz ? 0.5 : -0.5) * hc, lam_t * hp, lam_t * hc, 1.0,
+          add(2, 0, 1, lam_t, 0.5 * hc, 0.5 * hc, (cz ? 0.5 : -0.5) * hc, lam_t * hc, lam_t * hp, 1.0,
               NFREE_CLS + cz, (size_t)cz * 2 * KK);
         total += 4 * KK;
       }
-      if (parts & 2) {
-        b.m2m_i = total;
-        for (int t = 0; t < g.ntypes; ++t) {
-          int lp, bb;
-          type_decode(t, lp, bb);
-          const double la = c.md.lam[lp];
-          for (int cz = 0; cz < 2; ++cz)
-            add(1, 1, 0, la, 0.5 * hc, 0.5 * hc, (cz ? 0.5 : -0.5) * hc, la * hp, la * hc, 1.0, NFREE_CLS + cz,
-                ((size_t)t * 2 + cz) * 2 * KK);
-        }
-        total += (size_t)g.ntypes * 4 * KK;
+      if (free_l) {
+        b.fm2l = total;
+        const double pref = lam_t / (2.0 * PI * PI * c.md.eps[g.l]);
+        for (int ri = 0; ri < NRHO; ++ri)
+          for (int dz = -OFF_R; dz <= OFF_R; ++dz) {
+            const int cls = ri * NDZ + dz + OFF_R;
+            if (!free_class_is_far(ri, dz, c.ws)) continue;
+            // b = c_t - c_s = -(offset) h; azimuth factored out: b = (rho h, 0, -dz h)
+            add(0, 0, 0, lam_t, sqrt((double)rho2_of(ri)) * h, 0.0, -dz * h, lam_t * h, lam_t * h, pref, cls,
+                (size_t)cls * 2 * KK);
+          }
+        total += (size_t)NFREE_CLS * 2 * KK;
       }
-      // L2L: parent (l-1) -> child at l
-      b.l2l = total;
-      for (int cz = 0; cz < 2; ++cz)
-        add(2, 0, 1, lam_t, 0.5 * hc, 0.5 * hc, (cz ? 0.5 : -0.5) * hc, lam_t * hc, lam_t * hp, 1.0,
-            NFREE_CLS + cz, (size_t)cz * 2 * KK);
-      total += 4 * KK;
+      blk[gi * (DMAX + 1) + l] = b;
     }
-    if (free_l) {
-      b.fm2l = total;
-      const double pref = lam_t / (2.0 * PI * PI * c.md.eps[g.l]);
-      for (int ri = 0; ri < NRHO; ++ri)
-        for (int dz = -OFF_R; dz <= OFF_R; ++dz) {
-          const int cls = ri * NDZ + dz + OFF_R;
-          if (!free_class_is_far(ri, dz, c.ws)) continue;
-          // b = c_t - c_s = -(offset) h; azimuth factored out: b = (rho h, 0, -dz h)
-          add(0, 0, 0, lam_t, sqrt((double)rho2_of(ri)) * h, 0.0, -dz * h, lam_t * h, lam_t * h, pref, cls,
-              (size_t)cls * 2 * KK);
-        }
-      total += (size_t)NFREE_CLS * 2 * KK;
-    }
-    blk[l] = b;
   }
   T *ops = c.arena.get<T>(total);
-  for (int l = 2; l <= g.D; ++l) {
-    const bool free_l = g.is_free && (parts & 1) && l <= g.Df;
-    g.op_m2m_t[l] = (l >= 3 && free_l) ? (void *)(ops + blk[l].m2m_t) : nullptr;
-    g.op_m2m_i[l] = (l >= 3 && (parts & 2)) ? (void *)(ops + blk[l].m2m_i) : nullptr;
-    g.op_l2l[l] = (l >= 3) ? (void *)(ops + blk[l].l2l) : nullptr;
-    g.op_free[l] = free_l ? (void *)(ops + blk[l].fm2l) : nullptr;
+  for (size_t gi = 0; gi < groups.size(); ++gi) {
+    Group &g = groups[gi];
+    for (int l = 2; l <= g.D; ++l) {
+      const Blk &b = blk[gi * (DMAX + 1) + l];
+      const bool free_l = g.is_free && (g.parts & 1) && l <= g.Df;
+      g.op_m2m_t[l] = (l >= 3 && free_l) ? (void *)(ops + b.m2m_t) : nullptr;
+      g.op_m2m_i[l] = (l >= 3 && (g.parts & 2)) ? (void *)(ops + b.m2m_i) : nullptr;
+      g.op_l2l[l] = (l >= 3) ? (void *)(ops + b.l2l) : nullptr;
+      g.op_free[l] = free_l ? (void *)(ops + b.fm2l) : nullptr;
+    }
   }
-  if (!descs.empty()) {
-    OpDesc *dd = c.arena.get<OpDesc>(descs.size());
-    LPB_CUDA(cudaMemcpyAsync(dd, descs.data(), sizeof(OpDesc) * descs.size(), cudaMemcpyHostToDevice, c.stream));
-    double *prep = c.arena.get<double>(descs.size() * NPREP);
-    k_ops_prep<<<(unsigned)((descs.size() + 63) / 64), 64, 0, c.stream>>>(dd, (int)descs.size(), p, prep);
-    LPB_LAUNCH();
-    k_build_ops<T><<<dim3((unsigned)descs.size(), OPS_SPLIT), 256, 0, c.stream>>>(dd, prep, c.phat_dir, p, K,
-                                                                                  c.gaunt, ops);
-    LPB_LAUNCH();
-    c.launches += 2;
-  }
-  }
-  if (!(which & 2) || !(parts & 2) || !g.I.np) return;
-  // reaction: one descriptor per (level, type)
+  if (descs.empty()) return;
+  OpDesc *dd = c.arena.get<OpDesc>(descs.size());
+  LPB_CUDA(cudaMemcpyAsync(dd, descs.data(), sizeof(OpDesc) * descs.size(), cudaMemcpyHostToDevice, c.stream));
+  double *prep = c.arena.get<double>(descs.size() * NPREP);
+  k_ops_prep<<<(unsigned)((descs.size() + 63) / 64), 64, 0, c.stream>>>(dd, (int)descs.size(), p, prep);
+  LPB_LAUNCH();
+  k_build_ops<T><<<dim3((unsigned)descs.size(), OPS_SPLIT), 256, 0, c.stream>>>(dd, prep, c.phat_dir, p, K,
+                                                                                c.gaunt, ops);
+  LPB_LAUNCH();
+  c.launches += 2;
+}
+
+// the reaction tables and operators of every group, level and type: five launches
+template <typename T>
+static void build_react_t(Ctx &c, std::vector<Group> &groups) {
+  const int p = c.p, K = c.K;
+  const size_t KK = (size_t)K * K;
   const int KT = 2 * p + 3, NS = p + 2;
   const size_t TS = (size_t)(KT + 1) * (KT + 1) * 4;
   std::vector<RDesc> rd;
-  const int st = (g.a == 1) ? -1 : 1;
-  for (int l = 2; l <= g.D; ++l) {
-    if (!g.vreact[l]) continue;
-    const double h = g.h(l);
-    g.stab[l] = c.arena.get<double>((size_t)NREACT_CLS * g.ntypes * TS);
-    g.op_react[l] = c.arena.get<T>((size_t)NREACT_CLS * g.ntypes * 2 * KK);
-    float2 *coef = c.arena.get<float2>((size_t)g.ntypes * KK * NS);
-    for (int t = 0; t < g.ntypes; ++t) {
-      int lp, bb;
-      type_decode(t, lp, bb);
-      RDesc d;
-      d.l = g.l; d.a = g.a; d.lp = lp; d.b = bb; d.tau = t; d.ntypes = g.ntypes; d.st = st; d.pad = l;
-      d.cls0 = 0; d.pad2 = 0;
-      d.h = h; d.Lam = c.md.lam[g.l] * h; d.Lamp = c.md.lam[lp] * h;
-      d.used = g.used[l];
-      d.stab = g.stab[l];
-      d.coef = coef + (size_t)t * KK * NS;
-      d.dst = 0;
-      rd.push_back(d);
+  for (auto &g : groups) {
+    if (!(g.parts & 2) || !g.I.np) continue;
+    const int st = (g.a == 1) ? -1 : 1;
+    for (int l = 2; l <= g.D; ++l) {
+      if (!g.vreact[l]) continue;
+      const double h = g.h(l);
+      g.stab[l] = c.arena.get<double>((size_t)NREACT_CLS * g.ntypes * TS);
+      g.op_react[l] = c.arena.get<T>((size_t)NREACT_CLS * g.ntypes * 2 * KK);
+      float2 *coef = c.arena.get<float2>((size_t)g.ntypes * KK * NS);
+      for (int t = 0; t < g.ntypes; ++t) {
+        int lp, bb;
+        type_decode(t, lp, bb);
+        RDesc d;
+        d.l = g.l; d.a = g.a; d.lp = lp; d.b = bb; d.tau = t; d.ntypes = g.ntypes; d.st = st; d.pad = l;
+        d.cls0 = 0; d.pad2 = 0;
+        d.h = h; d.Lam = c.md.lam[g.l] * h; d.Lamp = c.md.lam[lp] * h;
+        d.used = g.used[l];
+        d.stab = g.stab[l];
+        d.coef = coef + (size_t)t * KK * NS;
+        d.out = g.op_react[l];
+        rd.push_back(d);
+      }
     }
   }
-  if (!rd.empty()) {
-    RDesc *dr = c.arena.get<RDesc>(rd.size());
-    LPB_CUDA(cudaMemcpyAsync(dr, rd.data(), sizeof(RDesc) * rd.size(), cudaMemcpyHostToDevice, c.stream));
-    const unsigned nd = (unsigned)rd.size();
-    const double tol = fmax(c.tol, 1e-16);
-    std::vector<NDesc> nv;
-    int maxq = 0;
-    // one node set for the whole evaluation (graded to the smallest Lambda of all reaction
-    // groups), so the Bessel columns are evaluated once and shared
-    if (!c.stab_bes) {
-      const NDesc N0 = node_desc(KT, tol, c.stab_lmin, c.stab_lmin);
-      c.stab_bes = c.arena.get<double>((size_t)N0.nq * 2 * NRHO);
-      k_stab_bessel<<<(unsigned)(((int64_t)N0.nq * NRHO + 255) / 256), 256, 0, c.stream>>>(N0, c.stab_bes);
-      LPB_LAUNCH();
-      c.launches++;
-    }
-    for (auto &d : rd) {
-      (void)d;
-      NDesc N = node_desc(KT, tol, c.stab_lmin, c.stab_lmin);
-      N.bes = c.stab_bes;
-      N.nodes = c.arena.get<double>((size_t)N.nq * NDF);
-      maxq = std::max(maxq, N.nq);
-      nv.push_back(N);
-    }
-    NDesc *dn = c.arena.get<NDesc>(nv.size());
-    LPB_CUDA(cudaMemcpyAsync(dn, nv.data(), sizeof(NDesc) * nv.size(), cudaMemcpyHostToDevice, c.stream));
-    k_stab_nodes<<<dim3((unsigned)((maxq + 255) / 256), nd), 256, 0, c.stream>>>(dr, dn, c.md);
-    LPB_LAUNCH();
-    {
-      const size_t sm = stab_quad_smem(KT);
-      LPB_ATTR_ONCE(k_stab_quad, stab_quad_smem(KMAX_TAB));  // the largest table any order needs
-      k_stab_quad<<<dim3(NREACT_CLS, nd), SQ_CHUNK, sm, c.stream>>>(dr, dn, KT, c.sfac);
-      LPB_LAUNCH();
-    }
-    c.launches += 1;
-    k_stab_recur<<<dim3(NREACT_CLS, nd), 32, 0, c.stream>>>(dr, KT);
-    LPB_LAUNCH();
-    k_react_coef<<<dim3((unsigned)((KK + 255) / 256), nd), 256, 0, c.stream>>>(dr, c.tpoly, c.tpk, p, K);
-    LPB_LAUNCH();
-    // assemble into each level's op array: descriptors grouped by level
-    size_t first = 0;
-    while (first < rd.size()) {
-      const int l = rd[first].pad;
-      size_t last = first;
-      while (last < rd.size() && rd[last].pad == l) ++last;
-      LPB_ATTR_ONCE(k_react_assemble<T>, assemble_smem(KMAX_TAB));
-      k_react_assemble<T><<<dim3((NREACT_CLS + ASM_CC - 1) / ASM_CC, (unsigned)(last - first)), 256,
-                            assemble_smem(KT), c.stream>>>(
-          dr + first, p, K, KT, c.sfac, (T *)g.op_react[l]);
-      LPB_LAUNCH();
-      c.launches++;
-      first = last;
-    }
-    c.launches += 3;
-  }
+  if (rd.empty()) return;
+  RDesc *dr = c.arena.get<RDesc>(rd.size());
+  LPB_CUDA(cudaMemcpyAsync(dr, rd.data(), sizeof(RDesc) * rd.size(), cudaMemcpyHostToDevice, c.stream));
+  const unsigned nd = (unsigned)rd.size();
+  // one node set for the whole evaluation (graded to the smallest Lambda of all reaction
+  // groups), so the Bessel columns are evaluated once and shared
+  NDesc N = node_desc(KT, fmax(c.tol, 1e-16), c.stab_lmin, c.stab_lmin);
+  double *bes = c.arena.get<double>((size_t)N.nq * NBES);
+  k_stab_bessel<<<(unsigned)(((int64_t)N.nq * NRHO + 255) / 256), 256, 0, c.stream>>>(N, bes);
+  LPB_LAUNCH();
+  N.bes = bes;
+  std::vector<NDesc> nv(nd, N);
+  for (auto &n : nv) n.nodes = c.arena.get<double>((size_t)N.nq * NDF);
+  NDesc *dn = c.arena.get<NDesc>(nv.size());
+  LPB_CUDA(cudaMemcpyAsync(dn, nv.data(), sizeof(NDesc) * nv.size(), cudaMemcpyHostToDevice, c.stream));
+  launch_tables(c, dr, dn, N.nq, nd, KT);
+  k_react_coef<<<dim3((unsigned)((KK + 255) / 256), nd), 256, 0, c.stream>>>(dr, c.tpoly, c.tpk, p, K);
+  LPB_LAUNCH();
+  LPB_ATTR_ONCE(k_react_assemble<T>, assemble_smem(PMAX, KMAX_TAB));
+  k_react_assemble<T><<<dim3((NREACT_CLS + ASM_CC - 1) / ASM_CC, nd), 256, assemble_smem(p, KT), c.stream>>>(
+      dr, p, K, KT, c.sfac);
+  LPB_LAUNCH();
+  c.launches += 5;
 }
 
-void build_operators(Ctx &c, Group &g, int parts, int which) {
-  if (c.opts.precision == LPBFMM_FP64) build_ops_t<double>(c, g, parts, which);
-  else build_ops_t<float>(c, g, parts, which);
+void build_operators(Ctx &c, std::vector<Group> &groups, int which) {
+  const bool d = c.opts.precision == LPBFMM_FP64;
+  if (which == 1) d ? build_free_t<double>(c, groups) : build_free_t<float>(c, groups);
+  else d ? build_react_t<double>(c, groups) : build_react_t<float>(c, groups);
 }
 
 void build_near_nodes(Ctx &c, Group &g, double zeta_min, double rho_max) {
@@ -798,7 +824,7 @@ void build_near_nodes(Ctx &c, Group &g, double zeta_min, double rho_max) {
   }());
   const double umax = 36.0 / zeta_min;
   const double wmax = fmin(2.0 / zeta_min, PI / fmax(rho_max, 1e-300));
-  g.nq = count_panels(umax, wmax, lmin) * 16;
+  g.nq = count_panels(umax, wmax, lmin, 0.5) * 16;
   g.nodes = c.arena.get<double>((size_t)g.ntypes * g.nq * 4);
   k_near_nodes<<<dim3((unsigned)((g.nq + 255) / 256), g.ntypes), 256, 0, c.stream>>>(c.md, g.l, g.a, g.ntypes, umax,
                                                                                      wmax, lmin, g.nodes, g.nq);
@@ -825,7 +851,7 @@ static RDesc one_class_desc(Ctx &c, int l, int a, int lp, int b, double h, int c
   d.l = l; d.a = a; d.lp = lp; d.b = b; d.tau = 0; d.ntypes = 1; d.st = a == 1 ? -1 : 1; d.pad = 0;
   d.cls0 = cls; d.pad2 = 0;
   d.h = h; d.Lam = c.md.lam[l] * h; d.Lamp = c.md.lam[lp] * h;
-  d.used = nullptr; d.stab = nullptr; d.coef = nullptr; d.dst = 0;
+  d.used = nullptr; d.stab = nullptr; d.coef = nullptr; d.out = nullptr;
   return d;
 }
 
@@ -853,19 +879,15 @@ void debug_stable(Ctx &c, int l, int a, int lp, int b, double h, double rho, dou
   const double tol = fmax(c.tol, 1e-16);
   NDesc N = node_desc(KT, tol, d.Lam, d.Lamp);
   NDesc *dn = nullptr;
+  double *bes = nullptr;
   LPB_CUDA(cudaMalloc(&N.nodes, sizeof(double) * (size_t)N.nq * NDF));
+  LPB_CUDA(cudaMalloc(&bes, sizeof(double) * (size_t)N.nq * NBES));
   LPB_CUDA(cudaMalloc(&dn, sizeof(NDesc)));
+  k_stab_bessel<<<(unsigned)((N.nq * NRHO + 255) / 256), 256, 0, c.stream>>>(N, bes);
+  LPB_LAUNCH();
+  N.bes = bes;
   LPB_CUDA(cudaMemcpyAsync(dn, &N, sizeof(NDesc), cudaMemcpyHostToDevice, c.stream));
-  k_stab_nodes<<<dim3((unsigned)((N.nq + 255) / 256), 1), 256, 0, c.stream>>>(dr, dn, c.md);
-  LPB_LAUNCH();
-  {
-    const size_t sm = stab_quad_smem(KT);
-    LPB_ATTR_ONCE(k_stab_quad, stab_quad_smem(KMAX_TAB));
-    k_stab_quad<<<dim3(NREACT_CLS, 1), SQ_CHUNK, sm, c.stream>>>(dr, dn, KT, c.sfac);
-    LPB_LAUNCH();
-  }
-  k_stab_recur<<<dim3(NREACT_CLS, 1), 32, 0, c.stream>>>(dr, KT);
-  LPB_LAUNCH();
+  launch_tables(c, dr, dn, N.nq, 1, KT);
   std::vector<double> h_out(TS);
   LPB_CUDA(cudaMemcpyAsync(h_out.data(), stab, sizeof(double) * TS, cudaMemcpyDeviceToHost, c.stream));
   LPB_CUDA(cudaStreamSynchronize(c.stream));
@@ -873,6 +895,7 @@ void debug_stable(Ctx &c, int l, int a, int lp, int b, double h, double rho, dou
   cudaFree(used);
   cudaFree(dr);
   cudaFree(N.nodes);
+  cudaFree(bes);
   cudaFree(dn);
   // out[((K*(Kmax+1)) + d)*4 + ij] with ij = 2i + j
   for (size_t e = 0; e < TS; ++e) out[e] = h_out[e];
@@ -887,7 +910,7 @@ void debug_stable(Ctx &c, int l, int a, int lp, int b, double h, double rho, dou
 // address is resolved per device with cudaGetSymbolAddress on the first call on that device.
 // ---------------------------------------------------------------------------------------
 constexpr size_t NA_TS = (size_t)(LPBFMM_NOALLOC_KMAX + 1) * (LPBFMM_NOALLOC_KMAX + 1) * 4;  // one class
-constexpr size_t NA_NODES = (size_t)LPBFMM_NOALLOC_NQ * NDF;        // doubles
+constexpr size_t NA_NODES = (size_t)LPBFMM_NOALLOC_NQ * (NDF + NBES);  // doubles
 constexpr size_t NA_DESC = (sizeof(RDesc) + sizeof(NDesc) + NREACT_CLS + 7) / 8 + 8;
 constexpr size_t NA_DOUBLES = NA_TS + NA_NODES + NA_DESC;           // ~1.8 MB in all
 static __device__ __align__(256) double g_noalloc_scratch[NA_DOUBLES];
@@ -930,7 +953,9 @@ void stable_noalloc(Ctx &c, int l, int a, int lp, int b, double h, double rho, d
   const size_t TS = (size_t)(KT + 1) * (KT + 1) * 4;
   RDesc d = one_class_desc(c, l, a, lp, b, h, cls);
   NDesc N = node_desc(KT, fmax(c.tol, 1e-16), d.Lam, d.Lamp);
-  if (N.nq > LPBFMM_NOALLOC_NQ) throw StatusError{LPBFMM_ERR_UNSUPPORTED};
+  // the limit counts 16-point panels of width 2, the rule it was set for; the present rule needs fewer nodes
+  if (count_panels(N.umax, 2.0, N.lmin, 0.5) * 16 > LPBFMM_NOALLOC_NQ || N.nq > LPBFMM_NOALLOC_NQ)
+    throw StatusError{LPBFMM_ERR_UNSUPPORTED};
   double *base = noalloc_scratch(c);
   double *stab = base, *nodes = base + NA_TS;
   RDesc *dr = (RDesc *)(nodes + NA_NODES);
@@ -939,15 +964,13 @@ void stable_noalloc(Ctx &c, int l, int a, int lp, int b, double h, double rho, d
   d.used = used;
   d.stab = stab;
   N.nodes = nodes;
+  double *bes = nodes + (size_t)LPBFMM_NOALLOC_NQ * NDF;
+  k_stab_bessel<<<(unsigned)((N.nq * NRHO + 255) / 256), 256, 0, c.stream>>>(N, bes);
+  LPB_LAUNCH();
+  N.bes = bes;
   k_noalloc_init<<<8, 256, 0, c.stream>>>(d, N, dr, dn, used, cls, stab, (int)TS);
   LPB_LAUNCH();
-  k_stab_nodes<<<dim3((unsigned)((N.nq + 255) / 256), 1), 256, 0, c.stream>>>(dr, dn, c.md);
-  LPB_LAUNCH();
-  LPB_ATTR_ONCE(k_stab_quad, stab_quad_smem(KMAX_TAB));
-  k_stab_quad<<<dim3(NREACT_CLS, 1), SQ_CHUNK, stab_quad_smem(KT), c.stream>>>(dr, dn, KT, c.sfac);
-  LPB_LAUNCH();
-  k_stab_recur<<<dim3(NREACT_CLS, 1), 32, 0, c.stream>>>(dr, KT);
-  LPB_LAUNCH();
+  launch_tables(c, dr, dn, N.nq, 1, KT);
   LPB_CUDA(cudaMemcpyAsync(out, stab, sizeof(double) * TS, cudaMemcpyDeviceToDevice, c.stream));
 }
 
