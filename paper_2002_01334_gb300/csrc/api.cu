@@ -251,12 +251,8 @@ static void eval_front(Ctx &c, int64_t n, const double *q, const double *xyz, co
   }
   const double xlo = unord(hs.xlo), xhi = unord(hs.xhi), ylo = unord(hs.ylo), yhi = unord(hs.yhi);
   // per-layer stable ranks
-  uint32_t *rank[MAXLAYER] = {};
-  for (int k = 0; k <= L; ++k)
-    if (cnt[k]) {
-      rank[k] = c.arena.get<uint32_t>(n);
-      layer_rank(c, n, layer, k, rank[k]);
-    }
+  RankPtrs rank;
+  layer_ranks(c, n, layer, cnt, rank);
   // target groups (l, a) and their roots (exact extremes of monotone expressions)
   const double cx = 0.5 * (xlo + xhi), cy = 0.5 * (ylo + yhi);
   for (int l = 0; l <= L; ++l) {
@@ -289,37 +285,13 @@ static void eval_front(Ctx &c, int64_t n, const double *q, const double *xyz, co
       c.groups.push_back(g);
     }
   }
-  // per-group streams (the groups' trees are independent): fork from / join into c.stream; in a
-  // batched evaluation the systems already run concurrently, and the groups stay on c.stream
-  const int NGS = c.def.on ? 0 : std::min<int>(Ctx::GROUP_STREAMS, (int)c.groups.size());
-  auto fork_groups = [&]() {
-    LPB_CUDA(cudaEventRecord(c.ev_gfork, c.stream));
-    for (int k = 0; k < NGS; ++k) LPB_CUDA(cudaStreamWaitEvent(c.gs[k], c.ev_gfork, 0));
-  };
-  auto join_groups = [&]() {
-    for (int k = 0; k < NGS; ++k) {
-      LPB_CUDA(cudaEventRecord(c.ev_gjoin[k], c.gs[k]));
-      LPB_CUDA(cudaStreamWaitEvent(c.stream, c.ev_gjoin[k], 0));
-    }
-  };
-  auto per_group = [&](auto &&f) {
-    fork_groups();
-    for (size_t k = 0; k < c.groups.size(); ++k) {
-      OnStream on(c, NGS ? c.gs[k % NGS] : c.stream);
-      f((int)k, c.groups[k]);
-    }
-    join_groups();
-  };
   const int G = (int)c.groups.size();
   uint32_t *dc = nullptr;  // occupied boxes per level and group (automatic depth)
   if (c.opts.uniform_depth <= 0) {
     dc = c.arena.get<uint32_t>((size_t)G * (DMAX + 1));
     LPB_CUDA(cudaMemsetAsync(dc, 0, sizeof(uint32_t) * G * (DMAX + 1), c.stream));
   }
-  per_group([&](int k, Group &g) {
-    build_group_targets(c, g, n, q, xyz, layer, rank, cnt);
-    if (dc) count_levels(c, g, dc + (size_t)k * (DMAX + 1));
-  });
+  build_targets(c, c.groups, n, q, xyz, layer, rank, cnt, dc);
   // smallest distances of the group's targets and images to its interface (exact extremes of
   // monotone expressions of the z ranges)
   auto z_gaps = [&](const Group &g, double &zt, double &zs) {
@@ -370,39 +342,20 @@ static void eval_front(Ctx &c, int64_t n, const double *q, const double *xyz, co
     build_operators(c, c.groups, 1);
     LPB_CUDA(cudaEventRecord(c.ev_free, c.side));
   }
-  per_group([&](int, Group &g) {
-    build_group_images(c, g, n, q, xyz, layer, rank, cnt);
-    build_group_boxes(c, g);
-  });
+  build_images(c, c.groups, n, q, xyz, layer, rank, cnt);
   // box counts to host
   {
-    std::vector<const uint32_t *> srcs;
-    for (auto &g : c.groups) {
-      for (int l = 2; l <= g.D; ++l) {
-        srcs.push_back(g.T.lev[l].d_n);
-        srcs.push_back(g.I.lev[l].d_n);
-      }
-      srcs.push_back(g.I.d_nseg);
-    }
-    uint32_t *dd = c.arena.get<uint32_t>(srcs.size());
-    LPB_CUDA(cudaMemsetAsync(dd, 0, sizeof(uint32_t) * srcs.size(), c.stream));
-    for (size_t k = 0; k < srcs.size(); ++k)
-      if (srcs[k]) LPB_CUDA(cudaMemcpyAsync(dd + k, srcs[k], sizeof(uint32_t), cudaMemcpyDeviceToDevice, c.stream));
-    uint32_t *hh = (uint32_t *)c.h_pinned;
-    LPB_CUDA(cudaMemcpyAsync(hh, dd, sizeof(uint32_t) * srcs.size(), cudaMemcpyDeviceToHost, c.stream));
-    LPB_CUDA(cudaStreamSynchronize(c.stream));
-    size_t k = 0;
-    for (auto &g : c.groups) {
-      for (int l = 2; l <= g.D; ++l) {
-        g.T.lev[l].n = g.T.np ? hh[k] : 0;
-        g.I.lev[l].n = g.I.np ? hh[k + 1] : 0;
-        k += 2;
-      }
-      g.I.nseg = g.I.np ? hh[k] : 0;
-      ++k;
+    uint32_t *dd = nullptr;
+    size_t nc = 0;
+    build_boxes(c, c.groups, &dd, &nc);
+    if (nc) {
+      uint32_t *hh = (uint32_t *)c.h_pinned;
+      LPB_CUDA(cudaMemcpyAsync(hh, dd, sizeof(uint32_t) * nc, cudaMemcpyDeviceToHost, c.stream));
+      LPB_CUDA(cudaStreamSynchronize(c.stream));
+      read_box_counts(c.groups, hh);
     }
   }
-  per_group([&](int, Group &g) { build_group_lists(c, g, g.parts); });
+  build_lists(c, c.groups);
   prof_mark(c, "tree");
   // the FP32 free-space near field needs only the trees and near lists: on its own stream, beside
   // the operators, the upward pass and the M2L (the downward pass waits for it).  In a batched
@@ -410,9 +363,9 @@ static void eval_front(Ctx &c, int64_t n, const double *q, const double *xyz, co
   c.near_async = !c.def.on && c.opts.precision != LPBFMM_FP64;
   if (c.near_async) {
     LPB_CUDA(cudaEventRecord(c.ev_gfork, c.stream));
-    LPB_CUDA(cudaStreamWaitEvent(c.gs[0], c.ev_gfork, 0));
-    run_near_free(c, c.groups, phi, field, c.gs[0]);
-    LPB_CUDA(cudaEventRecord(c.ev_near, c.gs[0]));
+    LPB_CUDA(cudaStreamWaitEvent(c.near, c.ev_gfork, 0));
+    run_near_free(c, c.groups, phi, field, c.near);
+    LPB_CUDA(cudaEventRecord(c.ev_near, c.near));
   } else {
     run_near_free(c, c.groups, phi, field, c.stream);
   }
@@ -570,10 +523,7 @@ int lpbfmm_create(int n_iface, const double *z_iface, const double *eps, const d
     LPB_CUDA(cudaEventCreateWithFlags(&c->ev_near, cudaEventDisableTiming));
     LPB_CUDA(cudaEventCreate(&c->ev_p2p[0]));
     LPB_CUDA(cudaEventCreate(&c->ev_p2p[1]));
-    for (int k = 0; k < Ctx::GROUP_STREAMS; ++k) {
-      LPB_CUDA(cudaStreamCreateWithFlags(&c->gs[k], cudaStreamNonBlocking));
-      LPB_CUDA(cudaEventCreateWithFlags(&c->ev_gjoin[k], cudaEventDisableTiming));
-    }
+    LPB_CUDA(cudaStreamCreateWithFlags(&c->near, cudaStreamNonBlocking));
     LPB_CUDA(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
     init_fmm_tables(*c);
   } catch (const CudaError &e) {
@@ -856,8 +806,7 @@ void lpbfmm_destroy(lpbfmm_t h) {
   cudaStreamSynchronize(h->stream);
   if (h->side) cudaStreamSynchronize(h->side);
   if (h->far) cudaStreamSynchronize(h->far);
-  for (int k = 0; k < Ctx::GROUP_STREAMS; ++k)
-    if (h->gs[k]) cudaStreamSynchronize(h->gs[k]);
+  if (h->near) cudaStreamSynchronize(h->near);
   h->arena.release();
   if (h->adj) cudaFree(h->adj);
   if (h->gaunt) cudaFree(h->gaunt);
@@ -874,10 +823,7 @@ void lpbfmm_destroy(lpbfmm_t h) {
   if (h->ev_near) cudaEventDestroy(h->ev_near);
   for (int k = 0; k < 2; ++k)
     if (h->ev_p2p[k]) cudaEventDestroy(h->ev_p2p[k]);
-  for (int k = 0; k < Ctx::GROUP_STREAMS; ++k) {
-    if (h->ev_gjoin[k]) cudaEventDestroy(h->ev_gjoin[k]);
-    if (h->gs[k]) cudaStreamDestroy(h->gs[k]);
-  }
+  if (h->near) cudaStreamDestroy(h->near);
   if (h->ev_join) cudaEventDestroy(h->ev_join);
   if (h->side) cudaStreamDestroy(h->side);
   if (h->far) cudaStreamDestroy(h->far);

@@ -288,13 +288,10 @@ struct Ctx {
   // with the upward pass (the M2L waits for them, ev_join)
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_free = nullptr, ev_join = nullptr;
-  // the target groups' trees and lists are independent: built on one stream per group
-  // (group k on gs[k % GROUP_STREAMS]), forked from and joined into the evaluation stream
-  static constexpr int GROUP_STREAMS = 4;
-  cudaStream_t gs[GROUP_STREAMS] = {};
-  cudaEvent_t ev_gfork = nullptr, ev_gjoin[GROUP_STREAMS] = {};
-  // the FP32 free-space near field runs on gs[0] beside the upward pass and the M2L; the downward
+  cudaEvent_t ev_gfork = nullptr;
+  // the FP32 free-space near field runs on a stream of its own beside the upward pass and the M2L; the downward
   // pass (which also adds into the outputs) waits for ev_near.  ev_p2p[2] time its launch.
+  cudaStream_t near = nullptr;
   cudaEvent_t ev_near = nullptr, ev_p2p[2] = {};
   bool near_async = false, p2p_timed = false;
   // beside it, the upward pass and the M2L run on a high-priority stream (far), so that their
@@ -321,16 +318,18 @@ struct Stats {
   unsigned long long zlo[MAXLAYER], zhi[MAXLAYER];
 };
 void scan_u32(Ctx &c, const uint32_t *in, uint32_t *out, int64_t n, uint32_t *d_total);
-void radix_sort(Ctx &c, uint64_t *&keys, uint32_t *&vals, int64_t n, int bits, int lo);
 void launch_validate(Ctx &c, int64_t n, const double *q, const double *xyz, const int32_t *layer, Stats *st);
-void build_group_targets(Ctx &c, Group &g, int64_t n, const double *q, const double *xyz, const int32_t *layer,
-                         uint32_t *const *rank, const int64_t *cnt);
-void build_group_images(Ctx &c, Group &g, int64_t n, const double *q, const double *xyz, const int32_t *layer,
-                        uint32_t *const *rank, const int64_t *cnt);
-void count_levels(Ctx &c, Group &g, uint32_t *d_counts);
-void build_group_boxes(Ctx &c, Group &g);
-void build_group_lists(Ctx &c, Group &g, int parts);
-void layer_rank(Ctx &c, int64_t n, const int32_t *layer, int lay, uint32_t *rank);
+struct RankPtrs {
+  uint32_t *r[MAXLAYER];
+};
+void layer_ranks(Ctx &c, int64_t n, const int32_t *layer, const int64_t *cnt, RankPtrs &rank);
+void build_targets(Ctx &c, std::vector<Group> &groups, int64_t n, const double *q, const double *xyz,
+                   const int32_t *layer, const RankPtrs &rank, const int64_t *cnt, uint32_t *dc);
+void build_images(Ctx &c, std::vector<Group> &groups, int64_t n, const double *q, const double *xyz,
+                  const int32_t *layer, const RankPtrs &rank, const int64_t *cnt);
+void build_boxes(Ctx &c, std::vector<Group> &groups, uint32_t **dcounts, size_t *ncounts);
+void read_box_counts(std::vector<Group> &groups, const uint32_t *h);
+void build_lists(Ctx &c, std::vector<Group> &groups);
 // adaptive dual-tree lists of group g's free-space target tree with itself (diagnostic): records
 // of 5 int64 (kind 0 V / 1 U / 2 W / 3 X, target level, target key, source level, source key)
 void adaptive_lists(Ctx &c, Group &g, int s, int ws, std::vector<int64_t> &rec);

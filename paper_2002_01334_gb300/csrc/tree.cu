@@ -5,6 +5,8 @@
 #include "internal.h"
 #include "prims.cuh"
 
+#include <algorithm>
+
 namespace lpb {
 
 // ---------------------------------------------------------------------------------------
@@ -32,24 +34,97 @@ void scan_u32(Ctx &c, const uint32_t *in, uint32_t *out, int64_t n, uint32_t *d_
   c.launches += 2 + (tiles > 1) + (n > 0 ? 0 : -1);
 }
 
-// stable sort by key bits [lo, bits): lower bits must not matter for the order (zero, or a
-// field equal within a run that the caller does not need sorted)
-void radix_sort(Ctx &c, uint64_t *&keys, uint32_t *&vals, int64_t n, int bits, int lo) {
-  if (n <= 1) return;
-  const int nblocks = (int)((n + RS_TILE - 1) / RS_TILE);
-  uint64_t *k2 = c.arena.get<uint64_t>(n);
-  uint32_t *v2 = c.arena.get<uint32_t>(n);
-  uint32_t *hist = c.arena.get<uint32_t>((size_t)256 * nblocks);
-  uint32_t *offs = c.arena.get<uint32_t>((size_t)256 * nblocks);
-  for (int shift = lo; shift < bits; shift += 8) {
-    k_radix_hist<<<nblocks, RS_THREADS, 0, c.stream>>>(keys, n, shift, hist, nblocks);
+// the scans of several arrays
+static void scan_batch(Ctx &c, ScanJobs &J, int nj) {
+  int64_t nmax = 0;
+  for (int k = 0; k < nj; ++k) nmax = std::max(nmax, J.j[k].n);
+  if (!nj || !nmax) return;
+  if (nmax <= 8192) {
+    k_scan_one_b<<<nj, 1024, 0, c.stream>>>(J);
     LPB_LAUNCH();
-    scan_u32(c, hist, offs, (int64_t)256 * nblocks, nullptr);
-    k_radix_scatter<<<nblocks, RS_THREADS, 0, c.stream>>>(keys, vals, k2, v2, n, shift, offs, nblocks);
+    c.launches++;
+    return;
+  }
+  const unsigned tiles = (unsigned)((nmax + SCAN_TILE - 1) / SCAN_TILE);
+  for (int k = 0; k < nj; ++k) J.j[k].sums = c.arena.get<uint32_t>((size_t)(J.j[k].n + SCAN_TILE - 1) / SCAN_TILE + 1);
+  k_scan_tiles_b<<<dim3(tiles, nj), SCAN_THREADS, 0, c.stream>>>(J);
+  LPB_LAUNCH();
+  k_scan_sums_b<<<nj, 1024, 0, c.stream>>>(J);
+  LPB_LAUNCH();
+  k_scan_add_b<<<dim3(tiles, nj), SCAN_THREADS, 0, c.stream>>>(J);
+  LPB_LAUNCH();
+  c.launches += 3;
+}
+
+// stable sorts of several arrays by key bits [lo, bits) of each: lower bits must not matter for the order
+// (zero, or a field equal within a run that the caller does not need sorted)
+struct SortReq {
+  uint64_t **keys;
+  uint32_t **vals;
+  int64_t n;
+  int bits, lo;
+};
+static void sort_batch(Ctx &c, const std::vector<SortReq> &reqs) {
+  SortJobs small{}, large{};
+  ScanJobs sc{};
+  std::vector<const SortReq *> rs, rl;
+  for (const SortReq &r : reqs) {
+    if (r.n <= 1) continue;
+    SortJob j{};
+    j.k = *r.keys; j.v = *r.vals; j.n = r.n; j.lo = r.lo; j.bits = r.bits;
+    j.ok = c.arena.get<uint64_t>(r.n);
+    j.ov = c.arena.get<uint32_t>(r.n);
+    if (r.n <= RS_SMALL) {
+      small.j[rs.size()] = j;
+      rs.push_back(&r);
+    } else {
+      j.nblocks = (int)((r.n + RS_TILE - 1) / RS_TILE);
+      j.hist = c.arena.get<uint32_t>((size_t)256 * j.nblocks);
+      j.offs = c.arena.get<uint32_t>((size_t)256 * j.nblocks);
+      large.j[rl.size()] = j;
+      rl.push_back(&r);
+    }
+  }
+  if (!rs.empty()) {
+    k_radix_small<<<(unsigned)rs.size(), 1024, 0, c.stream>>>(small);
+    LPB_LAUNCH();
+    c.launches++;
+    for (size_t k = 0; k < rs.size(); ++k)
+      if (((rs[k]->bits - rs[k]->lo + 7) / 8) & 1) {
+        *rs[k]->keys = small.j[k].ok;
+        *rs[k]->vals = small.j[k].ov;
+      }
+  }
+  for (int pass = 0; !rl.empty(); ++pass) {
+    SortJobs J{};
+    std::vector<int> who;
+    unsigned nb = 0;
+    for (size_t k = 0; k < rl.size(); ++k)
+      if (large.j[k].lo + 8 * pass < large.j[k].bits) {
+        J.j[who.size()] = large.j[k];
+        sc.j[who.size()] = ScanJob{large.j[k].hist, large.j[k].offs, nullptr, (int64_t)256 * large.j[k].nblocks};
+        who.push_back((int)k);
+        nb = std::max(nb, (unsigned)large.j[k].nblocks);
+      }
+    if (who.empty()) break;
+    const int nj = (int)who.size();
+    k_radix_hist<<<dim3(nb, nj), RS_THREADS, 0, c.stream>>>(J, pass);
+    LPB_LAUNCH();
+    scan_batch(c, sc, nj);
+    k_radix_scatter<<<dim3(nb, nj), RS_THREADS, 0, c.stream>>>(J, pass);
     LPB_LAUNCH();
     c.launches += 2;
-    uint64_t *tk = keys; keys = k2; k2 = tk;
-    uint32_t *tv = vals; vals = v2; v2 = tv;
+    for (int k : who) {
+      SortJob &j = large.j[k];
+      uint64_t *tk = const_cast<uint64_t *>(j.k);
+      uint32_t *tv = const_cast<uint32_t *>(j.v);
+      j.k = j.ok; j.ok = tk;
+      j.v = j.ov; j.ov = tv;
+    }
+  }
+  for (size_t k = 0; k < rl.size(); ++k) {
+    *rl[k]->keys = const_cast<uint64_t *>(large.j[k].k);
+    *rl[k]->vals = const_cast<uint32_t *>(large.j[k].v);
   }
 }
 
@@ -160,16 +235,30 @@ void launch_validate(Ctx &c, int64_t n, const double *q, const double *xyz, cons
   c.launches++;
 }
 
-__global__ void k_flag_layer(int64_t n, const int32_t *layer, int lay, uint32_t *f) {
+// flags of every layer present (f[k] may be null)
+__global__ void k_flag_layers(int64_t n, const int32_t *layer, int nl, RankPtrs f) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) f[i] = layer[i] == lay ? 1u : 0u;
+  if (i >= n) return;
+  const int lay = layer[i];
+  for (int k = 0; k < nl; ++k)
+    if (f.r[k]) f.r[k][i] = lay == k ? 1u : 0u;
 }
-void layer_rank(Ctx &c, int64_t n, const int32_t *layer, int lay, uint32_t *rank) {
-  uint32_t *f = c.arena.get<uint32_t>(n);
-  k_flag_layer<<<(unsigned)((n + 255) / 256), 256, 0, c.stream>>>(n, layer, lay, f);
+// stable rank of every charge within its layer (layers without charges: null)
+void layer_ranks(Ctx &c, int64_t n, const int32_t *layer, const int64_t *cnt, RankPtrs &rank) {
+  RankPtrs f{};
+  ScanJobs J{};
+  int nj = 0;
+  for (int k = 0; k <= c.md.L; ++k) {
+    rank.r[k] = nullptr;
+    if (!cnt[k]) continue;
+    f.r[k] = c.arena.get<uint32_t>(n);
+    rank.r[k] = c.arena.get<uint32_t>(n);
+    J.j[nj++] = ScanJob{f.r[k], rank.r[k], nullptr, n};
+  }
+  k_flag_layers<<<(unsigned)((n + 255) / 256), 256, 0, c.stream>>>(n, layer, c.md.L + 1, f);
   LPB_LAUNCH();
   c.launches++;
-  scan_u32(c, f, rank, n, nullptr);
+  scan_batch(c, J, nj);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -201,56 +290,92 @@ __device__ __forceinline__ uint64_t morton_of(double x, double y, double z, cons
   return (spread3(cell_of(x, o[0], s)) << 2) | (spread3(cell_of(y, o[1], s)) << 1) | spread3(cell_of(z, o[2], s));
 }
 
-struct RankPtrs {
-  uint32_t *r[MAXLAYER];
-};
 struct GroupGeom {
   double o[3];  // lower corner of the root cube
   double s;     // 2^DMAX / (2H)
-  int l, a;
+  int l, a, D;
   int64_t type_off[2 * MAXLAYER];
+  uint64_t *key;
+  uint32_t *src;
+};
+struct GroupGeoms {
+  GroupGeom g[MAXJOB];
+};
+struct GatherJob {
+  int64_t np;
+  const uint64_t *key;
+  const uint32_t *src;
+  int l, a;
+  double *x, *y, *z, *q;
+  uint32_t *cnt;  // targets: non-empty boxes per level (null: not counted)
+};
+struct GatherJobs {
+  GatherJob j[MAXJOB];
 };
 
-__global__ void k_make_targets(int64_t n, const double *xyz, const int32_t *layer, RankPtrs rk, GroupGeom gg,
-                               uint64_t *key, uint32_t *src) {
+__global__ void k_make_targets(int64_t n, const double *xyz, const int32_t *layer, RankPtrs rk, int ng,
+                               const __grid_constant__ GroupGeoms G) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || layer[i] != gg.l) return;
-  const uint32_t pos = rk.r[gg.l][i];
-  key[pos] = morton_of(xyz[3 * i], xyz[3 * i + 1], xyz[3 * i + 2], gg.o, gg.s) << 4;
-  src[pos] = (uint32_t)i;
+  if (i >= n) return;
+  const int lay = layer[i];
+  const double x = xyz[3 * i], y = xyz[3 * i + 1], z = xyz[3 * i + 2];
+  for (int k = 0; k < ng; ++k) {
+    const GroupGeom &gg = G.g[k];
+    if (lay != gg.l) continue;
+    const uint32_t pos = rk.r[gg.l][i];
+    gg.key[pos] = morton_of(x, y, z, gg.o, gg.s) << 4;
+    gg.src[pos] = (uint32_t)i;
+  }
 }
 
-__global__ void k_make_images(int64_t n, const double *xyz, const int32_t *layer, Medium md, RankPtrs rk,
-                              GroupGeom gg, int D, uint64_t *key, uint32_t *src) {
+__global__ void k_make_images(int64_t n, const double *xyz, const int32_t *layer, Medium md, RankPtrs rk, int ng,
+                              const __grid_constant__ GroupGeoms G) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int lp = layer[i];
-  for (int b = 1; b <= 2; ++b) {
-    if ((b == 1 && lp == md.L) || (b == 2 && lp == 0)) continue;
-    const int t = type_index(lp, b);
-    const int64_t pos = gg.type_off[t] + rk.r[lp][i];
-    const double zi = image_z(md, gg.l, gg.a, lp, b, xyz[3 * i + 2]);
-    key[pos] = ((morton_of(xyz[3 * i], xyz[3 * i + 1], zi, gg.o, gg.s) >> (3 * (DMAX - D))) << 4) | (uint64_t)t;
-    src[pos] = (uint32_t)i;
+  const double x = xyz[3 * i], y = xyz[3 * i + 1], z = xyz[3 * i + 2];
+  const uint32_t rank = rk.r[lp][i];
+  for (int k = 0; k < ng; ++k) {
+    const GroupGeom &gg = G.g[k];
+    for (int b = 1; b <= 2; ++b) {
+      if ((b == 1 && lp == md.L) || (b == 2 && lp == 0)) continue;
+      const int t = type_index(lp, b);
+      const int64_t pos = gg.type_off[t] + rank;
+      const double zi = image_z(md, gg.l, gg.a, lp, b, z);
+      gg.key[pos] = ((morton_of(x, y, zi, gg.o, gg.s) >> (3 * (DMAX - gg.D))) << 4) | (uint64_t)t;
+      gg.src[pos] = (uint32_t)i;
+    }
   }
 }
 
-__global__ void k_gather_points(int64_t np, const uint64_t *key, const uint32_t *src, const double *q,
-                                const double *xyz, Medium md, int l, int a, int images, double *x, double *y,
-                                double *z, double *qq, const int32_t *layer) {
+// sorted points of every group; with cnt, also the number of non-empty target boxes at every level
+// 2..DMAX (automatic depth rule)
+__global__ void k_gather_points(const double *q, const double *xyz, Medium md, int images,
+                                const __grid_constant__ GatherJobs J) {
+  const GatherJob &j = J.j[blockIdx.y];
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= np) return;
-  const uint32_t i = src[k];
-  x[k] = xyz[3 * i];
-  y[k] = xyz[3 * i + 1];
+  if (j.cnt)
+    for (int l = 2; l <= DMAX; ++l) {
+      bool f = false;
+      if (k < j.np) {
+        const int sh = 4 + 3 * (DMAX - l);
+        f = (k == 0) || ((j.key[k] >> sh) != (j.key[k - 1] >> sh));
+      }
+      const unsigned b = __popc(__ballot_sync(0xffffffffu, f));
+      if ((threadIdx.x & 31) == 0 && b) atomicAdd(&j.cnt[l], b);
+    }
+  if (k >= j.np) return;
+  const uint32_t i = j.src[k];
+  j.x[k] = xyz[3 * (size_t)i];
+  j.y[k] = xyz[3 * (size_t)i + 1];
+  double z = xyz[3 * (size_t)i + 2];
   if (images) {
     int lp, b;
-    type_decode((int)(key[k] & 15ull), lp, b);
-    z[k] = image_z(md, l, a, lp, b, xyz[3 * i + 2]);
-  } else {
-    z[k] = xyz[3 * i + 2];
+    type_decode((int)(j.key[k] & 15ull), lp, b);
+    z = image_z(md, j.l, j.a, lp, b, z);
   }
-  qq[k] = q[i];
+  j.z[k] = z;
+  j.q[k] = q[i];
 }
 
 static GroupGeom group_geom(Ctx &c, const Group &g, const int64_t *cnt) {
@@ -262,6 +387,7 @@ static GroupGeom group_geom(Ctx &c, const Group &g, const int64_t *cnt) {
   gg.s = double(1 << DMAX) / (2.0 * H);
   gg.l = g.l;
   gg.a = g.a;
+  gg.D = g.D;
   int64_t off = 0;
   for (int t = 0; t < 2 * c.md.L; ++t) {
     int lp, b;
@@ -272,138 +398,180 @@ static GroupGeom group_geom(Ctx &c, const Group &g, const int64_t *cnt) {
   return gg;
 }
 
-static void gather(Ctx &c, Group &g, PointSet &P, int images, const double *q, const double *xyz,
-                   const int32_t *layer) {
-  P.x = c.arena.get<double>(P.np);
-  P.y = c.arena.get<double>(P.np);
-  P.z = c.arena.get<double>(P.np);
-  P.q = c.arena.get<double>(P.np);
-  if (P.np) {
-    k_gather_points<<<(unsigned)((P.np + 255) / 256), 256, 0, c.stream>>>(P.np, P.key, P.src, q, xyz, c.md, g.l,
-                                                                          g.a, images, P.x, P.y, P.z, P.q, layer);
-    LPB_LAUNCH();
-    c.launches++;
+static void gather(Ctx &c, std::vector<Group> &groups, int images, const double *q, const double *xyz, uint32_t *dc) {
+  GatherJobs J{};
+  int nj = 0;
+  int64_t nmax = 0;
+  for (size_t k = 0; k < groups.size(); ++k) {
+    Group &g = groups[k];
+    PointSet &P = images ? g.I : g.T;
+    P.x = c.arena.get<double>(P.np);
+    P.y = c.arena.get<double>(P.np);
+    P.z = c.arena.get<double>(P.np);
+    P.q = c.arena.get<double>(P.np);
+    if (!P.np) continue;
+    J.j[nj++] = GatherJob{P.np, P.key, P.src, g.l, g.a, P.x, P.y, P.z, P.q, dc ? dc + k * (DMAX + 1) : nullptr};
+    nmax = std::max(nmax, P.np);
   }
-}
-
-// targets of the group, sorted by their depth-DMAX Morton keys (every coarser key is a prefix)
-void build_group_targets(Ctx &c, Group &g, int64_t n, const double *q, const double *xyz, const int32_t *layer,
-                         uint32_t *const *rank, const int64_t *cnt) {
-  GroupGeom gg = group_geom(c, g, cnt);
-  RankPtrs rk;
-  for (int k = 0; k <= c.md.L; ++k) rk.r[k] = rank[k];
-  g.T.np = cnt[g.l];
-  g.T.key = c.arena.get<uint64_t>(g.T.np);
-  g.T.src = c.arena.get<uint32_t>(g.T.np);
-  k_make_targets<<<(unsigned)((n + 255) / 256), 256, 0, c.stream>>>(n, xyz, layer, rk, gg, g.T.key, g.T.src);
+  if (!nj) return;
+  k_gather_points<<<dim3((unsigned)((nmax + 255) / 256), nj), 256, 0, c.stream>>>(q, xyz, c.md, images, J);
   LPB_LAUNCH();
   c.launches++;
-  radix_sort(c, g.T.key, g.T.src, g.T.np, DMAX * 3 + 4, 4);  // target keys: low 4 bits are zero
-  gather(c, g, g.T, 0, q, xyz, layer);
 }
 
-// images of the group, sorted by (depth-D leaf key, type, input order): every (leaf box,
+// targets of every group, sorted by their depth-DMAX Morton keys (every coarser key is a prefix); dc (may be
+// null): non-empty boxes per group and level [G][DMAX + 1]
+void build_targets(Ctx &c, std::vector<Group> &groups, int64_t n, const double *q, const double *xyz,
+                   const int32_t *layer, const RankPtrs &rank, const int64_t *cnt, uint32_t *dc) {
+  if (groups.empty()) return;
+  GroupGeoms G{};
+  std::vector<SortReq> reqs;
+  for (size_t k = 0; k < groups.size(); ++k) {
+    Group &g = groups[k];
+    g.T.np = cnt[g.l];
+    g.T.key = c.arena.get<uint64_t>(g.T.np);
+    g.T.src = c.arena.get<uint32_t>(g.T.np);
+    G.g[k] = group_geom(c, g, cnt);
+    G.g[k].key = g.T.key;
+    G.g[k].src = g.T.src;
+    reqs.push_back(SortReq{&g.T.key, &g.T.src, g.T.np, DMAX * 3 + 4, 4});  // the low 4 bits are zero
+  }
+  k_make_targets<<<(unsigned)((n + 255) / 256), 256, 0, c.stream>>>(n, xyz, layer, rank, (int)groups.size(), G);
+  LPB_LAUNCH();
+  c.launches++;
+  sort_batch(c, reqs);
+  gather(c, groups, 0, q, xyz, dc);
+}
+
+// images of every group, sorted by (depth-D leaf key, type, input order): every (leaf box,
 // type) pair is one contiguous run
-void build_group_images(Ctx &c, Group &g, int64_t n, const double *q, const double *xyz, const int32_t *layer,
-                        uint32_t *const *rank, const int64_t *cnt) {
-  GroupGeom gg = group_geom(c, g, cnt);
-  RankPtrs rk;
-  for (int k = 0; k <= c.md.L; ++k) rk.r[k] = rank[k];
+void build_images(Ctx &c, std::vector<Group> &groups, int64_t n, const double *q, const double *xyz,
+                  const int32_t *layer, const RankPtrs &rank, const int64_t *cnt) {
+  if (groups.empty()) return;
   int64_t tot = 0;
   for (int t = 0; t < 2 * c.md.L; ++t) {
     int lp, b;
     type_decode(t, lp, b);
     tot += cnt[lp];
   }
-  g.I.np = tot;
-  g.I.key = c.arena.get<uint64_t>(g.I.np);
-  g.I.src = c.arena.get<uint32_t>(g.I.np);
-  k_make_images<<<(unsigned)((n + 255) / 256), 256, 0, c.stream>>>(n, xyz, layer, c.md, rk, gg, g.D, g.I.key,
-                                                                   g.I.src);
-  LPB_LAUNCH();
-  c.launches++;
-  radix_sort(c, g.I.key, g.I.src, g.I.np, g.D * 3 + 4, 0);
-  gather(c, g, g.I, 1, q, xyz, layer);
-}
-
-// number of non-empty target boxes at every level 2..DMAX (automatic depth rule)
-__global__ void k_count_levels(int64_t np, const uint64_t *key, uint32_t *cnt) {
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  for (int l = 2; l <= DMAX; ++l) {
-    bool f = false;
-    if (k < np) {
-      const int sh = 4 + 3 * (DMAX - l);
-      f = (k == 0) || ((key[k] >> sh) != (key[k - 1] >> sh));
-    }
-    const unsigned b = __popc(__ballot_sync(0xffffffffu, f));
-    if ((threadIdx.x & 31) == 0 && b) atomicAdd(&cnt[l], b);
+  GroupGeoms G{};
+  std::vector<SortReq> reqs;
+  for (size_t k = 0; k < groups.size(); ++k) {
+    Group &g = groups[k];
+    g.I.np = tot;
+    g.I.key = c.arena.get<uint64_t>(g.I.np);
+    g.I.src = c.arena.get<uint32_t>(g.I.np);
+    G.g[k] = group_geom(c, g, cnt);
+    G.g[k].key = g.I.key;
+    G.g[k].src = g.I.src;
+    reqs.push_back(SortReq{&g.I.key, &g.I.src, g.I.np, g.D * 3 + 4, 0});
   }
-}
-void count_levels(Ctx &c, Group &g, uint32_t *d_counts) {
-  if (!g.T.np) return;
-  k_count_levels<<<(unsigned)((g.T.np + 255) / 256), 256, 0, c.stream>>>(g.T.np, g.T.key, d_counts);
+  k_make_images<<<(unsigned)((n + 255) / 256), 256, 0, c.stream>>>(n, xyz, layer, c.md, rank, (int)groups.size(), G);
   LPB_LAUNCH();
   c.launches++;
+  sort_batch(c, reqs);
+  gather(c, groups, 1, q, xyz, nullptr);
 }
 
 // ---------------------------------------------------------------------------------------
-// boxes per level
+// boxes of every level of every point set.  The points are sorted by key, so the boxes of a level are
+// the runs of equal key prefix: for each (set, level) a scan of the run starts numbers the boxes
+// (k_box_tiles, k_box_sums), every run start writes its box, every point keeps its box number
+// (k_box_fill), and the links between levels follow from the box numbers of the run starts (k_box_links).
+// Four launches for all sets and levels.  Image sets also number their (leaf box, type) segments.
 // ---------------------------------------------------------------------------------------
-__global__ void k_leaf_flags(int64_t np, const uint64_t *key, int sh, uint32_t *f) {
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < np) f[k] = (k == 0 || (key[k] >> sh) != (key[k - 1] >> sh)) ? 1u : 0u;
+struct BoxJob {
+  const uint64_t *pkey;
+  int64_t np, tile0, box0, cap;  // first tile / first box slot of this job in the flattened launches
+  int sh, seg;                   // key prefix: key >> sh; seg: (leaf box, type) segments
+  uint32_t *idx, *sums, *total;  // box of every point, per-tile counts, number of boxes
+  uint64_t *key;
+  uint32_t *pstart, *pcount;     // segments: seg_start, seg_count
+  uint32_t *start, *count;       // children (null at the leaf level)
+  const uint32_t *cidx, *ctotal; // the finer level's box numbers and total
+  uint32_t *parent;              // (null at level 2)
+  const uint32_t *pidx;          // the coarser level's box numbers
+  uint32_t *sbox, *stype;        // segments: leaf box (cidx: the leaf level's numbers), type
+};
+__device__ __forceinline__ bool box_starts(const BoxJob &j, int64_t k) {
+  return k == 0 || (j.pkey[k] >> j.sh) != (j.pkey[k - 1] >> j.sh);
 }
-__global__ void k_seg_flags(int64_t np, const uint64_t *key, int sh, uint32_t *f) {
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= np) return;
-  const uint64_t a = ((key[k] >> 4) >> sh << 4) | (key[k] & 15ull);
-  const uint64_t b = k ? (((key[k - 1] >> 4) >> sh << 4) | (key[k - 1] & 15ull)) : 0ull;
-  f[k] = (k == 0 || a != b) ? 1u : 0u;
+template <int64_t BoxJob::*M>
+__device__ __forceinline__ int box_find(const BoxJob *jobs, int nj, int64_t g) {
+  int lo = 0, hi = nj - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (jobs[mid].*M <= g) lo = mid; else hi = mid - 1;
+  }
+  return lo;
 }
-// flagged item k starts box idx[k]
-__global__ void k_leaf_boxes(int64_t np, const uint64_t *key, int sh, const uint32_t *f, const uint32_t *idx,
-                             uint64_t *bkey, uint32_t *bstart) {
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < np && f[k]) {
-    bkey[idx[k]] = key[k] >> sh;
-    bstart[idx[k]] = (uint32_t)k;
+__global__ void k_box_tiles(const BoxJob *jobs, int nj) {
+  const BoxJob j = jobs[box_find<&BoxJob::tile0>(jobs, nj, blockIdx.x)];
+  __shared__ uint32_t sm[32];
+  const int64_t tile = (int64_t)blockIdx.x - j.tile0;
+  const int64_t base = tile * SCAN_TILE + (int64_t)threadIdx.x * SCAN_ITEMS;
+  uint32_t f = 0;
+#pragma unroll
+  for (int k = 0; k < SCAN_ITEMS; ++k)
+    if (base + k < j.np && box_starts(j, base + k)) f |= 1u << k;
+  uint32_t tot;
+  uint32_t run = block_exclusive_scan(__popc(f), sm, &tot);
+#pragma unroll
+  for (int k = 0; k < SCAN_ITEMS; ++k) {
+    run += (f >> k) & 1u;
+    if (base + k < j.np) j.idx[base + k] = run;  // run starts of the tile up to and including this point
+  }
+  if (threadIdx.x == 0) j.sums[tile] = tot;
+}
+__global__ void k_box_sums(const BoxJob *jobs) {
+  const BoxJob &j = jobs[blockIdx.x];
+  __shared__ uint32_t sm[32];
+  const int64_t m = (j.np + SCAN_TILE - 1) / SCAN_TILE;
+  uint32_t carry = 0;
+  for (int64_t c = 0; c < m; c += blockDim.x) {
+    const int64_t i = c + threadIdx.x;
+    const uint32_t v = i < m ? j.sums[i] : 0u;
+    uint32_t tot;
+    const uint32_t ex = block_exclusive_scan(v, sm, &tot);
+    if (i < m) j.sums[i] = carry + ex;
+    carry += tot;
+  }
+  if (threadIdx.x == 0) *j.total = carry;
+}
+__global__ void k_box_fill(const BoxJob *jobs, int nj) {
+  const BoxJob j = jobs[box_find<&BoxJob::tile0>(jobs, nj, blockIdx.x)];
+  const int64_t tile = (int64_t)blockIdx.x - j.tile0;
+  const uint32_t before = j.sums[tile];
+  for (int x = threadIdx.x; x < SCAN_TILE; x += blockDim.x) {
+    const int64_t k = tile * SCAN_TILE + x;
+    if (k >= j.np) break;
+    const uint32_t b = before + j.idx[k] - 1u;
+    j.idx[k] = b;
+    if (!box_starts(j, k)) continue;
+    j.pstart[b] = (uint32_t)k;
+    if (j.seg) j.stype[b] = (uint32_t)(j.pkey[k] & 15ull);
+    else j.key[b] = j.pkey[k] >> j.sh;
   }
 }
-__global__ void k_counts_from_starts(const uint32_t *d_n, const uint32_t *start, uint32_t total, uint32_t *cnt,
-                                     int64_t cap) {
-  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t n = *d_n;
-  if (b < n && b < cap) cnt[b] = ((b + 1 < n) ? start[b + 1] : total) - start[b];
-}
-__global__ void k_seg_fill(int64_t np, const uint64_t *key, const uint32_t *f, const uint32_t *sidx,
-                           const uint32_t *bf, const uint32_t *bidx, uint32_t *sstart, uint32_t *sbox,
-                           uint32_t *stype) {
-  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (k < np && f[k]) {
-    const uint32_t s = sidx[k];
-    sstart[s] = (uint32_t)k;
-    sbox[s] = bidx[k] + bf[k] - 1u;
-    stype[s] = (uint32_t)(key[k] & 15ull);
+__global__ void k_box_links(const BoxJob *jobs, int nj, int64_t ntot) {
+  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= ntot) return;
+  const BoxJob &j = jobs[box_find<&BoxJob::box0>(jobs, nj, g)];
+  const int64_t b = g - j.box0;
+  const uint32_t n = *j.total;
+  if (b >= n || b >= j.cap) return;
+  const uint32_t s = j.pstart[b], e = b + 1 < n ? j.pstart[b + 1] : (uint32_t)j.np;
+  j.pcount[b] = e - s;
+  if (j.seg) {
+    j.sbox[b] = j.cidx[s];
+    return;
   }
-}
-// parents of level l+1 boxes
-__global__ void k_parent_flags(const uint32_t *d_n, const uint64_t *ckey, uint32_t *f, int64_t cap) {
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t n = *d_n;
-  if (j < n && j < cap) f[j] = (j == 0 || (ckey[j] >> 3) != (ckey[j - 1] >> 3)) ? 1u : 0u;
-  else if (j < cap) f[j] = 0u;
-}
-__global__ void k_parent_fill(const uint32_t *d_n, const uint64_t *ckey, const uint32_t *f, const uint32_t *idx,
-                              uint32_t *cparent, uint64_t *pkey, uint32_t *pstart, int64_t cap) {
-  const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t n = *d_n;
-  if (j >= n || j >= cap) return;
-  const uint32_t pid = idx[j] + f[j] - 1u;
-  cparent[j] = pid;
-  if (f[j]) {
-    pkey[pid] = ckey[j] >> 3;
-    pstart[pid] = (uint32_t)j;
+  if (j.start) {
+    const uint32_t c0 = j.cidx[s], c1 = b + 1 < n ? j.cidx[e] : *j.ctotal;
+    j.start[b] = c0;
+    j.count[b] = c1 - c0;
   }
+  if (j.parent) j.parent[b] = j.pidx[s];
 }
 
 static int64_t level_cap(int64_t np, int l) {
@@ -412,111 +580,97 @@ static int64_t level_cap(int64_t np, int l) {
   return c < np ? c : np;
 }
 
-static void build_levels(Ctx &c, PointSet &P, int D, bool images) {
-  const int64_t np = P.np;
-  const unsigned pb = (unsigned)((np + 255) / 256);
-  for (int l = 0; l <= DMAX; ++l) P.lev[l] = Level();
-  if (!np) return;
-  // targets carry depth-DMAX keys, images depth-D keys (both shifted by 4 type bits)
-  const int sh = images ? 4 : 4 + 3 * (DMAX - D);
-  uint32_t *f = c.arena.get<uint32_t>(np), *idx = c.arena.get<uint32_t>(np);
-  Level &Lf = P.lev[D];
-  const int64_t capD = level_cap(np, D);
-  Lf.key = c.arena.get<uint64_t>(capD);
-  Lf.start = c.arena.get<uint32_t>(capD);
-  Lf.count = c.arena.get<uint32_t>(capD);
-  Lf.d_n = c.arena.get<uint32_t>(1);
-  k_leaf_flags<<<pb, 256, 0, c.stream>>>(np, P.key, sh, f);
-  LPB_LAUNCH();
-  scan_u32(c, f, idx, np, Lf.d_n);
-  k_leaf_boxes<<<pb, 256, 0, c.stream>>>(np, P.key, sh, f, idx, Lf.key, Lf.start);
-  LPB_LAUNCH();
-  k_counts_from_starts<<<(unsigned)((capD + 255) / 256), 256, 0, c.stream>>>(Lf.d_n, Lf.start, (uint32_t)np,
-                                                                              Lf.count, capD);
-  LPB_LAUNCH();
-  c.launches += 3;
-  if (images) {
-    uint32_t *sf = c.arena.get<uint32_t>(np), *sidx = c.arena.get<uint32_t>(np);
-    P.seg_start = c.arena.get<uint32_t>(np);
-    P.seg_count = c.arena.get<uint32_t>(np);
-    P.seg_box = c.arena.get<uint32_t>(np);
-    P.seg_type = c.arena.get<uint32_t>(np);
-    P.d_nseg = c.arena.get<uint32_t>(1);
-    k_seg_flags<<<pb, 256, 0, c.stream>>>(np, P.key, 0, sf);
-    LPB_LAUNCH();
-    scan_u32(c, sf, sidx, np, P.d_nseg);
-    k_seg_fill<<<pb, 256, 0, c.stream>>>(np, P.key, sf, sidx, f, idx, P.seg_start, P.seg_box, P.seg_type);
-    LPB_LAUNCH();
-    k_counts_from_starts<<<pb, 256, 0, c.stream>>>(P.d_nseg, P.seg_start, (uint32_t)np, P.seg_count, np);
-    LPB_LAUNCH();
-    c.launches += 3;
-  }
-  for (int l = D - 1; l >= 2; --l) {
-    Level &C = P.lev[l + 1], &Pa = P.lev[l];
-    const int64_t ccap = level_cap(np, l + 1), pcap = level_cap(np, l);
-    uint32_t *cf = c.arena.get<uint32_t>(ccap), *cidx = c.arena.get<uint32_t>(ccap);
-    Pa.key = c.arena.get<uint64_t>(pcap);
-    Pa.start = c.arena.get<uint32_t>(pcap);
-    Pa.count = c.arena.get<uint32_t>(pcap);
-    Pa.d_n = c.arena.get<uint32_t>(1);
-    C.parent = c.arena.get<uint32_t>(ccap);
-    const unsigned cb = (unsigned)((ccap + 255) / 256);
-    k_parent_flags<<<cb, 256, 0, c.stream>>>(C.d_n, C.key, cf, ccap);
-    LPB_LAUNCH();
-    scan_u32(c, cf, cidx, ccap, Pa.d_n);
-    k_parent_fill<<<cb, 256, 0, c.stream>>>(C.d_n, C.key, cf, cidx, C.parent, Pa.key, Pa.start, ccap);
-    LPB_LAUNCH();
-    k_counts_from_starts<<<(unsigned)((pcap + 255) / 256), 256, 0, c.stream>>>(Pa.d_n, Pa.start, 0u, Pa.count,
-                                                                                pcap);
-    LPB_LAUNCH();
-    c.launches += 3;
-  }
-}
-
-__global__ void k_fix_last_count(const uint32_t *d_nc, const uint32_t *d_np, const uint32_t *pstart,
-                                 uint32_t *pcount) {
-  // the last parent's count is (number of children) - start
-  const uint32_t np = *d_np;
-  if (np) pcount[np - 1] = *d_nc - pstart[np - 1];
-}
-
-// points of every box of a coarser target level: its first child's first point, up to the next
-// box's first point (points are sorted by key, so a box's points are one contiguous run)
-__global__ void k_point_ranges(const uint32_t *d_n, const uint32_t *start, const uint32_t *cpstart, uint32_t np,
-                               uint32_t *pstart, uint32_t *pcount, int64_t cap) {
-  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t n = *d_n;
-  if (b >= n || b >= cap) return;
-  const uint32_t s = cpstart[start[b]];
-  pstart[b] = s;
-  pcount[b] = ((b + 1 < n) ? cpstart[start[b + 1]] : np) - s;
-}
-
-void build_group_boxes(Ctx &c, Group &g) {
-  build_levels(c, g.T, g.D, false);
-  build_levels(c, g.I, g.D, true);
-  if (g.T.np) {
-    g.T.lev[g.D].pstart = g.T.lev[g.D].start;
-    g.T.lev[g.D].pcount = g.T.lev[g.D].count;
-    for (int l = g.D - 1; l >= 2; --l) {
-      Level &P = g.T.lev[l];
-      const int64_t cap = level_cap(g.T.np, l);
-      P.pstart = c.arena.get<uint32_t>(cap);
-      P.pcount = c.arena.get<uint32_t>(cap);
-      k_point_ranges<<<(unsigned)((cap + 255) / 256), 256, 0, c.stream>>>(P.d_n, P.start, g.T.lev[l + 1].pstart,
-                                                                         (uint32_t)g.T.np, P.pstart, P.pcount, cap);
-      LPB_LAUNCH();
-      c.launches++;
+// the box arrays of every group; *dcounts, *ncounts: the device array of box counts in the order of
+// read_box_counts
+void build_boxes(Ctx &c, std::vector<Group> &groups, uint32_t **dcounts, size_t *ncounts) {
+  std::vector<BoxJob> jobs;
+  size_t nc = 0;
+  for (auto &g : groups) nc += 2 * (size_t)(g.D - 1) + 1;
+  uint32_t *counts = c.arena.get<uint32_t>(nc);
+  LPB_CUDA(cudaMemsetAsync(counts, 0, sizeof(uint32_t) * nc, c.stream));
+  *dcounts = counts;
+  *ncounts = nc;
+  int64_t tiles = 0, boxes = 0;
+  size_t at = 0;
+  for (auto &g : groups)
+    for (int which = 0; which < 2; ++which) {
+      PointSet &P = which ? g.I : g.T;
+      const int64_t np = P.np, nt = (np + SCAN_TILE - 1) / SCAN_TILE;
+      for (int l = 0; l <= DMAX; ++l) P.lev[l] = Level();
+      for (int l = 2; l <= g.D; ++l, ++at) {
+        if (!np) continue;
+        Level &L = P.lev[l];
+        BoxJob j{};
+        j.pkey = P.key; j.np = np; j.tile0 = tiles; j.box0 = boxes; j.cap = level_cap(np, l);
+        // targets carry depth-DMAX keys, images depth-D keys (both shifted by 4 type bits)
+        j.sh = 4 + 3 * ((which ? g.D : DMAX) - l);
+        j.idx = c.arena.get<uint32_t>(np);
+        j.sums = c.arena.get<uint32_t>(nt);
+        j.total = L.d_n = counts + at;
+        j.key = L.key = c.arena.get<uint64_t>(j.cap);
+        j.pstart = L.pstart = c.arena.get<uint32_t>(j.cap);
+        j.pcount = L.pcount = c.arena.get<uint32_t>(j.cap);
+        if (l < g.D) {
+          j.start = L.start = c.arena.get<uint32_t>(j.cap);
+          j.count = L.count = c.arena.get<uint32_t>(j.cap);
+        } else {
+          L.start = L.pstart;
+          L.count = L.pcount;
+        }
+        if (l > 2) {
+          j.parent = L.parent = c.arena.get<uint32_t>(j.cap);
+          j.pidx = jobs.back().idx;
+          jobs.back().cidx = j.idx;
+          jobs.back().ctotal = j.total;
+        }
+        jobs.push_back(j);
+        tiles += nt;
+        boxes += j.cap;
+      }
+      if (which) {
+        if (np) {
+          BoxJob j = jobs.back();  // the leaf level's keys with their type bits
+          j.tile0 = tiles; j.box0 = boxes; j.cap = np; j.sh = 0; j.seg = 1;
+          j.cidx = j.idx;
+          j.idx = c.arena.get<uint32_t>(np);
+          j.sums = c.arena.get<uint32_t>(nt);
+          j.total = P.d_nseg = counts + at;
+          j.pstart = P.seg_start = c.arena.get<uint32_t>(np);
+          j.pcount = P.seg_count = c.arena.get<uint32_t>(np);
+          j.sbox = P.seg_box = c.arena.get<uint32_t>(np);
+          j.stype = P.seg_type = c.arena.get<uint32_t>(np);
+          j.start = j.count = j.parent = nullptr;
+          jobs.push_back(j);
+          tiles += nt;
+          boxes += np;
+        }
+        ++at;
+      }
     }
-  }
-  for (int which = 0; which < 2; ++which) {
-    PointSet &P = which ? g.I : g.T;
-    if (!P.np) continue;
-    for (int l = g.D - 1; l >= 2; --l) {
-      k_fix_last_count<<<1, 1, 0, c.stream>>>(P.lev[l + 1].d_n, P.lev[l].d_n, P.lev[l].start, P.lev[l].count);
-      LPB_LAUNCH();
-      c.launches++;
+  if (jobs.empty()) return;
+  const int nj = (int)jobs.size();
+  BoxJob *dj = c.arena.get<BoxJob>(jobs.size());
+  LPB_CUDA(cudaMemcpyAsync(dj, jobs.data(), sizeof(BoxJob) * jobs.size(), cudaMemcpyHostToDevice, c.stream));
+  k_box_tiles<<<(unsigned)tiles, SCAN_THREADS, 0, c.stream>>>(dj, nj);
+  LPB_LAUNCH();
+  k_box_sums<<<nj, 1024, 0, c.stream>>>(dj);
+  LPB_LAUNCH();
+  k_box_fill<<<(unsigned)tiles, SCAN_THREADS, 0, c.stream>>>(dj, nj);
+  LPB_LAUNCH();
+  k_box_links<<<(unsigned)((boxes + 255) / 256), 256, 0, c.stream>>>(dj, nj, boxes);
+  LPB_LAUNCH();
+  c.launches += 4;
+}
+
+// the counts of build_boxes, on the host, into the groups
+void read_box_counts(std::vector<Group> &groups, const uint32_t *h) {
+  for (auto &g : groups) {
+    for (int which = 0; which < 2; ++which) {
+      PointSet &P = which ? g.I : g.T;
+      for (int l = 2; l <= g.D; ++l) P.lev[l].n = P.np ? *h : 0, ++h;
     }
+    g.I.nseg = g.I.np ? *h : 0;
+    ++h;
   }
 }
 
@@ -539,132 +693,176 @@ __device__ __forceinline__ int64_t find_key(const uint64_t *keys, int64_t n, uin
 
 // dense box index of a level: grid[Morton key] = box index or -1 (levels up to GRID_LEV_MAX)
 constexpr int GRID_LEV_MAX = 8;
-__global__ void k_grid_fill(const uint64_t *key, const uint32_t *d_n, int32_t *grid, int64_t cap) {
-  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (b < *d_n && b < cap) grid[key[b]] = (int32_t)b;
-}
-static const int32_t *level_grid(Ctx &c, const Level &L, int lev, int64_t np) {
-  if (lev > GRID_LEV_MAX || !L.n) return nullptr;
-  const size_t cells = (size_t)1 << (3 * lev);
-  int32_t *grid = c.arena.get<int32_t>(cells);
-  LPB_CUDA(cudaMemsetAsync(grid, 0xff, sizeof(int32_t) * cells, c.stream));
-  const int64_t cap = level_cap(np, lev);
-  k_grid_fill<<<(unsigned)((cap + 255) / 256), 256, 0, c.stream>>>(L.key, L.d_n, grid, cap);
-  LPB_LAUNCH();
-  c.launches++;
-  return grid;
+struct GridJob {
+  const uint64_t *key;
+  int32_t *grid;
+  int64_t n, box0;
+};
+__global__ void k_grid_fill(const GridJob *jobs, int nj, int64_t ntot) {
+  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= ntot) return;
+  int lo = 0, hi = nj - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (jobs[mid].box0 <= g) lo = mid; else hi = mid - 1;
+  }
+  const GridJob &j = jobs[lo];
+  const int64_t b = g - j.box0;
+  if (b < j.n) j.grid[j.key[b]] = (int32_t)b;
 }
 
-// far = 1: V list over NOFF slots; far = 0: near list over NNEAR slots
-// react: reaction list (targets vs images): also records the classes in use
-// sgrid: dense box index of the source level (nullptr: binary search in skey)
-__global__ void k_lists(const uint64_t *tkey, const uint32_t *d_nt, const uint64_t *skey, const uint32_t *d_ns,
-                        const int32_t *sgrid, int lev, int far, int react, int a, int ws, int32_t *out,
-                        uint8_t *used) {
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int nslot = far ? NOFF : NNEAR;
-  const int64_t t = gid / nslot;
-  const int o = (int)(gid % nslot);
-  const int64_t nt = *d_nt;
-  if (t >= nt) return;
-  int dx, dy, dz;
-  if (far) off_decode(o, dx, dy, dz);
-  else near_decode(o, dx, dy, dz);
-  const uint64_t k = tkey[t];
-  const int ix = compact3(k >> 2), iy = compact3(k >> 1), iz = compact3(k);
-  const int jx = ix + dx, jy = iy + dy, jz = iz + dz, nc = 1 << lev;
-  int32_t res = -1;
-  const int cheb = cheb3(dx, dy, dz);
-  bool ok = jx >= 0 && jy >= 0 && jz >= 0 && jx < nc && jy < nc && jz < nc;
-  if (far) {
-    ok = ok && cheb > ws && abs((jx >> 1) - (ix >> 1)) <= ws && abs((jy >> 1) - (iy >> 1)) <= ws &&
-         abs((jz >> 1) - (iz >> 1)) <= ws;
-  } else {
-    ok = ok && cheb <= ws;
+// One list of one level: far = 1: V list over NOFF slots; far = 0: near list over NNEAR slots; react:
+// targets against images (the far list also records the classes in use and sorts the target boxes into
+// their rows, box layers k_t = 0 .. 2 ws from the interface).  One block per target box, every list of
+// every group in one launch.
+struct ListJob {
+  const uint64_t *tkey, *skey;
+  const int32_t *sgrid;  // dense box index of the source level (nullptr: binary search in skey)
+  int64_t nt, ns, box0;
+  int lev, far, react, a;
+  int32_t *out;
+  uint8_t *used;
+  int32_t *rows, *ktrow;
+  uint32_t *nrows;
+};
+constexpr int LIST_THREADS = 128;
+__global__ void __launch_bounds__(LIST_THREADS) k_lists(const ListJob *jobs, int nj, int ws) {
+  int lo = 0, hi = nj - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (jobs[mid].box0 <= (int64_t)blockIdx.x) lo = mid; else hi = mid - 1;
   }
-  const int64_t ns = *d_ns;
-  if (ok && ns > 0) {
-    const uint64_t sk = (spread3(jx) << 2) | (spread3(jy) << 1) | spread3(jz);
-    const int64_t s = sgrid ? (int64_t)sgrid[sk] : find_key(skey, ns, sk);
-    if (s >= 0) {
-      res = (int32_t)s;
-      if (react && far && used) {
-        const int half = 1 << (lev - 1);
-        const int kt = (a == 1) ? iz - half : half - 1 - iz;
-        const int ks = (a == 1) ? half - 1 - jz : jz - half;
-        const int kk = kk_index(kt, ks);
-        if (kk >= 0) used[rho_index(dx, dy) * NKK + kk] = 1;
+  const ListJob &J = jobs[lo];
+  const int64_t t = (int64_t)blockIdx.x - J.box0, ns = J.ns;
+  const int nslot = J.far ? NOFF : NNEAR, lev = J.lev, far = J.far, a = J.a;
+  const uint64_t *skey = J.skey;
+  const int32_t *sgrid = J.sgrid;
+  uint8_t *used = J.used;
+  int32_t *out = J.out + t * nslot;
+  const uint64_t k = J.tkey[t];
+  const int ix = compact3(k >> 2), iy = compact3(k >> 1), iz = compact3(k), nc = 1 << lev, half = nc >> 1;
+  const int kt = a == 1 ? iz - half : half - 1 - iz;
+  const bool react_far = J.react && far;
+  if (react_far && threadIdx.x == 0) {
+    J.ktrow[t] = kt;
+    if (kt >= 0 && kt < 2 * ws + 1) {
+      const uint32_t pos = atomicAdd(&J.nrows[kt], 1u);
+      J.rows[kt * J.nt + pos] = (int32_t)t;
+    }
+  }
+  // images lie across the interface: a box more than 2 ws layers from it has no image box in reach
+  const bool none = ns <= 0 || (J.react && kt > 2 * ws);
+  for (int o = threadIdx.x; o < nslot; o += LIST_THREADS) {
+    int32_t res = -1;
+    if (!none) {
+      int dx, dy, dz;
+      if (far) off_decode(o, dx, dy, dz);
+      else near_decode(o, dx, dy, dz);
+      const int jx = ix + dx, jy = iy + dy, jz = iz + dz;
+      const int cheb = cheb3(dx, dy, dz);
+      bool ok = jx >= 0 && jy >= 0 && jz >= 0 && jx < nc && jy < nc && jz < nc;
+      if (far) {
+        ok = ok && cheb > ws && abs((jx >> 1) - (ix >> 1)) <= ws && abs((jy >> 1) - (iy >> 1)) <= ws &&
+             abs((jz >> 1) - (iz >> 1)) <= ws;
+      } else {
+        ok = ok && cheb <= ws;
+      }
+      if (ok) {
+        const uint64_t sk = (spread3(jx) << 2) | (spread3(jy) << 1) | spread3(jz);
+        const int64_t s = sgrid ? (int64_t)sgrid[sk] : find_key(skey, ns, sk);
+        if (s >= 0) {
+          res = (int32_t)s;
+          if (react_far) {
+            const int ks = (a == 1) ? half - 1 - jz : jz - half;
+            const int kk = kk_index(kt, ks);
+            if (kk >= 0) used[rho_index(dx, dy) * NKK + kk] = 1;
+          }
+        }
       }
     }
-  }
-  out[t * nslot + o] = res;
-}
-
-// reaction target rows: boxes at k_t = 0 .. 2 ws box layers from the interface, per row
-__global__ void k_rows(const uint64_t *tkey, const uint32_t *d_nt, int lev, int a, int nkt, int32_t *rows,
-                       uint32_t *nrows, int32_t *ktrow, int64_t cap) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= *d_nt) return;
-  const int iz = compact3(tkey[t]);
-  const int half = 1 << (lev - 1);
-  const int kt = (a == 1) ? iz - half : half - 1 - iz;
-  ktrow[t] = kt;
-  if (kt >= 0 && kt < nkt) {
-    const uint32_t pos = atomicAdd(&nrows[kt], 1u);
-    rows[kt * cap + pos] = (int32_t)t;
+    out[o] = res;
   }
 }
 
-void build_group_lists(Ctx &c, Group &g, int parts) {
-  const int ws = c.ws, nkt = 2 * c.ws + 1;
-  for (int l = 2; l <= g.D; ++l) {
-    const Level &T = g.T.lev[l];
-    const Level &I = g.I.lev[l];
-    const int64_t nt = T.n;
-    if (!nt) continue;
-    const unsigned fb = (unsigned)((nt * NOFF + 255) / 256);
-    if (g.is_free && (parts & 1) && l <= g.Df) {
-      g.vfree[l] = c.arena.get<int32_t>(nt * NOFF);
-      const int32_t *tg = level_grid(c, T, l, g.T.np);
-      k_lists<<<fb, 256, 0, c.stream>>>(T.key, T.d_n, T.key, T.d_n, tg, l, 1, 0, g.a, ws, g.vfree[l], nullptr);
-      LPB_LAUNCH();
-      c.launches++;
+void build_lists(Ctx &c, std::vector<Group> &groups) {
+  std::vector<GridJob> gj;
+  std::vector<ListJob> lj;
+  int64_t gboxes = 0, lboxes = 0;
+  size_t cells = 0, zb = 0;
+  // pass 0 sizes the grids and the zeroed records, pass 1 hands them out
+  int32_t *grids = nullptr;
+  uint8_t *zero = nullptr;
+  for (int pass = 0; pass < 2; ++pass) {
+    if (pass) {
+      grids = c.arena.get<int32_t>(cells);
+      zero = c.arena.get<uint8_t>(zb);
+      if (cells) LPB_CUDA(cudaMemsetAsync(grids, 0xff, sizeof(int32_t) * cells, c.stream));
+      if (zb) LPB_CUDA(cudaMemsetAsync(zero, 0, zb, c.stream));
+      cells = zb = 0;
     }
-    if ((parts & 2) && I.n) {
-      g.vreact[l] = c.arena.get<int32_t>(nt * NOFF);
-      g.used[l] = c.arena.get<uint8_t>(NREACT_CLS);
-      LPB_CUDA(cudaMemsetAsync(g.used[l], 0, NREACT_CLS, c.stream));
-      const int32_t *ig = level_grid(c, I, l, g.I.np);
-      k_lists<<<fb, 256, 0, c.stream>>>(T.key, T.d_n, I.key, I.d_n, ig, l, 1, 1, g.a, ws, g.vreact[l], g.used[l]);
-      LPB_LAUNCH();
-      g.rows[l] = c.arena.get<int32_t>((size_t)NKT * nt);
-      g.nrows[l] = c.arena.get<uint32_t>(NKT);
-      g.ktrow[l] = c.arena.get<int32_t>(nt);
-      LPB_CUDA(cudaMemsetAsync(g.nrows[l], 0, NKT * sizeof(uint32_t), c.stream));
-      k_rows<<<(unsigned)((nt + 255) / 256), 256, 0, c.stream>>>(T.key, T.d_n, l, g.a, nkt, g.rows[l], g.nrows[l],
-                                                                 g.ktrow[l], nt);
-      LPB_LAUNCH();
-      c.launches += 2;
+    auto grid = [&](const Level &L, int lev) -> const int32_t * {
+      if (lev > GRID_LEV_MAX || !L.n) return nullptr;
+      int32_t *g = pass ? grids + cells : nullptr;
+      cells += (size_t)1 << (3 * lev);
+      if (pass) {
+        gj.push_back(GridJob{L.key, g, L.n, gboxes});
+        gboxes += L.n;
+      }
+      return g;
+    };
+    for (auto &g : groups) {
+      const bool fr = g.is_free && (g.parts & 1), re = g.parts & 2;
+      const int32_t *tgf = nullptr, *igd = nullptr;  // grids of the leaf levels
+      auto list = [&](int lev, const Level &S, const int32_t *sg, int far, int react, int32_t *&out) {
+        const Level &T = g.T.lev[lev];
+        ListJob j{};
+        if (far && react) {
+          uint8_t *z = zero + zb;
+          zb += (NREACT_CLS + 3) / 4 * 4 + NKT * sizeof(uint32_t);
+          zb = (zb + 15) / 16 * 16;
+          if (pass) {
+            g.used[lev] = j.used = z;
+            g.nrows[lev] = j.nrows = (uint32_t *)(z + (NREACT_CLS + 3) / 4 * 4);
+            g.rows[lev] = j.rows = c.arena.get<int32_t>((size_t)NKT * T.n);
+            g.ktrow[lev] = j.ktrow = c.arena.get<int32_t>(T.n);
+          }
+        }
+        if (!pass) return;
+        out = c.arena.get<int32_t>((size_t)T.n * (far ? NOFF : NNEAR));
+        j.tkey = T.key; j.skey = S.key; j.sgrid = sg; j.nt = T.n; j.ns = S.n; j.box0 = lboxes;
+        j.lev = lev; j.far = far; j.react = react; j.a = g.a; j.out = out;
+        lj.push_back(j);
+        lboxes += T.n;
+      };
+      for (int l = 2; l <= g.D; ++l) {
+        const Level &T = g.T.lev[l], &I = g.I.lev[l];
+        if (!T.n) continue;
+        if (fr && l <= g.Df) {
+          const int32_t *tg = grid(T, l);
+          if (l == g.Df) tgf = tg;
+          list(l, T, tg, 1, 0, g.vfree[l]);
+        }
+        if (re && I.n) {
+          const int32_t *ig = grid(I, l);
+          if (l == g.D) igd = ig;
+          list(l, I, ig, 1, 1, g.vreact[l]);
+        }
+      }
+      if (fr && g.T.lev[g.Df].n) list(g.Df, g.T.lev[g.Df], tgf, 0, 0, g.ufree);
+      if (re && g.T.lev[g.D].n && g.I.lev[g.D].n) list(g.D, g.I.lev[g.D], igd, 0, 1, g.ureact);
     }
   }
-  const int Df = g.Df;
-  const int64_t ntf = g.T.lev[Df].n;
-  if (g.is_free && (parts & 1) && ntf) {
-    g.ufree = c.arena.get<int32_t>(ntf * NNEAR);
-    k_lists<<<(unsigned)((ntf * NNEAR + 255) / 256), 256, 0, c.stream>>>(
-        g.T.lev[Df].key, g.T.lev[Df].d_n, g.T.lev[Df].key, g.T.lev[Df].d_n, nullptr, Df, 0, 0, g.a, ws, g.ufree,
-        nullptr);
+  if (!gj.empty()) {
+    GridJob *dg = c.arena.get<GridJob>(gj.size());
+    LPB_CUDA(cudaMemcpyAsync(dg, gj.data(), sizeof(GridJob) * gj.size(), cudaMemcpyHostToDevice, c.stream));
+    k_grid_fill<<<(unsigned)((gboxes + 255) / 256), 256, 0, c.stream>>>(dg, (int)gj.size(), gboxes);
     LPB_LAUNCH();
     c.launches++;
   }
-  const int D = g.D;
-  const int64_t nt = g.T.lev[D].n;
-  if (!nt) return;
-  const unsigned nb = (unsigned)((nt * NNEAR + 255) / 256);
-  if ((parts & 2) && g.I.lev[D].n) {
-    g.ureact = c.arena.get<int32_t>(nt * NNEAR);
-    k_lists<<<nb, 256, 0, c.stream>>>(g.T.lev[D].key, g.T.lev[D].d_n, g.I.lev[D].key, g.I.lev[D].d_n, nullptr, D, 0,
-                                      1, g.a, ws, g.ureact, nullptr);
+  if (!lj.empty()) {
+    ListJob *dl = c.arena.get<ListJob>(lj.size());
+    LPB_CUDA(cudaMemcpyAsync(dl, lj.data(), sizeof(ListJob) * lj.size(), cudaMemcpyHostToDevice, c.stream));
+    k_lists<<<(unsigned)lboxes, LIST_THREADS, 0, c.stream>>>(dl, (int)lj.size(), c.ws);
     LPB_LAUNCH();
     c.launches++;
   }
