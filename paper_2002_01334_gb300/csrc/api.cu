@@ -355,6 +355,7 @@ static void eval_front(Ctx &c, int64_t n, const double *q, const double *xyz, co
       read_box_counts(c.groups, hh);
     }
   }
+  build_type_masks(c, c.groups);
   build_lists(c, c.groups);
   prof_mark(c, "tree");
   // the FP32 free-space near field needs only the trees and near lists: on its own stream, beside
@@ -387,6 +388,10 @@ static void eval_front(Ctx &c, int64_t n, const double *q, const double *xyz, co
       if ((g.parts & 2) && g.ureact) {
         double zt, zs;
         z_gaps(g, zt, zs);
+        // no target box is near an image box (a box's layer is at least this, up to rounding far below
+        // the margin): no near field, no nodes for it
+        const double h = g.h(g.D);
+        if (std::floor(zt / h - 1e-6) + std::floor(zs / h - 1e-6) >= c.ws) continue;
         build_near_nodes(c, g, std::max(zt + zs, 1e-12), (c.ws + 1) * std::sqrt(2.0) * g.h(g.D));
       }
     }

@@ -123,190 +123,7 @@ __device__ __forceinline__ T wsum(T v) {
   return v;
 }
 
-struct LamTab {
-  double v[2 * MAXLAYER];
-};
-
-// ---------------------------------------------------------------------------------------
-// P2M: one warp per leaf (box, type) segment
-// ---------------------------------------------------------------------------------------
-template <typename T, int PT>
-__global__ void k_p2m(const uint32_t *d_nseg, const uint32_t *seg_start, const uint32_t *seg_count,
-                      const uint32_t *seg_box, const uint32_t *seg_type, int ntypes, const uint64_t *box_key,
-                      const double *x, const double *y, const double *z, const double *q, Geo geo, LamTab lt,
-                      int p, int K, typename C2<T>::t *M) {
-  typedef typename C2<T>::t T2;
-  __shared__ T2 acc[4][KHALF_MAX];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t seg = (int64_t)blockIdx.x * 4 + warp;
-  if (seg >= *d_nseg) return;
-  for (int e = lane; e < K; e += 32) acc[warp][e] = T2{0, 0};
-  const uint32_t st = seg_start[seg], cnt = seg_count[seg];
-  const uint32_t box = seg_box ? seg_box[seg] : (uint32_t)seg;
-  const uint32_t type = seg_type ? seg_type[seg] : 0u;
-  double cx, cy, cz;
-  box_center(box_key[box], geo, cx, cy, cz);
-  const double ih = 1.0 / geo.h;
-  const T lh = (T)(lt.v[type] * geo.h);
-  __syncwarp();
-  for (uint32_t b0 = 0; b0 < cnt; b0 += 32) {
-    const uint32_t j = b0 + lane;
-    const bool valid = j < cnt;
-    const uint32_t k = st + (valid ? j : 0);
-    const T rx = (T)((x[k] - cx) * ih), ry = (T)((y[k] - cy) * ih), rz = (T)((z[k] - cz) * ih);
-    const T qq = valid ? (T)(q[k] * 4.0 * PI) : T(0);
-    const T r2 = rx * rx + ry * ry + rz * rz;
-    T it[PT + 2];
-    itilde_all<T, PT + 1>(lh * lh * r2, it);
-    T2 Rmm = T2{(T)(0.5 / sqrt(PI)), T(0)};
-#pragma unroll
-    for (int m = 0; m <= PT; ++m) {
-      if (m > p) break;
-      if (m > 0) {
-        const T s = CK<T>::sect(m);
-        const T2 t = T2{Rmm.x * rx - Rmm.y * ry, Rmm.x * ry + Rmm.y * rx};
-        Rmm = T2{s * t.x, s * t.y};
-      }
-      T2 p1 = T2{0, 0}, p2 = T2{0, 0};
-#pragma unroll
-      for (int n = m; n <= PT; ++n) {
-        if (n > p) break;
-        T2 R;
-        if (n == m) R = Rmm;
-        else if (n == m + 1) { const T s = CK<T>::sub(m) * rz; R = T2{s * p1.x, s * p1.y}; }
-        else {
-          const T a = CK<T>::A(n, m) * rz, b = CK<T>::B(n, m) * r2;
-          R = T2{a * p1.x - b * p2.x, a * p1.y - b * p2.y};
-        }
-        p2 = p1;
-        p1 = R;
-        const T c = qq * it[n];
-        const T vr = wsum(c * R.x), vi = wsum(-c * R.y);
-        if (lane == 0) {
-          T2 &A = acc[warp][hidx(n, m)];
-          A.x += vr;
-          A.y += vi;
-        }
-      }
-    }
-  }
-  __syncwarp();
-  T2 *out = M + ((size_t)box * ntypes + type) * K;
-  for (int e = lane; e < K; e += 32) out[e] = acc[warp][e];
-}
-
-// ---------------------------------------------------------------------------------------
-// M2M (children -> parent) and L2L (parent -> child): azimuth-factored dense operators
-// ---------------------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ void rot_of_octant(uint64_t ckey, int m, const T *rot4, T &c, T &s) {
-  const int oct = (int)(ckey & 7ull);
-  const int dir = ((oct >> 2) & 1) * 2 + ((oct >> 1) & 1);
-  c = rot4[(dir * (PMAX + 1) + m) * 2];
-  s = rot4[(dir * (PMAX + 1) + m) * 2 + 1];
-}
-
-// One CTA per (parent, source type), one thread per output row.  All children's rotated
-// multipoles are staged at once; a thread reads each operator row once per z-half (child octant
-// bit cz) and applies it to the (at most four) children with that cz.
-constexpr int M2M_THREADS = 96;  // >= K for p <= 12 handled in one pass; larger K loops
-template <typename T>
-__global__ void __launch_bounds__(M2M_THREADS) k_m2m(const uint32_t *d_np, const uint32_t *pstart,
-                                                     const uint32_t *pcount, const uint64_t *ckey, int ntypes,
-                                                     const typename C2<T>::t *Mc, typename C2<T>::t *Mp,
-                                                     const T *ops, const T *rot4, int K) {
-  typedef typename C2<T>::t T2;
-  __shared__ T xr[8][KHALF_MAX], xi[8][KHALF_MAX];
-  __shared__ int slot[2][4], nslot[2];
-  __shared__ uint64_t ck_s[8];
-  const uint32_t box = blockIdx.x, type = blockIdx.y;
-  if (box >= *d_np) return;
-  const size_t KK = (size_t)K * K;
-  const uint32_t c0 = pstart[box], nc = min(pcount[box], 8u);
-  if (threadIdx.x < nc) ck_s[threadIdx.x] = ckey[c0 + threadIdx.x];
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    nslot[0] = nslot[1] = 0;
-    for (uint32_t c = 0; c < nc; ++c) {
-      const int cz = (int)(ck_s[c] & 1ull);
-      slot[cz][nslot[cz]++] = (int)c;
-    }
-  }
-  for (uint32_t e = threadIdx.x; e < nc * (uint32_t)K; e += blockDim.x) {
-    const int c = (int)(e / K), k = (int)(e % K);
-    T cs, sn;
-    rot_of_octant(ck_s[c], cK.mof[k], rot4, cs, sn);
-    const T2 v = Mc[((size_t)(c0 + c) * ntypes + type) * K + k];
-    xr[c][k] = cs * v.x - sn * v.y;
-    xi[c][k] = sn * v.x + cs * v.y;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < K; i += blockDim.x) {
-    const int m = cK.mof[i];
-    T ar = 0, ai = 0;
-    for (int cz = 0; cz < 2; ++cz) {
-      const int ns = nslot[cz];
-      if (ns == 0) continue;
-      const T *P = ops + ((size_t)type * 2 + cz) * 2 * KK + (size_t)i * K, *Q = P + KK;
-      T yr[4] = {0, 0, 0, 0}, yi[4] = {0, 0, 0, 0};
-      int sl[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) sl[j] = j < ns ? slot[cz][j] : slot[cz][0];
-#pragma unroll 2
-      for (int k = 0; k < K; ++k) {
-        const T pv = P[k], qv = Q[k];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          yr[j] += pv * xr[sl[j]][k];
-          yi[j] += qv * xi[sl[j]][k];
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        if (j >= ns) break;
-        T cs, sn;
-        rot_of_octant(ck_s[sl[j]], m, rot4, cs, sn);
-        ar += cs * yr[j] + sn * yi[j];
-        ai += cs * yi[j] - sn * yr[j];
-      }
-    }
-    Mp[((size_t)box * ntypes + type) * K + i] = T2{ar, ai};
-  }
-}
-
-template <typename T>
-__global__ void k_l2l(const uint32_t *d_nc, const uint32_t *cparent, const uint64_t *ckey,
-                      const typename C2<T>::t *Lp, typename C2<T>::t *Lc, const T *ops, const T *rot4, int K) {
-  typedef typename C2<T>::t T2;
-  __shared__ T xr[KHALF_MAX], xi[KHALF_MAX];
-  const uint32_t c = blockIdx.x;
-  if (c >= *d_nc) return;
-  const uint64_t ck = ckey[c];
-  const int cz = (int)(ck & 1ull);
-  const size_t KK = (size_t)K * K;
-  const T *P = ops + (size_t)cz * 2 * KK, *Q = P + KK;
-  const uint32_t par = cparent[c];
-  for (int e = threadIdx.x; e < K; e += blockDim.x) {
-    T cs, sn;
-    rot_of_octant(ck, cK.mof[e], rot4, cs, sn);
-    const T2 v = Lp[(size_t)par * K + e];
-    xr[e] = cs * v.x - sn * v.y;
-    xi[e] = sn * v.x + cs * v.y;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < K; i += blockDim.x) {
-    T yr = 0, yi = 0;
-    for (int k = 0; k < K; ++k) {
-      yr += P[(size_t)i * K + k] * xr[k];
-      yi += Q[(size_t)i * K + k] * xi[k];
-    }
-    T cs, sn;
-    rot_of_octant(ck, cK.mof[i], rot4, cs, sn);
-    T2 &dst = Lc[(size_t)c * K + i];
-    dst.x += cs * yr + sn * yi;
-    dst.y += cs * yi - sn * yr;
-  }
-}
+#include "passes.cuh"
 
 // ---------------------------------------------------------------------------------------
 // M2L: one launch for every (group, level, free / reaction row) job.  A work item is
@@ -691,7 +508,7 @@ __global__ void __launch_bounds__(256, 1) k_m2l_f32(const XJob *jobs, int njobs,
   }
 }
 
-// L[box][k] += sum over the partial slots, in slot order (deterministic)
+// L[box][k] += sum over the box's written partial slots, in slot order (deterministic)
 template <typename T>
 __global__ void k_m2l_reduce(const RJob *jobs, int njobs, int K) {
   typedef typename C2<T>::t T2;
@@ -707,97 +524,14 @@ __global__ void k_m2l_reduce(const RJob *jobs, int njobs, int K) {
   const int64_t box = e / K, k = e % K;
   const T2 *P = (const T2 *)J.part + box * M2L_NSLOT * K + k;
   T sx = 0, sy = 0;
-#pragma unroll
-  for (int s = 0; s < M2L_NSLOT; ++s) {
+  for (uint32_t m = J.smask ? J.smask[box] : (1u << M2L_NSLOT) - 1u; m; m &= m - 1) {
+    const int s = __ffs(m) - 1;
     sx += P[(size_t)s * K].x;
     sy += P[(size_t)s * K].y;
   }
   T2 &d = ((T2 *)J.L)[e];
   d.x += sx;
   d.y += sy;
-}
-
-// ---------------------------------------------------------------------------------------
-// L2P with field: one warp per leaf box
-// ---------------------------------------------------------------------------------------
-template <typename T, int PT>
-__global__ void k_l2p(const uint32_t *d_nb, const uint64_t *bkey, const uint32_t *bstart, const uint32_t *bcount,
-                      const double *x, const double *y, const double *z, const uint32_t *src, Geo geo, double lam,
-                      int p, int K, const typename C2<T>::t *L, double *phi, double *field) {
-  typedef typename C2<T>::t T2;
-  __shared__ T2 Ls[4][KHALF_MAX];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t box = (int64_t)blockIdx.x * 4 + warp;
-  if (box >= *d_nb) return;
-  for (int e = lane; e < K; e += 32) Ls[warp][e] = L[(size_t)box * K + e];
-  __syncwarp();
-  double cx, cy, cz;
-  box_center(bkey[box], geo, cx, cy, cz);
-  const double ih = 1.0 / geo.h;
-  const T lh = (T)(lam * geo.h);
-  const uint32_t st = bstart[box], cnt = bcount[box];
-  const T2 *Lw = Ls[warp];
-  for (uint32_t j = lane; j < cnt; j += 32) {
-    const uint32_t k = st + j;
-    const T rx = (T)((x[k] - cx) * ih), ry = (T)((y[k] - cy) * ih), rz = (T)((z[k] - cz) * ih);
-    const T r2 = rx * rx + ry * ry + rz * rz;
-    T it[PT + 3];
-    itilde_all<T, PT + 2>(lh * lh * r2, it);
-    T ph = 0, S1 = 0, Gz = 0, Gpr = 0, Gpi = 0;
-    T2 Rmm = T2{(T)(0.5 / sqrt(PI)), T(0)};
-#pragma unroll
-    for (int m = 0; m <= PT; ++m) {
-      if (m > p) break;
-      if (m > 0) {
-        const T s = CK<T>::sect(m);
-        const T2 t = T2{Rmm.x * rx - Rmm.y * ry, Rmm.x * ry + Rmm.y * rx};
-        Rmm = T2{s * t.x, s * t.y};
-      }
-      const T wm = m ? T(2) : T(1);
-      T2 p1 = T2{0, 0}, p2 = T2{0, 0};
-#pragma unroll
-      for (int n = m; n <= PT; ++n) {
-        if (n > p) break;
-        T2 R;
-        if (n == m) R = Rmm;
-        else if (n == m + 1) { const T s = CK<T>::sub(m) * rz; R = T2{s * p1.x, s * p1.y}; }
-        else {
-          const T a = CK<T>::A(n, m) * rz, b = CK<T>::B(n, m) * r2;
-          R = T2{a * p1.x - b * p2.x, a * p1.y - b * p2.y};
-        }
-        p2 = p1;
-        p1 = R;
-        const T2 Lnm = Lw[hidx(n, m)];
-        const T re = Lnm.x * R.x - Lnm.y * R.y;
-        ph += wm * it[n] * re;
-        S1 += wm * it[n + 1] / T(2 * n + 3) * re;
-        if (n < p) {
-          const T in1 = it[n + 1];
-          const T2 Lz = Lw[hidx(n + 1, m)];
-          Gz += wm * in1 * CK<T>::gz(n, m) * (Lz.x * R.x - Lz.y * R.y);
-          if (m >= 1) {
-            const T2 La = Lw[hidx(n + 1, m - 1)];
-            const T ca = in1 * CK<T>::ga(n, m);
-            Gpr += ca * (La.x * R.x - La.y * R.y);
-            Gpi += ca * (La.x * R.y + La.y * R.x);
-          }
-          const T2 Lb = Lw[hidx(n + 1, m + 1)];
-          const T cb = in1 * CK<T>::gb(n, m);
-          // - conj(Lb R)
-          Gpr -= cb * (Lb.x * R.x - Lb.y * R.y);
-          Gpi += cb * (Lb.x * R.y + Lb.y * R.x);
-        }
-      }
-    }
-    const uint32_t i = src[k];
-    phi[i] += (double)ph;
-    if (field) {
-      const double l2h = lam * lam * geo.h;  // lambda^2 r = lambda^2 h r_u
-      field[3 * i] -= l2h * (double)rx * (double)S1 + (double)Gpr * ih;
-      field[3 * i + 1] -= l2h * (double)ry * (double)S1 + (double)Gpi * ih;
-      field[3 * i + 2] -= l2h * (double)rz * (double)S1 + (double)Gz * ih;
-    }
-  }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1137,24 +871,34 @@ void init_fmm_tables(Ctx &c) {
 }
 
 template <typename T, int PT>
-static void launch_p2m(Ctx &c, const uint32_t *d_nseg, int64_t nseg_cap, const uint32_t *sst, const uint32_t *scnt,
-                       const uint32_t *sbox, const uint32_t *styp, int ntypes, const uint64_t *bkey,
-                       const PointSet &P, Geo geo, const LamTab &lt, void *M) {
-  typedef typename C2<T>::t T2;
-  k_p2m<T, PT><<<(unsigned)((nseg_cap + 3) / 4), 128, 0, c.stream>>>(d_nseg, sst, scnt, sbox, styp, ntypes, bkey,
-                                                                      P.x, P.y, P.z, P.q, geo, lt, c.p, c.K,
-                                                                      (T2 *)M);
-  LPB_LAUNCH();
-  c.launches++;
+static void launch_p2m(Ctx &c, const std::vector<P2MJob> &dense, const std::vector<P2MJob> &sparse, int64_t nd,
+                       int64_t ns) {
+  if (nd) {
+    k_p2m<T, PT><<<(unsigned)nd, 128, 0, c.stream>>>(upload_jobs(c, dense), (int)dense.size(), c.p, c.K);
+    LPB_LAUNCH();
+    c.launches++;
+  }
+  if (ns) {
+    k_p2m_sparse<T, PT><<<(unsigned)ns, 128, 0, c.stream>>>(upload_jobs(c, sparse), (int)sparse.size(), c.p, c.K);
+    LPB_LAUNCH();
+    c.launches++;
+  }
 }
 template <typename T, int PT>
-static void launch_l2p(Ctx &c, const Level &Lv, int64_t nb, const PointSet &P, Geo geo, double lam, const void *L,
-                       double *phi, double *field) {
-  typedef typename C2<T>::t T2;
-  k_l2p<T, PT><<<(unsigned)((nb + 3) / 4), 128, 0, c.stream>>>(Lv.d_n, Lv.key, Lv.start, Lv.count, P.x, P.y, P.z,
-                                                                P.src, geo, lam, c.p, c.K, (const T2 *)L, phi, field);
-  LPB_LAUNCH();
-  c.launches++;
+static void launch_l2p(Ctx &c, const std::vector<L2PJob> &dense, const std::vector<L2PJob> &sparse, int64_t nd,
+                       int64_t ns, double *phi, double *field) {
+  if (nd) {
+    k_l2p<T, PT, false><<<(unsigned)nd, 128, 0, c.stream>>>(upload_jobs(c, dense), (int)dense.size(), c.p, c.K, phi,
+                                                            field);
+    LPB_LAUNCH();
+    c.launches++;
+  }
+  if (ns) {
+    k_l2p<T, PT, true><<<(unsigned)ns, 128, 0, c.stream>>>(upload_jobs(c, sparse), (int)sparse.size(), c.p, c.K, phi,
+                                                           field);
+    LPB_LAUNCH();
+    c.launches++;
+  }
 }
 
 template <typename T, int TPT, int NR>
@@ -1189,52 +933,86 @@ static Geo geo_at(const Group &g, int l) {
   return G;
 }
 
-// P2M and M2M of one group; local expansions of every level zeroed
+// P2M and M2M of every group; local expansions of every level zeroed
 template <typename T>
-static void upward_t(Ctx &c, Group &g, int parts) {
+static void upward_t(Ctx &c, std::vector<Group> &groups) {
   typedef typename C2<T>::t T2;
-  const int K = c.K, D = g.D, Df = g.Df;
+  const int K = c.K;
   const Tables &tb = sizeof(T) == 8 ? g_tab_d[c.device] : g_tab_f[c.device];
-  const bool dofree = g.is_free && (parts & 1);
-  const bool doreact = (parts & 2) && g.I.np > 0;
-  LamTab lt_t, lt_i;
-  for (int k = 0; k < 2 * MAXLAYER; ++k) lt_t.v[k] = lt_i.v[k] = c.md.lam[g.l];
-  for (int t = 0; t < g.ntypes; ++t) {
-    int lp, b;
-    type_decode(t, lp, b);
-    lt_i.v[t] = c.md.lam[lp];
-  }
-  for (int l = 2; l <= D; ++l) {
-    const int64_t ntb = g.T.lev[l].n, nib = g.I.lev[l].n;
-    g.Lt[l] = c.arena.get<T2>(ntb * K);
-    LPB_CUDA(cudaMemsetAsync(g.Lt[l], 0, sizeof(T2) * ntb * K, c.stream));
-    if (dofree && l <= Df) g.Mfree[l] = c.arena.get<T2>(ntb * K);
-    if (doreact) g.Mimg[l] = c.arena.get<T2>(nib * g.ntypes * K);
-  }
-  // free-space P2M at the free-space leaves (level Df; their point ranges)
-  if (dofree)
-    PT_DISPATCH(launch_p2m, c, g.T.lev[Df].d_n, g.T.lev[Df].n, g.T.lev[Df].pstart, g.T.lev[Df].pcount, nullptr,
-                nullptr, 1, g.T.lev[Df].key, g.T, geo_at<T>(g, Df), lt_t, g.Mfree[Df]);
-  if (doreact) {
-    LPB_CUDA(cudaMemsetAsync(g.Mimg[D], 0, sizeof(T2) * g.I.lev[D].n * g.ntypes * K, c.stream));
-    PT_DISPATCH(launch_p2m, c, g.I.d_nseg, g.I.nseg, g.I.seg_start, g.I.seg_count, g.I.seg_box, g.I.seg_type,
-                g.ntypes, g.I.lev[D].key, g.I, geo_at<T>(g, D), lt_i, g.Mimg[D]);
-  }
-  for (int l = D; l >= 3; --l) {
-    if (dofree && l <= Df && g.T.lev[l - 1].n) {
-      k_m2m<T><<<dim3((unsigned)g.T.lev[l - 1].n, 1), M2M_THREADS, 0, c.stream>>>(
-          g.T.lev[l - 1].d_n, g.T.lev[l - 1].start, g.T.lev[l - 1].count, g.T.lev[l].key, 1, (const T2 *)g.Mfree[l],
-          (T2 *)g.Mfree[l - 1], (const T *)g.op_m2m_t[l], (const T *)tb.rot4, K);
-      LPB_LAUNCH();
-      c.launches++;
+  int64_t nl = 0;
+  int Dmax = 2;
+  for (auto &g : groups)
+    for (int l = 2; l <= g.D; ++l) nl += g.T.lev[l].n;
+  T2 *Lt = c.arena.get<T2>(nl * K);
+  LPB_CUDA(cudaMemsetAsync(Lt, 0, sizeof(T2) * nl * K, c.stream));
+  // absent (box, type) rows are neither written nor read; the SIMT M2L of the mixed mode (p > 10) reads them all
+  const bool zero_img = sizeof(T) == 4 && tc_chunks(c.p) > 4;
+  std::vector<P2MJob> dense, sparse;
+  int64_t nd = 0, ns = 0;
+  auto p2m = [&](const Group &g, const PointSet &P, int lev, const uint32_t *sst, const uint32_t *scnt,
+                 const uint32_t *sbox, const uint32_t *styp, int64_t nseg, int ntypes, void *M) {
+    P2MJob j;
+    j.sst = sst; j.scnt = scnt; j.sbox = sbox; j.styp = styp; j.nseg = nseg; j.ntypes = ntypes;
+    j.bkey = P.lev[lev].key; j.x = P.x; j.y = P.y; j.z = P.z; j.q = P.q; j.geo = geo_at<T>(g, lev); j.M = M;
+    for (int t = 0; t < 2 * MAXLAYER; ++t) j.lam[t] = c.md.lam[g.l];
+    if (styp)
+      for (int t = 0; t < ntypes; ++t) {
+        int lp, b;
+        type_decode(t, lp, b);
+        j.lam[t] = c.md.lam[lp];
+      }
+    if (P.np < P2M_SPARSE * nseg) {
+      j.item0 = ns;
+      ns += (nseg + 127) / 128;
+      sparse.push_back(j);
+    } else {
+      j.item0 = nd;
+      nd += (nseg + 3) / 4;
+      dense.push_back(j);
     }
-    if (doreact && g.I.lev[l - 1].n) {
-      k_m2m<T><<<dim3((unsigned)g.I.lev[l - 1].n, g.ntypes), M2M_THREADS, 0, c.stream>>>(
-          g.I.lev[l - 1].d_n, g.I.lev[l - 1].start, g.I.lev[l - 1].count, g.I.lev[l].key, g.ntypes,
-          (const T2 *)g.Mimg[l], (T2 *)g.Mimg[l - 1], (const T *)g.op_m2m_i[l], (const T *)tb.rot4, K);
-      LPB_LAUNCH();
-      c.launches++;
+  };
+  for (auto &g : groups) {
+    const bool dofree = g.is_free && (g.parts & 1), doreact = (g.parts & 2) && g.I.np > 0;
+    Dmax = std::max(Dmax, g.D);
+    for (int l = 2; l <= g.D; ++l) {
+      const int64_t ntb = g.T.lev[l].n, nib = g.I.lev[l].n;
+      g.Lt[l] = Lt;
+      Lt += ntb * K;
+      if (dofree && l <= g.Df) g.Mfree[l] = c.arena.get<T2>(ntb * K);
+      if (doreact) {
+        g.Mimg[l] = c.arena.get<T2>(nib * g.ntypes * K);
+        if (zero_img) LPB_CUDA(cudaMemsetAsync(g.Mimg[l], 0, sizeof(T2) * nib * g.ntypes * K, c.stream));
+      }
     }
+    // free-space P2M at the free-space leaves (level Df; their point ranges)
+    const Level &Lf = g.T.lev[g.Df];
+    if (dofree && Lf.n) p2m(g, g.T, g.Df, Lf.pstart, Lf.pcount, nullptr, nullptr, Lf.n, 1, g.Mfree[g.Df]);
+    if (doreact && g.I.nseg)
+      p2m(g, g.I, g.D, g.I.seg_start, g.I.seg_count, g.I.seg_box, g.I.seg_type, g.I.nseg, g.ntypes, g.Mimg[g.D]);
+  }
+  PT_DISPATCH(launch_p2m, c, dense, sparse, nd, ns);
+  const int threads = std::min(256, (K + 31) / 32 * 32);
+  for (int l = Dmax; l >= 3; --l) {
+    std::vector<M2MJob> jobs;
+    int64_t items = 0;
+    auto m2m = [&](const PointSet &P, const uint32_t *const *mask, int ntypes, const void *Mc, void *Mp, const void *ops) {
+      if (!P.lev[l - 1].n) return;
+      M2MJob j;
+      j.pstart = P.lev[l - 1].start; j.pcount = P.lev[l - 1].count; j.ckey = P.lev[l].key;
+      j.pmask = mask ? mask[l - 1] : nullptr; j.cmask = mask ? mask[l] : nullptr;
+      j.Mc = Mc; j.Mp = Mp; j.ops = ops; j.np = P.lev[l - 1].n; j.item0 = items; j.ntypes = ntypes;
+      items += j.np;
+      jobs.push_back(j);
+    };
+    for (auto &g : groups) {
+      if (l > g.D) continue;
+      if (g.is_free && (g.parts & 1) && l <= g.Df) m2m(g.T, nullptr, 1, g.Mfree[l], g.Mfree[l - 1], g.op_m2m_t[l]);
+      if ((g.parts & 2) && g.I.np > 0) m2m(g.I, g.tmask, g.ntypes, g.Mimg[l], g.Mimg[l - 1], g.op_m2m_i[l]);
+    }
+    if (jobs.empty()) continue;
+    k_m2m<T><<<(unsigned)items, threads, 0, c.stream>>>(upload_jobs(c, jobs), (int)jobs.size(), (const T *)tb.rot4, K);
+    LPB_LAUNCH();
+    c.launches++;
   }
 }
 
@@ -1262,15 +1040,8 @@ static void m2l_all_f64(Ctx &c, std::vector<Group> &groups) {
           ncls.push_back(NFREE_CLS);
         }
         if (kind == 1 && react_far && g.vreact[l]) {
-          const int64_t nib = g.I.lev[l].n, rows = nib * g.ntypes;
-          uint32_t *tmask = c.arena.get<uint32_t>((size_t)nib);
-          LPB_CUDA(cudaMemsetAsync(tmask, 0, sizeof(uint32_t) * nib, c.stream));
-          k_pair_types<<<(unsigned)((rows + 7) / 8), 256, 0, c.stream>>>((const double2 *)g.Mimg[l], rows, c.K,
-                                                                         g.ntypes, tmask);
-          LPB_LAUNCH();
-          c.launches++;
           j.vlist = g.vreact[l]; j.cls = tb.cls_react + (size_t)(g.a - 1) * NKT * NOFF; j.ktrow = g.ktrow[l];
-          j.tmask = tmask; j.M = (const double2 *)g.Mimg[l]; j.ops = (const double *)g.op_react[l];
+          j.tmask = g.tmask[l]; j.M = (const double2 *)g.Mimg[l]; j.ops = (const double *)g.op_react[l];
           j.ntypes = g.ntypes; j.nkt = 2 * c.ws + 1;
           jobs.push_back(j);
           ncls.push_back(NREACT_CLS);
@@ -1282,6 +1053,19 @@ static void m2l_all_f64(Ctx &c, std::vector<Group> &groups) {
   launch_pair_m2l(c, jobs, ncls, (const double *)tb.rot);
 }
 
+template <int P>
+static void launch_pack_w_p(const PackWJob *jobs, int njobs, int64_t items, int ws, cudaStream_t st) {
+  constexpr int K = (P + 1) * (P + 2) / 2;
+  k_tc_pack_w<P><<<(unsigned)items, PACKW_THREADS, sizeof(float) * 2 * K * K, st>>>(jobs, njobs, ws);
+}
+static void launch_pack_w(int p, const PackWJob *jobs, int njobs, int64_t items, int ws, cudaStream_t st) {
+  switch (p) {
+#define LPB_TC_CASE(P) case P: launch_pack_w_p<P>(jobs, njobs, items, ws, st); break;
+    LPB_TC_CASE(2) LPB_TC_CASE(3) LPB_TC_CASE(4) LPB_TC_CASE(5) LPB_TC_CASE(6) LPB_TC_CASE(7) LPB_TC_CASE(8)
+    LPB_TC_CASE(9) LPB_TC_CASE(10)
+#undef LPB_TC_CASE
+  }
+}
 template <int P>
 static void launch_tc_p(const TJob *jobs, int njobs, int64_t items, int *status, cudaStream_t st) {
   LPB_ATTR_ONCE(k_m2l_tc<P>, tc_smem(tc_chunks(P)));
@@ -1311,6 +1095,17 @@ static void m2l_all_f32(Ctx &c, std::vector<Group> &groups) {
   const bool use_tc = tc_nc <= 4;  // p <= 10
   std::vector<TJob> tjobs;
   int64_t titems = 0;
+  std::vector<PackRowJob> prow;
+  std::vector<PackWJob> pw;
+  int64_t row_items = 0, img_items = 0;
+  uint32_t *smasks = nullptr;
+  if (use_tc) {
+    int64_t nb = 0;
+    for (auto &g : groups)
+      for (int l = 2; l <= g.D; ++l) nb += g.T.lev[l].n;
+    smasks = c.arena.get<uint32_t>(nb);
+    LPB_CUDA(cudaMemsetAsync(smasks, 0, sizeof(uint32_t) * nb, c.stream));
+  }
   auto add = [&](const int32_t *tlist, const uint32_t *d_ntl, int64_t ntb, const int32_t *vlist,
                  const int32_t *cls_of, const void *M, const void *ops, void *part, int ntypes, int slot0,
                  const Level *par, const Level *lev) {
@@ -1332,34 +1127,40 @@ static void m2l_all_f32(Ctx &c, std::vector<Group> &groups) {
       const int64_t ntb = g.T.lev[l].n;
       if (!ntb || !(dofree || (react_far && g.vreact[l]))) continue;
       T2 *part = c.arena.get<T2>((size_t)ntb * M2L_NSLOT * c.K);
-      LPB_CUDA(cudaMemsetAsync(part, 0, sizeof(T2) * ntb * M2L_NSLOT * c.K, c.stream));
+      uint32_t *smask = nullptr;  // partial slots written (the SIMT kernels write or leave zero every slot)
+      if (use_tc) {
+        smask = smasks;
+        smasks += ntb;
+      } else {
+        LPB_CUDA(cudaMemsetAsync(part, 0, sizeof(T2) * ntb * M2L_NSLOT * c.K, c.stream));
+      }
       RJob r;
-      r.part = part; r.L = g.Lt[l]; r.n = ntb * c.K; r.e0 = relem;
+      r.part = part; r.L = g.Lt[l]; r.n = ntb * c.K; r.e0 = relem; r.smask = smask;
       rjobs.push_back(r);
       relem += r.n;
       const int N = 32 * tc_nc;
-      // split source rows and their masks; operator images
-      auto pack = [&](TJob &j, const void *M, int64_t nsb, const Level &sl, int side, const void *ops, int kind,
+      // split source rows; operator images
+      auto pack = [&](TJob &j, const void *M, const Level &sl, const uint32_t *mask, int side, const void *ops, int kind,
                       int ntypes, const uint8_t *used, int ncls) {
-        __half *rows = c.arena.get<__half>((size_t)nsb * ntypes * 2 * N);
-        float *rs = c.arena.get<float>((size_t)nsb * ntypes), *wsc = c.arena.get<float>((size_t)ncls * ntypes);
-        uint32_t *tmask = c.arena.get<uint32_t>((size_t)nsb);
-        unsigned char *wimg = c.arena.get<unsigned char>((size_t)ncls * ntypes * N * N * 4);
-        LPB_CUDA(cudaMemsetAsync(tmask, 0, sizeof(uint32_t) * nsb, c.stream));
-        const int64_t nr = nsb * ntypes;
-        k_tc_pack_rows<<<(unsigned)((nr + 7) / 8), 256, 0, c.stream>>>((const float2 *)M, nr, c.K, c.p, tc_nc, ntypes,
-                                                                        sl.key, l, side, c.ws, rows, rs, tmask);
-        LPB_LAUNCH();
-        k_tc_pack_w<<<ncls * ntypes, PACKW_THREADS, sizeof(float) * 2 * c.K * c.K, c.stream>>>(
-            (const float *)ops, kind, ntypes, used, c.ws, c.K, c.p, tc_nc, wimg, wsc);
-        LPB_LAUNCH();
-        c.launches += 2;
-        j.rows = rows; j.rscale = rs; j.tmask = tmask; j.wimg = wimg; j.wscale = wsc; j.ntypes = ntypes;
-        j.L = (float2 *)part; j.ntb = ntb;
+        PackRowJob r;
+        r.M = (const float2 *)M; r.nrows = sl.n * ntypes; r.item0 = row_items; r.ntypes = ntypes; r.mask = mask;
+        r.bkey = sl.key; r.lev = l; r.side = side;
+        r.rows = c.arena.get<__half>((size_t)r.nrows * 2 * N);
+        r.rscale = c.arena.get<float>((size_t)r.nrows);
+        row_items += (r.nrows + 7) / 8;
+        prow.push_back(r);
+        PackWJob w;
+        w.ops = (const float *)ops; w.kind = kind; w.ntypes = ntypes; w.used = used; w.item0 = img_items;
+        w.wimg = c.arena.get<unsigned char>((size_t)ncls * ntypes * N * N * 4);
+        w.wscale = c.arena.get<float>((size_t)ncls * ntypes);
+        img_items += (int64_t)ncls * ntypes;
+        pw.push_back(w);
+        j.rows = r.rows; j.rscale = r.rscale; j.tmask = mask; j.wimg = w.wimg; j.wscale = w.wscale; j.ntypes = ntypes;
+        j.L = (float2 *)part; j.smask = smask; j.ntb = ntb;
       };
       if (dofree && use_tc) {
         TJob j;
-        pack(j, g.Mfree[l], ntb, g.T.lev[l], 0, g.op_free[l], 0, 1, nullptr, TC_NFREE);
+        pack(j, g.Mfree[l], g.T.lev[l], nullptr, 0, g.op_free[l], 0, 1, nullptr, TC_NFREE);
         j.vlist = g.vfree[l]; j.cls_of = tb.tc_free; j.tlist = nullptr; j.d_ntl = nullptr;
         j.item0 = titems; j.slot0 = 0;
         const Level *par = l >= 3 ? &g.T.lev[l - 1] : nullptr;
@@ -1376,7 +1177,7 @@ static void m2l_all_f32(Ctx &c, std::vector<Group> &groups) {
       }
       if (react_far && g.vreact[l] && use_tc && g.ntypes <= 16) {
         TJob j;
-        pack(j, g.Mimg[l], g.I.lev[l].n, g.I.lev[l], g.a, g.op_react[l], 1, g.ntypes, g.used[l], TC_NREACT);
+        pack(j, g.Mimg[l], g.I.lev[l], g.tmask[l], g.a, g.op_react[l], 1, g.ntypes, g.used[l], TC_NREACT);
         j.vlist = g.vreact[l]; j.slot0 = M2L_NSLICE;
         j.pstart = nullptr; j.pcount = nullptr; j.ckey = nullptr; j.npar = 0;
         // a row is one layer of boxes: at most 4^l of them
@@ -1397,6 +1198,13 @@ static void m2l_all_f32(Ctx &c, std::vector<Group> &groups) {
     }
   }
   if (jobs.empty() && tjobs.empty()) return;
+  if (!prow.empty()) {
+    k_tc_pack_rows<<<(unsigned)row_items, 256, 0, c.stream>>>(upload_jobs(c, prow), (int)prow.size(), c.K, c.p, tc_nc, c.ws);
+    LPB_LAUNCH();
+    launch_pack_w(c.p, upload_jobs(c, pw), (int)pw.size(), img_items, c.ws, c.stream);
+    LPB_LAUNCH();
+    c.launches += 2;
+  }
   prof_mark(c, "m2l_prep");
   if (c.def.on && !tjobs.empty() && jobs.empty()) {
     // batched evaluation: the tensor-core M2L and the slot sums join a grouped launch
@@ -1482,25 +1290,56 @@ static void near_free_f64(Ctx &c, std::vector<Group> &groups, double *phi, doubl
   c.launches++;
 }
 
-// L2L (adding the parent's shifted expansion), L2P and the reaction near field of one group
+// L2L (adding the parent's shifted expansion), L2P and the reaction near field of every group
 template <typename T>
-static void downward_t(Ctx &c, Group &g, int parts, double *phi, double *field) {
-  typedef typename C2<T>::t T2;
-  const int K = c.K, D = g.D;
+static void downward_t(Ctx &c, std::vector<Group> &groups, double *phi, double *field) {
+  const int K = c.K;
   const Tables &tb = sizeof(T) == 8 ? g_tab_d[c.device] : g_tab_f[c.device];
-  const bool doreact = (parts & 2) && g.I.np > 0;
-  const bool react_near = doreact && !(parts & 4);
-  for (int l = 3; l <= D; ++l) {
-    const int64_t ntb = g.T.lev[l].n;
-    if (!ntb) continue;
-    k_l2l<T><<<(unsigned)ntb, 128, 0, c.stream>>>(g.T.lev[l].d_n, g.T.lev[l].parent, g.T.lev[l].key,
-                                                  (const T2 *)g.Lt[l - 1], (T2 *)g.Lt[l], (const T *)g.op_l2l[l],
-                                                  (const T *)tb.rot4, K);
+  int Dmax = 2;
+  for (auto &g : groups) Dmax = std::max(Dmax, g.D);
+  const int threads = std::min(256, (K + 31) / 32 * 32);
+  for (int l = 3; l <= Dmax; ++l) {
+    std::vector<L2LJob> jobs;
+    int64_t items = 0;
+    for (auto &g : groups) {
+      if (l > g.D || !g.T.lev[l].n) continue;
+      jobs.push_back(L2LJob{g.T.lev[l].parent, g.T.lev[l].key, g.Lt[l - 1], g.op_l2l[l], g.Lt[l], g.T.lev[l].n, items});
+      items += g.T.lev[l].n;
+    }
+    if (jobs.empty()) continue;
+    k_l2l<T><<<(unsigned)items, threads, 0, c.stream>>>(upload_jobs(c, jobs), (int)jobs.size(), (const T *)tb.rot4, K);
     LPB_LAUNCH();
     c.launches++;
   }
-  PT_DISPATCH(launch_l2p, c, g.T.lev[D], g.T.lev[D].n, g.T, geo_at<T>(g, D), c.md.lam[g.l], g.Lt[D], phi, field);
-  if (react_near && g.ureact && g.nodes) {
+  // the two groups of a layer add into the same outputs: one side after the other
+  for (int a = 1; a <= 2; ++a) {
+    std::vector<L2PJob> dense, sparse;
+    int64_t nd = 0, ns = 0;
+    for (auto &g : groups) {
+      const Level &Lv = g.T.lev[g.D];
+      if (g.a != a || !Lv.n) continue;
+      L2PJob j;
+      j.bkey = Lv.key; j.bstart = Lv.start; j.bcount = Lv.count; j.pbox = g.T.pbox;
+      j.x = g.T.x; j.y = g.T.y; j.z = g.T.z; j.src = g.T.src; j.L = g.Lt[g.D]; j.geo = geo_at<T>(g, g.D);
+      j.lam = c.md.lam[g.l];
+      if (g.T.np < P2M_SPARSE * Lv.n) {
+        j.n = g.T.np;
+        j.item0 = ns;
+        ns += (j.n + 127) / 128;
+        sparse.push_back(j);
+      } else {
+        j.n = Lv.n;
+        j.item0 = nd;
+        nd += (j.n + 3) / 4;
+        dense.push_back(j);
+      }
+    }
+    PT_DISPATCH(launch_l2p, c, dense, sparse, nd, ns, phi, field);
+  }
+  for (auto &g : groups) {
+    const bool react_near = (g.parts & 2) && g.I.np > 0 && !(g.parts & 4);
+    if (!react_near || !g.ureact || !g.nodes) continue;
+    const int D = g.D;
     k_p2p_react<T><<<(unsigned)g.T.lev[D].n, P2P_THREADS, 0, c.stream>>>(
         g.T.lev[D].d_n, g.T.lev[D].key, g.T.lev[D].start, g.T.lev[D].count, g.ureact, g.T.x, g.T.y, g.T.z, g.T.src,
         g.I.lev[D].start, g.I.lev[D].count, g.I.x, g.I.y, g.I.z, g.I.q, g.I.key, geo_at<T>(g, D), g.dI,
@@ -1529,7 +1368,7 @@ void run_fmm_front(Ctx &c, std::vector<Group> &groups) {
   const bool d = c.opts.precision == LPBFMM_FP64;
   // the free-space operators (side stream) are complete before the upward pass
   if (c.ev_free) LPB_CUDA(cudaStreamWaitEvent(c.stream, c.ev_free, 0));
-  for (auto &g : groups) d ? upward_t<double>(c, g, g.parts) : upward_t<float>(c, g, g.parts);
+  d ? upward_t<double>(c, groups) : upward_t<float>(c, groups);
   prof_mark(c, "upward");
   // the reaction tables and operators (side stream) are complete before any M2L
   if (c.ev_join) LPB_CUDA(cudaStreamWaitEvent(c.stream, c.ev_join, 0));
@@ -1580,8 +1419,7 @@ void run_fmm_back(Ctx &c, std::vector<Group> &groups, double *phi, double *field
   // outputs, are complete first
   if (c.far_async) LPB_CUDA(cudaStreamWaitEvent(c.stream, c.ev_far, 0));
   if (c.near_async) LPB_CUDA(cudaStreamWaitEvent(c.stream, c.ev_near, 0));
-  for (auto &g : groups)
-    d ? downward_t<double>(c, g, g.parts, phi, field) : downward_t<float>(c, g, g.parts, phi, field);
+  d ? downward_t<double>(c, groups, phi, field) : downward_t<float>(c, groups, phi, field);
   if (d) near_free_f64(c, groups, phi, field);
   prof_mark(c, "downward");
 }

@@ -159,6 +159,7 @@ struct PointSet {
   int64_t nseg = 0;
   uint32_t *seg_start = nullptr, *seg_count = nullptr, *seg_box = nullptr, *seg_type = nullptr;
   uint32_t *d_nseg = nullptr;
+  uint32_t *pbox = nullptr;  // leaf box of every point
 };
 
 struct Group {
@@ -177,6 +178,7 @@ struct Group {
   uint32_t *nrows[DMAX + 1] = {};  // [NKT]
   uint8_t *used[DMAX + 1] = {};  // reaction classes in use, NREACT_CLS per level
   int32_t *ktrow[DMAX + 1] = {};
+  uint32_t *tmask[DMAX + 1] = {};  // image boxes: source types present
   // expansions
   void *Mfree[DMAX + 1] = {}, *Mimg[DMAX + 1] = {}, *Lt[DMAX + 1] = {};
   // operators
@@ -198,7 +200,7 @@ struct Group {
 struct TJob {
   const void *rows;         // source rows [nsb][ntypes][NC][32 hi | 32 lo], split FP16 (k_tc_pack_rows)
   const float *rscale;      // [nsb][ntypes] inverse power of two of each row
-  const uint32_t *tmask;    // [nsb] source types with a nonzero row (the others are not written)
+  const uint32_t *tmask;    // [nsb] source types present (nullptr: type 0); other rows are not written
   const void *wimg;         // [ncls][ntypes] operator images (k_tc_pack_w)
   const float *wscale;      // [ncls][ntypes] inverse power of two of each image
   const int32_t *vlist;     // [ntb][NOFF]
@@ -206,6 +208,7 @@ struct TJob {
   const int32_t *tlist;     // target boxes (nullptr: octant or plain tiles over 0..ntb-1)
   const uint32_t *d_ntl;    // number of entries of tlist (device)
   float2 *L;                // partial sums [ntb][M2L_NSLOT][K]
+  uint32_t *smask;          // [ntb] slots written
   int64_t ntb, item0, ntiles;
   int slot0, ntypes;
   const uint32_t *pstart, *pcount;  // octant tiles (nullptr: plain tiles of 128)
@@ -215,6 +218,7 @@ struct TJob {
 // Sum of a level's M2L partial slots into its local expansions (k_m2l_reduce).
 struct RJob {
   const void *part;
+  const uint32_t *smask;  // [boxes] slots written (nullptr: all)
   void *L;
   int64_t n;     // boxes x K
   int64_t e0;    // first element of this job in the flattened launch
@@ -330,6 +334,7 @@ void build_images(Ctx &c, std::vector<Group> &groups, int64_t n, const double *q
 void build_boxes(Ctx &c, std::vector<Group> &groups, uint32_t **dcounts, size_t *ncounts);
 void read_box_counts(std::vector<Group> &groups, const uint32_t *h);
 void build_lists(Ctx &c, std::vector<Group> &groups);
+void build_type_masks(Ctx &c, std::vector<Group> &groups);
 // adaptive dual-tree lists of group g's free-space target tree with itself (diagnostic): records
 // of 5 int64 (kind 0 V / 1 U / 2 W / 3 X, target level, target key, source level, source key)
 void adaptive_lists(Ctx &c, Group &g, int s, int ws, std::vector<int64_t> &rec);

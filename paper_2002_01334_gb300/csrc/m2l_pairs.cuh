@@ -1,6 +1,6 @@
 // FP64 multipole-to-local over lists of translations sorted by operator.
 //
-// A translation is one (target box, offset, source type) with a nonzero source expansion.  All
+// A translation is one (target box, offset, source type) with charges of that type in the source box.  All
 // translations of one operator (class and source type) of a (group, level) job are gathered into
 // batches of PAIR_C columns, whatever targets they belong to; one CTA multiplies a batch by the
 // operator and writes every column's translated expansion to the translation's own slot.  Slots are
@@ -24,7 +24,7 @@ struct PairJob {
   const int32_t *vlist;      // [ntb][NOFF] source box or -1
   const int32_t *cls;        // [NOFF] (free) or [NKT][NOFF] (reaction, row ktrow[t]) operator class or -1
   const int32_t *ktrow;      // reaction: target row k_t of every box (nullptr: free)
-  const uint32_t *tmask;     // [nsb] source types with a nonzero expansion (nullptr: type 0 of every box)
+  const uint32_t *tmask;     // [nsb] source types present (nullptr: type 0 of every box)
   const double2 *M;          // [nsb][ntypes][K]
   const double *ops;         // [ncls][ntypes][2][K][K]
   double2 *L;                // [ntb][K], added to
@@ -45,19 +45,6 @@ __device__ __forceinline__ int pair_find_job(const PairJob *jobs, int njobs, int
     if (jobs[mid].t0 <= g) lo = mid; else hi = mid - 1;
   }
   return lo;
-}
-
-// types with a nonzero source expansion, per source box: one warp per (box, type) row
-__global__ void k_pair_types(const double2 *M, int64_t nrows, int K, int ntypes, uint32_t *tmask) {
-  const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (row >= nrows) return;
-  bool nz = false;
-  for (int k = threadIdx.x & 31; k < K; k += 32) {
-    const double2 v = M[row * K + k];
-    nz |= v.x != 0.0 || v.y != 0.0;
-  }
-  if (__any_sync(0xffffffffu, nz) && (threadIdx.x & 31) == 0)
-    atomicOr(&tmask[row / ntypes], 1u << (int)(row % ntypes));
 }
 
 // MODE 0: translations of every target (cnt[g]); 1: bin counts of the translations numbered

@@ -116,30 +116,41 @@ __device__ __forceinline__ void tc_split(float x, int e, __half &h, __half &l) {
 // W of one (canonical class, type) as the shared-memory image the MMA reads: NC K-chunks of 32
 // columns, each N rows of 128 bytes [32 hi | 32 lo] in the 128-byte swizzled K-major layout, so that one
 // bulk copy moves a chunk.  One CTA per image; classes that no far list uses are skipped.
-// kind 0: free space (class (a, b), dz), 1: reaction (class (a, b), kk; used[] per (rho^2, kk)).
+// kind 0: free space (class (a, b), dz), 1: reaction (class (a, b), kk; used[] per (rho^2, kk)).  Every
+// level of every group in one launch.
+struct PackWJob {
+  const float *ops;
+  const uint8_t *used;
+  unsigned char *wimg;
+  float *wscale;
+  int64_t item0;
+  int kind, ntypes;
+};
 constexpr int PACKW_THREADS = 256;
-__global__ void __launch_bounds__(PACKW_THREADS) k_tc_pack_w(const float *ops, int kind, int ntypes,
-                                                             const uint8_t *used, int ws, int K, int p, int NC,
-                                                             unsigned char *wimg, float *wscale) {
+template <int P>
+__global__ void __launch_bounds__(PACKW_THREADS) k_tc_pack_w(const PackWJob *jobs, int nj, int ws) {
+  constexpr int NC = tc_chunks(P), N = 32 * NC, K = (P + 1) * (P + 2) / 2;
   extern __shared__ float pq[];  // P, Q
-  __shared__ int code[128];
-  __shared__ float tc_[128], ts_[128];  // cos, sin of m phi_c of every column's coefficient
+  __shared__ int code[N];
+  __shared__ float tc_[N], ts_[N];  // cos, sin of m phi_c of every column's coefficient
   __shared__ float red[PACKW_THREADS / 32];
-  const int ct = blockIdx.x, cls = ct / ntypes, tau = ct % ntypes, N = 32 * NC;
+  const PackWJob &J = job_of(jobs, nj, (int64_t)blockIdx.x);
+  const int kind = J.kind, ntypes = J.ntypes;
+  const int ct = (int)((int64_t)blockIdx.x - J.item0), cls = ct / ntypes, tau = ct % ntypes;
   const int per = kind ? NKK : NDZ, ci = cls / per, sub = cls % per;
   int a, b;
   can_decode(ci, a, b);
   const int src = rho_index(a, b) * per + sub;  // the (rho^2, ...) class of the operators
-  if (kind ? !used[src] : max(a, abs(sub - OFF_R)) <= ws) return;
-  const float *P = ops + ((size_t)src * ntypes + tau) * 2 * K * K;
+  if (kind ? !J.used[src] : max(a, abs(sub - OFF_R)) <= ws) return;
+  const float *op = J.ops + ((size_t)src * ntypes + tau) * 2 * K * K;
   float mx = 0.f;
   for (int e = threadIdx.x; e < 2 * K * K; e += blockDim.x) {
-    const float v = P[e];
+    const float v = op[e];
     pq[e] = v;
     mx = fmaxf(mx, fabsf(v));
   }
   for (int c = threadIdx.x; c < N; c += blockDim.x) {
-    const int cd = tc_remap(c, p);
+    const int cd = tc_remap(c, P);
     const int m = cd == -1 ? 0 : cK.mof[cd >= 0 ? cd : -cd - 2];
     code[c] = cd;
     tc_[c] = c_trig[ci][m][0];
@@ -153,9 +164,11 @@ __global__ void __launch_bounds__(PACKW_THREADS) k_tc_pack_w(const float *ops, i
   for (int w = 0; w < PACKW_THREADS / 32; ++w) mx = fmaxf(mx, red[w]);
   // the entries of W are bounded by the largest of P and Q
   const int e2 = tc_exponent(mx);
-  if (threadIdx.x == 0) wscale[ct] = scalbnf(1.f, -e2);
+  if (threadIdx.x == 0) J.wscale[ct] = scalbnf(1.f, -e2);
+  // 2^e2 in two factors, each an ordinary number
+  const float f1 = scalbnf(1.f, e2 / 2), f2 = scalbnf(1.f, e2 - e2 / 2);
   const float *Pm = pq, *Qm = pq + K * K;
-  unsigned char *img = wimg + (size_t)ct * N * NC * 128;
+  unsigned char *img = J.wimg + (size_t)ct * N * NC * 128;
   for (int e = threadIdx.x; e < N * (N / 2); e += blockDim.x) {
     const int r = e / (N / 2), cp = 2 * (e % (N / 2));  // row, first column of the pair
     const int ro = code[r], k0 = code[cp], k1 = code[cp + 1];
@@ -179,9 +192,11 @@ __global__ void __launch_bounds__(PACKW_THREADS) k_tc_pack_w(const float *ops, i
         if (k1 >= 0) w1 = f * Pm[i * K + k1];
       }
     }
-    __half2 h, l;
-    tc_split(w0, e2, h.x, l.x);
-    tc_split(w1, e2, h.y, l.y);
+    w0 = w0 * f1 * f2;
+    w1 = w1 * f1 * f2;
+    const __half2 h = __floats2half2_rn(w0, w1);
+    const float2 hf = __half22float2(h);
+    const __half2 l = __floats2half2_rn(w0 - hf.x, w1 - hf.y);
     unsigned char *row = img + ((size_t)(cp >> 5) * N + r) * 128;
     const int by = (cp & 31) * 2;  // byte of the hi pair in the row
     *(__half2 *)(row + ((((by >> 4)) ^ (r & 7)) << 4) + (by & 15)) = h;
@@ -189,23 +204,32 @@ __global__ void __launch_bounds__(PACKW_THREADS) k_tc_pack_w(const float *ops, i
   }
 }
 
-// source rows as split FP16 (per 32-column chunk [32 hi | 32 lo]), with the row's inverse power of two and,
-// per box, the mask of types with a nonzero row (zero rows are neither written nor read).  One warp
-// per (box, type) row.  side: 0 free space; 1, 2 reaction side a: only image boxes within 2 ws box
-// layers of the interface can be in a far list, the others are skipped.
-__global__ void __launch_bounds__(256) k_tc_pack_rows(const float2 *M, int64_t nrows, int K, int p, int NC,
-                                                      int ntypes, const uint64_t *bkey, int lev, int side, int ws,
-                                                      __half *rows, float *rscale, uint32_t *tmask) {
+// source rows as split FP16 (per 32-column chunk [32 hi | 32 lo]), with the row's inverse power of two; rows
+// of absent types are neither written nor read.  One warp per (box, type) row, every level of every group in one
+// launch.  side: 0 free space; 1, 2 reaction side a: only image boxes within 2 ws box layers of the
+// interface can be in a far list, the others are skipped.
+struct PackRowJob {
+  const float2 *M;
+  const uint32_t *mask;  // types present (nullptr: all)
+  const uint64_t *bkey;
+  __half *rows;
+  float *rscale;
+  int64_t nrows, item0;
+  int ntypes, lev, side;
+};
+__global__ void __launch_bounds__(256) k_tc_pack_rows(const PackRowJob *jobs, int nj, int K, int p, int NC, int ws) {
   __shared__ int code[128];
   const int N = 32 * NC, lane = threadIdx.x & 31;
   for (int c = threadIdx.x; c < N; c += blockDim.x) code[c] = tc_remap(c, p);
   __syncthreads();
-  const int64_t row = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (row >= nrows) return;
-  const int64_t box = row / ntypes;
-  if (side) {
-    const int iz = (int)compact3_(bkey[box]), half = 1 << (lev - 1);
-    if ((side == 1 ? half - 1 - iz : iz - half) > 2 * ws) return;
+  const PackRowJob &J = job_of(jobs, nj, (int64_t)blockIdx.x);
+  const int64_t row = ((int64_t)blockIdx.x - J.item0) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if (row >= J.nrows) return;
+  const int64_t box = row / J.ntypes;
+  if (J.mask && !((J.mask[box] >> (int)(row % J.ntypes)) & 1u)) return;
+  if (J.side) {
+    const int iz = (int)compact3_(J.bkey[box]), half = 1 << (J.lev - 1);
+    if ((J.side == 1 ? half - 1 - iz : iz - half) > 2 * ws) return;
   }
   float v[4], mx = 0.f;
 #pragma unroll
@@ -214,18 +238,17 @@ __global__ void __launch_bounds__(256) k_tc_pack_rows(const float2 *M, int64_t n
     if (ch < NC) {
       const int cd = code[ch * 32 + lane];
       if (cd != -1) {
-        const float2 m = M[row * K + (cd >= 0 ? cd : -cd - 2)];
+        const float2 m = J.M[row * K + (cd >= 0 ? cd : -cd - 2)];
         v[ch] = cd >= 0 ? m.x : m.y;
       }
     }
     mx = fmaxf(mx, fabsf(v[ch]));
-    if (v[ch] != v[ch]) mx = INFINITY;  // a NaN row stays in the mask
+    if (v[ch] != v[ch]) mx = INFINITY;  // a NaN row stays one
   }
 #pragma unroll
   for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (mx == 0.f) return;
   const int e2 = tc_exponent(mx);
-  __half *out = rows + row * 2 * N;
+  __half *out = J.rows + row * 2 * N;
 #pragma unroll
   for (int ch = 0; ch < 4; ++ch) {
     if (ch >= NC) break;
@@ -234,10 +257,7 @@ __global__ void __launch_bounds__(256) k_tc_pack_rows(const float2 *M, int64_t n
     out[ch * 64 + lane] = h;
     out[ch * 64 + 32 + lane] = l;
   }
-  if (lane == 0) {
-    rscale[row] = scalbnf(1.f, -e2);
-    atomicOr(&tmask[box], 1u << (int)(row % ntypes));
-  }
+  if (lane == 0) J.rscale[row] = scalbnf(1.f, -e2);
 }
 
 constexpr int TC_MAXSTEP = SLICE_OFFS * 2 * (MAXLAYER - 1);
@@ -370,7 +390,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TJob *jobs, int 
       for (int b = 0; b < KB; ++b) {
         const int k = 32 * b + lane;
         const int sb = k < SLICE_OFFS ? Jvlist[(size_t)t * NOFF + slice * SLICE_OFFS + k] : -1;
-        if (sb >= 0) acc[b] |= Jtm[sb];
+        if (sb >= 0) acc[b] |= Jtm ? Jtm[sb] : 1u;
       }
     }
 #pragma unroll
@@ -495,7 +515,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TJob *jobs, int 
     const int32_t *const lrow = Jvlist + (size_t)(lt >= 0 ? lt : 0) * NOFF;
     auto src_of = [&](int i) { return i < ns && lt >= 0 ? lrow[steps[i] >> 4] : -1; };
     int s1 = src_of(0), s2 = src_of(1);                // sources of the next step and the one after
-    unsigned m1 = s1 >= 0 ? Jtm[s1] : 0u;              // type mask of the next step's source
+    unsigned m1 = s1 >= 0 ? (Jtm ? Jtm[s1] : 1u) : 0u;              // type mask of the next step's source
     float rs = 0.f, wsc = 0.f;                         // scales of the loaded step (lanes 0..15)
     uint4 buf[NC][4];                                  // the loaded step: per chunk, one unit of four rows
     auto load = [&](int i) {
@@ -511,7 +531,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TJob *jobs, int 
         for (int kc = 0; kc < NC; ++kc) buf[kc][g] = r >= 0 ? __ldg(at + kc * 8) : make_uint4(0u, 0u, 0u, 0u);
       }
       s1 = s2;
-      m1 = s1 >= 0 ? Jtm[s1] : 0u;
+      m1 = s1 >= 0 ? (Jtm ? Jtm[s1] : 1u) : 0u;
       s2 = src_of(i + 2);
     };
     load(0);
@@ -559,6 +579,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TJob *jobs, int 
     if (!fail && !fold(ns - 1)) fail = true;
     if (!fail && myt >= 0) {
       float2 *Lrow = J.L + ((size_t)myt * M2L_NSLOT + J.slot0 + slice) * K;
+      if (hf == 0) atomicOr(&J.smask[myt], 1u << (J.slot0 + slice));
 #pragma unroll
       for (int j = 0; j < NH; ++j) {
         const int code = remap_s[hf * NH + j];

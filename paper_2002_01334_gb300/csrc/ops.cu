@@ -112,8 +112,10 @@ __global__ void k_build_ops(const OpDesc *descs, const double *prep, const doubl
       P = r[0] + r1;
       Q = r[0] - r1;
     }
-    out[d.dst + (size_t)o * K + i] = (T)P;
-    out[d.dst + (size_t)K * K + (size_t)o * K + i] = (T)Q;
+    // M2L operators row by row; M2M and L2L with the output row fastest (their kernels own a row per thread)
+    const size_t at = d.dst + (d.kind == 0 ? (size_t)o * K + i : (size_t)i * K + o);
+    out[at] = (T)P;
+    out[at + (size_t)K * K] = (T)Q;
   }
 }
 

@@ -626,6 +626,7 @@ void build_boxes(Ctx &c, std::vector<Group> &groups, uint32_t **dcounts, size_t 
         jobs.push_back(j);
         tiles += nt;
         boxes += j.cap;
+        if (l == g.D) P.pbox = j.idx;
       }
       if (which) {
         if (np) {
@@ -660,6 +661,62 @@ void build_boxes(Ctx &c, std::vector<Group> &groups, uint32_t **dcounts, size_t 
   k_box_links<<<(unsigned)((boxes + 255) / 256), 256, 0, c.stream>>>(dj, nj, boxes);
   LPB_LAUNCH();
   c.launches += 4;
+}
+
+// source types present in every image box: each segment marks its leaf and climbs until an ancestor is marked
+// already (whoever marked it climbs on)
+struct MaskJob {
+  const uint32_t *sbox, *stype;
+  int64_t nseg, item0;
+  int D;
+  const uint32_t *parent[DMAX + 1];
+  uint32_t *mask[DMAX + 1];
+};
+__global__ void k_type_masks(const MaskJob *jobs, int nj, int64_t ntot) {
+  const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (g >= ntot) return;
+  int lo = 0, hi = nj - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (jobs[mid].item0 <= g) lo = mid; else hi = mid - 1;
+  }
+  const MaskJob &J = jobs[lo];
+  const int64_t s = g - J.item0;
+  if (s >= J.nseg) return;
+  uint32_t b = J.sbox[s];
+  const uint32_t bit = 1u << J.stype[s];
+  for (int l = J.D; l >= 2; --l) {
+    if ((l < J.D && (*(volatile uint32_t *)&J.mask[l][b] & bit)) || (atomicOr(&J.mask[l][b], bit) & bit)) return;
+    if (l > 2) b = J.parent[l][b];
+  }
+}
+void build_type_masks(Ctx &c, std::vector<Group> &groups) {
+  std::vector<MaskJob> jobs;
+  int64_t segs = 0, boxes = 0;
+  for (auto &g : groups)
+    if ((g.parts & 2) && g.I.np)
+      for (int l = 2; l <= g.D; ++l) boxes += g.I.lev[l].n;
+  if (!boxes) return;
+  uint32_t *m = c.arena.get<uint32_t>(boxes);
+  LPB_CUDA(cudaMemsetAsync(m, 0, sizeof(uint32_t) * boxes, c.stream));
+  for (auto &g : groups) {
+    if (!((g.parts & 2) && g.I.np)) continue;
+    MaskJob j{};
+    j.sbox = g.I.seg_box; j.stype = g.I.seg_type; j.nseg = g.I.nseg; j.item0 = segs; j.D = g.D;
+    segs += j.nseg;
+    for (int l = 2; l <= g.D; ++l) {
+      g.tmask[l] = j.mask[l] = m;
+      j.parent[l] = g.I.lev[l].parent;
+      m += g.I.lev[l].n;
+    }
+    jobs.push_back(j);
+  }
+  if (!segs) return;
+  MaskJob *dj = c.arena.get<MaskJob>(jobs.size());
+  LPB_CUDA(cudaMemcpyAsync(dj, jobs.data(), sizeof(MaskJob) * jobs.size(), cudaMemcpyHostToDevice, c.stream));
+  k_type_masks<<<(unsigned)((segs + 255) / 256), 256, 0, c.stream>>>(dj, (int)jobs.size(), segs);
+  LPB_LAUNCH();
+  c.launches++;
 }
 
 // the counts of build_boxes, on the host, into the groups
