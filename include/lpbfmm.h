@@ -152,8 +152,10 @@ int lpbfmm_eval_groups(lpbfmm_t h, int64_t n, const double *q, const double *xyz
  *   g_xyz[j] = sum_i g_phi[i] d phi_i / d r_j = -(q_j field[g_phi](r_j) + g_phi[j] field[q](r_j))
  * using the reciprocity G_{l l'}(r, r') = G_{l' l}(r', r) of the layered Green's function (the
  * vector-Jacobian product of phi).  For E = 1/2 sum q_i phi_i: dE/dq = g_q with g_phi = q, and
- * dE/dr = g_xyz with g_phi = q / 2 (so the force on charge j is -g_xyz[j]).  Two evaluations
- * are run.  Device arrays; g_q[n], g_xyz[n*3] are outputs.  The context keeps a work space of
+ * dE/dr = g_xyz with g_phi = q / 2 (so the force on charge j is -g_xyz[j]).  The two
+ * charge vectors g and q are evaluated in turn on one set of trees, lists, tables and operators
+ * (lpbfmm_last_profile and the launch count of lpbfmm_last_counts are those of the second, without them).
+ * Device arrays; g_q[n], g_xyz[n*3] are outputs.  The context keeps a work space of
  * 7 n doubles between calls (allocated when n first exceeds its size); g_q and g_xyz are written
  * in stream order on the context's stream.
  */

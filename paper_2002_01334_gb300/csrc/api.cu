@@ -20,6 +20,7 @@ void init_fmm_tables(Ctx &c);
 void *Arena::alloc(size_t bytes) {
   bytes = (bytes + 255) & ~size_t(255);
   used_total += bytes;
+  peak = std::max(peak, used_total);
   for (auto &ch : chunks)
     if (ch.size - ch.used >= bytes) {
       void *p = ch.p + ch.used;
@@ -37,12 +38,12 @@ void *Arena::alloc(size_t bytes) {
   return p;
 }
 void Arena::reset() {
-  if (chunks.size() > 1 || (chunks.size() == 1 && chunks[0].size < used_total)) {
-    want = std::max(want, used_total + (used_total >> 3));
+  if (chunks.size() > 1 || (chunks.size() == 1 && chunks[0].size < peak)) {
+    want = std::max(want, peak + (peak >> 3));
     release();
   }
   for (auto &ch : chunks) ch.used = 0;
-  used_total = 0;
+  used_total = peak = 0;
 }
 void Arena::release() {
   for (auto &ch : chunks) cudaFree(ch.p);
@@ -210,12 +211,41 @@ static double unord(unsigned long long u) {
 // ---------------------------------------------------------------------------------------
 // evaluation
 // ---------------------------------------------------------------------------------------
+static void start_near(Ctx &c, double *phi, double *field) {
+  // the FP32 free-space near field needs only the trees and near lists: on its own stream, beside
+  // the operators, the upward pass and the M2L (the downward pass waits for it).  In a batched
+  // evaluation it is recorded for the batch's grouped launch.
+  c.near_async = !c.def.on && c.opts.precision != LPBFMM_FP64;
+  if (c.near_async) {
+    LPB_CUDA(cudaEventRecord(c.ev_gfork, c.stream));
+    LPB_CUDA(cudaStreamWaitEvent(c.near, c.ev_gfork, 0));
+    run_near_free(c, c.groups, phi, field, c.near);
+    LPB_CUDA(cudaEventRecord(c.ev_near, c.near));
+  } else {
+    run_near_free(c, c.groups, phi, field, c.stream);
+  }
+}
+static void start_far(Ctx &c) {
+  c.far_async = c.near_async;
+  if (c.far_async) {
+    // the far field on the high-priority stream, beside the near field
+    LPB_CUDA(cudaEventRecord(c.ev_gfork, c.stream));
+    LPB_CUDA(cudaStreamWaitEvent(c.far, c.ev_gfork, 0));
+    OnStream on(c, c.far);
+    run_fmm_front(c, c.groups);
+    LPB_CUDA(cudaEventRecord(c.ev_far, c.far));
+  } else {
+    run_fmm_front(c, c.groups);
+  }
+}
+
 // parts: bits 0, 1 free-space / reaction part, bits 2, 3 diagnostics (lpbfmm_eval_parts); gmask (host,
 // may be null): per target group (l, a) at index 2 l + a - 1, the parts it computes (bits 0, 1)
 // validation, trees, lists, tables, operators, upward pass and M2L of one evaluation (eval_back
 // finishes it); with c.def.on the tensor-core M2L is only recorded
-static void eval_front(Ctx &c, int64_t n, const double *q, const double *xyz, const int32_t *layer, int parts,
-                       const int32_t *gmask, double *phi, double *field) {
+// q2 (may be null): a second charge vector on the same positions that eval_again will evaluate; only checked here
+static void eval_front(Ctx &c, int64_t n, const double *q, const double *q2, const double *xyz, const int32_t *layer,
+                       int parts, const int32_t *gmask, double *phi, double *field) {
   c.def.clear();
   c.arena.reset();
   c.launches = 0;
@@ -236,7 +266,7 @@ static void eval_front(Ctx &c, int64_t n, const double *q, const double *xyz, co
   for (int k = 0; k <= L; ++k) hs.zlo[k] = ~0ull;
   Stats *ds = c.arena.get<Stats>(1);
   LPB_CUDA(cudaMemcpyAsync(ds, &hs, sizeof hs, cudaMemcpyHostToDevice, c.stream));
-  launch_validate(c, n, q, xyz, layer, ds);
+  launch_validate(c, n, q, q2, xyz, layer, ds);
   Stats *hp = (Stats *)c.h_pinned;
   LPB_CUDA(cudaMemcpyAsync(hp, ds, sizeof(Stats), cudaMemcpyDeviceToHost, c.stream));
   LPB_CUDA(cudaStreamSynchronize(c.stream));
@@ -358,18 +388,7 @@ static void eval_front(Ctx &c, int64_t n, const double *q, const double *xyz, co
   build_type_masks(c, c.groups);
   build_lists(c, c.groups);
   prof_mark(c, "tree");
-  // the FP32 free-space near field needs only the trees and near lists: on its own stream, beside
-  // the operators, the upward pass and the M2L (the downward pass waits for it).  In a batched
-  // evaluation it is recorded for the batch's grouped launch.
-  c.near_async = !c.def.on && c.opts.precision != LPBFMM_FP64;
-  if (c.near_async) {
-    LPB_CUDA(cudaEventRecord(c.ev_gfork, c.stream));
-    LPB_CUDA(cudaStreamWaitEvent(c.near, c.ev_gfork, 0));
-    run_near_free(c, c.groups, phi, field, c.near);
-    LPB_CUDA(cudaEventRecord(c.ev_near, c.near));
-  } else {
-    run_near_free(c, c.groups, phi, field, c.stream);
-  }
+  start_near(c, phi, field);
   {
     double lmin = 1e300, hmin = 1e300;
     for (int k = 0; k <= L; ++k) lmin = std::min(lmin, c.md.lam[k]);
@@ -398,17 +417,9 @@ static void eval_front(Ctx &c, int64_t n, const double *q, const double *xyz, co
     LPB_CUDA(cudaEventRecord(c.ev_join, c.side));
   }
   prof_mark(c, "tables+ops");
-  c.far_async = c.near_async;
-  if (c.far_async) {
-    // the far field on the high-priority stream, beside the near field
-    LPB_CUDA(cudaEventRecord(c.ev_gfork, c.stream));
-    LPB_CUDA(cudaStreamWaitEvent(c.far, c.ev_gfork, 0));
-    OnStream on(c, c.far);
-    run_fmm_front(c, c.groups);
-    LPB_CUDA(cudaEventRecord(c.ev_far, c.far));
-  } else {
-    run_fmm_front(c, c.groups);
-  }
+  reserve_images(c, c.groups);
+  c.charge_mark = c.arena.mark();
+  start_far(c);
 }
 // the downward pass and near fields of the evaluation eval_front began
 static void eval_back(Ctx &c, double *phi, double *field) {
@@ -417,7 +428,24 @@ static void eval_back(Ctx &c, double *phi, double *field) {
 }
 static void eval_impl(Ctx &c, int64_t n, const double *q, const double *xyz, const int32_t *layer, int parts,
                       const int32_t *gmask, double *phi, double *field) {
-  eval_front(c, n, q, xyz, layer, parts, gmask, phi, field);
+  eval_front(c, n, q, nullptr, xyz, layer, parts, gmask, phi, field);
+  eval_back(c, phi, field);
+}
+// another charge vector on the positions, trees, lists and operators of the evaluation just issued: its passes
+// take the memory of that evaluation's, which they follow in stream order (every side stream has been
+// joined by then)
+static void eval_again(Ctx &c, int64_t n, const double *q, double *phi, double *field) {
+  c.arena.rewind(c.charge_mark);
+  c.launches = 0;
+  c.nev = 0;
+  c.prof_names.clear();
+  c.prof_launch.clear();
+  prof_mark(c, "start");
+  LPB_CUDA(cudaMemsetAsync(phi, 0, sizeof(double) * n, c.stream));
+  if (field) LPB_CUDA(cudaMemsetAsync(field, 0, sizeof(double) * 3 * n, c.stream));
+  recharge_points(c, c.groups, q);
+  start_near(c, phi, field);
+  start_far(c);
   eval_back(c, phi, field);
 }
 
@@ -600,8 +628,18 @@ int lpbfmm_adjoint(lpbfmm_t h, int64_t n, const double *q, const double *xyz, co
     h->adj_cap = need;
   }
   double *fg = h->adj, *pq = h->adj + 3 * n, *fq = h->adj + 4 * n;
-  int rc = lpbfmm_eval(h, n, g_phi, xyz, layer_id, g_q, fg);
-  if (rc == LPBFMM_OK) rc = lpbfmm_eval(h, n, q, xyz, layer_id, pq, fq);
+  if (n >= (int64_t)1 << 31) return LPBFMM_ERR_UNSUPPORTED;
+  int rc = LPBFMM_OK;
+  try {
+    // one set of trees, lists, tables and operators for both charge vectors
+    eval_front(*h, n, g_phi, q, xyz, layer_id, 3, nullptr, g_q, fg);
+    eval_back(*h, g_q, fg);
+    eval_again(*h, n, q, pq, fq);
+  } catch (const CudaError &e) {
+    rc = map_error(e);
+  } catch (const StatusError &e) {
+    rc = e.code;
+  }
   if (rc == LPBFMM_OK) {
     k_adjoint_combine<<<(unsigned)((n + 255) / 256), 256, 0, h->stream>>>(n, q, g_phi, fq, fg, g_xyz);
     if (cudaGetLastError() != cudaSuccess) rc = LPBFMM_ERR_CUDA;
@@ -718,7 +756,7 @@ int lpbfmm_eval_batched(int nsys, const lpbfmm_t *ctxs, const int64_t *offsets, 
       const int64_t o = offsets[s], n = offsets[s + 1] - offsets[s];
       ctx->def.on = true;
       const int rc = guarded([&] {
-        eval_front(*ctx, n, q + o, xyz + 3 * o, layer_id + o, 3, nullptr, phi + o, field ? field + 3 * o : nullptr);
+        eval_front(*ctx, n, q + o, nullptr, xyz + 3 * o, layer_id + o, 3, nullptr, phi + o, field ? field + 3 * o : nullptr);
       });
       if (rc) {
         ctx->def.on = false;

@@ -1080,6 +1080,22 @@ static void launch_tc(int p, const TJob *jobs, int njobs, int64_t items, int *st
   }
 }
 
+void reserve_images(Ctx &c, std::vector<Group> &groups) {
+  c.images_ready = false;
+  const int NC = tc_chunks(c.p), N = 32 * NC;
+  if (c.opts.precision == LPBFMM_FP64 || NC > 4) return;
+  for (auto &g : groups)
+    for (int l = 2; l <= g.D; ++l)
+      for (int kind = 0; kind < 2; ++kind) {
+        if (!g.T.lev[l].n) continue;
+        if (kind == 0 ? !(g.is_free && (g.parts & 1) && l <= g.Df)
+                      : !((g.parts & 2) && g.I.np > 0 && !(g.parts & 8) && g.vreact[l])) continue;
+        const size_t n = kind ? (size_t)TC_NREACT * g.ntypes : (size_t)TC_NFREE;
+        g.wimg[kind][l] = c.arena.get<unsigned char>(n * N * N * 4);
+        g.wscale[kind][l] = c.arena.get<float>(n);
+      }
+}
+
 // mixed mode: every multipole-to-local translation of every group and level in one launch
 static void m2l_all_f32(Ctx &c, std::vector<Group> &groups) {
   typedef float T;
@@ -1139,7 +1155,7 @@ static void m2l_all_f32(Ctx &c, std::vector<Group> &groups) {
       rjobs.push_back(r);
       relem += r.n;
       const int N = 32 * tc_nc;
-      // split source rows; operator images
+      // split source rows; operator images (once per evaluation, also for several charge vectors)
       auto pack = [&](TJob &j, const void *M, const Level &sl, const uint32_t *mask, int side, const void *ops, int kind,
                       int ntypes, const uint8_t *used, int ncls) {
         PackRowJob r;
@@ -1149,13 +1165,12 @@ static void m2l_all_f32(Ctx &c, std::vector<Group> &groups) {
         r.rscale = c.arena.get<float>((size_t)r.nrows);
         row_items += (r.nrows + 7) / 8;
         prow.push_back(r);
-        PackWJob w;
-        w.ops = (const float *)ops; w.kind = kind; w.ntypes = ntypes; w.used = used; w.item0 = img_items;
-        w.wimg = c.arena.get<unsigned char>((size_t)ncls * ntypes * N * N * 4);
-        w.wscale = c.arena.get<float>((size_t)ncls * ntypes);
-        img_items += (int64_t)ncls * ntypes;
-        pw.push_back(w);
-        j.rows = r.rows; j.rscale = r.rscale; j.tmask = mask; j.wimg = w.wimg; j.wscale = w.wscale; j.ntypes = ntypes;
+        if (!c.images_ready) {
+          pw.push_back(PackWJob{(const float *)ops, used, g.wimg[kind][l], g.wscale[kind][l], img_items, kind, ntypes});
+          img_items += (int64_t)ncls * ntypes;
+        }
+        j.rows = r.rows; j.rscale = r.rscale; j.tmask = mask; j.ntypes = ntypes;
+        j.wimg = g.wimg[kind][l]; j.wscale = g.wscale[kind][l];
         j.L = (float2 *)part; j.smask = smask; j.ntb = ntb;
       };
       if (dofree && use_tc) {
@@ -1201,9 +1216,13 @@ static void m2l_all_f32(Ctx &c, std::vector<Group> &groups) {
   if (!prow.empty()) {
     k_tc_pack_rows<<<(unsigned)row_items, 256, 0, c.stream>>>(upload_jobs(c, prow), (int)prow.size(), c.K, c.p, tc_nc, c.ws);
     LPB_LAUNCH();
-    launch_pack_w(c.p, upload_jobs(c, pw), (int)pw.size(), img_items, c.ws, c.stream);
-    LPB_LAUNCH();
-    c.launches += 2;
+    c.launches++;
+    if (!pw.empty()) {
+      launch_pack_w(c.p, upload_jobs(c, pw), (int)pw.size(), img_items, c.ws, c.stream);
+      LPB_LAUNCH();
+      c.launches++;
+      c.images_ready = true;
+    }
   }
   prof_mark(c, "m2l_prep");
   if (c.def.on && !tjobs.empty() && jobs.empty()) {

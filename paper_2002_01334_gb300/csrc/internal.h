@@ -129,7 +129,23 @@ struct Arena {
     size_t size, used;
   };
   std::vector<Chunk> chunks;
-  size_t want = 0, used_total = 0;
+  size_t want = 0, used_total = 0, peak = 0;
+  // a point to go back to: what was allocated since may be overwritten by work that follows, in stream
+  // order, the work that used it
+  struct Mark {
+    std::vector<size_t> used;
+    size_t total = 0;
+  };
+  Mark mark() const {
+    Mark m;
+    for (const auto &ch : chunks) m.used.push_back(ch.used);
+    m.total = used_total;
+    return m;
+  }
+  void rewind(const Mark &m) {
+    for (size_t k = 0; k < chunks.size(); ++k) chunks[k].used = k < m.used.size() ? m.used[k] : 0;
+    used_total = m.total;
+  }
   void *alloc(size_t bytes);
   template <typename T>
   T *get(size_t n) {
@@ -179,6 +195,9 @@ struct Group {
   uint8_t *used[DMAX + 1] = {};  // reaction classes in use, NREACT_CLS per level
   int32_t *ktrow[DMAX + 1] = {};
   uint32_t *tmask[DMAX + 1] = {};  // image boxes: source types present
+  // operator images of the tensor-core M2L, [0] free space, [1] reaction
+  unsigned char *wimg[2][DMAX + 1] = {};
+  float *wscale[2][DMAX + 1] = {};
   // expansions
   void *Mfree[DMAX + 1] = {}, *Mimg[DMAX + 1] = {}, *Lt[DMAX + 1] = {};
   // operators
@@ -279,6 +298,10 @@ struct Ctx {
   void *h_pinned = nullptr;  // pinned staging
   Arena arena;
   std::vector<Group> groups;
+  // of the evaluation in progress: what is allocated for one charge vector starts here; the operator images
+  // are filled
+  Arena::Mark charge_mark;
+  bool images_ready = false;
   // profile of the last evaluation
   std::vector<std::string> prof_names;
   std::vector<float> prof_ms;
@@ -322,7 +345,9 @@ struct Stats {
   unsigned long long zlo[MAXLAYER], zhi[MAXLAYER];
 };
 void scan_u32(Ctx &c, const uint32_t *in, uint32_t *out, int64_t n, uint32_t *d_total);
-void launch_validate(Ctx &c, int64_t n, const double *q, const double *xyz, const int32_t *layer, Stats *st);
+// q2 (may be null): a second charge vector, checked for finite values
+void launch_validate(Ctx &c, int64_t n, const double *q, const double *q2, const double *xyz, const int32_t *layer,
+                     Stats *st);
 struct RankPtrs {
   uint32_t *r[MAXLAYER];
 };
@@ -335,6 +360,8 @@ void build_boxes(Ctx &c, std::vector<Group> &groups, uint32_t **dcounts, size_t 
 void read_box_counts(std::vector<Group> &groups, const uint32_t *h);
 void build_lists(Ctx &c, std::vector<Group> &groups);
 void build_type_masks(Ctx &c, std::vector<Group> &groups);
+// the charges of every group's sorted points replaced
+void recharge_points(Ctx &c, std::vector<Group> &groups, const double *q);
 // adaptive dual-tree lists of group g's free-space target tree with itself (diagnostic): records
 // of 5 int64 (kind 0 V / 1 U / 2 W / 3 X, target level, target key, source level, source key)
 void adaptive_lists(Ctx &c, Group &g, int s, int ws, std::vector<int64_t> &rec);
@@ -353,6 +380,8 @@ void debug_stable(Ctx &c, int l, int a, int lp, int b, double h, double rho, dou
 // upward pass and M2L of every group (with c.def.on the tensor-core M2L and its slot sums are
 // recorded in c.def instead of launched)
 void run_fmm_front(Ctx &c, std::vector<Group> &groups);
+// memory for the tensor-core M2L's operator images of every group (filled by the first run_fmm_front)
+void reserve_images(Ctx &c, std::vector<Group> &groups);
 // the FP32 free-space near field of every group (mixed precision): point splitting and one P2P
 // launch on stream st, or, with c.def.on, the launch recorded in c.def for a grouped one
 void run_near_free(Ctx &c, std::vector<Group> &groups, double *phi, double *field, cudaStream_t st);

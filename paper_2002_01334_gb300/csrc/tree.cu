@@ -148,7 +148,7 @@ __device__ __forceinline__ unsigned long long wmax(unsigned long long v) {
 // the FP64 coordinates) and per-layer counts; they are reduced per warp by shuffles, per block
 // in shared memory, and merged into the global statistics with one atomic per block and field.
 constexpr int VAL_THREADS = 256;
-__global__ void __launch_bounds__(VAL_THREADS) k_validate(int64_t n, const double *q, const double *xyz,
+__global__ void __launch_bounds__(VAL_THREADS) k_validate(int64_t n, const double *q, const double *q2, const double *xyz,
                                                           const int32_t *layer, Medium md, double thr, Stats *st) {
   const unsigned long long HI = ~0ull, LO = 0ull;
   unsigned long long xlo = HI, xhi = LO, ylo = HI, yhi = LO, zlo[MAXLAYER], zhi[MAXLAYER];
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(VAL_THREADS) k_validate(int64_t n, const doubl
     const double qq = q[i];
     const int lay = layer[i];
     int code = 0;
-    if (!isfinite(x) || !isfinite(y) || !isfinite(z) || !isfinite(qq)) {
+    if (!isfinite(x) || !isfinite(y) || !isfinite(z) || !isfinite(qq) || (q2 && !isfinite(q2[i]))) {
       code = LPBFMM_ERR_NONFINITE;
     } else {
       int l = 0;
@@ -225,12 +225,13 @@ __global__ void __launch_bounds__(VAL_THREADS) k_validate(int64_t n, const doubl
   }
 }
 
-void launch_validate(Ctx &c, int64_t n, const double *q, const double *xyz, const int32_t *layer, Stats *st) {
+void launch_validate(Ctx &c, int64_t n, const double *q, const double *q2, const double *xyz, const int32_t *layer,
+                     Stats *st) {
   double scale = 1.0;
   for (int k = 0; k < c.md.L; ++k) scale = fmax(scale, fabs(c.md.d[k]));
   const double thr = 1e-12 * scale;
   const unsigned blocks = (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + VAL_THREADS - 1) / VAL_THREADS, 152 * 4));
-  k_validate<<<blocks, VAL_THREADS, 0, c.stream>>>(n, q, xyz, layer, c.md, thr, st);
+  k_validate<<<blocks, VAL_THREADS, 0, c.stream>>>(n, q, q2, xyz, layer, c.md, thr, st);
   LPB_LAUNCH();
   c.launches++;
 }
@@ -415,6 +416,35 @@ static void gather(Ctx &c, std::vector<Group> &groups, int images, const double 
   }
   if (!nj) return;
   k_gather_points<<<dim3((unsigned)((nmax + 255) / 256), nj), 256, 0, c.stream>>>(q, xyz, c.md, images, J);
+  LPB_LAUNCH();
+  c.launches++;
+}
+
+struct ChargeJob {
+  int64_t np;
+  const uint32_t *src;
+  double *q;
+};
+struct ChargeJobs {
+  ChargeJob j[2 * MAXJOB];
+};
+__global__ void k_recharge(const double *q, const __grid_constant__ ChargeJobs J) {
+  const ChargeJob &j = J.j[blockIdx.y];
+  const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (k < j.np) j.q[k] = q[j.src[k]];
+}
+void recharge_points(Ctx &c, std::vector<Group> &groups, const double *q) {
+  ChargeJobs J{};
+  int nj = 0;
+  int64_t nmax = 0;
+  for (auto &g : groups)
+    for (PointSet *P : {&g.T, &g.I}) {
+      if (!P->np) continue;
+      J.j[nj++] = ChargeJob{P->np, P->src, P->q};
+      nmax = std::max(nmax, P->np);
+    }
+  if (!nj) return;
+  k_recharge<<<dim3((unsigned)((nmax + 255) / 256), nj), 256, 0, c.stream>>>(q, J);
   LPB_LAUNCH();
   c.launches++;
 }
