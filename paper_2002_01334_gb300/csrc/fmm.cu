@@ -991,17 +991,14 @@ static void upward_t(Ctx &c, std::vector<Group> &groups) {
       p2m(g, g.I, g.D, g.I.seg_start, g.I.seg_count, g.I.seg_box, g.I.seg_type, g.I.nseg, g.ntypes, g.Mimg[g.D]);
   }
   PT_DISPATCH(launch_p2m, c, dense, sparse, nd, ns);
-  const int threads = std::min(256, (K + 31) / 32 * 32);
   for (int l = Dmax; l >= 3; --l) {
     std::vector<M2MJob> jobs;
-    int64_t items = 0;
     auto m2m = [&](const PointSet &P, const uint32_t *const *mask, int ntypes, const void *Mc, void *Mp, const void *ops) {
       if (!P.lev[l - 1].n) return;
       M2MJob j;
       j.pstart = P.lev[l - 1].start; j.pcount = P.lev[l - 1].count; j.ckey = P.lev[l].key;
       j.pmask = mask ? mask[l - 1] : nullptr; j.cmask = mask ? mask[l] : nullptr;
-      j.Mc = Mc; j.Mp = Mp; j.ops = ops; j.np = P.lev[l - 1].n; j.item0 = items; j.ntypes = ntypes;
-      items += j.np;
+      j.Mc = Mc; j.Mp = Mp; j.ops = ops; j.np = P.lev[l - 1].n; j.ntypes = ntypes;
       jobs.push_back(j);
     };
     for (auto &g : groups) {
@@ -1010,7 +1007,15 @@ static void upward_t(Ctx &c, std::vector<Group> &groups) {
       if ((g.parts & 2) && g.I.np > 0) m2m(g.I, g.tmask, g.ntypes, g.Mimg[l], g.Mimg[l - 1], g.op_m2m_i[l]);
     }
     if (jobs.empty()) continue;
-    k_m2m<T><<<(unsigned)items, threads, 0, c.stream>>>(upload_jobs(c, jobs), (int)jobs.size(), (const T *)tb.rot4, K);
+    int64_t np = 0, items = 0;
+    for (auto &j : jobs) np += j.np;
+    for (auto &j : jobs) {
+      j.tsplit = np <= M2M_TSPLIT_MAX ? j.ntypes : 1;
+      j.item0 = items;
+      items += j.np * j.tsplit;
+    }
+    k_m2m<T><<<(unsigned)items, oct_threads(K, c.p, items), oct_smem<T>(K, c.p), c.stream>>>(
+        upload_jobs(c, jobs), (int)jobs.size(), (const T *)tb.rot4, K, c.p);
     LPB_LAUNCH();
     c.launches++;
   }
@@ -1316,17 +1321,18 @@ static void downward_t(Ctx &c, std::vector<Group> &groups, double *phi, double *
   const Tables &tb = sizeof(T) == 8 ? g_tab_d[c.device] : g_tab_f[c.device];
   int Dmax = 2;
   for (auto &g : groups) Dmax = std::max(Dmax, g.D);
-  const int threads = std::min(256, (K + 31) / 32 * 32);
   for (int l = 3; l <= Dmax; ++l) {
     std::vector<L2LJob> jobs;
     int64_t items = 0;
     for (auto &g : groups) {
       if (l > g.D || !g.T.lev[l].n) continue;
-      jobs.push_back(L2LJob{g.T.lev[l].parent, g.T.lev[l].key, g.Lt[l - 1], g.op_l2l[l], g.Lt[l], g.T.lev[l].n, items});
-      items += g.T.lev[l].n;
+      const Level &P = g.T.lev[l - 1];
+      jobs.push_back(L2LJob{P.start, P.count, g.T.lev[l].key, g.Lt[l - 1], g.op_l2l[l], g.Lt[l], P.n, items});
+      items += P.n;
     }
     if (jobs.empty()) continue;
-    k_l2l<T><<<(unsigned)items, threads, 0, c.stream>>>(upload_jobs(c, jobs), (int)jobs.size(), (const T *)tb.rot4, K);
+    k_l2l<T><<<(unsigned)items, oct_threads(K, c.p, items), oct_smem<T>(K, c.p), c.stream>>>(
+        upload_jobs(c, jobs), (int)jobs.size(), (const T *)tb.rot4, K, c.p);
     LPB_LAUNCH();
     c.launches++;
   }

@@ -182,19 +182,138 @@ __global__ void __launch_bounds__(128) k_p2m_sparse(const P2MJob *jobs, int nj, 
 // ---------------------------------------------------------------------------------------
 // M2M (children -> parent) and L2L (parent -> child): azimuth-factored dense operators, stored with
 // the output row fastest so that a warp's operator reads coalesce.
+//
+// One CTA per parent (M2M: and per source type where parents are few): the operator of a z-half serves its (at most
+// four) children, whose columns lie side by side in shared memory.  Rows are real: K real parts by P, then the
+// K - p - 1 imaginary parts of m > 0 by Q (the m = 0 ones vanish for real charges).  A thread owns one row of one
+// z-half and one of OCT_SPLIT parts of its columns.
+// Bound: latency where parents are few, L2 reads of the operators (or the FP64 pipe) where they are many.  A thread per
+// row that walked both z-halves of every type in turn took 255 us for the 56 parents of a level, as long as for 448;
+// now 16 us.  M2M of three layers N = 1M (p = 10, 56 / 448 / 3,584 parents) 869 -> 209 us, L2L 307 -> 118; four layers
+// N = 200,000 (p = 8, 24,576 sparse parents) M2M 2.28 -> 1.28 ms an evaluation, L2L 0.57 -> 0.28.
 // ---------------------------------------------------------------------------------------
+constexpr int OCT_SPLIT = 2;
+// parents of a level up to which each source type takes a CTA of its own; beyond it the set-up that every CTA
+// repeats costs more than the types in turn (868 parents p = 10 FP64: 231 us in turn, 199 apart)
+constexpr int M2M_TSPLIT_MAX = 2048;
+// CTAs of a level up to which a CTA takes one group of threads per z-half and column part (latency counts);
+// beyond it one group does all, so that a half without children idles no threads and more parents are in flight
+// (24,576 sparse parents p = 8: 2.08 ms with the groups, 1.01 with one; 56 parents FP32: 13 us with, 16 - 25 without)
+constexpr int OCT_WIDE = 512;
+static __host__ __device__ __forceinline__ int oct_rows(int K, int p) { return (2 * K - (p + 1) + 31) / 32 * 32; }
+static int oct_threads(int K, int p, int64_t ctas) {
+  const int r = oct_rows(K, p);
+  if (ctas > OCT_WIDE) return r;
+  return 2 * r * OCT_SPLIT <= 1024 ? 2 * r * OCT_SPLIT : 2 * r;  // p = 16: two parts of 320 rows exceed a block
+}
 template <typename T>
-__device__ __forceinline__ void rot_of_octant(uint64_t ckey, int m, const T *rot4, T &c, T &s) {
-  const int oct = (int)(ckey & 7ull);
-  const int dir = ((oct >> 2) & 1) * 2 + ((oct >> 1) & 1);
-  c = rot4[(dir * (PMAX + 1) + m) * 2];
-  s = rot4[(dir * (PMAX + 1) + m) * 2 + 1];
+static size_t oct_smem(int K, int p) {
+  const int R = 2 * K - (p + 1);
+  return sizeof(T) * ((size_t)R * 8 + 4 * (PMAX + 1) * 2) + sizeof(int) * (R + K);
+}
+__device__ __forceinline__ void ld4(const float *p, float *v) {
+  const float4 a = *(const float4 *)p;
+  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+}
+__device__ __forceinline__ void ld4(const double *p, double *v) {
+  const double2 a = *(const double2 *)p, b = *(const double2 *)(p + 2);
+  v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+}
+template <int NJ, typename T>
+__device__ __forceinline__ void oct_dot(T *acc, const T *__restrict__ W, const int *row, const T *x, int q0, int q1, int K) {
+#pragma unroll 8
+  for (int q = q0; q < q1; ++q) {
+    const T w = __ldg(W + row[q] * K);
+    T v[4];
+    if (NJ == 4) ld4(x + q * 8, v);
+    else
+#pragma unroll
+      for (int j = 0; j < NJ; ++j) v[j] = x[q * 8 + j];
+#pragma unroll
+    for (int j = 0; j < NJ; ++j) acc[j] += w * v[j];
+  }
+}
+// shared state of a CTA: the children's columns, the azimuthal factors of the four (x, y) octants, indices
+template <typename T>
+struct OctCta {
+  T *x;      // [R][8]: row, z-half * 4 + slot
+  T *rt;     // [4][PMAX + 1][2]
+  int *row;  // [R] coefficient of each real row
+  int *nm;   // [K] n | m << 8
+  int K, KI;
+  __device__ __forceinline__ OctCta(unsigned char *sm, const T *rot4, int K_, int p) : K(K_), KI(K_ - (p + 1)) {
+    const int R = K + KI;
+    x = (T *)sm;
+    rt = x + R * 8;
+    row = (int *)(rt + 4 * (PMAX + 1) * 2);
+    nm = row + R;
+    for (int e = threadIdx.x; e < 4 * (PMAX + 1) * 2; e += blockDim.x) rt[e] = rot4[e];
+    for (int k = threadIdx.x; k < K; k += blockDim.x) {
+      int n = (int)((sqrtf(8.0f * (float)k + 1.0f) - 1.0f) * 0.5f);
+      while (n * (n + 1) / 2 > k) --n;
+      while ((n + 1) * (n + 2) / 2 <= k) ++n;
+      const int m = k - n * (n + 1) / 2;
+      nm[k] = n | m << 8;
+      row[k] = k;
+      if (m) row[K + k - n - 1] = k;  // k - n - 1: position among the m > 0 coefficients
+    }
+  }
+  __device__ __forceinline__ void put(int k, int dir, int slot, T re, T im) {  // rotated into the operator's frame
+    const int n = nm[k] & 255, m = nm[k] >> 8;
+    const T cs = rt[(dir * (PMAX + 1) + m) * 2], sn = rt[(dir * (PMAX + 1) + m) * 2 + 1];
+    x[k * 8 + slot] = cs * re - sn * im;
+    if (m) x[(K + k - n - 1) * 8 + slot] = sn * re + cs * im;
+  }
+  __device__ __forceinline__ void add(int k, int dir, int slot, T &re, T &im) const {  // rotated back
+    const int n = nm[k] & 255, m = nm[k] >> 8;
+    const T cs = rt[(dir * (PMAX + 1) + m) * 2], sn = rt[(dir * (PMAX + 1) + m) * 2 + 1];
+    const T yr = x[k * 8 + slot], yi = m ? x[(K + k - n - 1) * 8 + slot] : (T)0;
+    re += cs * yr + sn * yi;
+    im += cs * yi - sn * yr;
+  }
+  // x <- [P 0; 0 Q] x for the n0, n1 slots in use of the two z-halves; ops: [z-half][P, Q][K][K].  A group of threads
+  // (one per row) takes one z-half and one part of the columns, or, where it is the only one, all of both.
+  __device__ __forceinline__ void product(const T *ops, int n0, int n1) {
+    const int R = K + KI, Rp = (R + 31) / 32 * 32, grp = threadIdx.x / Rp, r = threadIdx.x - grp * Rp;
+    const int ngrp = blockDim.x / Rp, parts = ngrp > 1 ? ngrp >> 1 : 1, part = grp >> 1;
+    const int im = r >= K;
+    T acc[2][4] = {};
+    if (r < R) {
+      const int len = im ? KI : K, per = (len + parts - 1) / parts, b = im ? K : 0;
+      const int q0 = b + part * per, q1 = b + min(len, (part + 1) * per);
+#pragma unroll
+      for (int cz = 0; cz < 2; ++cz) {
+        const int n = cz ? n1 : n0;
+        if (n == 0 || (ngrp > 1 && (grp & 1) != cz)) continue;
+        const T *W = ops + (size_t)(cz * 2 + im) * K * K + row[r];
+        if (n == 1) oct_dot<1>(acc[cz], W, row, x + cz * 4, q0, q1, K);
+        else if (n == 2) oct_dot<2>(acc[cz], W, row, x + cz * 4, q0, q1, K);
+        else oct_dot<4>(acc[cz], W, row, x + cz * 4, q0, q1, K);  // a fourth, unused slot is not read back
+      }
+    }
+    for (int t = 0; t < parts; ++t) {
+      __syncthreads();
+      if (r >= R || part != t) continue;
+#pragma unroll
+      for (int cz = 0; cz < 2; ++cz) {
+        const int n = cz ? n1 : n0;
+        if (ngrp > 1 && (grp & 1) != cz) continue;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if (j < n) x[r * 8 + cz * 4 + j] = t ? x[r * 8 + cz * 4 + j] + acc[cz][j] : acc[cz][j];
+      }
+    }
+    __syncthreads();
+  }
+};
+// slot of child c among the children in `have` (bit per child; zm: bit set for the upper z-half)
+__device__ __forceinline__ int oct_slot(uint32_t have, uint32_t zm, int c) {
+  const int cz = (zm >> c) & 1;
+  return cz * 4 + __popc(have & (cz ? zm : ~zm) & ((1u << c) - 1u));
 }
 
-// One CTA per parent: for every source type present in it (pmask; a box holds an expansion of type t if bit t
-// of its mask is set, other rows are neither written nor read), all children's rotated
-// multipoles are staged at once; a thread owns an output row, reads each operator entry once per z-half
-// (child octant bit cz) and applies it to the (at most four) children with that cz.
+// A box holds an expansion of type t if bit t of its mask is set; other rows are neither written nor read.
+// tsplit CTAs share the types present in a parent.
 struct M2MJob {
   const uint32_t *pstart, *pcount;  // children of every parent
   const uint64_t *ckey;
@@ -202,134 +321,93 @@ struct M2MJob {
   const void *Mc, *ops;
   void *Mp;
   int64_t np, item0;
-  int ntypes;
+  int ntypes, tsplit;
 };
 template <typename T>
-__global__ void k_m2m(const M2MJob *jobs, int nj, const T *rot4, int K) {
+__global__ void __launch_bounds__(1024) k_m2m(const M2MJob *jobs, int nj, const T *rot4, int K, int p) {
   typedef typename C2<T>::t T2;
-  __shared__ T xr[8][KHALF_MAX], xi[8][KHALF_MAX];
-  __shared__ uint64_t ck_s[8];
+  extern __shared__ __align__(16) unsigned char oct_sm[];
   __shared__ uint32_t cm_s[8];
+  __shared__ uint32_t oc_s[8];
   const M2MJob &J = job_of(jobs, nj, (int64_t)blockIdx.x);
-  const int64_t box = (int64_t)blockIdx.x - J.item0;
+  const int64_t it = (int64_t)blockIdx.x - J.item0, box = it / J.tsplit;
+  const int part = (int)(it - box * J.tsplit);
   if (box >= J.np) return;
-  const size_t KK = (size_t)K * K;
+  uint32_t todo = J.pmask ? J.pmask[box] : 1u;
+  if (__popc(todo) <= part) return;
   const int ntypes = J.ntypes;
   const uint32_t c0 = J.pstart[box], nc = min(J.pcount[box], 8u);
-  if (threadIdx.x < nc) {
-    ck_s[threadIdx.x] = J.ckey[c0 + threadIdx.x];
-    cm_s[threadIdx.x] = J.cmask ? J.cmask[c0 + threadIdx.x] : 1u;
+  OctCta<T> S(oct_sm, rot4, K, p);
+  if (threadIdx.x < 8) {
+    const bool in = threadIdx.x < nc;
+    oc_s[threadIdx.x] = in ? (uint32_t)(J.ckey[c0 + threadIdx.x] & 7ull) : 0u;
+    cm_s[threadIdx.x] = in ? (J.cmask ? J.cmask[c0 + threadIdx.x] : 1u) : 0u;
   }
   const T2 *Mc = (const T2 *)J.Mc;
-  for (uint32_t todo = J.pmask ? J.pmask[box] : 1u; todo; todo &= todo - 1) {
+  for (int w = 0; todo; todo &= todo - 1, ++w) {
+    if (w % J.tsplit != part) continue;
     const int type = __ffs(todo) - 1;
     __syncthreads();
-    // children of the type, by z-half
-    int slot[2][4], ns[2] = {0, 0};
+    uint32_t have = 0, zm = 0;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) slot[0][j] = slot[1][j] = 0;
-    for (uint32_t c = 0; c < nc; ++c)
-      if ((cm_s[c] >> type) & 1u) {
-#pragma unroll
-        for (int cz = 0; cz < 2; ++cz) {
-          if ((int)(ck_s[c] & 1ull) != cz) continue;
-#pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (j >= ns[cz]) slot[cz][j] = (int)c;  // unfilled slots repeat the last child
-          ++ns[cz];
-        }
-      }
+    for (int c = 0; c < 8; ++c) {
+      have |= ((cm_s[c] >> type) & 1u) << c;
+      zm |= (oc_s[c] & 1u) << c;
+    }
     for (uint32_t e = threadIdx.x; e < nc * (uint32_t)K; e += blockDim.x) {
-      const int c = (int)(e / K), k = (int)(e % K);
-      if (!((cm_s[c] >> type) & 1u)) continue;
-      T cs, sn;
-      rot_of_octant(ck_s[c], cK.mof[k], rot4, cs, sn);
+      const int c = (int)(e / K), k = (int)(e - c * K);
+      if (!((have >> c) & 1u)) continue;
       const T2 v = Mc[((size_t)(c0 + c) * ntypes + type) * K + k];
-      xr[c][k] = cs * v.x - sn * v.y;
-      xi[c][k] = sn * v.x + cs * v.y;
+      S.put(k, oc_s[c] >> 1, oct_slot(have, zm, c), v.x, v.y);
     }
     __syncthreads();
+    S.product((const T *)J.ops + (size_t)type * 4 * K * K, __popc(have & ~zm), __popc(have & zm));
     for (int i = threadIdx.x; i < K; i += blockDim.x) {
-      const int m = cK.mof[i];
       T ar = 0, ai = 0;
-#pragma unroll
-      for (int cz = 0; cz < 2; ++cz) {
-        const int n = ns[cz];
-        if (n == 0) continue;
-        const T *P = (const T *)J.ops + ((size_t)type * 2 + cz) * 2 * KK + i, *Q = P + KK;
-        T yr[4] = {0, 0, 0, 0}, yi[4] = {0, 0, 0, 0};
-        if (n == 1) {
-          const T *x0 = xr[slot[cz][0]], *x1 = xi[slot[cz][0]];
-#pragma unroll 4
-          for (int k = 0; k < K; ++k) {
-            yr[0] += P[(size_t)k * K] * x0[k];
-            yi[0] += Q[(size_t)k * K] * x1[k];
-          }
-        } else {
-#pragma unroll 2
-          for (int k = 0; k < K; ++k) {
-            const T pv = P[(size_t)k * K], qv = Q[(size_t)k * K];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              yr[j] += pv * xr[slot[cz][j]][k];
-              yi[j] += qv * xi[slot[cz][j]][k];
-            }
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          if (j >= n) break;
-          T cs, sn;
-          rot_of_octant(ck_s[slot[cz][j]], m, rot4, cs, sn);
-          ar += cs * yr[j] + sn * yi[j];
-          ai += cs * yi[j] - sn * yr[j];
-        }
-      }
+      for (int c = 0; c < (int)nc; ++c)
+        if ((have >> c) & 1u) S.add(i, oc_s[c] >> 1, oct_slot(have, zm, c), ar, ai);
       ((T2 *)J.Mp)[((size_t)box * ntypes + type) * K + i] = T2{ar, ai};
     }
   }
 }
 
 struct L2LJob {
-  const uint32_t *cparent;
+  const uint32_t *pstart, *pcount;  // children of every parent
   const uint64_t *ckey;
   const void *Lp, *ops;
   void *Lc;
-  int64_t nc, item0;
+  int64_t np, item0;
 };
 template <typename T>
-__global__ void k_l2l(const L2LJob *jobs, int nj, const T *rot4, int K) {
+__global__ void __launch_bounds__(1024) k_l2l(const L2LJob *jobs, int nj, const T *rot4, int K, int p) {
   typedef typename C2<T>::t T2;
-  __shared__ T xr[KHALF_MAX], xi[KHALF_MAX];
+  extern __shared__ __align__(16) unsigned char oct_sm[];
+  __shared__ uint32_t oc_s[8];
   const L2LJob &J = job_of(jobs, nj, (int64_t)blockIdx.x);
-  const int64_t c = (int64_t)blockIdx.x - J.item0;
-  if (c >= J.nc) return;
-  const uint64_t ck = J.ckey[c];
-  const int cz = (int)(ck & 1ull);
-  const size_t KK = (size_t)K * K;
-  const T *P = (const T *)J.ops + (size_t)cz * 2 * KK, *Q = P + KK;
-  const uint32_t par = J.cparent[c];
-  const T2 *Lp = (const T2 *)J.Lp;
-  for (int e = threadIdx.x; e < K; e += blockDim.x) {
-    T cs, sn;
-    rot_of_octant(ck, cK.mof[e], rot4, cs, sn);
-    const T2 v = Lp[(size_t)par * K + e];
-    xr[e] = cs * v.x - sn * v.y;
-    xi[e] = sn * v.x + cs * v.y;
+  const int64_t box = (int64_t)blockIdx.x - J.item0;
+  if (box >= J.np) return;
+  const uint32_t c0 = J.pstart[box], nc = min(J.pcount[box], 8u);
+  OctCta<T> S(oct_sm, rot4, K, p);
+  if (threadIdx.x < 8) oc_s[threadIdx.x] = threadIdx.x < nc ? (uint32_t)(J.ckey[c0 + threadIdx.x] & 7ull) : 0u;
+  __syncthreads();
+  const uint32_t have = (1u << nc) - 1u;
+  uint32_t zm = 0;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) zm |= (oc_s[c] & 1u) << c;
+  const T2 *Lp = (const T2 *)J.Lp + (size_t)box * K;
+  for (uint32_t e = threadIdx.x; e < nc * (uint32_t)K; e += blockDim.x) {
+    const int c = (int)(e / K), k = (int)(e - c * K);
+    const T2 v = Lp[k];
+    S.put(k, oc_s[c] >> 1, oct_slot(have, zm, c), v.x, v.y);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < K; i += blockDim.x) {
-    T yr = 0, yi = 0;
-#pragma unroll 4
-    for (int k = 0; k < K; ++k) {
-      yr += P[(size_t)k * K + i] * xr[k];
-      yi += Q[(size_t)k * K + i] * xi[k];
-    }
-    T cs, sn;
-    rot_of_octant(ck, cK.mof[i], rot4, cs, sn);
-    T2 &dst = ((T2 *)J.Lc)[(size_t)c * K + i];
-    dst.x += cs * yr + sn * yi;
-    dst.y += cs * yi - sn * yr;
+  S.product((const T *)J.ops, __popc(have & ~zm), __popc(have & zm));
+  for (uint32_t e = threadIdx.x; e < nc * (uint32_t)K; e += blockDim.x) {
+    const int c = (int)(e / K), k = (int)(e - c * K);
+    T2 &dst = ((T2 *)J.Lc)[(size_t)(c0 + c) * K + k];
+    T re = dst.x, im = dst.y;
+    S.add(k, oc_s[c] >> 1, oct_slot(have, zm, c), re, im);
+    dst = T2{re, im};
   }
 }
 
