@@ -364,23 +364,37 @@ static void eval_front(Ctx &c, int64_t n, const double *q, const double *q2, con
       }
     }
   }
-  // the free-space operators on the side stream, concurrently with the image trees and lists
+  // beside the image trees and lists: the free-space operators on the far stream, whose upward pass needs
+  // them first, and on the side stream what the reaction tables need of depths and medium alone
   LPB_CUDA(cudaEventRecord(c.ev_fork, c.stream));
   LPB_CUDA(cudaStreamWaitEvent(c.side, c.ev_fork, 0));
+  LPB_CUDA(cudaStreamWaitEvent(c.far, c.ev_fork, 0));
   {
-    OnStream on(c, c.side);
-    build_operators(c, c.groups, 1);
-    LPB_CUDA(cudaEventRecord(c.ev_free, c.side));
+    OnStream on(c, c.far);
+    build_free_operators(c, c.groups);
+    LPB_CUDA(cudaEventRecord(c.ev_free, c.far));
   }
   build_images(c, c.groups, n, q, xyz, layer, rank, cnt);
+  {
+    double lmin = 1e300, hmin = 1e300;
+    for (int k = 0; k <= L; ++k) lmin = std::min(lmin, c.md.lam[k]);
+    for (auto &g : c.groups)
+      if (g.I.np) hmin = std::min(hmin, g.h(g.D));
+    c.stab_lmin = hmin < 1e300 ? lmin * hmin : lmin;
+  }
+  ReactPlan plan;
   // box counts to host
   {
     uint32_t *dd = nullptr;
     size_t nc = 0;
     build_boxes(c, c.groups, &dd, &nc);
+    uint32_t *hh = (uint32_t *)c.h_pinned;
+    if (nc) LPB_CUDA(cudaMemcpyAsync(hh, dd, sizeof(uint32_t) * nc, cudaMemcpyDeviceToHost, c.stream));
+    {
+      OnStream on(c, c.side);
+      begin_react_operators(c, c.groups, plan);
+    }
     if (nc) {
-      uint32_t *hh = (uint32_t *)c.h_pinned;
-      LPB_CUDA(cudaMemcpyAsync(hh, dd, sizeof(uint32_t) * nc, cudaMemcpyDeviceToHost, c.stream));
       LPB_CUDA(cudaStreamSynchronize(c.stream));
       read_box_counts(c.groups, hh);
     }
@@ -389,20 +403,13 @@ static void eval_front(Ctx &c, int64_t n, const double *q, const double *q2, con
   build_lists(c, c.groups);
   prof_mark(c, "tree");
   start_near(c, phi, field);
-  {
-    double lmin = 1e300, hmin = 1e300;
-    for (int k = 0; k <= L; ++k) lmin = std::min(lmin, c.md.lam[k]);
-    for (auto &g : c.groups)
-      if (g.I.np) hmin = std::min(hmin, g.h(g.D));
-    c.stab_lmin = hmin < 1e300 ? lmin * hmin : lmin;
-  }
   // reaction tables, operators and near-field nodes on the side stream, after the lists (the M2L
   // waits for them)
   LPB_CUDA(cudaEventRecord(c.ev_fork, c.stream));
   {
     OnStream on(c, c.side);
     LPB_CUDA(cudaStreamWaitEvent(c.side, c.ev_fork, 0));
-    build_operators(c, c.groups, 2);
+    build_react_operators(c, c.groups, plan);
     for (auto &g : c.groups) {
       if ((g.parts & 2) && g.ureact) {
         double zt, zs;

@@ -1391,7 +1391,7 @@ void run_fmm_front(Ctx &c, std::vector<Group> &groups) {
   c.def.red.clear();
   c.def.tc_items = c.def.red_elems = 0;
   const bool d = c.opts.precision == LPBFMM_FP64;
-  // the free-space operators (side stream) are complete before the upward pass
+  // the free-space operators (far stream) are complete before the upward pass
   if (c.ev_free) LPB_CUDA(cudaStreamWaitEvent(c.stream, c.ev_free, 0));
   d ? upward_t<double>(c, groups) : upward_t<float>(c, groups);
   prof_mark(c, "upward");

@@ -310,9 +310,9 @@ struct Ctx {
   int nev = 0;
   int launches = 0;
   Deferred def;
-  // operators are built on a second stream: the free-space ones concurrently with the image
-  // trees and lists (the upward pass waits for them, ev_free), the reaction ones concurrently
-  // with the upward pass (the M2L waits for them, ev_join)
+  // operators are built beside the trees and lists: the free-space ones on the far stream (the upward pass
+  // waits for them, ev_free), the reaction tables and operators on the side stream (the M2L waits for
+  // them, ev_join).  One after the other on one stream the tables waited for the free-space operators.
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_free = nullptr, ev_join = nullptr;
   cudaEvent_t ev_gfork = nullptr;
@@ -367,9 +367,26 @@ void recharge_points(Ctx &c, std::vector<Group> &groups, const double *q);
 void adaptive_lists(Ctx &c, Group &g, int s, int ws, std::vector<int64_t> &rec);
 
 // ops.cu
-// which: 1 the free-space operators (M2M, L2L, free M2L; need only the depths and roots),
-// 2 the reaction tables and operators (need the interaction lists)
-void build_operators(Ctx &c, std::vector<Group> &groups, int which);
+// one reaction table and operator set: a (group, level, source type)
+struct RDesc {
+  int l, a, lp, b, tau, ntypes, st, lev;
+  int cls0, group;       // lev, group: where the classes in use are found; the table array holds classes cls0, cls0 + 1, ... (0: every class)
+  double h, Lam, Lamp;
+  const uint8_t *used;   // [NREACT_CLS]
+  double *stab;          // [NREACT_CLS][ntypes][TS]
+  float2 *coef;          // [K*K][NS] double-float (hi, lo) coefficients C_s
+  void *out;             // operators of class 0, type 0 of this level [NREACT_CLS][ntypes][2][K][K]
+};
+struct NDesc;
+struct ReactPlan {
+  std::vector<RDesc> desc;
+  const NDesc *nodes = nullptr;  // device, one per descriptor
+};
+// the free-space operators (M2M, L2L, free M2L; need only the depths and roots)
+void build_free_operators(Ctx &c, std::vector<Group> &groups);
+// the reaction tables and operators: what depths and medium give, then what needs the interaction lists
+void begin_react_operators(Ctx &c, std::vector<Group> &groups, ReactPlan &plan);
+void build_react_operators(Ctx &c, std::vector<Group> &groups, ReactPlan &plan);
 void build_near_nodes(Ctx &c, Group &g, double zeta_min, double rho_max);
 void stable_noalloc(Ctx &c, int l, int a, int lp, int b, double h, double rho, double zt, double zs, int Kmax,
                     double *out);

@@ -122,16 +122,6 @@ __global__ void k_build_ops(const OpDesc *descs, const double *prep, const doubl
 // ---------------------------------------------------------------------------------------
 // Reaction operators
 // ---------------------------------------------------------------------------------------
-struct RDesc {
-  int l, a, lp, b, tau, ntypes, st, pad;
-  int cls0, pad2;        // the table array holds classes cls0, cls0 + 1, ... (0: every class)
-  double h, Lam, Lamp;
-  const uint8_t *used;   // [NREACT_CLS]
-  double *stab;          // [NREACT_CLS][ntypes][TS]
-  float2 *coef;          // [K*K][NS] double-float (hi, lo) coefficients C_s
-  void *out;             // operators of class 0, type 0 of this level [NREACT_CLS][ntypes][2][K][K]
-};
-
 constexpr int MAXPANEL = 1024;
 
 __device__ __forceinline__ int stab_index(int KT, int K, int d, int ij) { return ((K * (KT + 1)) + d) * 4 + ij; }
@@ -443,15 +433,30 @@ static NDesc node_desc(int KT, double tol, double Lam, double Lamp) {
   return N;
 }
 
-// C_s(n,m,nu,mu) = sum_{k+k'=s} c^{nm}_k c^{nu mu}_{k'} Lam^{n-m-2k} Lamp^{nu-mu-2k'}
+// C_s(n,m,nu,mu) = sum_{k+k'=s} c^{nm}_k c^{nu mu}_{k'} Lam^{n-m-2k} Lamp^{nu-mu-2k'}, s <= (n-m+1)/2 + (nu-mu+1)/2
+// (the assembly reads no others).  Bound: the FP64 pipe, so the powers go into the two factors once per CTA and
+// a term is one FMA (four FP64 operations before): 0.110 -> 0.040 ms at p = 10, 0.57 -> 0.20 ms for four layers at p = 12.
 __global__ void k_react_coef(const RDesc *descs, const double *tpoly, int tpk, int p, int K) {
   const RDesc D = descs[blockIdx.y];
-  __shared__ double pl[PMAX + 3], plp[PMAX + 3];  // Lam^e, Lamp^e for e = -1..p+1 at index e+1
-  if (threadIdx.x == 0) {
-    pl[0] = 1.0 / D.Lam;
-    plp[0] = 1.0 / D.Lamp;
-    pl[1] = plp[1] = 1.0;
-    for (int e = 2; e <= p + 2; ++e) { pl[e] = pl[e - 1] * D.Lam; plp[e] = plp[e - 1] * D.Lamp; }
+  __shared__ double pl[2][PMAX + 3];  // Lam^e, Lamp^e for e = -1..p+1 at index e+1
+  extern __shared__ double coef_sm[];
+  double *A = coef_sm, *B = A + (size_t)K * tpk;  // c^{nm}_k Lam^{n-m-2k}, c^{nu mu}_k Lamp^{nu-mu-2k}
+  if (threadIdx.x < 2) {
+    const double v = threadIdx.x ? D.Lamp : D.Lam;
+    double *t = pl[threadIdx.x];
+    t[0] = 1.0 / v;
+    t[1] = 1.0;
+    for (int e = 2; e <= p + 2; ++e) t[e] = t[e - 1] * v;
+  }
+  __syncthreads();
+  for (int x = threadIdx.x; x < K * tpk; x += blockDim.x) {
+    const int o = x / tpk, k = x % tpk;
+    int n, m;
+    hdecode(o, n, m);
+    const int e = n - m - 2 * k + 1;
+    const double c = e >= 0 ? tpoly[x] : 0.0;
+    A[x] = e >= 0 ? c * pl[0][e] : 0.0;
+    B[x] = e >= 0 ? c * pl[1][e] : 0.0;
   }
   __syncthreads();
   const int NS = p + 2;
@@ -462,20 +467,19 @@ __global__ void k_react_coef(const RDesc *descs, const double *tpoly, int tpk, i
   hdecode(o, n, m);
   hdecode(i, nu, mu);
   const int k1 = (n - m + 1) / 2, k2 = (nu - mu + 1) / 2;
-  for (int s = 0; s < NS; ++s) {
+  const double *a = A + o * tpk, *b = B + i * tpk;
+  for (int s = 0; s <= k1 + k2; ++s) {
     double acc = 0.0;
-    for (int k = 0; k <= k1; ++k) {
-      const int kp = s - k;
-      if (kp < 0 || kp > k2) continue;
-      acc += tpoly[o * tpk + k] * tpoly[i * tpk + kp] * pl[n - m - 2 * k + 1] * plp[nu - mu - 2 * kp + 1];
-    }
+    for (int k = max(0, s - k2); k <= min(k1, s); ++k) acc = fma(a[k], b[s - k], acc);
     const float h = (float)acc;
     D.coef[(size_t)e * NS + s] = make_float2(h, (float)(acc - (double)h));
   }
 }
 
 // double-float arithmetic (value = hi + lo, two FP32 numbers; about 44 significant bits) on
-// the FP32 pipes: exact products by FMA, sums by the two-sum of Knuth, then renormalised.
+// the FP32 pipes: exact products by FMA, sums by the two-sum of Knuth, whose error joins the low part.  The
+// two parts of a sum are not renormalised on the way (the two-sum asks for no order of its operands, the low
+// part stays a few ulps of the partial sums): 12 operations a term instead of 15, assembly 0.77 -> 0.73 ms at p = 10.
 // The _rn intrinsics keep the compiler from contracting the error-free transformations.
 __device__ __forceinline__ float2 df_split(double v) {
   const float h = (float)v;
@@ -496,10 +500,8 @@ __device__ __forceinline__ void df_fma(float2 a, float2 b, float2 &acc) {
   e = fmaf(a.y, b.x, e);
   const float s = __fadd_rn(acc.x, p);
   const float v = __fsub_rn(s, acc.x);
-  float t = __fadd_rn(__fsub_rn(acc.x, __fsub_rn(s, v)), __fsub_rn(p, v));
-  t = __fadd_rn(t, __fadd_rn(acc.y, e));
-  const float hi = __fadd_rn(s, t);
-  acc = make_float2(hi, __fsub_rn(t, __fsub_rn(hi, s)));
+  const float t = __fadd_rn(__fsub_rn(acc.x, __fsub_rn(s, v)), __fsub_rn(p, v));
+  acc = make_float2(s, __fadd_rn(t, __fadd_rn(acc.y, e)));
 }
 
 // ASM_CC classes per CTA share each entry's decode and coefficient loads.  The tables sit in shared memory by
@@ -649,10 +651,12 @@ __global__ void k_near_nodes(Medium md, int l, int a, int ntypes, double umax, d
   }
 }
 
-// nodes and tables of nd descriptors (two launches)
-static void launch_tables(Ctx &c, const RDesc *dr, const NDesc *dn, int nq, unsigned nd, int KT) {
+// nodes, then tables, of nd descriptors
+static void launch_nodes(Ctx &c, const RDesc *dr, const NDesc *dn, int nq, unsigned nd) {
   k_stab_nodes<<<dim3((unsigned)((nq + 127) / 128), nd), 128, 0, c.stream>>>(dr, dn, c.md);
   LPB_LAUNCH();
+}
+static void launch_tables(Ctx &c, const RDesc *dr, const NDesc *dn, unsigned nd, int KT) {
   LPB_ATTR_ONCE(k_stab_table, stab_table_smem(KMAX_TAB));  // the largest table any order needs
   k_stab_table<<<dim3(NKK * (NRHO / ST_NC), nd), ST_THREADS, stab_table_smem(KT), c.stream>>>(dr, dn, KT, c.sfac);
   LPB_LAUNCH();
@@ -755,19 +759,21 @@ static void build_free_t(Ctx &c, std::vector<Group> &groups) {
   c.launches += 2;
 }
 
-// the reaction tables and operators of every group, level and type: five launches
+// What the reaction tables and operators need of depths and medium alone: quadrature nodes, Bessel columns and
+// Legendre-product coefficients of every group, level and type (three launches).  They run beside the trees and
+// lists; in line with the tables, and those behind the free-space operators on one stream, they held up each
+// small evaluation (N = 3,000, p = 10: 3.50 -> 3.31 ms with k_react_coef's and the assembly's shorter sums).
 template <typename T>
-static void build_react_t(Ctx &c, std::vector<Group> &groups) {
+static void begin_react_t(Ctx &c, std::vector<Group> &groups, ReactPlan &plan) {
   const int p = c.p, K = c.K;
   const size_t KK = (size_t)K * K;
   const int KT = 2 * p + 3, NS = p + 2;
   const size_t TS = (size_t)(KT + 1) * (KT + 1) * 4;
-  std::vector<RDesc> rd;
+  std::vector<RDesc> &rd = plan.desc;
   for (auto &g : groups) {
-    if (!(g.parts & 2) || !g.I.np) continue;
+    if (!(g.parts & 2) || !g.I.np || !g.T.np) continue;
     const int st = (g.a == 1) ? -1 : 1;
     for (int l = 2; l <= g.D; ++l) {
-      if (!g.vreact[l]) continue;
       const double h = g.h(l);
       g.stab[l] = c.arena.get<double>((size_t)NREACT_CLS * g.ntypes * TS);
       g.op_react[l] = c.arena.get<T>((size_t)NREACT_CLS * g.ntypes * 2 * KK);
@@ -776,10 +782,10 @@ static void build_react_t(Ctx &c, std::vector<Group> &groups) {
         int lp, bb;
         type_decode(t, lp, bb);
         RDesc d;
-        d.l = g.l; d.a = g.a; d.lp = lp; d.b = bb; d.tau = t; d.ntypes = g.ntypes; d.st = st; d.pad = l;
-        d.cls0 = 0; d.pad2 = 0;
+        d.l = g.l; d.a = g.a; d.lp = lp; d.b = bb; d.tau = t; d.ntypes = g.ntypes; d.st = st; d.lev = l;
+        d.cls0 = 0; d.group = (int)(&g - groups.data());
         d.h = h; d.Lam = c.md.lam[g.l] * h; d.Lamp = c.md.lam[lp] * h;
-        d.used = g.used[l];
+        d.used = nullptr;
         d.stab = g.stab[l];
         d.coef = coef + (size_t)t * KK * NS;
         d.out = g.op_react[l];
@@ -802,20 +808,38 @@ static void build_react_t(Ctx &c, std::vector<Group> &groups) {
   for (auto &n : nv) n.nodes = c.arena.get<double>((size_t)N.nq * NDF);
   NDesc *dn = c.arena.get<NDesc>(nv.size());
   LPB_CUDA(cudaMemcpyAsync(dn, nv.data(), sizeof(NDesc) * nv.size(), cudaMemcpyHostToDevice, c.stream));
-  launch_tables(c, dr, dn, N.nq, nd, KT);
-  k_react_coef<<<dim3((unsigned)((KK + 255) / 256), nd), 256, 0, c.stream>>>(dr, c.tpoly, c.tpk, p, K);
+  plan.nodes = dn;
+  launch_nodes(c, dr, dn, N.nq, nd);
+  k_react_coef<<<dim3((unsigned)((KK + 255) / 256), nd), 256, sizeof(double) * 2 * K * c.tpk, c.stream>>>(
+      dr, c.tpoly, c.tpk, p, K);
   LPB_LAUNCH();
+  c.launches += 3;
+}
+// the tables and operators of the classes that the lists use (two launches)
+template <typename T>
+static void build_react_t(Ctx &c, std::vector<Group> &groups, ReactPlan &plan) {
+  if (plan.desc.empty()) return;
+  const int p = c.p, KT = 2 * p + 3;
+  for (auto &d : plan.desc) d.used = groups[d.group].used[d.lev];
+  const unsigned nd = (unsigned)plan.desc.size();
+  RDesc *dr = c.arena.get<RDesc>(nd);
+  LPB_CUDA(cudaMemcpyAsync(dr, plan.desc.data(), sizeof(RDesc) * nd, cudaMemcpyHostToDevice, c.stream));
+  launch_tables(c, dr, plan.nodes, nd, KT);
   LPB_ATTR_ONCE(k_react_assemble<T>, assemble_smem(PMAX, KMAX_TAB));
   k_react_assemble<T><<<dim3((NREACT_CLS + ASM_CC - 1) / ASM_CC, nd), 256, assemble_smem(p, KT), c.stream>>>(
-      dr, p, K, KT, c.sfac);
+      dr, p, c.K, KT, c.sfac);
   LPB_LAUNCH();
-  c.launches += 5;
+  c.launches += 2;
 }
 
-void build_operators(Ctx &c, std::vector<Group> &groups, int which) {
-  const bool d = c.opts.precision == LPBFMM_FP64;
-  if (which == 1) d ? build_free_t<double>(c, groups) : build_free_t<float>(c, groups);
-  else d ? build_react_t<double>(c, groups) : build_react_t<float>(c, groups);
+void build_free_operators(Ctx &c, std::vector<Group> &groups) {
+  c.opts.precision == LPBFMM_FP64 ? build_free_t<double>(c, groups) : build_free_t<float>(c, groups);
+}
+void begin_react_operators(Ctx &c, std::vector<Group> &groups, ReactPlan &plan) {
+  c.opts.precision == LPBFMM_FP64 ? begin_react_t<double>(c, groups, plan) : begin_react_t<float>(c, groups, plan);
+}
+void build_react_operators(Ctx &c, std::vector<Group> &groups, ReactPlan &plan) {
+  c.opts.precision == LPBFMM_FP64 ? build_react_t<double>(c, groups, plan) : build_react_t<float>(c, groups, plan);
 }
 
 void build_near_nodes(Ctx &c, Group &g, double zeta_min, double rho_max) {
@@ -850,8 +874,8 @@ static int class_of_request(double h, double rho, double zt, double zs) {
 
 static RDesc one_class_desc(Ctx &c, int l, int a, int lp, int b, double h, int cls) {
   RDesc d;
-  d.l = l; d.a = a; d.lp = lp; d.b = b; d.tau = 0; d.ntypes = 1; d.st = a == 1 ? -1 : 1; d.pad = 0;
-  d.cls0 = cls; d.pad2 = 0;
+  d.l = l; d.a = a; d.lp = lp; d.b = b; d.tau = 0; d.ntypes = 1; d.st = a == 1 ? -1 : 1; d.lev = 0;
+  d.cls0 = cls; d.group = 0;
   d.h = h; d.Lam = c.md.lam[l] * h; d.Lamp = c.md.lam[lp] * h;
   d.used = nullptr; d.stab = nullptr; d.coef = nullptr; d.out = nullptr;
   return d;
@@ -889,7 +913,8 @@ void debug_stable(Ctx &c, int l, int a, int lp, int b, double h, double rho, dou
   LPB_LAUNCH();
   N.bes = bes;
   LPB_CUDA(cudaMemcpyAsync(dn, &N, sizeof(NDesc), cudaMemcpyHostToDevice, c.stream));
-  launch_tables(c, dr, dn, N.nq, 1, KT);
+  launch_nodes(c, dr, dn, N.nq, 1);
+  launch_tables(c, dr, dn, 1, KT);
   std::vector<double> h_out(TS);
   LPB_CUDA(cudaMemcpyAsync(h_out.data(), stab, sizeof(double) * TS, cudaMemcpyDeviceToHost, c.stream));
   LPB_CUDA(cudaStreamSynchronize(c.stream));
@@ -972,7 +997,8 @@ void stable_noalloc(Ctx &c, int l, int a, int lp, int b, double h, double rho, d
   N.bes = bes;
   k_noalloc_init<<<8, 256, 0, c.stream>>>(d, N, dr, dn, used, cls, stab, (int)TS);
   LPB_LAUNCH();
-  launch_tables(c, dr, dn, N.nq, 1, KT);
+  launch_nodes(c, dr, dn, N.nq, 1);
+  launch_tables(c, dr, dn, 1, KT);
   LPB_CUDA(cudaMemcpyAsync(out, stab, sizeof(double) * TS, cudaMemcpyDeviceToDevice, c.stream));
 }
 
