@@ -16,7 +16,11 @@
 // (the m = 0 imaginary parts vanish for real charges): K^2 + (K - p - 1)^2 FMAs, not 2 K^2.
 #pragma once
 
-constexpr int PAIR_C = 8;    // columns of a batch: 4 per thread, two threads per operator row
+// Columns of a batch: two threads per operator row, every other column each, so that a partial batch of n columns
+// costs ceil(n / 2) quarters of a full one, not all of it (first and second half each: N = 2,003 p = 12 adjoint 52.5 ms,
+// so 49.5; N = 100,000 p = 10 87.7 -> 86.0).
+constexpr int PAIR_C = 8;
+__device__ __forceinline__ int pair_pos(int c) { return (c & 1) * (PAIR_C / 2) + (c >> 1); }
 constexpr int PAIR_KC = 16;  // operator columns staged at a time (16 doubles = one 128-byte line per row)
 constexpr size_t PAIR_WINDOW_BYTES = (size_t)6 << 30;  // slots held at a time (longer lists run in windows)
 
@@ -101,6 +105,23 @@ __global__ void k_pair_batches(const uint32_t *bins, int nbins, uint32_t *nbatch
   if (b < nbins) nbatch[b] = (bins[b] + PAIR_C - 1) / PAIR_C;
 }
 
+// acc[j] += W(row, k) X(k, j) over kn operator columns for the first CN of a thread's columns
+template <int CN>
+__device__ __forceinline__ void pair_dot(double *acc, const double *w, int ld, const double *x, int kn) {
+#pragma unroll 4
+  for (int kk = 0; kk < kn; ++kk) {
+    const double wv = w[kk * ld];
+    const double2 xa = *(const double2 *)(x + kk * PAIR_C);
+    acc[0] = fma(wv, xa.x, acc[0]);
+    if (CN > 1) acc[1] = fma(wv, xa.y, acc[1]);
+    if (CN > 2) {
+      const double2 xc = *(const double2 *)(x + kk * PAIR_C + 2);
+      acc[2] = fma(wv, xc.x, acc[2]);
+      if (CN > 3) acc[3] = fma(wv, xc.y, acc[3]);
+    }
+  }
+}
+
 // One CTA per batch: 2 threads per real operator row, PAIR_C / 2 columns each.
 __global__ void k_pair_m2l(const PairJob *jobs, int njobs, int nbins, const uint32_t *bins, const uint32_t *bin_batch,
                            const uint32_t *d_nbatch, const PairEnt *list, const double *rot, int K, int p,
@@ -155,8 +176,8 @@ __global__ void k_pair_m2l(const PairJob *jobs, int njobs, int nbins, const uint
         vr = cs * v.x - sn * v.y;
         vi = sn * v.x + cs * v.y;
       }
-      X[k * PAIR_C + c] = vr;
-      if (iof[k] >= 0) X[(K + iof[k]) * PAIR_C + c] = vi;
+      X[k * PAIR_C + pair_pos(c)] = vr;
+      if (iof[k] >= 0) X[(K + iof[k]) * PAIR_C + pair_pos(c)] = vi;
     }
     const double *P = J.ops + (size_t)ct * 2 * K * K, *Q = P + (size_t)K * K;
     double acc[PAIR_C / 2];
@@ -176,16 +197,13 @@ __global__ void k_pair_m2l(const PairJob *jobs, int njobs, int nbins, const uint
       }
       __syncthreads();
       const int kn = min(PAIR_KC, (im ? KI : K) - k0);
-      if (r < R && (cg < nc)) {
-        const double *xb = X + (size_t)((im ? K : 0) + k0) * PAIR_C + cg;
-#pragma unroll 4
-        for (int kk = 0; kk < kn; ++kk) {
-          const double w = W[kk * LD + r];
-          const double2 xa = *(const double2 *)(xb + kk * PAIR_C), xc = *(const double2 *)(xb + kk * PAIR_C + 2);
-          acc[0] = fma(w, xa.x, acc[0]);
-          acc[1] = fma(w, xa.y, acc[1]);
-          acc[2] = fma(w, xc.x, acc[2]);
-          acc[3] = fma(w, xc.y, acc[3]);
+      if (r < R) {
+        const double *xb = X + (size_t)((im ? K : 0) + k0) * PAIR_C + cg, *wb = W + r;
+        switch ((nc + 1) >> 1) {  // columns of this thread (the last one empty for odd nc and the odd thread)
+          case 1: pair_dot<1>(acc, wb, LD, xb, kn); break;
+          case 2: pair_dot<2>(acc, wb, LD, xb, kn); break;
+          case 3: pair_dot<3>(acc, wb, LD, xb, kn); break;
+          default: pair_dot<4>(acc, wb, LD, xb, kn);
         }
       }
     }
@@ -200,7 +218,7 @@ __global__ void k_pair_m2l(const PairJob *jobs, int njobs, int nbins, const uint
       const PairEnt en = ent[c];
       const int m = cK.mof[k];
       const double cs = rot[((size_t)en.o * (PMAX + 1) + m) * 2], sn = rot[((size_t)en.o * (PMAX + 1) + m) * 2 + 1];
-      const double yr = X[k * PAIR_C + c], yi = iof[k] >= 0 ? X[(K + iof[k]) * PAIR_C + c] : 0.0;
+      const double yr = X[k * PAIR_C + pair_pos(c)], yi = iof[k] >= 0 ? X[(K + iof[k]) * PAIR_C + pair_pos(c)] : 0.0;
       Y[(size_t)en.e * K + k] = make_double2(cs * yr + sn * yi, cs * yi - sn * yr);
     }
   }
@@ -249,7 +267,7 @@ __global__ void k_pair_sum(const PairJob *jobs, int njobs, int64_t g0, const uin
 }
 
 // every FP64 translation of the jobs (free-space jobs first; t0, bin0 filled in here)
-static void launch_pair_m2l(Ctx &c, std::vector<PairJob> &jobs, const std::vector<int> &ncls, const double *rot) {
+static void launch_pair_m2l_part(Ctx &c, std::vector<PairJob> &jobs, const std::vector<int> &ncls, const double *rot) {
   int64_t ntot = 0, nfree = 0;
   int nbins = 0;
   for (size_t k = 0; k < jobs.size(); ++k) {
@@ -306,4 +324,37 @@ static void launch_pair_m2l(Ctx &c, std::vector<PairJob> &jobs, const std::vecto
       c.launches++;
     }
   }
+}
+
+// the jobs in parts of at most 2^32 - 1 translations (their numbers are 32-bit), whole targets each, in the jobs' order,
+// so that a target's free-space and reaction sums are added as in one part
+static void launch_pair_m2l(Ctx &c, const std::vector<PairJob> &jobs, const std::vector<int> &ncls, const double *rot) {
+  std::vector<PairJob> part;
+  std::vector<int> pcls;
+  uint64_t room = UINT32_MAX;
+  const Arena::Mark mark = c.arena.mark();  // a part follows the one before it in stream order, in its memory
+  for (size_t k = 0; k < jobs.size(); ++k) {
+    const PairJob &J = jobs[k];
+    const uint64_t per = (uint64_t)NOFF * J.ntypes;  // at most, per target
+    for (int32_t t = 0; t < J.ntb;) {
+      if (room < per) {
+        launch_pair_m2l_part(c, part, pcls, rot);
+        c.arena.rewind(mark);
+        part.clear();
+        pcls.clear();
+        room = UINT32_MAX;
+      }
+      const int32_t n = (int32_t)std::min<uint64_t>((uint64_t)(J.ntb - t), room / per);
+      PairJob p = J;
+      p.vlist += (size_t)t * NOFF;
+      if (p.ktrow) p.ktrow += t;
+      p.L += (size_t)t * c.K;
+      p.ntb = n;
+      part.push_back(p);
+      pcls.push_back(ncls[k]);
+      room -= per * (uint64_t)n;
+      t += n;
+    }
+  }
+  launch_pair_m2l_part(c, part, pcls, rot);
 }
