@@ -413,17 +413,17 @@ def run_ours(args, rank, world, local_rank):
         peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
     except Exception:
         pass
-    # FP32 / FP64: FMA chains timed on this device now (lpbfmm_measure_peak); TF32 tensor: the
-    # measured bf16 burst x the nominal TF32 / BF16 ratio 1.1 / 2.25; HBM: the measured copy
+    # FP32 / FP64: FMA chains timed on this device now (lpbfmm_measure_peak); FP16 tensor: the
+    # measured bf16 burst (the same nominal rate); HBM: the measured copy
     fp32_peak = F.measure_peak(F.PEAK_FP32_FMA)
     fp64_peak = F.measure_peak(F.PEAK_FP64_FMA)
     bf16 = peaks.get("bf16_tflops")
-    tf32_peak = (bf16 if bf16 else 1900.0) * 1.1 / 2.25
+    fp16_peak = bf16 if bf16 else 1900.0
     hbm_peak = peaks.get("hbm_gbs") or 6800.0
-    peak_info = {"fp32_fma_tflops": fp32_peak, "fp64_fma_tflops": fp64_peak, "tf32_tflops": tf32_peak,
+    peak_info = {"fp32_fma_tflops": fp32_peak, "fp64_fma_tflops": fp64_peak, "fp16_tflops": fp16_peak,
                  "hbm_gbs": hbm_peak, "sms": torch.cuda.get_device_properties(dev).multi_processor_count,
-                 "how": "fp32/fp64: measured FMA chains (lpbfmm_measure_peak); tf32: measured bf16 burst "
-                        "(MEASURED_PEAKS.json) x 1.1/2.25; hbm: measured copy (MEASURED_PEAKS.json)" +
+                 "how": "fp32/fp64: measured FMA chains (lpbfmm_measure_peak); fp16: measured bf16 burst "
+                        "(MEASURED_PEAKS.json); hbm: measured copy (MEASURED_PEAKS.json)" +
                         ("" if peaks.get("hbm_gbs") else " [fallback 6800 GB/s: file absent]")}
     per = lambda nm: phase_ms.get(nm, float("nan")) / args.steps
 
@@ -441,8 +441,8 @@ def run_ours(args, rank, world, local_rank):
                           24.0 * counts["p2p_pairs"], per("p2p"), fp32_peak, "24 per pair (+2 SFU)"))
     if "m2l_tc" in phase_ms:
         tr = counts["m2l_free"] + counts["m2l_react"]
-        roofs.append(roof("k_m2l_tc (free-space and reaction M2L, tcgen05 3xTF32)", "tensor", 2.0 * R * R * tr,
-                          per("m2l_tc"), tf32_peak,
+        roofs.append(roof("k_m2l_tc (free-space and reaction M2L, tcgen05, split FP16)", "tensor", 2.0 * R * R * tr,
+                          per("m2l_tc"), fp16_peak,
                           "2 R^2 = %d per translation (R = %d real coordinates)" % (2 * R * R, R)))
     if "m2l_simt" in phase_ms:
         roofs.append(roof("k_m2l_f32 (M2L, FP32 SIMT)", "alu", 4.0 * K * K * counts["m2l_react"], per("m2l_simt"),

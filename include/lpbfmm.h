@@ -56,7 +56,7 @@ extern "C" {
 
 /* precision modes */
 #define LPBFMM_FP64 0  /* every step in FP64                                                  */
-#define LPBFMM_MIXED 1 /* FP32 P2P, P2M/M2M/L2L/L2P; M2L on the tensor cores in 3xTF32 for
+#define LPBFMM_MIXED 1 /* FP32 P2P, P2M/M2M/L2L/L2P; M2L on the tensor cores in split FP16 for
                           p <= 10 (FP32 otherwise); FP64 tables, operators and final sums  */
 
 typedef struct lpbfmm_ctx *lpbfmm_t;
