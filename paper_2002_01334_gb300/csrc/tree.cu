@@ -839,6 +839,13 @@ __global__ void __launch_bounds__(LIST_THREADS) k_lists(const ListJob *jobs, int
   }
   // images lie across the interface: a box more than 2 ws layers from it has no image box in reach
   const bool none = ns <= 0 || (J.react && kt > 2 * ws);
+  // classes in use are gathered per block and written once where they are new: a global store per found source
+  // box kept every block's stores on the same few lines (139,000 leaf boxes of four layers: lists 0.93 -> 0.51 ms)
+  __shared__ uint8_t seen[NREACT_CLS];
+  if (react_far && !none) {
+    for (int e = threadIdx.x; e < NREACT_CLS; e += LIST_THREADS) seen[e] = 0;
+    __syncthreads();
+  }
   for (int o = threadIdx.x; o < nslot; o += LIST_THREADS) {
     int32_t res = -1;
     if (!none) {
@@ -862,12 +869,17 @@ __global__ void __launch_bounds__(LIST_THREADS) k_lists(const ListJob *jobs, int
           if (react_far) {
             const int ks = (a == 1) ? half - 1 - jz : jz - half;
             const int kk = kk_index(kt, ks);
-            if (kk >= 0) used[rho_index(dx, dy) * NKK + kk] = 1;
+            if (kk >= 0) seen[rho_index(dx, dy) * NKK + kk] = 1;
           }
         }
       }
     }
     out[o] = res;
+  }
+  if (react_far && !none) {
+    __syncthreads();
+    for (int e = threadIdx.x; e < NREACT_CLS; e += LIST_THREADS)
+      if (seen[e] && !used[e]) used[e] = 1;
   }
 }
 
