@@ -490,8 +490,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TJob *jobs, int 
 #pragma unroll
         for (int c1 = 0; c1 < NH; c1 += 16) {
           uint32_t v[16];
-          tc::tmem_ld16_nw(at + (uint32_t)c1, v);
-          tc::tmem_wait_ld();
+          tc::tmem_ld16(at + (uint32_t)c1, v);
 #pragma unroll
           for (int j = 0; j < 16; j += 2) {
             const int g = tc_segment(P, (c1 + j) / 2);
