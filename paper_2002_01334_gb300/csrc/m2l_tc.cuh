@@ -591,34 +591,42 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TJob *jobs, int 
       }
     }
   } else if (tid == TC_WORKERS) {
-    // the MMA thread: stage after stage, once the workers and the bulk copy have filled it; a step's first
-    // chunk waits until the workers have read the accumulator two steps back
+    // the MMA thread: a step's cross products (hi lo, lo hi) of every chunk as it is filled, by the workers and the bulk
+    // copy, then its hi hi ones; a step starts once the workers have read the accumulator two steps back
     constexpr uint32_t IDESC = tc::idesc_f16(TC_ROWS, N);
     int last = -1;
-    for (int sc = 0; sc < S; ++sc) {
-      const int b = sc % NST, si = sc / NC, kc = sc % NC;
-      if (!tc::mbar_wait(&full[b], (uint32_t)((sc / NST) & 1), TC_WAIT) ||
-          !tc::mbar_wait(&wfull[b], (uint32_t)((sc / NST) & 1), TC_WAIT)) {
+    for (int si = 0; si < ns && !fail; ++si) {
+      if (si >= 2 && !tc::mbar_wait(&foldbar[si & 1], (uint32_t)(((si - 2) >> 1) & 1), TC_WAIT)) {
         fail = true;
         break;
       }
-      if (kc == 0 && si >= 2 && !tc::mbar_wait(&foldbar[si & 1], (uint32_t)(((si - 2) >> 1) & 1), TC_WAIT)) {
-        fail = true;
-        break;
-      }
-      tc::fence_after();
-      const uint32_t ah = tc::smem_u32(sbase + (size_t)b * tc_stage_bytes(NC)), wh = ah + SA;
       const uint32_t dacc = tmem + (uint32_t)((si & 1) * N);
+      for (int kc = 0; kc < NC; ++kc) {
+        const int sc = si * NC + kc, b = sc % NST;
+        if (!tc::mbar_wait(&full[b], (uint32_t)((sc / NST) & 1), TC_WAIT) ||
+            !tc::mbar_wait(&wfull[b], (uint32_t)((sc / NST) & 1), TC_WAIT)) {
+          fail = true;
+          break;
+        }
+        tc::fence_after();
+        const uint32_t ah = tc::smem_u32(sbase + (size_t)b * tc_stage_bytes(NC)), wh = ah + SA;
 #pragma unroll
-      for (int kk = 0; kk < 2; ++kk) {  // 16 columns: 32 bytes of hi, their lo 64 bytes on
-        const uint32_t o = kk * 32;
-        tc::mma_f16(dacc, tc::sdesc(ah + o), tc::sdesc(wh + o), IDESC, (kc | kk) ? 1u : 0u);
-        tc::mma_f16(dacc, tc::sdesc(ah + o), tc::sdesc(wh + 64 + o), IDESC, 1u);
-        tc::mma_f16(dacc, tc::sdesc(ah + 64 + o), tc::sdesc(wh + o), IDESC, 1u);
+        for (int kk = 0; kk < 2; ++kk) {  // 16 columns: 32 bytes of hi, their lo 64 bytes on
+          const uint32_t o = kk * 32;
+          tc::mma_f16(dacc, tc::sdesc(ah + o), tc::sdesc(wh + 64 + o), IDESC, (kc | kk) ? 1u : 0u);
+          tc::mma_f16(dacc, tc::sdesc(ah + 64 + o), tc::sdesc(wh + o), IDESC, 1u);
+        }
       }
-      tc::commit(&empty[b]);
-      if (kc == NC - 1) tc::commit(&accbar[si & 1]);
-      last = sc;
+      if (fail) break;
+      for (int kc = 0; kc < NC; ++kc) {
+        const int sc = si * NC + kc, b = sc % NST;
+        const uint32_t ah = tc::smem_u32(sbase + (size_t)b * tc_stage_bytes(NC)), wh = ah + SA;
+#pragma unroll
+        for (int kk = 0; kk < 2; ++kk) tc::mma_f16(dacc, tc::sdesc(ah + kk * 32), tc::sdesc(wh + kk * 32), IDESC, 1u);
+        tc::commit(&empty[b]);
+        last = sc;
+      }
+      tc::commit(&accbar[si & 1]);
     }
     // every MMA has completed once the last committed stage's barrier phase completes
     if (last >= 0) tc::mbar_wait(&empty[last % NST], (uint32_t)((last / NST) & 1), TC_WAIT);
