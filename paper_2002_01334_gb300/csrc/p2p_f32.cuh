@@ -3,7 +3,7 @@
 // Every point of the target tree carries its offset from its own leaf centre as FP32 hi + lo pairs
 // (k_split_points, once per evaluation, one array per component).  A source of a near leaf whose centre lies
 // delta * h away is moved into the target leaf's frame by an exact FP32 two-sum with h = hh + hl.  Sources are staged
-// with cp.async, one chunk ahead of the one being summed.  Per-chunk sums are folded into
+// with cp.async, one chunk ahead of the one being summed.  Sums over 64 sources are folded into
 // Kahan-compensated FP32 totals; no FP64 in the pair loop.
 //
 // Bound: the FP32 pipes.  A pair is 17 FP32 operations (10 without the field) and two special-function
@@ -75,6 +75,12 @@ __device__ __forceinline__ float rsqrt_approx(float x) {
 }
 
 constexpr int P2P_WARPS = 4, P2P_CH = 128, P2P_GROUP = 64;  // warps per leaf, sources per chunk, targets per group
+// Sources between two folds into the compensated totals.  A lane adds P2P_FOLD / 2 of them to a running FP32 sum (fewer where
+// several lanes share a target), whose rounding grows with that number: a fold per chunk of 128, which may span
+// leaves, left sums of small leaves 12 % further from FP64 than a fold per leaf (four layers, N = 10,000, strong screening:
+// 1.55e-7 against 1.38e-7), a fold per 64 gives 1.17e-7.  Its cost, 40 of some 1,400 instructions, is 0.3 % of the kernel (N = 1M,
+// beside the far field, 11.65 -> 11.66 ms; N = 2.86M 32.29 -> 32.52).
+constexpr int P2P_FOLD = 64;
 constexpr float P2P_FAR = 1e18f;  // x of the records that fill a chunk up to fours (charge 0)
 
 // e^{-lambda r} = 2^{(-lambda log2 e) r}; field factor (1 + lambda r) / r^2 = (1/r)(1/r + lambda).
@@ -233,10 +239,7 @@ __device__ __forceinline__ void p2p_warp_pass(const P2PJob &J, int lane, uint32_
       }
     }
     __syncwarp();
-    float2 ap[2], ax[2], ay[2], az[2], pl[2][3];
-#pragma unroll
-    for (int t = 0; t < 2; ++t) ap[t] = ax[t] = ay[t] = az[t] = make_float2(0.f, 0.f);
-    const int nq = (nn + 3) >> 2;
+    float2 pl[2][3];
     if (near) {
 #pragma unroll
       for (int t = 0; t < 2; ++t)
@@ -245,17 +248,24 @@ __device__ __forceinline__ void p2p_warp_pass(const P2PJob &J, int lane, uint32_
           const float l = -pts[(4 + d) * ld + first + min(tl + (t << lg), nt - 1)];
           pl[t][d] = make_float2(l, l);
         }
-      p2p_f32_chunk<FIELD, true>(buf[b], nq, sub, nsub, ph, pl, nl2, lam, ap, ax, ay, az);
-    } else {
-      p2p_f32_chunk<FIELD, false>(buf[b], nq, sub, nsub, ph, pl, nl2, lam, ap, ax, ay, az);
     }
+    const int nq = (nn + 3) >> 2, step = max(P2P_FOLD / 4, nsub);  // at least a quad per lane
+#pragma unroll 1
+    for (int j0 = 0; j0 < nq; j0 += step) {
+      float2 ap[2], ax[2], ay[2], az[2];
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      kahan_add(tot[t][0], cmp[t][0], ap[t].x + ap[t].y);
-      if (FIELD) {
-        kahan_add(tot[t][1], cmp[t][1], ax[t].x + ax[t].y);
-        kahan_add(tot[t][2], cmp[t][2], ay[t].x + ay[t].y);
-        kahan_add(tot[t][3], cmp[t][3], az[t].x + az[t].y);
+      for (int t = 0; t < 2; ++t) ap[t] = ax[t] = ay[t] = az[t] = make_float2(0.f, 0.f);
+      const int j1 = min(nq, j0 + step);
+      if (near) p2p_f32_chunk<FIELD, true>(buf[b], j1, j0 + sub, nsub, ph, pl, nl2, lam, ap, ax, ay, az);
+      else p2p_f32_chunk<FIELD, false>(buf[b], j1, j0 + sub, nsub, ph, pl, nl2, lam, ap, ax, ay, az);
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        kahan_add(tot[t][0], cmp[t][0], ap[t].x + ap[t].y);
+        if (FIELD) {
+          kahan_add(tot[t][1], cmp[t][1], ax[t].x + ax[t].y);
+          kahan_add(tot[t][2], cmp[t][2], ay[t].x + ay[t].y);
+          kahan_add(tot[t][3], cmp[t][3], az[t].x + az[t].y);
+        }
       }
     }
     __syncwarp();  // buffer b is refilled by the next issue

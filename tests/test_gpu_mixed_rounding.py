@@ -45,3 +45,13 @@ def test_tensor_core_m2l(layout, n, p, phi, fld):
     e = rounding(layout, n, p, 2 + 4, 1.0)
     assert e[0] <= phi * 1.05 and e[1] <= fld * 1.05, e
 
+
+
+@pytest.mark.parametrize("layout,n,phi", [("four_layer", 10000, 1.382e-7), ("three_layer", 3000, 1.451e-7),
+                                          ("three_layer", 30000, 1.145e-7)])
+def test_fp32_near_field_sums(layout, n, phi):
+    """The free-space part under screening that leaves little but the near field, in leaves of some tens to a hundred
+    charges, no further off than sums folded into the compensated totals leaf by leaf on the same inputs; 5 % for the
+    mean's own spread."""
+    e = rounding(layout, n, 5, 1, 60.0)
+    assert e[0] <= phi * 1.05, e
