@@ -271,6 +271,15 @@ int lpbfmm_debug_array(lpbfmm_t h, int l, int a, const char *name, int lev, void
                        int64_t *bytes);
 
 /*
+ * Diagnostics: limits for this context's later evaluations, so that tests reach on small inputs what large ones need.
+ * window: bytes of translated expansions that the FP64 multipole-to-local holds at a time (default 2 GB; halved as
+ * often as device memory asks for); part: translations it numbers at a time (default 2^32 - 1; at least one target's longest
+ * list); memory: device bytes that the context's work space may hold, beyond which an evaluation returns
+ * LPBFMM_ERR_OOM as if the device had no more (default: no limit).  0 restores a default.
+ */
+int lpbfmm_debug_limits(lpbfmm_t h, int64_t window, int64_t part, int64_t memory);
+
+/*
  * Work counts of the last lpbfmm_eval (host int64 out[8]): [0] free-space multipole-to-local
  * translations, [1] reaction translations (box pairs x source types), [2] free-space P2P pairs
  * (including the excluded self pairs), [3] reaction near-field pairs, [4] targets summed over

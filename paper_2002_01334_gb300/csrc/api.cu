@@ -19,22 +19,31 @@ void init_fmm_tables(Ctx &c);
 // ---------------------------------------------------------------------------------------
 void *Arena::alloc(size_t bytes) {
   bytes = (bytes + 255) & ~size_t(255);
-  used_total += bytes;
-  peak = std::max(peak, used_total);
+  void *p = nullptr;
   for (auto &ch : chunks)
     if (ch.size - ch.used >= bytes) {
-      void *p = ch.p + ch.used;
+      p = ch.p + ch.used;
       ch.used += bytes;
-      return p;
+      break;
     }
-  size_t sz = std::max(bytes, std::max(want, (size_t)64 << 20));
-  char *p = nullptr;
-  cudaError_t e = cudaMalloc(&p, sz);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    throw StatusError{LPBFMM_ERR_OOM};
+  if (!p) {
+    // the merged chunk of an earlier, larger evaluation may not fit any more where this piece alone does
+    auto grow = [&](size_t sz) {
+      if (sz > limit || held > limit - sz) return false;
+      if (cudaMalloc(&p, sz) == cudaSuccess) {
+        held += sz;
+        chunks.push_back(Chunk{(char *)p, sz, bytes});
+        return true;
+      }
+      cudaGetLastError();
+      p = nullptr;
+      return false;
+    };
+    const size_t chunk = std::max(bytes, (size_t)64 << 20);
+    if (!(want > chunk && grow(want)) && !grow(chunk) && !grow(bytes)) throw StatusError{LPBFMM_ERR_OOM};
   }
-  chunks.push_back(Chunk{p, sz, bytes});
+  used_total += bytes;
+  peak = std::max(peak, used_total);
   return p;
 }
 void Arena::reset() {
@@ -48,6 +57,7 @@ void Arena::reset() {
 void Arena::release() {
   for (auto &ch : chunks) cudaFree(ch.p);
   chunks.clear();
+  held = 0;
 }
 
 void prof_mark(Ctx &c, const char *name) {
@@ -1047,6 +1057,17 @@ int lpbfmm_debug_array(lpbfmm_t h, int l, int a, const char *name, int lev, void
   if ((int64_t)nb > cap) return LPBFMM_ERR_ARG;
   if (cudaStreamSynchronize(h->stream) != cudaSuccess) return LPBFMM_ERR_CUDA;
   if (cudaMemcpy(dst, src, nb, cudaMemcpyDeviceToHost) != cudaSuccess) return LPBFMM_ERR_CUDA;
+  return LPBFMM_OK;
+}
+
+int lpbfmm_debug_limits(lpbfmm_t h, int64_t window, int64_t part, int64_t memory) {
+  if (!h || window < 0 || part < 0 || memory < 0) return LPBFMM_ERR_ARG;
+  // a part takes whole targets, so it holds at least one target's longest list
+  h->pair_window = window ? (size_t)window : PAIR_WINDOW_BYTES;
+  h->pair_part = part ? std::min<uint64_t>(std::max<uint64_t>((uint64_t)part, (uint64_t)NOFF * 2 * (MAXLAYER - 1)),
+                                           PAIR_PART_MAX)
+                      : PAIR_PART_MAX;
+  h->arena.limit = memory ? (size_t)memory : SIZE_MAX;
   return LPBFMM_OK;
 }
 

@@ -129,7 +129,8 @@ struct Arena {
     size_t size, used;
   };
   std::vector<Chunk> chunks;
-  size_t want = 0, used_total = 0, peak = 0;
+  size_t want = 0, used_total = 0, peak = 0, held = 0;
+  size_t limit = SIZE_MAX;  // device bytes the chunks may hold (lpbfmm_debug_limits)
   // a point to go back to: what was allocated since may be overwritten by work that follows, in stream
   // order, the work that used it
   struct Mark {
@@ -275,8 +276,17 @@ struct Deferred {
   }
 };
 
+// FP64 multipole-to-local: bytes of translation slots a context holds at a time (longer lists run in windows, which are
+// halved where memory is short), and translations numbered at a time (their numbers are 32-bit).  A window costs two
+// walks over its targets' lists and a partial batch per operator: N = 100,000, p = 10 in one window 85.5 ms, 1 GB 86.7,
+// 256 MB 88.6, 64 MB 96.6; 2,003 charges, p = 12, adjoint 50.5 in one (0.9 GB), 52.8 at 256 MB, 59.9 at 64 MB.
+constexpr size_t PAIR_WINDOW_BYTES = (size_t)2 << 30;
+constexpr uint64_t PAIR_PART_MAX = UINT32_MAX;
+
 struct Ctx {
   Medium md;
+  size_t pair_window = PAIR_WINDOW_BYTES;
+  uint64_t pair_part = PAIR_PART_MAX;
   int p = 10, K = 66;
   int ws = 2;  // separation of the interaction lists (boxes)
   double tol = 1e-14;

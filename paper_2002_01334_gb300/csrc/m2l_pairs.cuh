@@ -21,8 +21,8 @@
 // so 49.5; N = 100,000 p = 10 87.7 -> 86.0).
 constexpr int PAIR_C = 8;
 __device__ __forceinline__ int pair_pos(int c) { return (c & 1) * (PAIR_C / 2) + (c >> 1); }
+constexpr uint64_t PAIR_WINDOW_MIN = 4096;  // translations below which a window is not halved for want of memory
 constexpr int PAIR_KC = 16;  // operator columns staged at a time (16 doubles = one 128-byte line per row)
-constexpr size_t PAIR_WINDOW_BYTES = (size_t)6 << 30;  // slots held at a time (longer lists run in windows)
 
 struct PairJob {
   const int32_t *vlist;      // [ntb][NOFF] source box or -1
@@ -64,9 +64,10 @@ __global__ void k_pair_walk(const PairJob *jobs, int njobs, int64_t ntot, uint32
   const int64_t g = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (g >= ntot) return;
   const int lane = threadIdx.x & 31;
+  uint32_t e = MODE ? e0[g] : 0u, total = 0;
+  if (MODE && (e >= w1 || e + cnt[g] <= w0)) return;  // no translation of this target in the window
   const PairJob &J = jobs[pair_find_job(jobs, njobs, g)];
   const int64_t t = g - J.t0;
-  uint32_t e = MODE ? e0[g] : 0u, total = 0;
   if (!J.ktrow || (J.ktrow[t] >= 0 && J.ktrow[t] < J.nkt)) {
     for (int o0 = 0; o0 < NOFF; o0 += 32) {
       const int o = o0 + lane;
@@ -293,11 +294,21 @@ static void launch_pair_m2l_part(Ctx &c, std::vector<PairJob> &jobs, const std::
   LPB_CUDA(cudaStreamSynchronize(c.stream));
   const uint64_t total = h[0];
   if (!total) return;
-  const uint64_t win = std::min<uint64_t>(total, std::max<uint64_t>(PAIR_WINDOW_BYTES / (sizeof(double2) * K), 1));
-  double2 *Y = c.arena.get<double2>((size_t)win * K);
-  PairEnt *list = c.arena.get<PairEnt>((size_t)win + (size_t)nbins * PAIR_C);
   uint32_t *bins = c.arena.get<uint32_t>(nbins), *nbt = c.arena.get<uint32_t>(nbins),
            *bb = c.arena.get<uint32_t>(nbins), *cur = c.arena.get<uint32_t>(nbins);
+  uint64_t win = std::min<uint64_t>(total, std::max<uint64_t>(c.pair_window / (sizeof(double2) * K), 1));
+  double2 *Y = nullptr;
+  PairEnt *list = nullptr;
+  for (const Arena::Mark mark = c.arena.mark(); !list;) {  // smaller windows where memory is short
+    try {
+      Y = c.arena.get<double2>((size_t)win * K);
+      list = c.arena.get<PairEnt>((size_t)win + (size_t)nbins * PAIR_C);
+    } catch (const StatusError &) {
+      if (win <= PAIR_WINDOW_MIN) throw;
+      c.arena.rewind(mark);
+      win = (win + 1) / 2;
+    }
+  }
   const int R = 2 * K - (c.p + 1), threads = (2 * R + 31) / 32 * 32;
   LPB_ATTR_ONCE(k_pair_m2l, pair_smem(KHALF_MAX, PMAX));
   for (uint64_t w0 = 0; w0 < total; w0 += win) {
@@ -326,12 +337,12 @@ static void launch_pair_m2l_part(Ctx &c, std::vector<PairJob> &jobs, const std::
   }
 }
 
-// the jobs in parts of at most 2^32 - 1 translations (their numbers are 32-bit), whole targets each, in the jobs' order,
+// the jobs in parts of at most pair_part translations (their numbers are 32-bit), whole targets each, in the jobs' order,
 // so that a target's free-space and reaction sums are added as in one part
 static void launch_pair_m2l(Ctx &c, const std::vector<PairJob> &jobs, const std::vector<int> &ncls, const double *rot) {
   std::vector<PairJob> part;
   std::vector<int> pcls;
-  uint64_t room = UINT32_MAX;
+  uint64_t room = c.pair_part;
   const Arena::Mark mark = c.arena.mark();  // a part follows the one before it in stream order, in its memory
   for (size_t k = 0; k < jobs.size(); ++k) {
     const PairJob &J = jobs[k];
@@ -342,7 +353,7 @@ static void launch_pair_m2l(Ctx &c, const std::vector<PairJob> &jobs, const std:
         c.arena.rewind(mark);
         part.clear();
         pcls.clear();
-        room = UINT32_MAX;
+        room = c.pair_part;
       }
       const int32_t n = (int32_t)std::min<uint64_t>((uint64_t)(J.ntb - t), room / per);
       PairJob p = J;
@@ -357,4 +368,5 @@ static void launch_pair_m2l(Ctx &c, const std::vector<PairJob> &jobs, const std:
     }
   }
   launch_pair_m2l_part(c, part, pcls, rot);
+  c.arena.rewind(mark);  // what follows on this stream may take the slots' memory
 }

@@ -59,6 +59,7 @@ def lib():
         L.lpbfmm_stable_noalloc.argtypes = [vp, C.c_int, C.c_int, C.c_int, C.c_int, C.c_double, C.c_double,
                                             C.c_double, C.c_double, C.c_int, vp]
         L.lpbfmm_debug_array.argtypes = [vp, C.c_int, C.c_int, C.c_char_p, C.c_int, vp, i64, C.POINTER(i64)]
+        L.lpbfmm_debug_limits.argtypes = [vp, i64, i64, i64]
         L.lpbfmm_last_counts.argtypes = [vp, C.POINTER(i64)]
         L.lpbfmm_status.argtypes = [vp]
         L.lpbfmm_strerror.argtypes = [C.c_int]
@@ -232,6 +233,10 @@ class Context:
         _check(lib().lpbfmm_debug_array(self.h, l, a, name.encode(), lev, C.c_void_p(out.ctypes.data), nb.value,
                                         C.byref(nb)), "debug_array")
         return out.view(dtype)
+
+    def debug_limits(self, window=0, part=0, memory=0):
+        """Limits of later evaluations (lpbfmm_debug_limits); 0 restores a default."""
+        _check(lib().lpbfmm_debug_limits(self.h, int(window), int(part), int(memory)), "lpbfmm_debug_limits")
 
     def debug_stable(self, l, a, lp, b, h, rho, zt, zs, Kmax):
         import numpy as np
