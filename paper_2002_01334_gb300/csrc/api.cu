@@ -443,10 +443,24 @@ static void eval_back(Ctx &c, double *phi, double *field) {
   run_fmm_back(c, c.groups, phi, field);
   prof_mark(c, "end");
 }
+// f(); where it throws, the context's stream is ordered after the work already issued on its other streams: they write the
+// caller's outputs and the work space, both of which the caller may reuse once the error is returned
+template <typename F>
+static void settled(Ctx &c, F &&f) {
+  try {
+    f();
+  } catch (...) {
+    for (cudaStream_t s : {c.side, c.far, c.near})
+      if (cudaEventRecord(c.ev_gfork, s) == cudaSuccess) cudaStreamWaitEvent(c.stream, c.ev_gfork, 0);
+    throw;
+  }
+}
 static void eval_impl(Ctx &c, int64_t n, const double *q, const double *xyz, const int32_t *layer, int parts,
                       const int32_t *gmask, double *phi, double *field) {
-  eval_front(c, n, q, nullptr, xyz, layer, parts, gmask, phi, field);
-  eval_back(c, phi, field);
+  settled(c, [&] {
+    eval_front(c, n, q, nullptr, xyz, layer, parts, gmask, phi, field);
+    eval_back(c, phi, field);
+  });
 }
 // another charge vector on the positions, trees, lists and operators of the evaluation just issued: its passes
 // take the memory of that evaluation's, which they follow in stream order (every side stream has been
@@ -649,9 +663,11 @@ int lpbfmm_adjoint(lpbfmm_t h, int64_t n, const double *q, const double *xyz, co
   int rc = LPBFMM_OK;
   try {
     // one set of trees, lists, tables and operators for both charge vectors
-    eval_front(*h, n, g_phi, q, xyz, layer_id, 3, nullptr, g_q, fg);
-    eval_back(*h, g_q, fg);
-    eval_again(*h, n, q, pq, fq);
+    settled(*h, [&] {
+      eval_front(*h, n, g_phi, q, xyz, layer_id, 3, nullptr, g_q, fg);
+      eval_back(*h, g_q, fg);
+      eval_again(*h, n, q, pq, fq);
+    });
   } catch (const CudaError &e) {
     rc = map_error(e);
   } catch (const StatusError &e) {
@@ -773,7 +789,9 @@ int lpbfmm_eval_batched(int nsys, const lpbfmm_t *ctxs, const int64_t *offsets, 
       const int64_t o = offsets[s], n = offsets[s + 1] - offsets[s];
       ctx->def.on = true;
       const int rc = guarded([&] {
-        eval_front(*ctx, n, q + o, nullptr, xyz + 3 * o, layer_id + o, 3, nullptr, phi + o, field ? field + 3 * o : nullptr);
+        settled(*ctx, [&] {
+          eval_front(*ctx, n, q + o, nullptr, xyz + 3 * o, layer_id + o, 3, nullptr, phi + o, field ? field + 3 * o : nullptr);
+        });
       });
       if (rc) {
         ctx->def.on = false;

@@ -71,3 +71,32 @@ def test_short_memory_halves_the_windows():
         b, fb = ctx.eval(*args, parts=3 + 4)
         assert ctx.counts()["launches"] > n["launches"]
         assert rel(b, a) < 1e-13 and rel(fb, fa) < 1e-13, (rel(b, a), rel(fb, fa))
+
+
+@pytest.mark.parametrize("prec", [F.FP64, F.MIXED])
+def test_nothing_runs_on_after_an_error(prec):
+    """Out of memory at every stage that a growing limit reaches: once the error is returned, the outputs are the caller's
+    again (no kernel of another stream adds into them later), and the context goes on to give the same results."""
+    ctx, args = problem("three_layer", 100000, 5, 0, prec)
+    a, fa = ctx.eval(*args)
+    ctx.close()
+    phi, fld = torch.empty_like(a), torch.empty_like(fa)
+    seen = 0
+    for mb in range(64, 100 * 64, 64):
+        ctx, args = problem("three_layer", 100000, 5, 0, prec)
+        ctx.debug_limits(memory=mb << 20)
+        try:
+            ctx.eval(*args, out=(phi, fld))
+            break
+        except F.LpbfmmError as e:
+            assert e.code == 7
+        seen += 1
+        phi.fill_(3.0)
+        fld.fill_(4.0)
+        torch.cuda.synchronize()
+        assert bool((phi == 3.0).all()) and bool((fld == 4.0).all()), mb
+        ctx.debug_limits()
+        b, fb = ctx.eval(*args)
+        assert rel(b, a) < 1e-13 and rel(fb, fa) < 1e-13 and ctx.status() == 0
+        ctx.close()
+    assert seen >= 2
