@@ -1262,7 +1262,8 @@ static void m2l_all_f32(Ctx &c, std::vector<Group> &groups) {
       it += m2l_tiles(j, F32_TT) * M2L_NSLICE;
     }
     const size_t smem = m2l_f32_smem(c.K);
-    LPB_ATTR_ONCE(k_m2l_f32, m2l_f32_smem(F32_KR));  // the largest K of this kernel
+    // the largest K of this kernel, p = 11; the K = 80 that its rows are padded to would ask for more than a block has
+    LPB_ATTR_ONCE(k_m2l_f32, m2l_f32_smem(12 * 13 / 2));
     XJob *dj = c.arena.get<XJob>(jobs.size());
     LPB_CUDA(cudaMemcpyAsync(dj, jobs.data(), sizeof(XJob) * jobs.size(), cudaMemcpyHostToDevice, c.stream));
     k_m2l_f32<<<(unsigned)it, 256, smem, c.stream>>>(dj, (int)jobs.size(), (const float *)tb.rot, c.K);
