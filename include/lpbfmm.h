@@ -264,7 +264,9 @@ int lpbfmm_stable_noalloc(lpbfmm_t h, int l, int a, int lp, int b, double hbox, 
  * level lev into the host buffer dst (capacity cap bytes); *bytes receives its size.  Names:
  * "Mimg", "Mfree", "Lt" (expansions, complex, working precision), "op_react", "op_free"
  * (translation operators), "stab" (FP64 Sommerfeld tables), "used" (uint8 reaction classes in
- * use), "vreact" (int32 far list), "ikeys", "tkeys" (uint64 box keys), "rows", "nrows".
+ * use), "vreact" (int32 far list), "ikeys", "tkeys" (uint64 box keys), "rows", "nrows".  "Mimg" is 0 for the
+ * source types without charges in a box, "stab" for classes not in use and for entries other than K - d odd, d < K;
+ * operators of classes not in use are undefined.
  * With dst == NULL only *bytes is set.
  */
 int lpbfmm_debug_array(lpbfmm_t h, int l, int a, const char *name, int lev, void *dst, int64_t cap,

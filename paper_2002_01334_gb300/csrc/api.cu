@@ -1075,6 +1075,26 @@ int lpbfmm_debug_array(lpbfmm_t h, int l, int a, const char *name, int lev, void
   if ((int64_t)nb > cap) return LPBFMM_ERR_ARG;
   if (cudaStreamSynchronize(h->stream) != cudaSuccess) return LPBFMM_ERR_CUDA;
   if (cudaMemcpy(dst, src, nb, cudaMemcpyDeviceToHost) != cudaSuccess) return LPBFMM_ERR_CUDA;
+  // what the evaluation neither writes nor reads, as zero
+  if (nm == "Mimg" && g->tmask[lev]) {
+    std::vector<uint32_t> mask(nib);
+    if (cudaMemcpy(mask.data(), g->tmask[lev], sizeof(uint32_t) * nib, cudaMemcpyDeviceToHost) != cudaSuccess)
+      return LPBFMM_ERR_CUDA;
+    const size_t row = (size_t)h->K * 2 * es;
+    for (int64_t b = 0; b < nib; ++b)
+      for (int t = 0; t < g->ntypes; ++t)
+        if (!((mask[b] >> t) & 1u)) std::memset((char *)dst + ((size_t)b * g->ntypes + t) * row, 0, row);
+  } else if (nm == "stab") {
+    uint8_t used[NREACT_CLS] = {};
+    if (g->used[lev] && cudaMemcpy(used, g->used[lev], NREACT_CLS, cudaMemcpyDeviceToHost) != cudaSuccess)
+      return LPBFMM_ERR_CUDA;
+    double *S = (double *)dst;
+    for (int cls = 0; cls < NREACT_CLS; ++cls)
+      for (int t = 0; t < g->ntypes; ++t)
+        for (int K = 0; K <= KT; ++K)
+          for (int d = 0; d <= KT; ++d, S += 4)
+            if (!used[cls] || d > K || !((K - d) & 1)) S[0] = S[1] = S[2] = S[3] = 0.0;
+  }
   return LPBFMM_OK;
 }
 
