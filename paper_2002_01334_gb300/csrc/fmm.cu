@@ -543,7 +543,9 @@ __device__ __forceinline__ double fexp(double x) { return exp(x); }
 // Bound: the FP64 pipe (half an FMA per clock and SM quarter), so the kernel minimises FP64
 // operations per pair and idle lanes and leaves everything else to the other pipes:
 //  * 28 FP64 operations per pair (21 without the field): 1/r from the special-function unit's
-//    approximation by one third-order step (5 operations), e^{-lambda r} by the table method (Tang,
+//    approximation y by one third-order step (5 operations): with e = 1 - x y^2, x^{-1/2} = y (1 - e)^{-1/2} =
+//    y (1 + e/2 + 3 e^2/8 + ...), the binomial series to second order, whose next term 5 e^3/16 is below 2^-58 for an
+//    approximation good to 2^-20; e^{-lambda r} by the table method (Tang,
 //    ACM TOMS 15, 1989: 2^(n/2048) from a table, a cubic for the remainder below 2^-12; 7 operations).
 //    The library's rsqrt and exp take about 45 in all.
 //  * no idle lanes in a leaf's last, partial group of targets: a group of 2^b targets gives each of

@@ -91,3 +91,24 @@ def test_near_field_of_exactly_n_targets_in_a_leaf(n, prec, tol):
     assert np.linalg.norm(fld[s] - ref_f[s]) <= tol * np.linalg.norm(ref_f[s])
     only, _ = ctx.eval(*a, parts=1, field=False)
     assert np.array_equal(only.cpu().numpy()[s], phi[s])
+
+
+def test_fp64_inverse_distance_over_many_binades():
+    """One charge and targets at distances 2^-500 to 0.5 on a line through it (a tenth of a binade apart), screening too weak to
+    count: phi is q / (4 pi eps r).  Roundings of the FP64 pair: r^2, 1/r (one step), r, the exponential's table and polynomial, two
+    products, the scale and two sums, at most 2^-53 each and 2^-52 for 1/r and the exponential: 12 * 2^-53; the field
+    along the line has two more 1/r and two products: 18 * 2^-53, where the 1 / r^3 in it is a finite number."""
+    k = np.arange(5001)
+    r = np.exp2(-k / 10.0 - 1.0)
+    x = np.column_stack([np.concatenate([[0.0], r]), np.zeros(len(r) + 1), np.full(len(r) + 1, -0.6)])
+    q = np.zeros(len(x))
+    q[0] = 1.0
+    eps, lam = 2.0, 1e-18
+    ctx = F.Context([0.0, -1.2], [1.0, eps, 5.0], [0.5, lam, 0.8], 4, uniform_depth=2)
+    phi, fld = (t.cpu().numpy()[1:] for t in ctx.eval(*dev(q, x, np.ones(len(x), np.int32)), parts=1))
+    L = np.longdouble
+    ref = 1 / (4 * L("3.14159265358979323846264338327950288") * L(eps) * r.astype(L))
+    assert np.all(np.abs(phi - ref) <= 12 * 2.0 ** -53 * ref)
+    fr = ref / r.astype(L)
+    ok = r > 1e-100
+    assert ok.sum() > 3300 and np.all(np.abs(fld[ok, 0] - fr[ok]) <= 18 * 2.0 ** -53 * fr[ok])
