@@ -274,7 +274,7 @@ int lpbfmm_debug_array(lpbfmm_t h, int l, int a, const char *name, int lev, void
 
 /*
  * Diagnostics: limits for this context's later evaluations, so that tests reach on small inputs what large ones need.
- * window: bytes of translated expansions that the FP64 multipole-to-local holds at a time (default 2 GB; halved as
+ * window: bytes of translated expansions that the FP64 multipole-to-local holds at a time (default 3 GB; halved as
  * often as device memory asks for); part: translations it numbers at a time (default 2^32 - 1; at least one target's longest
  * list); memory: device bytes that the context's work space may hold, beyond which an evaluation returns
  * LPBFMM_ERR_OOM as if the device had no more (default: no limit).  0 restores a default.

@@ -278,9 +278,9 @@ struct Deferred {
 
 // FP64 multipole-to-local: bytes of translation slots a context holds at a time (longer lists run in windows, which are
 // halved where memory is short), and translations numbered at a time (their numbers are 32-bit).  A window costs two
-// walks over its targets' lists and a partial batch per operator: N = 100,000, p = 10 in one window 85.5 ms, 1 GB 86.7,
-// 256 MB 88.6, 64 MB 96.6; 2,003 charges, p = 12, adjoint 50.5 in one (0.9 GB), 52.8 at 256 MB, 59.9 at 64 MB.
-constexpr size_t PAIR_WINDOW_BYTES = (size_t)2 << 30;
+// walks over its targets' lists and a partial batch per operator: N = 100,000, p = 10 in one window (2.6 GB) 85.5 ms, 2 GB
+// 86.3, 256 MB 88.6, 64 MB 96.6; 2,003 charges, p = 12, adjoint 50.5 in one (0.9 GB), 52.8 at 256 MB, 59.9 at 64 MB.
+constexpr size_t PAIR_WINDOW_BYTES = (size_t)3 << 30;
 constexpr uint64_t PAIR_PART_MAX = UINT32_MAX;
 
 struct Ctx {
