@@ -6,10 +6,14 @@
 // with cp.async, one chunk ahead of the one being summed.  Sums over 64 sources are folded into
 // Kahan-compensated FP32 totals; no FP64 in the pair loop.
 //
-// Bound: the FP32 pipes.  A pair is 17 FP32 operations (10 without the field) and two special-function
+// A pair is 17 FP32 operations (10 without the field; 23 and 16 for leaves that touch) and two special-function
 // operations (12 clocks of that unit per warp).  Two sources ride in one 64-bit register pair
 // (add / mul / fma.f32x2: two lanes' worth of FP32 per issue slot), so that the 17 operations no longer fill the
-// issue slots and the special functions, loads and loop run beside them.  The sources are packed, not
+// issue slots and the special functions, loads and loop run beside them.  Bound: latency ahead of any pipe.  N = 100,000, p = 10
+// with the field: FP32 pipe busy 60 % of the active cycles (a packed operation takes two), special functions 24 %, an
+// instruction issued in 49 % of the slots; warps wait for their own operations (1.8 cycles per issue), the block's barrier
+// (1.4) and the FP32 pipe (1.0), because 127 registers leave 16 warps an SM.  Without the field 53 %, 33 % and 53 %.
+// N = 1M, 10.3e9 pairs: 8.3 ms, 30 TFLOP/s at 24 a pair, 38 % of the measured FP32 peak.  The sources are packed, not
 // the targets: target coordinates are duplicated once per chunk, a packed source is one load.
 // One CTA of 4 warps per leaf: groups of 64 targets (two per lane), and the chunks of the near leaves
 // split over the warps a group has; a last group of at most 32, 16, ... targets gives each pair of targets 2, 4,

@@ -37,7 +37,11 @@ struct P2MJob {
   double lam[2 * MAXLAYER];                  // per type
   void *M;
 };
-constexpr int P2M_SPARSE = 6;  // mean points per segment below which a lane takes a segment
+// Mean points per segment below which a lane takes a segment; us by warps / by lanes: FP32 (N = 100,000) 8.9 points a segment
+// 179 / 406, 6.5: 316 / 507, 1.8: 810 / 452; FP64 (N = 20,000, p = 10; 3,000, p = 12) 13.1: 662 / 947, 11.7: 268 / 1,028, 2.3: 3,480 / 579,
+// 2.0: 1,349 / 334.  L2P takes the same line for points per leaf, although a lane per target was the faster form at
+// every occupancy measured there (FP32, N = 100,000, 65 points a leaf 48 / 24, 1.8: 203 / 34; FP64, N = 20,000, 104: 538 / 109).
+constexpr int P2M_SPARSE = 6;
 
 template <typename T>
 __device__ __forceinline__ T halve(T a, T b, bool hi, int o) {  // hi lanes keep b, the others a; the rest is exchanged
@@ -193,12 +197,15 @@ __global__ void __launch_bounds__(128) k_p2m_sparse(const P2MJob *jobs, int nj, 
 // N = 200,000 (p = 8, 24,576 sparse parents) M2M 2.28 -> 1.28 ms an evaluation, L2L 0.57 -> 0.28.
 // ---------------------------------------------------------------------------------------
 constexpr int OCT_SPLIT = 2;
-// parents of a level up to which each source type takes a CTA of its own; beyond it the set-up that every CTA
-// repeats costs more than the types in turn (868 parents p = 10 FP64: 231 us in turn, 199 apart)
+// parents of a level up to which each source type takes a CTA of its own; far beyond it the set-up that every CTA
+// repeats costs more than the types in turn.  us in turn / apart: FP32 448 parents (p = 10) 57 / 28, 3,584: 158 / 147, 5,120 (p = 8)
+// 222 / 200, 26,649 (p = 10) 755 / 827, 40,177 (p = 8) 935 / 1,119; FP64 448 (p = 10) 224 / 161, 3,574: 1,132 / 961, 4,596 (p = 12)
+// 921 / 876.  The two meet between 5,000 and 27,000 parents; the line is on the low side of that.
 constexpr int M2M_TSPLIT_MAX = 2048;
 // CTAs of a level up to which a CTA takes one group of threads per z-half and column part (latency counts);
-// beyond it one group does all, so that a half without children idles no threads and more parents are in flight
-// (24,576 sparse parents p = 8: 2.08 ms with the groups, 1.01 with one; 56 parents FP32: 13 us with, 16 - 25 without)
+// beyond it one group does all, so that a half without children idles no threads and more parents are in flight.  us with the
+// groups / with one: FP32 (p = 10) 152 CTAs 16 / 29, 384 (L2L, p = 8) 25 / 31, 1,216: 48 / 28, 26,649: 1,424 / 755; FP64 (p = 10) 152 CTAs
+// 32 / 82, 384 (L2L, p = 12) 111 / 114, 1,216: 164 / 160, 3,574: 1,053 / 1,110, 4,596 (p = 12) 1,343 / 942.
 constexpr int OCT_WIDE = 512;
 static __host__ __device__ __forceinline__ int oct_rows(int K, int p) { return (2 * K - (p + 1) + 31) / 32 * 32; }
 static int oct_threads(int K, int p, int64_t ctas) {
