@@ -302,6 +302,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TJob *jobs, int 
   constexpr int NC = tc_chunks(P), N = 32 * NC, NST = TC_NST, K = (P + 1) * (P + 2) / 2;
   constexpr int TCOLS = 2 * N <= 32 ? 32 : (2 * N <= 64 ? 64 : (2 * N <= 128 ? 128 : 256));
   static_assert(2 * N <= 256, "two accumulators of N columns");
+  static_assert(NC <= NST, "a step's chunks stay staged until its last products");
   constexpr uint32_t SA = TC_ROWS * 128, SB = N * 128;  // bytes of one A / W chunk tile
   extern __shared__ __align__(16) unsigned char tcsm[];  // base rounded up to 1024 below
   unsigned char *sbase = (unsigned char *)(((uintptr_t)tcsm + 1023) & ~(uintptr_t)1023);
@@ -318,8 +319,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TJob *jobs, int 
   // slowest warp, whose fold is one step behind (7 steps at one chunk per step)
   __shared__ float scl[TC_SCL][TC_ROWS];
   // full[b]: the worker warps have staged buffer b; wfull[b]: its operator chunk has landed; empty[b]: its
-  // MMAs are done; accbar[a]: a step's MMAs into accumulator a are done; foldbar[a]: the workers have read it
-  __shared__ uint64_t full[NST], empty[NST], accbar[2], foldbar[2], wfull[NST];
+  // MMAs are done; accbar[a]: a step's MMAs into accumulator a are done; foldbar[a]: the workers have read it; done: every MMA
+  __shared__ uint64_t full[NST], empty[NST], accbar[2], foldbar[2], wfull[NST], done;
   __shared__ uint32_t tbase;
   int lo = 0, hi = njobs - 1;
   while (lo < hi) {
@@ -448,6 +449,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TJob *jobs, int 
       tc::mbar_init(&accbar[a], 1);
       tc::mbar_init(&foldbar[a], TC_WORKERS / 32);
     }
+    tc::mbar_init(&done, 1);
     tc::mbar_fence_init();
   }
   tc::fence_before();
@@ -594,7 +596,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TJob *jobs, int 
     // the MMA thread: a step's cross products (hi lo, lo hi) of every chunk as it is filled, by the workers and the bulk
     // copy, then its hi hi ones; a step starts once the workers have read the accumulator two steps back
     constexpr uint32_t IDESC = tc::idesc_f16(TC_ROWS, N);
-    int last = -1;
     for (int si = 0; si < ns && !fail; ++si) {
       if (si >= 2 && !tc::mbar_wait(&foldbar[si & 1], (uint32_t)(((si - 2) >> 1) & 1), TC_WAIT)) {
         fail = true;
@@ -624,12 +625,13 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_m2l_tc(const TJob *jobs, int 
 #pragma unroll
         for (int kk = 0; kk < 2; ++kk) tc::mma_f16(dacc, tc::sdesc(ah + kk * 32), tc::sdesc(wh + kk * 32), IDESC, 1u);
         tc::commit(&empty[b]);
-        last = sc;
       }
       tc::commit(&accbar[si & 1]);
     }
-    // every MMA has completed once the last committed stage's barrier phase completes
-    if (last >= 0) tc::mbar_wait(&empty[last % NST], (uint32_t)((last / NST) & 1), TC_WAIT);
+    // no MMA may be in flight when the tensor memory is freed, also those of a step that a timeout cut short, whose chunks
+    // no other barrier covers
+    tc::commit(&done);
+    if (!tc::mbar_wait(&done, 0u, TC_WAIT)) fail = true;
   } else if (tid == TC_WORKERS + 32) {
     // the operator chunks, one bulk copy per stage
     int issued = 0;
