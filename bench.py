@@ -365,7 +365,7 @@ def run_ours(args, rank, world, local_rank):
     e2e_ms = max_over_ranks(e0.elapsed_time(e1), dist, dev)
     e2e_val = job_throughput(world, n, e2e_steps, e2e_ms)
 
-    # accuracy gate and the FP64 comparator (same tree rule, same inputs), untimed by the driver's clock
+    # accuracy gate and the FP64 comparator (same tree rule, same inputs), outside the timed region
     accuracy, fp64_value = None, None
     if not args.no_fp64:
         ctx64 = F.Context(m["d"], m["eps"], m["lam"], args.p, precision=F.FP64, stream=stream, **settings)
